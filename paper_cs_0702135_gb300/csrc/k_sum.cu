@@ -24,7 +24,8 @@
 //    result depends on neither the order of j, nor the j slices, nor which
 //    CTA computes what.  (The rounding avoids float-to-int64 conversions, which
 //    run on the FP64 pipe: three exact FP32 splits do it on the FP32 pipe.)
-//  NB_SUM_FP32  one thread per i, an FP32 running sum over j = 0, 1, ... .
+//  NB_SUM_FP32  per i an FP32 running sum over j = 0, 1, ... ; the terms are
+//    evaluated in parallel, only the additions are in order.
 //  NB_SUM_FP32_SORTED  one CTA per i: the pair-force magnitudes |mj dx/r^3|
 //    as keys, a stable radix sort of (key, j), then the FP32 running sum in
 //    increasing key (ties in increasing j).
@@ -203,50 +204,160 @@ __global__ void k_fixed_combine(ForceArgs fa, SumArgs sa)
 }
 
 // ---------------------------------------------------------------------------
-// FP32 running sum in index order: one thread per i over all j, in order.
+// FP32 running sum in index order.  The order fixes one chain of additions per
+// output (4 cycles a term), but nothing fixes who evaluates the terms: a CTA
+// owns I active particles; 16 warps evaluate the seven terms of a tile of T
+// sources, lane per source, into shared memory while 4 warps (one per
+// scheduler) add the tile before it in index order, one lane per (particle,
+// component).  Two tiles alternate with one barrier a tile.  A pair left out
+// (j = i, r2 = 0) and the padding past n enter as -0, which changes no sum.
+//
+// Bounds: with many particles the term evaluation's issue slots (two
+// particles share every packed operation), with few the chain of additions.
+// I spreads the block evenly over the resident CTAs, one per SM; T grows as I
+// shrinks (the buffers keep their size) so that the barrier stays a small part
+// of the tile's chain.  1820 active on 65536 bodies: 458 us; one thread per i
+// evaluating and adding its own terms kept 15 SMs busy and took 9.54 ms.  Of
+// the steps between, all with the same bits: tiles of 128 sources 627 us,
+// larger tiles and the next records loaded ahead 583 us, packed pairs and the
+// short 1/sqrt 502 us, tile lengths as compile-time constants 458 us.
 
-template <int NT>
-__global__ void __launch_bounds__(NT) k_force_seq(ForceArgs fa, JDS J)
+constexpr int kSeqI = 15;             // active particles per CTA at most
+constexpr int kSeqTermWarps = 16;     // warps that evaluate terms
+constexpr int kSeqSumWarps = kSeqNT / 32 - kSeqTermWarps;
+static_assert(kSeqSumWarps * 32 >= kSeqI * kComp, "one summing lane per (particle, component)");
+
+// Particles per CTA and sources per tile for a block of na on `slots` CTAs:
+// the fewest rounds of at most kSeqI particles, split evenly.
+__host__ __device__ inline void seq_shape(int na, int slots, int &I, int &T)
+{
+    const int rounds = cdiv(na, (long long)slots * kSeqI);
+    I = cdiv(na, (long long)slots * rounds);
+    T = I > 7 ? 256 : (I > 3 ? 512 : 1024);
+}
+
+// Rows of T terms are T + 4 floats apart: the summing lanes' 16-byte reads of
+// eight rows then fall into different banks.
+__host__ __device__ constexpr int seq_row(int T) { return T + 4; }
+constexpr int kSeqBufFloats = kSeqI * kComp * seq_row(256);   // the largest of the shapes
+static_assert(7 * seq_row(512) <= kSeqI * seq_row(256) && 3 * seq_row(1024) <= kSeqI * seq_row(256),
+              "every shape fits the buffers");
+constexpr int kSeqSmem = 2 * kSeqBufFloats * (int)sizeof(float);
+
+template <int T>
+__device__ __forceinline__ void seq_groups(const ForceArgs &fa, const JDS &J, int na, int I)
+{
+    extern __shared__ float4 s_dyn[];
+    float *const buf = reinterpret_cast<float *>(s_dyn);
+    __shared__ float2 s_i[(kSeqI + 1) / 2][10];   // two particles' records, negated, component by component
+    __shared__ int s_ii[kSeqI + 1];
+    __shared__ float s_sum[kSeqI * kComp];
+    constexpr int row = seq_row(T), nsub = T / 32;
+    const float eps2 = (float)fa.eps2;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n = fa.n;
+    const int ntile = cdiv(n, T), ngrp = cdiv(na, I);
+    // term warp w takes sub-tiles w mod nsub, + 16, ... and, with fewer
+    // sub-tiles than warps, every qstep-th pair of particles
+    const int qstep = nsub < kSeqTermWarps ? kSeqTermWarps / nsub : 1;
+    const int sub0 = nsub < kSeqTermWarps ? warp % nsub : warp, q0 = nsub < kSeqTermWarps ? warp / nsub : 0;
+    const int jlane = sub0 * 32 + lane;   // this lane's first source within a tile
+    for (int grp = blockIdx.x; grp < ngrp; grp += gridDim.x) {
+        const int a0 = grp * I, cnt = min(I, na - a0), npair = (cnt + 1) / 2;
+        __syncthreads();
+        if (tid < 2 * npair) {   // an odd count repeats the last particle, unstored
+            const int i = clamp_index(fa.act[a0 + min(tid, cnt - 1)], n);
+            const float4 p = J.pos_hi[i], l = J.pos_lo[i], v = J.vel[i];
+            const float c[9] = {p.x, p.y, p.z, l.x, l.y, l.z, v.x, v.y, v.z};
+            float *const d = reinterpret_cast<float *>(s_i[tid >> 1]) + (tid & 1);
+#pragma unroll
+            for (int e = 0; e < 9; ++e) d[2 * e] = -c[e];
+            s_ii[tid] = i;
+        }
+        __syncthreads();
+        const int chain = tid - kSeqTermWarps * 32;   // summing lanes: particle * 7 + component
+        float sum = 0.0f;
+        // a term warp's next source records are loaded while it works on the
+        // present ones (the index of padding lanes is clamped)
+        float4 np, nl, nv;
+        if (warp < kSeqTermWarps) {
+            const int jc = min(jlane, n - 1);
+            np = J.pos_hi[jc], nl = J.pos_lo[jc], nv = J.vel[jc];
+        }
+        for (int k = 0; k <= ntile; ++k) {
+            if (warp < kSeqTermWarps) {
+                if (k < ntile) {
+                    float *const dst = buf + (k & 1) * kSeqBufFloats;
+                    for (int sub = sub0; sub < nsub; sub += kSeqTermWarps) {
+                        const int jj = sub * 32 + lane, j = k * T + jj;
+                        Side2 Js;
+                        Js.h[0] = f2(np.x), Js.h[1] = f2(np.y), Js.h[2] = f2(np.z);
+                        Js.l[0] = f2(nl.x), Js.l[1] = f2(nl.y), Js.l[2] = f2(nl.z);
+                        Js.v[0] = f2(nv.x), Js.v[1] = f2(nv.y), Js.v[2] = f2(nv.z);
+                        Js.m = f2(np.w);
+                        const int jn = min(sub + kSeqTermWarps < nsub ? j + kSeqTermWarps * 32
+                                                                      : (k + 1) * T + jlane, n - 1);
+                        np = J.pos_hi[jn], nl = J.pos_lo[jn], nv = J.vel[jn];
+                        const int j0 = j - lane;
+                        const bool edge = j0 + 32 > n || !(eps2 > 0.0f);
+                        for (int q = q0; q < npair; q += qstep) {
+                            Side2 N;
+#pragma unroll
+                            for (int c = 0; c < 3; ++c)
+                                N.h[c] = s_i[q][c], N.l[c] = s_i[q][3 + c], N.v[c] = s_i[q][6 + c];
+                            float2 t[7];
+                            const float2 r2 = pair_rn2<true>(Js, N, eps2, 1.0f, 1.0f, 1.0f, t);
+                            const int ia = s_ii[2 * q], ib = s_ii[2 * q + 1];
+                            // pairs to leave out can only be here (uniform in the warp)
+                            if ((unsigned)(ia - j0) < 32u || (unsigned)(ib - j0) < 32u || edge) {
+                                const bool oa = j < n && j != ia && r2.x != 0.0f;
+                                const bool ob = j < n && j != ib && r2.y != 0.0f;
+#pragma unroll
+                                for (int c = 0; c < 7; ++c)
+                                    t[c] = make_float2(oa ? t[c].x : -0.0f, ob ? t[c].y : -0.0f);
+                            }
+                            float *const d = dst + 2 * q * kComp * row + jj;
+#pragma unroll
+                            for (int c = 0; c < 7; ++c) d[c * row] = t[c].x;
+                            if (2 * q + 1 < cnt)
+#pragma unroll
+                                for (int c = 0; c < 7; ++c) d[(kComp + c) * row] = t[c].y;
+                        }
+                    }
+                }
+            } else if (k > 0 && chain < cnt * kComp) {
+                const float4 *src = reinterpret_cast<const float4 *>(buf + ((k - 1) & 1) * kSeqBufFloats +
+                                                                     chain * row);
+#pragma unroll 8
+                for (int q = 0; q < T / 4; ++q) {
+                    const float4 t = src[q];
+                    sum = __fadd_rn(sum, t.x);
+                    sum = __fadd_rn(sum, t.y);
+                    sum = __fadd_rn(sum, t.z);
+                    sum = __fadd_rn(sum, t.w);
+                }
+            }
+            __syncthreads();
+        }
+        if (chain >= 0 && chain < cnt * kComp) s_sum[chain] = sum;
+        __syncthreads();
+        if (tid < cnt) {
+            double res[kComp];
+#pragma unroll
+            for (int c = 0; c < kComp; ++c) res[c] = (double)s_sum[tid * kComp + c];
+            store_result(fa.out, a0 + tid, res);
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kSeqNT, 1) k_force_seq(ForceArgs fa, JDS J, int slots)
 {
     const int na = read_na(fa);
     if (na <= 0) return;
-    __shared__ float4 s_p[NT], s_l[NT], s_v[NT];
-    const float eps2 = (float)fa.eps2;
-    const int tid = threadIdx.x, n = fa.n;
-    const int nblk = cdiv(na, NT);
-    for (int ib = blockIdx.x; ib < nblk; ib += gridDim.x) {
-        const int a = ib * NT + tid;
-        const int i = clamp_index(fa.act[a < na ? a : 0], n);
-        float xh[3], xl[3], vi[3];
-        load_i(J, i, xh, xl, vi);
-        float sum[7] = {0, 0, 0, 0, 0, 0, 0};
-        for (int jt = 0; jt < n; jt += NT) {
-            __syncthreads();
-            const int j = jt + tid;
-            if (j < n) {
-                s_p[tid] = J.pos_hi[j];
-                s_l[tid] = J.pos_lo[j];
-                s_v[tid] = J.vel[j];
-            }
-            __syncthreads();
-            const int jc = min(NT, n - jt);
-            for (int jj = 0; jj < jc; ++jj) {
-                float t[7];
-                const bool ok = pair_rn(s_p[jj], s_l[jj], s_v[jj], xh, xl, vi, eps2, 1.0f, 1.0f,
-                                        1.0f, t);
-                if (ok && jt + jj != i) {
-#pragma unroll
-                    for (int q = 0; q < 7; ++q) sum[q] = __fadd_rn(sum[q], t[q]);
-                }
-            }
-        }
-        if (a < na) {
-            double res[kComp];
-#pragma unroll
-            for (int q = 0; q < 7; ++q) res[q] = (double)sum[q];
-            store_result(fa.out, a, res);
-        }
-    }
+    int I, T;
+    seq_shape(na, slots, I, T);
+    if (T == 256) seq_groups<256>(fa, J, na, I);
+    else if (T == 512) seq_groups<512>(fa, J, na, I);
+    else seq_groups<1024>(fa, J, na, I);
 }
 
 // ---------------------------------------------------------------------------
@@ -399,7 +510,11 @@ int occupancy_sum(int mode, int *blocks_per_sm)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_force_fixed<kFixNT, kFixR>,
                                                           kFixNT, 0);
     else if (mode == NB_SUM_FP32)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_force_seq<kSeqNT>, kSeqNT, 0);
+    {
+        e = cudaFuncSetAttribute(k_force_seq, cudaFuncAttributeMaxDynamicSharedMemorySize, kSeqSmem);
+        if (e == cudaSuccess)
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_force_seq, kSeqNT, kSeqSmem);
+    }
     else
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_force_sorted, kSortNT, 0);
     return e == cudaSuccess ? 0 : -1;
@@ -413,9 +528,11 @@ int grid_summed(const ForceArgs &fa, const SumArgs &sa)
     long long items;
     if (sa.mode == NB_SUM_FIXED)
         items = fa.plan.p.items;
-    else if (sa.mode == NB_SUM_FP32)
-        items = cdiv(na, kSeqNT);
-    else
+    else if (sa.mode == NB_SUM_FP32) {
+        int I, T;
+        seq_shape(na, sa.slots, I, T);
+        items = cdiv(na, I);
+    } else
         items = na;
     return (int)(items < sa.slots ? items : sa.slots);
 }
@@ -435,7 +552,7 @@ int launch_force_summed(const ForceArgs &fa, const JDS &j, const SumArgs &sa, in
         return 3;
     }
     if (sa.mode == NB_SUM_FP32) {
-        k_force_seq<kSeqNT><<<grid, kSeqNT, 0, st>>>(fa, j);
+        k_force_seq<<<grid, kSeqNT, kSeqSmem, st>>>(fa, j, sa.slots);
         return 1;
     }
     k_force_sorted<<<grid, kSortNT, 0, st>>>(fa, j, sa);

@@ -546,6 +546,97 @@ __device__ __forceinline__ bool pair_rn(const float4 &p, const float4 &l, const 
     return r2 != 0.0f;
 }
 
+// Two-lane arithmetic for two pairs at once.  The assembler contracts a packed
+// product that feeds a packed sum into one multiply-add even where both carry
+// .rn (seen with the intrinsics and with add.rn/mul.rn.f32x2 in PTX), so such
+// a product (mul2s) is a packed multiply-add of -0, which rounds the product
+// itself and cannot be contracted; the -0 comes from constant memory, where
+// it is not known at compile time.
+static __constant__ float2 c_neg_zero2 = {-0.0f, -0.0f};
+
+__device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 mul2s(float2 a, float2 b) { return __ffma2_rn(a, b, c_neg_zero2); }
+
+// True where inv_sqrt_fast2 below does not give RN(1 / RN(sqrt(x))): x outside
+// [2^-87, 2^126], or within 6 ulps below a power of four (a square root whose
+// significand is all ones is the exception of Markstein's theorem).
+__device__ __forceinline__ bool inv_sqrt_hard(float x)
+{
+    const unsigned b = __float_as_uint(x);
+    return b - 0x14000000u > 0x6A800000u || ((b + 0x800006u) & 0xffffffu) < 6u;
+}
+
+// RN(1 / RN(sqrt(x))) for two x that are not inv_sqrt_hard, from the SFU's
+// approximate y ~ 1/sqrt(x) (relative error about 2^-22.9) by the final steps
+// of Markstein (IBM J. Res. Dev. 34, 1990): with s0 = x y and the exact
+// residual x - s0^2, s = RN(s0 + (x - s0^2) y/2) is the rounded square root;
+// y1 = RN(y + (1 - s y) y) is within an ulp of its reciprocal and, with the
+// exact residual 1 - s y1, RN(y1 + (1 - s y1) y1) is the rounded reciprocal.
+// Compared on the GB300 with __frcp_rn(__fsqrt_rn(x)) for every
+// single-precision x: the same bits wherever inv_sqrt_hard is false.  The
+// intrinsics cost about twice the instructions (a second SFU operation and a
+// range test with a branch each), and two x share every operation here.
+__device__ __forceinline__ float2 inv_sqrt_fast2(float2 x)
+{
+    const float2 y = make_float2(rsqrt_sfu(x.x), rsqrt_sfu(x.y));
+    const float2 s0 = mul2(x, y);
+    const float2 s = fma2(fma2(neg2(s0), s0, x), mul2(y, f2(0.5f)), s0);
+    const float2 y1 = fma2(fma2(neg2(s), y, f2(1.0f)), y, y);
+    return fma2(fma2(neg2(s), y1, f2(1.0f)), y1, y1);
+}
+
+__device__ __forceinline__ float2 inv_sqrt_rn2(float2 x)
+{
+    float2 r = inv_sqrt_fast2(x);
+    if (inv_sqrt_hard(x.x) || inv_sqrt_hard(x.y)) {
+        r.x = __frcp_rn(__fsqrt_rn(x.x));
+        r.y = __frcp_rn(__fsqrt_rn(x.y));
+    }
+    return r;
+}
+
+// One side of two pairs: hi and lo position words, velocity (of the i side
+// negated), mass.
+struct Side2 {
+    float2 h[3], l[3], v[3], m;
+};
+
+// pair_rn on two pairs: j of each lane (J), i of each lane negated (N).  Every
+// operation is pair_rn's, in its order, rounded per lane, so the bits are the
+// same.  UNIT: the scale factors are 1 and their multiplications are left out
+// (exact).  Returns r2 (a lane with r2 = 0 holds no numbers in t).
+template <bool UNIT>
+__device__ __forceinline__ float2 pair_rn2(const Side2 &J, const Side2 &N, float eps2, float sa, float sk,
+                                           float sp, float2 t[7])
+{
+    float2 dx[3], u[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        dx[c] = add2(add2(J.h[c], N.h[c]), add2(J.l[c], N.l[c]));
+        u[c] = add2(J.v[c], N.v[c]);
+    }
+    const float2 d2 = add2(add2(mul2s(dx[0], dx[0]), mul2s(dx[1], dx[1])), mul2s(dx[2], dx[2]));
+    const float2 r2 = add2(d2, f2(eps2));
+    const float2 rv = add2(add2(mul2s(dx[0], u[0]), mul2s(dx[1], u[1])), mul2s(dx[2], u[2]));
+    const float2 rinv = inv_sqrt_rn2(r2);
+    const float2 rinv2 = mul2(rinv, rinv);
+    const float2 mr = mul2(J.m, rinv);
+    const float2 mr3 = mul2(mr, rinv2);
+    const float2 b = mul2(mul2(f2(-3.0f), rv), rinv2);
+    const float2 fa = UNIT ? mr3 : mul2(mr3, f2(sa)), fk = UNIT ? mr3 : mul2(mr3, f2(sk));
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        t[c] = mul2(fa, dx[c]);
+        t[3 + c] = mul2(fk, add2(u[c], mul2s(b, dx[c])));
+    }
+    t[6] = neg2(UNIT ? mr : mul2(mr, f2(sp)));
+    return r2;
+}
+
 __device__ __forceinline__ void load_i(const JDS &J, int i, float xh[3], float xl[3], float vi[3])
 {
     const float4 p = J.pos_hi[i], l = J.pos_lo[i], v = J.vel[i];

@@ -354,7 +354,7 @@ struct SumArgs {
 constexpr int kFixNT = NB_FIX_NT;   // fixed point: threads per CTA (= j per tile)
 constexpr int kFixR = NB_FIX_R;     // fixed point: i per thread
 constexpr int kFixUnroll = NB_FIX_UNROLL;  // fixed point: j unrolling of the inner loop
-constexpr int kSeqNT = 128;         // FP32 index order: threads per CTA, one i each
+constexpr int kSeqNT = 640;         // FP32 index order: threads per CTA
 constexpr int kSortNT = 1024;       // FP32 sorted: one CTA per i
 constexpr int kErrFixedScale = 64;  // device error word: fixed-point scales out of range
 constexpr int kErrInput = 65;       // device error word: a non-finite value or a negative mass

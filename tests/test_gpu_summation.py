@@ -191,3 +191,72 @@ def test_million_body_sampled_bit_exact(nb, mode):
     got = _gpu_force(nb, m, x, v, eps, idx, MODES[mode][0], no_force=True)
     ref = oracle.force_summed(m, x, v, eps, idx, mode=MODES[mode][1], nthreads=oracle.max_threads())
     _assert_same(got, ref, "%s n=2^20" % mode)
+
+
+@pytest.mark.parametrize("na", [300, 456, 600, 1216, 1217, 2432, 2433])
+def test_fp32_particles_per_cta_bit_exact(nb, na):
+    # on 152 SMs: 2, 3, 4, 8, 9 and 16 particles per CTA (every tile length),
+    # then two rounds; 2500 bodies end inside a tile of each length.  The sums
+    # have a fixed order, so the tolerance is zero.
+    n = 2500
+    m, x, v = plummer(n, 31)
+    idx = sample_active(n, na, 5 + na)
+    got = _gpu_force(nb, m, x, v, EPS, idx, nb.NB_SUM_FP32)
+    ref = oracle.force_summed(m, x, v, EPS, idx, mode=oracle.SUM_FP32, nthreads=8)
+    _assert_same(got, ref, "fp32 na=%d" % na)
+
+
+@pytest.mark.parametrize("mode", ["fp32", "sorted"])
+def test_block_size_read_on_the_device(nb, mode):
+    # a device-driven block step equals predict, force and correct from the host
+    m, x, v = plummer(700, 37)
+    a = nb.Context(m, x, v, EPS, summation=MODES[mode][0])
+    b = nb.Context(m, x, v, EPS, summation=MODES[mode][0])
+    try:
+        for _ in range(3):
+            t, na = a.nb_step()
+            idx, _ = a.nb_get_active()
+            assert len(idx) == na
+            b.nb_predict(t)
+            b.nb_force(idx)
+            b.nb_correct(idx, t)
+            sa, sb = a.nb_get_state(), b.nb_get_state()
+            for key in sa:
+                assert np.array_equal(sa[key], sb[key]), key
+    finally:
+        a.nb_free()
+        b.nb_free()
+
+
+@pytest.mark.parametrize("mode", sorted(MODES))
+@pytest.mark.parametrize("case", ["below_a_power_of_four", "tiny", "tiny_light", "huge"])
+def test_square_root_exceptions_bit_exact(nb, mode, case):
+    # r^2 where the short 1/sqrt gives way to the intrinsics: single-precision
+    # values just below a power of four, below 2^-87 and above 2^126
+    if (mode, case) == ("fixed", "tiny"):
+        pytest.skip("m / r^3 is above the single-precision range: no fixed-point term")
+    n = 400
+    rng = np.random.RandomState(3)
+    m = np.full(n, 1.0 / n)
+    v = rng.normal(size=(n, 3))
+    if case == "below_a_power_of_four":
+        eps = 0.5   # r^2 = x^2 + 1/4 around 1, from consecutive single-precision x
+        x = np.zeros((n, 3))
+        d = np.float32(np.sqrt(0.75)).view(np.int32) + np.arange(-200, 199)
+        x[1:, 0] = d.astype(np.int32).view(np.float32)
+        r2 = (x[1:, 0].astype(np.float32) ** 2 + np.float32(0.25)).astype(np.float32).view(np.uint32)
+        assert np.any((r2 & 0xffffff) - 0x7ffffa < 6)
+        idx = np.array([0], dtype=np.int32)
+    elif case in ("tiny", "tiny_light"):
+        eps = 1e-14
+        if case == "tiny_light":
+            m = np.full(n, 1e-9)
+        x = rng.normal(size=(n, 3)) * 1e-14
+        idx = np.arange(n, dtype=np.int32)
+    else:
+        eps = 1.0 / 256
+        x = rng.normal(size=(n, 3)) * 7e18
+        idx = np.arange(n, dtype=np.int32)
+    got = _gpu_force(nb, m, x, v, eps, idx, MODES[mode][0], no_force=True)
+    ref = oracle.force_summed(m, x, v, eps, idx, mode=MODES[mode][1], nthreads=8)
+    _assert_same(got, ref, "%s %s" % (mode, case))
