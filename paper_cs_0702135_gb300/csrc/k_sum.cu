@@ -30,6 +30,7 @@
 //    as keys, a stable radix sort of (key, j), then the FP32 running sum in
 //    increasing key (ties in increasing j).
 #include <cfloat>
+#include <type_traits>
 
 #include "nb_device.cuh"
 
@@ -60,25 +61,33 @@ __global__ void k_fixed_bounds(JDS J, int n, unsigned *bounds)
     }
 }
 
-// One pair into the tile's split sums; the pair j = i adds zeros, so every
-// tile adds exactly NT terms.
+// Two pairs (j, j + 1) into the tile's split sums; the pair j = i adds zeros,
+// so every tile adds all its terms.
 template <bool GUARD>
-__device__ __forceinline__ void pair_fixed(const float4 &p, const float4 &l, const float4 &w,
-                                           const float xh[3], const float xl[3], const float vi[3],
-                                           float eps2, const Scale &S, unsigned a[3][7], int j = 0,
-                                           int i = 1)
+__device__ __forceinline__ void pair_fixed2(const Side2 &Js, const Side2 &N, float eps2, const Scale &S,
+                                            unsigned a[3][7], int j = 0, int i = 1)
 {
-    float t[7];
-    pair_rn(p, l, w, xh, xl, vi, eps2, S.sc[0], S.sc[1], S.sc[2], t);
+    float2 t[7];
+    pair_rn2<false>(Js, N, eps2, S.sc[0], S.sc[1], S.sc[2], t);
 #pragma unroll
-    for (int q = 0; q < 7; ++q) split_add(GUARD && j == i ? 0.0f : t[q], a[0][q], a[1][q], a[2][q]);
+    for (int q = 0; q < 7; ++q) {
+        if (GUARD) t[q] = make_float2(j == i ? 0.0f : t[q].x, j + 1 == i ? 0.0f : t[q].y);
+        split_add2(t[q], a[0][q], a[1][q], a[2][q]);
+    }
 }
 
-// i-parallel like the DS kernel: a CTA owns R * NT active i and one j slice,
-// tiles of NT j in shared memory; 64-bit tile sums, 128-bit totals; with
-// several slices the totals go to the partial buffer as (hi, lo) pairs.
-template <int NT, int R>
-__global__ void __launch_bounds__(NT) k_force_fixed(ForceArgs fa, JDS J, SumArgs sa)
+// i-parallel like the DS kernel: a CTA owns NT active i, one per thread, and
+// one j slice, tiles of TL j in shared memory; 64-bit tile sums, 128-bit
+// totals; with several slices the totals go to the partial buffer as (hi, lo)
+// pairs.  The j side lies in shared memory component by component, so that
+// one 16-byte read gives a component of four j, two packed operands: every
+// single-precision operation of the terms and of their splitting then serves
+// two pairs.  Bound by the FMA pipe (about 103 operations a pair, of which 49
+// split the terms); the scalar form was bound by issue at 132 instructions a
+// pair.  65536 bodies all active: 17.4 ms -> 14.6 ms packed, 13.5 ms with one
+// CTA per work item (grid_summed), 13.2 ms with more slices and ten CTAs a SM.
+template <int NT>
+__global__ void __launch_bounds__(NT, kFixCtas) k_force_fixed(ForceArgs fa, JDS J, SumArgs sa)
 {
     const ForcePlan F = load_plan(fa);
     const int na = F.na;
@@ -91,7 +100,9 @@ __global__ void __launch_bounds__(NT) k_force_fixed(ForceArgs fa, JDS J, SumArgs
     }
     const Plan P = F.p;
     long long *part = reinterpret_cast<long long *>(fa.part);
-    __shared__ float4 s_p[NT], s_l[NT], s_v[NT];
+    constexpr int TL = 2 * NT;   // j per shared-memory tile; TL 2^22 stays below 2^31 (split_add)
+    __shared__ float4 s_j[10][TL / 4];
+    float *const sj = reinterpret_cast<float *>(s_j);
     const int tid = threadIdx.x;
 
     for (int w = blockIdx.x; w < P.items; w += gridDim.x) {
@@ -100,76 +111,78 @@ __global__ void __launch_bounds__(NT) k_force_fixed(ForceArgs fa, JDS J, SumArgs
         const int j0 = sl * P.jslice;
         const int j1 = min(fa.n, j0 + P.jslice);
 
-        float xh[R][3], xl[R][3], vi[R][3];
-        int ia[R], ii[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int a = ib * NT * R + r * NT + tid;
-            ia[r] = a < na ? a : -1;
-            ii[r] = clamp_index(fa.act[a < na ? a : 0], fa.n);
-            load_i(J, ii[r], xh[r], xl[r], vi[r]);
+        const int a = ib * NT + tid;
+        const int ia = a < na ? a : -1;
+        const int ii = clamp_index(fa.act[a < na ? a : 0], fa.n);
+        Side2 N;
+        {
+            const float4 p = J.pos_hi[ii], l = J.pos_lo[ii], v = J.vel[ii];
+            N.h[0] = f2(-p.x), N.h[1] = f2(-p.y), N.h[2] = f2(-p.z);
+            N.l[0] = f2(-l.x), N.l[1] = f2(-l.y), N.l[2] = f2(-l.z);
+            N.v[0] = f2(-v.x), N.v[1] = f2(-v.y), N.v[2] = f2(-v.z);
         }
-        long long hi[R][7];
-        unsigned long long lo[R][7];
+        long long hi[7];
+        unsigned long long lo[7];
 #pragma unroll
-        for (int r = 0; r < R; ++r)
-#pragma unroll
-            for (int q = 0; q < 7; ++q) hi[r][q] = 0, lo[r][q] = 0;
+        for (int q = 0; q < 7; ++q) hi[q] = 0, lo[q] = 0;
 
-        for (int jt = j0; jt < j1; jt += NT) {
+        for (int jt = j0; jt < j1; jt += TL) {
             __syncthreads();
-            const int j = jt + tid;
-            const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);  // mass 0: contributes 0
-            s_p[tid] = j < j1 ? J.pos_hi[j] : z;
-            s_l[tid] = j < j1 ? J.pos_lo[j] : z;
-            s_v[tid] = j < j1 ? J.vel[j] : z;
+#pragma unroll
+            for (int u = 0; u < TL / NT; ++u) {
+                const int t = tid + u * NT, j = jt + t;
+                const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);  // mass 0: contributes 0
+                const float4 p = j < j1 ? J.pos_hi[j] : z, l = j < j1 ? J.pos_lo[j] : z,
+                             v = j < j1 ? J.vel[j] : z;
+                const float c[10] = {p.x, p.y, p.z, l.x, l.y, l.z, v.x, v.y, v.z, p.w};
+#pragma unroll
+                for (int e = 0; e < 10; ++e) sj[e * TL + t] = c[e];
+            }
             __syncthreads();
-            unsigned ch[R][3][7];
+            const int jc = (min(TL, j1 - jt) + 3) & ~3;   // whole reads of four; the padding adds zeros
+            unsigned ch[3][7];
 #pragma unroll
-            for (int r = 0; r < R; ++r)
+            for (int q = 0; q < 7; ++q) ch[0][q] = ch[1][q] = ch[2][q] = 0u;
+            auto four = [&](int jj, auto guard) {
+                float4 c[10];
 #pragma unroll
-                for (int q = 0; q < 7; ++q) ch[r][0][q] = ch[r][1][q] = ch[r][2][q] = 0u;
-            bool mine = false;
+                for (int e = 0; e < 10; ++e) c[e] = s_j[e][jj / 4];
 #pragma unroll
-            for (int r = 0; r < R; ++r) mine |= (unsigned)(ii[r] - jt) < (unsigned)NT;
-            if (__any_sync(kFull, mine)) {
-                for (int jj = 0; jj < NT; ++jj)
+                for (int h = 0; h < 2; ++h) {
+                    Side2 Js;
 #pragma unroll
-                    for (int r = 0; r < R; ++r)
-                        pair_fixed<true>(s_p[jj], s_l[jj], s_v[jj], xh[r], xl[r], vi[r], eps2, S,
-                                         ch[r], jt + jj, ii[r]);
+                    for (int e = 0; e < 3; ++e) {
+                        Js.h[e] = h ? make_float2(c[e].z, c[e].w) : make_float2(c[e].x, c[e].y);
+                        Js.l[e] = h ? make_float2(c[3 + e].z, c[3 + e].w) : make_float2(c[3 + e].x, c[3 + e].y);
+                        Js.v[e] = h ? make_float2(c[6 + e].z, c[6 + e].w) : make_float2(c[6 + e].x, c[6 + e].y);
+                    }
+                    Js.m = h ? make_float2(c[9].z, c[9].w) : make_float2(c[9].x, c[9].y);
+                    pair_fixed2<decltype(guard)::value>(Js, N, eps2, S, ch, jt + jj + 2 * h, ii);
+                }
+            };
+            if (__any_sync(kFull, (unsigned)(ii - jt) < (unsigned)TL)) {
+                for (int jj = 0; jj < jc; jj += 4) four(jj, std::true_type());
             } else {
-#pragma unroll (kFixUnroll)
-                for (int jj = 0; jj < NT; ++jj)
-#pragma unroll
-                    for (int r = 0; r < R; ++r)
-                        pair_fixed<false>(s_p[jj], s_l[jj], s_v[jj], xh[r], xl[r], vi[r], eps2, S,
-                                          ch[r]);
+                for (int jj = 0; jj < jc; jj += 4) four(jj, std::false_type());
             }
 #pragma unroll
-            for (int r = 0; r < R; ++r)
-#pragma unroll
-                for (int q = 0; q < 7; ++q)
-                    add128(hi[r][q], lo[r][q], tile_sum(ch[r][0][q], ch[r][1][q], ch[r][2][q], NT));
+            for (int q = 0; q < 7; ++q)
+                add128(hi[q], lo[q], tile_sum(ch[0][q], ch[1][q], ch[2][q], (unsigned)jc));
         }
 
+        if (ia < 0) continue;
+        if (P.S == 1) {
+            double res[kComp];
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            if (ia[r] < 0) continue;
-            if (P.S == 1) {
-                double res[kComp];
+            for (int q = 0; q < 7; ++q)
+                res[q] = __dmul_rn(i128_to_double(hi[q], lo[q]), S.inv[q < 3 ? 0 : (q < 6 ? 1 : 2)]);
+            store_result(fa.out, ia, res);
+        } else {
 #pragma unroll
-                for (int q = 0; q < 7; ++q)
-                    res[q] = __dmul_rn(i128_to_double(hi[r][q], lo[r][q]),
-                                       S.inv[q < 3 ? 0 : (q < 6 ? 1 : 2)]);
-                store_result(fa.out, ia[r], res);
-            } else {
-#pragma unroll
-                for (int q = 0; q < 7; ++q) {
-                    long long *pp = part + 2 * (((long long)sl * kComp + q) * na + ia[r]);
-                    pp[0] = hi[r][q];
-                    pp[1] = (long long)lo[r][q];
-                }
+            for (int q = 0; q < 7; ++q) {
+                long long *pp = part + 2 * (((long long)sl * kComp + q) * na + ia);
+                pp[0] = hi[q];
+                pp[1] = (long long)lo[q];
             }
         }
     }
@@ -507,7 +520,7 @@ int occupancy_sum(int mode, int *blocks_per_sm)
 {
     cudaError_t e;
     if (mode == NB_SUM_FIXED)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_force_fixed<kFixNT, kFixR>,
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_force_fixed<kFixNT>,
                                                           kFixNT, 0);
     else if (mode == NB_SUM_FP32)
     {
@@ -527,7 +540,10 @@ int grid_summed(const ForceArgs &fa, const SumArgs &sa)
     if (na <= 0) return 0;
     long long items;
     if (sa.mode == NB_SUM_FIXED)
-        items = fa.plan.p.items;
+        // one CTA per item, dealt out as CTAs end: with four warps a scheduler
+        // the resident CTAs progress unevenly, and items dealt in turn left
+        // 28% of the warps idle on average
+        return fa.plan.p.items;
     else if (sa.mode == NB_SUM_FP32) {
         int I, T;
         seq_shape(na, sa.slots, I, T);
@@ -545,7 +561,7 @@ int launch_force_summed(const ForceArgs &fa, const JDS &j, const SumArgs &sa, in
         cudaMemsetAsync(sa.bounds, 0, 2 * sizeof(unsigned), st);
         const int gb = (int)(cdiv(fa.n, 256) < 1024 ? cdiv(fa.n, 256) : 1024);
         k_fixed_bounds<<<gb, 256, 0, st>>>(j, fa.n, sa.bounds);
-        k_force_fixed<kFixNT, kFixR><<<grid, kFixNT, 0, st>>>(fa, j, sa);
+        k_force_fixed<kFixNT><<<grid, kFixNT, 0, st>>>(fa, j, sa);
         long long gc = fa.na_dev ? 1024 : cdiv((long long)fa.na_host * kComp, 256);
         if (gc > 4096) gc = 4096;
         k_fixed_combine<<<(int)gc, 256, 0, st>>>(fa, sa);

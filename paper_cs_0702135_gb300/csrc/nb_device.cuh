@@ -630,10 +630,12 @@ __device__ __forceinline__ float2 pair_rn2(const Side2 &J, const Side2 &N, float
     const float2 fa = UNIT ? mr3 : mul2(mr3, f2(sa)), fk = UNIT ? mr3 : mul2(mr3, f2(sk));
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        t[c] = mul2(fa, dx[c]);
-        t[3 + c] = mul2(fk, add2(u[c], mul2s(b, dx[c])));
+        const float2 q = add2(u[c], mul2s(b, dx[c]));
+        // scaled terms go on into packed sums (split_add2)
+        t[c] = UNIT ? mul2(fa, dx[c]) : mul2s(fa, dx[c]);
+        t[3 + c] = UNIT ? mul2(fk, q) : mul2s(fk, q);
     }
-    t[6] = neg2(UNIT ? mr : mul2(mr, f2(sp)));
+    t[6] = UNIT ? neg2(mr) : mul2s(mr, f2(-sp));
     return r2;
 }
 
@@ -708,6 +710,21 @@ __device__ __forceinline__ void split_add(float t, unsigned &a1, unsigned &a2, u
     a1 += __float_as_uint(s1);
     a2 += __float_as_uint(s2);
     a3 += __float_as_uint(s3);
+}
+
+// split_add on two terms: the same roundings per lane, C - s taken as the
+// exact multiply-add s (-1) + C; the terms must not be plain packed products
+// (see mul2s).
+__device__ __forceinline__ void split_add2(float2 t, unsigned &a1, unsigned &a2, unsigned &a3)
+{
+    const float2 s1 = add2(t, f2(kC1));
+    const float2 r = add2(t, fma2(s1, f2(-1.0f), f2(kC1)));
+    const float2 s2 = add2(r, f2(kC2));
+    const float2 r2 = add2(r, fma2(s2, f2(-1.0f), f2(kC2)));
+    const float2 s3 = add2(r2, f2(kC3));
+    a1 += __float_as_uint(s1.x) + __float_as_uint(s1.y);
+    a2 += __float_as_uint(s2.x) + __float_as_uint(s2.y);
+    a3 += __float_as_uint(s3.x) + __float_as_uint(s3.y);
 }
 
 // The integer sum of a tile of `cnt` split terms.

@@ -345,15 +345,14 @@ struct SumArgs {
 #ifndef NB_FIX_NT
 #define NB_FIX_NT 64
 #endif
-#ifndef NB_FIX_R
-#define NB_FIX_R 1
-#endif
-#ifndef NB_FIX_UNROLL
-#define NB_FIX_UNROLL 4
-#endif
-constexpr int kFixNT = NB_FIX_NT;   // fixed point: threads per CTA (= j per tile)
-constexpr int kFixR = NB_FIX_R;     // fixed point: i per thread
-constexpr int kFixUnroll = NB_FIX_UNROLL;  // fixed point: j unrolling of the inner loop
+constexpr int kFixNT = NB_FIX_NT;   // fixed point: threads per CTA, one i each (slices: multiples of it)
+// fixed point: CTAs per SM the registers are held to (8, 9, 10, 12: 13.29, 13.23, 13.22, 13.36 ms
+// on 65536 bodies all active)
+constexpr int kFixCtas = 10;
+// fixed point: blocks of at least an eighth of the slots in i-blocks plan as if there were this
+// many times the slots, so that the items are short against the launch (1, 2, 4: 13.45, 13.45,
+// 13.29 ms); smaller blocks have too few j a slice for it
+constexpr int kFixWaves = 4;
 constexpr int kSeqNT = 640;         // FP32 index order: threads per CTA
 constexpr int kSortNT = 1024;       // FP32 sorted: one CTA per i
 constexpr int kErrFixedScale = 64;  // device error word: fixed-point scales out of range
@@ -366,7 +365,8 @@ __host__ __device__ inline ForcePlan make_force_plan(const ForceArgs &fa, int na
     f.regime = kRegIpar;
     if (na <= 0) return f;
     if (fa.summation == NB_SUM_FIXED) {
-        f.p = plan_ipar(na, fa.n, kFixNT * kFixR, kFixNT, fa.slots_sum, fa.split, fa.part_cap / 2);
+        f.p = plan_ipar(na, fa.n, kFixNT, kFixNT,
+                        fa.slots_sum * (8LL * cdiv(na, kFixNT) >= fa.slots_sum ? kFixWaves : 1), fa.split, fa.part_cap / 2);
         return f;
     }
     if (fa.summation != NB_SUM_COMPENSATED) return f;   // no slices
