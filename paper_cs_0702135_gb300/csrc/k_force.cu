@@ -206,38 +206,6 @@ __global__ void __launch_bounds__(NT) k_force_ipar_ds(ForceArgs fa, JDS J)
 // partials in slice order: the result depends only on the plan, and no
 // second launch is needed.
 
-// Lane l ends up holding, for value index e = l >> (5 - log2 P), the DS sum of
-// value e over all 32 lanes; P is a power of two <= 32.
-template <int P>
-__device__ __forceinline__ void warp_reduce_scatter(float (&h)[P], float (&lo)[P], int lane)
-{
-    int c = P;
-#pragma unroll
-    for (int off = 16; off >= 1; off >>= 1) {
-        if (c > 1) {
-            const bool up = (lane & off) != 0;
-            const int half = c / 2;
-#pragma unroll
-            for (int k = 0; k < P / 2; ++k) {
-                if (k < half) {
-                    const float sh = up ? h[k] : h[k + half], sl = up ? lo[k] : lo[k + half];
-                    float kh = up ? h[k + half] : h[k], kl = up ? lo[k + half] : lo[k];
-                    const float rh = __shfl_xor_sync(0xffffffffu, sh, off);
-                    const float rl = __shfl_xor_sync(0xffffffffu, sl, off);
-                    ds_add(kh, kl, rh, rl);
-                    h[k] = kh;
-                    lo[k] = kl;
-                }
-            }
-            c = half;
-        } else {
-            const float rh = __shfl_xor_sync(0xffffffffu, h[0], off);
-            const float rl = __shfl_xor_sync(0xffffffffu, lo[0], off);
-            ds_add(h[0], lo[0], rh, rl);
-        }
-    }
-}
-
 template <int NT, int IC, bool SOFT>
 __device__ __forceinline__ void jpar_ds_items(const ForceArgs &fa, const JDS &J, int na, const Plan &P)
 {

@@ -10,50 +10,50 @@
 // on each GPU when the library's module is loaded there and keeps until the
 // process exits.
 //
-// The kernels are a variant of the j-parallel force: each CTA takes up to four
-// active particles and one slice of the j range, every thread takes every
-// 256th j of the slice, positions are split into double-single form as they
-// are read, the CTA reduces with a warp-shuffle tree in double-single, and the
-// per-slice partial sums go to the scratch array; a second kernel sums the
-// slices in slice order.  Each thread adds its pair terms in FP32 runs of at
-// most eight and folds every run into double-single sums.  Every partial is
-// written before it is read in the same call, so nothing in the scratch array
-// needs clearing between calls.
+// The sums are fixed as runs: the j range falls into slices (as many as give
+// two per SM for four active particles a CTA), a slice into groups of 2048 j,
+// and run t of a group is the plain FP32 sum of its pairs with j = t, t + 256,
+// ... (at most eight).  Everything beyond a run is added in double-single or
+// FP64, so which thread adds which run does not show in single precision.
+//
+// A CTA takes a range of groups and up to 64 active particles.  Each thread
+// loads its eight j of a group straight from the FP64 arrays and splits them
+// into double-single form once, in registers, then walks the active particles
+// (in shared memory): eight pairs, and a warp reduce-scatter into the warp's
+// double-single totals.  The CTA adds its warps and writes one FP64 partial
+// per value; a second kernel adds the ranges, a warp per value.  Every partial
+// is written before it is read in the same call, so nothing in the scratch
+// array needs clearing between calls.
+//
+// The first form held four active particles per CTA and split every j again
+// for each four, on the FP64 pipe: 16 conversions a j at 2 lanes a clock per
+// SM were nearly all of its time (64 active on 2^18 + 37 bodies: 148 us).
 #include <climits>
 #include <cmath>
 #include <mutex>
 
 #include "nb.h"
-#include <cuda_runtime.h>
+#include "nb_device.cuh"
 
 namespace {
 
 constexpr int kNT = 256;                    // threads per CTA
-constexpr int kIC = 4;                      // active particles per CTA
+constexpr int kIC = 4;                      // active particles that the slice count is chosen for
 constexpr int kComp = 7;                    // acc xyz, jerk xyz, pot
-constexpr int kMaxSlices = 2048;            // j slices at most
-constexpr int kRun = 8;                     // FP32 pair terms per thread between promotions
+constexpr int kMaxSlices = 2048;            // j slices, and j ranges, at most
+constexpr int kRun = 8;                     // FP32 pair terms per run
+constexpr int kGroup = kNT * kRun;          // j per group of runs
 constexpr long long kScratchDoubles = (long long)kMaxSlices * kComp * NB_NOALLOC_MAX_ACTIVE;
 constexpr int kMaxDevices = 64;
 
-// Slice partials: part[(s * 7 + c) * n_active + a].  7 MiB per GPU.
+// Partials of the j ranges: part[(b * 7 + c) * n_active + a].  7 MiB per GPU.
 static __device__ __align__(256) double g_scratch[kScratchDoubles];
 
-__device__ __forceinline__ float rsqrt_sfu(float x)
-{
-    float y;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-__device__ __forceinline__ void ds_add(float &h, float &l, float h2, float l2)
-{
-    float s = h + h2;
-    float bb = s - h;
-    float e = (h - (s - bb)) + (h2 - bb);
-    h = s;
-    l = (l + l2) + e;
-}
+using nbk::dev::ds_add;
+using nbk::dev::rsqrt_sfu;
+using nbk::dev::split_ds_int;
+using nbk::dev::to_float_int;
+using nbk::dev::warp_reduce_scatter;
 
 struct DSPoint {
     float xh[3], xl[3], v[3], m;
@@ -65,18 +65,18 @@ __device__ __forceinline__ DSPoint load_point(const double *m, const double *x, 
     DSPoint p;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        const double xc = x[3 * j + c];
-        p.xh[c] = __double2float_rn(xc);
-        p.xl[c] = __double2float_rn(__dsub_rn(xc, (double)p.xh[c]));
-        p.v[c] = __double2float_rn(v[3 * j + c]);
+        split_ds_int(x[3 * j + c], p.xh[c], p.xl[c]);
+        p.v[c] = to_float_int(v[3 * j + c]);
     }
-    p.m = __double2float_rn(m[j]);
+    p.m = to_float_int(m[j]);
     return p;
 }
 
 // FP32 pair terms (Eq. 1 with the pair terms of the Appendix A kernel) on
-// double-single positions; the pair j = i and, with eps = 0, any pair at r = 0
-// contribute nothing.
+// double-single positions; a pair to be skipped and, with eps = 0, any pair at
+// r = 0 contribute nothing.  (Packing two j an instruction outside the running
+// sums left 64 active on 2^18 + 37 bodies at 52.1 against 50.5 us: about half
+// the instructions are the warp reductions', and the registers spill.)
 __device__ __forceinline__ void pair(const DSPoint &J, const DSPoint &I, float eps2, bool skip,
                                      float acc[3], float jk[3], float &pot)
 {
@@ -102,100 +102,95 @@ __device__ __forceinline__ void pair(const DSPoint &J, const DSPoint &I, float e
     pot -= mr;
 }
 
-__global__ void __launch_bounds__(kNT) k_few_partials(long long n, const double *m, const double *x,
-                                                      const double *v, float eps2, const int *act,
-                                                      int na, int S, long long jslice,
-                                                      double *part)
+// CTA (b, ch): j groups [b G / B, (b + 1) G / B) of the G = S gps groups (gps a
+// slice), active particles [ch IC, (ch + 1) IC).
+__global__ void __launch_bounds__(kNT, 2) k_few_partials(long long n, const double *m, const double *x,
+                                                         const double *v, float eps2, const int *act,
+                                                         int na, long long jslice, int gps, long long G,
+                                                         int B, int IC, int chunks, double *part)
 {
     constexpr int NW = kNT / 32;
-    constexpr int NV = kIC * kComp;
+    constexpr int NV = NB_NOALLOC_MAX_ACTIVE * kComp;
+    __shared__ DSPoint s_i[NB_NOALLOC_MAX_ACTIVE];
+    __shared__ long long s_ii[NB_NOALLOC_MAX_ACTIVE];
     __shared__ float s_h[NW][NV], s_l[NW][NV];
-    const int chunks = (na + kIC - 1) / kIC;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int w = blockIdx.x; w < chunks * S; w += gridDim.x) {
-        const int ch = w % chunks, sl = w / chunks;
-        const long long j0 = sl * jslice;
-        const long long j1 = j0 + jslice < n ? j0 + jslice : n;
-        DSPoint ip[kIC];
-        long long ii[kIC];
+    const int ch = blockIdx.x % chunks, b = blockIdx.x / chunks;
+    const int cnt = min(IC, na - ch * IC);
+    if (tid < cnt) {
+        long long i = act[ch * IC + tid];
+        i = i < 0 ? 0 : (i >= n ? n - 1 : i);
+        s_ii[tid] = i;
+        s_i[tid] = load_point(m, x, v, i);
+    }
+    for (int e = lane; e < cnt * kComp; e += 32) s_h[warp][e] = s_l[warp][e] = 0.0f;
+    __syncthreads();
+    const long long g1 = (b + 1) * G / B;
+    for (long long g = b * G / B; g < g1; ++g) {
+        const long long sl = g / gps;
+        const long long j0 = sl * jslice + (g - sl * gps) * kGroup;
+        const long long j1 = (sl + 1) * jslice < n ? (sl + 1) * jslice : n;
+        if (j0 >= j1) continue;   // past the end of a short slice
+        DSPoint jp[kRun];
 #pragma unroll
-        for (int q = 0; q < kIC; ++q) {
-            const int a = ch * kIC + q;
-            long long i = act[a < na ? a : 0];
-            i = i < 0 ? 0 : (i >= n ? n - 1 : i);
-            ii[q] = i;
-            ip[q] = load_point(m, x, v, i);
+        for (int u = 0; u < kRun; ++u) {
+            const long long j = j0 + u * kNT + tid;
+            jp[u] = load_point(m, x, v, j < j1 ? j : j1 - 1);
         }
-        // Plain FP32 runs of at most kRun pair terms per thread, each folded
-        // into the double-single sums (h, lo) by TwoSum, so the rounding error
-        // of a thread's sum does not grow with the slice length.
-        float h[NV], lo[NV];
+        const int left = (int)(j1 - j0 < kGroup ? j1 - j0 : kGroup);   // j of this group
+        for (int a = 0; a < cnt; ++a) {
+            const DSPoint I = s_i[a];
+            // this thread's j that is the particle itself, as a run position
+            const long long own = s_ii[a] - j0 - tid;
+            float a3[3] = {0.0f, 0.0f, 0.0f}, k3[3] = {0.0f, 0.0f, 0.0f}, pp = 0.0f;
+            if (left < kGroup || (unsigned long long)(s_ii[a] - j0) < (unsigned long long)kGroup) {
 #pragma unroll
-        for (int e = 0; e < NV; ++e) h[e] = lo[e] = 0.0f;
-        for (long long jb = j0 + tid; jb < j1; jb += (long long)kNT * kRun) {
-            float t[NV];
+                for (int u = 0; u < kRun; ++u)
+                    pair(jp[u], I, eps2, u * kNT + tid >= left || own == u * kNT, a3, k3, pp);
+            } else {
 #pragma unroll
-            for (int e = 0; e < NV; ++e) t[e] = 0.0f;
-#pragma unroll 1
-            for (int u = 0; u < kRun; ++u) {
-                const long long j = jb + (long long)u * kNT;
-                if (j >= j1) break;
-                const DSPoint jp = load_point(m, x, v, j);
-#pragma unroll
-                for (int q = 0; q < kIC; ++q) {
-                    float a3[3] = {t[q * kComp], t[q * kComp + 1], t[q * kComp + 2]};
-                    float k3[3] = {t[q * kComp + 3], t[q * kComp + 4], t[q * kComp + 5]};
-                    float pp = t[q * kComp + 6];
-                    pair(jp, ip[q], eps2, j == ii[q], a3, k3, pp);
-                    t[q * kComp] = a3[0]; t[q * kComp + 1] = a3[1]; t[q * kComp + 2] = a3[2];
-                    t[q * kComp + 3] = k3[0]; t[q * kComp + 4] = k3[1]; t[q * kComp + 5] = k3[2];
-                    t[q * kComp + 6] = pp;
-                }
+                for (int u = 0; u < kRun; ++u) pair(jp[u], I, eps2, false, a3, k3, pp);
             }
-#pragma unroll
-            for (int e = 0; e < NV; ++e) ds_add(h[e], lo[e], t[e], 0.0f);
+            float h[8] = {a3[0], a3[1], a3[2], k3[0], k3[1], k3[2], pp, 0.0f};
+            float lo[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+            warp_reduce_scatter<8>(h, lo, lane);
+            const int e = lane >> 2;
+            if ((lane & 3) == 0 && e < kComp)
+                ds_add(s_h[warp][a * kComp + e], s_l[warp][a * kComp + e], h[0], lo[0]);
         }
+    }
+    __syncthreads();
+    for (int t = tid; t < cnt * kComp; t += kNT) {
+        float th = s_h[0][t], tl = s_l[0][t];
 #pragma unroll
-        for (int off = 16; off >= 1; off >>= 1)
-#pragma unroll
-            for (int e = 0; e < NV; ++e) {
-                const float h2 = __shfl_xor_sync(0xffffffffu, h[e], off);
-                const float l2 = __shfl_xor_sync(0xffffffffu, lo[e], off);
-                ds_add(h[e], lo[e], h2, l2);
-            }
-        if (lane == 0)
-#pragma unroll
-            for (int e = 0; e < NV; ++e) {
-                s_h[warp][e] = h[e];
-                s_l[warp][e] = lo[e];
-            }
-        __syncthreads();
-        if (tid < NV) {
-            float th = s_h[0][tid], tl = s_l[0][tid];
-            for (int ww = 1; ww < NW; ++ww) ds_add(th, tl, s_h[ww][tid], s_l[ww][tid]);
-            const int q = tid / kComp, c = tid % kComp;
-            const int a = ch * kIC + q;
-            if (a < na) part[((long long)sl * kComp + c) * na + a] = (double)th + (double)tl;
-        }
-        __syncthreads();
+        for (int ww = 1; ww < NW; ++ww) ds_add(th, tl, s_h[ww][t], s_l[ww][t]);
+        const int q = t / kComp, c = t % kComp;
+        part[((long long)b * kComp + c) * na + ch * IC + q] = (double)th + (double)tl;
     }
 }
 
-__global__ void k_few_combine(int na, int S, const double *part, double *acc, double *jerk,
+// One warp per value: lanes over the ranges in a fixed stride, then a fixed
+// tree (one thread per value, adding the ranges in turn, waited for its loads
+// four at a time: ~15 us for one active particle on 2^18 bodies).
+__global__ void k_few_combine(int na, int B, const double *part, double *acc, double *jerk,
                               double *pot)
 {
-    const int total = na * kComp;
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
-        const int c = e / na, a = e % na;
-        double s = 0.0;
-        for (int q = 0; q < S; ++q) s += part[((long long)q * kComp + c) * na + a];
-        if (c < 3) {
-            if (acc) acc[3 * a + c] = s;
-        } else if (c < 6) {
-            if (jerk) jerk[3 * a + (c - 3)] = s;
-        } else if (pot) {
-            pot[a] = s;
-        }
+    const int lane = threadIdx.x & 31;
+    const int e = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (e >= na * kComp) return;
+    const int c = e / na, a = e % na;
+    double s = 0.0;
+#pragma unroll 4
+    for (int q = lane; q < B; q += 32) s += part[((long long)q * kComp + c) * na + a];
+#pragma unroll
+    for (int off = 16; off >= 1; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if (lane != 0) return;
+    if (c < 3) {
+        if (acc) acc[3 * a + c] = s;
+    } else if (c < 6) {
+        if (jerk) jerk[3 * a + (c - 3)] = s;
+    } else if (pot) {
+        pot[a] = s;
     }
 }
 
@@ -261,14 +256,25 @@ extern "C" int nb_force_few_noalloc(int64_t n, const double *d_m, const double *
     if (S < 1) S = 1;
     const long long jslice = ((n + S - 1) / S + kNT - 1) / kNT * kNT;
     S = (n + jslice - 1) / jslice;
-    const long long items = (long long)chunks * S;
-    const int grid = (int)(items < 4LL * s.sms ? items : 4LL * s.sms);
+    // Work: G groups of runs by the active particles, two CTAs resident an SM.
+    // With fewer groups than CTAs the particles are divided too, no further than
+    // one round of CTAs (each splits its j again: 64 active on 2^18 + 37 bodies
+    // take 49 us so, 55 and 66 us with two and four times the CTAs); otherwise
+    // a CTA takes several groups.
+    const int gps = (int)((jslice + kGroup - 1) / kGroup);
+    const long long G = S * gps, slots = 2LL * s.sms;
+    const long long rounds = (G + slots - 1) / slots;
+    const int B = (int)((G + rounds - 1) / rounds);
+    int parts = (int)(slots / B < n_active ? slots / B : n_active);
+    if (parts < 1) parts = 1;
+    const int IC = (n_active + parts - 1) / parts;
+    const int ichunks = (n_active + IC - 1) / IC;
 
     cudaStream_t st = (cudaStream_t)stream;
-    k_few_partials<<<grid, kNT, 0, st>>>(n, d_m, d_x, d_v, (float)(eps * eps), d_active_idx,
-                                         n_active, (int)S, jslice, s.scratch);
+    k_few_partials<<<B * ichunks, kNT, 0, st>>>(n, d_m, d_x, d_v, (float)(eps * eps), d_active_idx,
+                                                n_active, jslice, gps, G, B, IC, ichunks, s.scratch);
     if (cudaGetLastError() != cudaSuccess) return NB_ECUDA;
-    k_few_combine<<<(n_active * kComp + 255) / 256, 256, 0, st>>>(n_active, (int)S, s.scratch,
-                                                                  d_acc, d_jerk, d_pot);
+    k_few_combine<<<(n_active * kComp * 32 + 255) / 256, 256, 0, st>>>(n_active, B, s.scratch, d_acc,
+                                                                       d_jerk, d_pot);
     return cudaGetLastError() == cudaSuccess ? NB_OK : NB_ECUDA;
 }

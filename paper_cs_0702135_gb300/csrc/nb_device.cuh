@@ -50,6 +50,38 @@ __device__ __forceinline__ void ds_add(float &h, float &l, float h2, float l2)
     l = (l + l2) + e;
 }
 
+// Lane l ends up holding, for value index e = l >> (5 - log2 P), the DS sum of
+// value e over all 32 lanes; P is a power of two <= 32.
+template <int P>
+__device__ __forceinline__ void warp_reduce_scatter(float (&h)[P], float (&lo)[P], int lane)
+{
+    int c = P;
+#pragma unroll
+    for (int off = 16; off >= 1; off >>= 1) {
+        if (c > 1) {
+            const bool up = (lane & off) != 0;
+            const int half = c / 2;
+#pragma unroll
+            for (int k = 0; k < P / 2; ++k) {
+                if (k < half) {
+                    const float sh = up ? h[k] : h[k + half], sl = up ? lo[k] : lo[k + half];
+                    float kh = up ? h[k + half] : h[k], kl = up ? lo[k + half] : lo[k];
+                    const float rh = __shfl_xor_sync(0xffffffffu, sh, off);
+                    const float rl = __shfl_xor_sync(0xffffffffu, sl, off);
+                    ds_add(kh, kl, rh, rl);
+                    h[k] = kh;
+                    lo[k] = kl;
+                }
+            }
+            c = half;
+        } else {
+            const float rh = __shfl_xor_sync(0xffffffffu, h[0], off);
+            const float rl = __shfl_xor_sync(0xffffffffu, lo[0], off);
+            ds_add(h[0], lo[0], rh, rl);
+        }
+    }
+}
+
 // a / C rounded to nearest, for the constants C = 3, 12, 20 of the predictor
 // and corrector, without an FP64 division (a long sequence on the GB300's
 // narrow FP64 pipe): q0 = RN(a y) with y = RN(1/C) is within one ulp of a/C
@@ -116,6 +148,50 @@ __device__ __forceinline__ void split_ds(double x, float &hi, float &lo)
 {
     hi = __double2float_rn(x);
     lo = __double2float_rn(__dsub_rn(x, (double)hi));
+}
+
+// RN32(x) and RN32(x - RN32(x)) on the integer pipe.  A conversion between
+// FP64 and FP32 runs on the GB300's FP64 pipe like an FP64 operation (2 lanes
+// a clock per SM, 64 cycles), so a split costs four of those; these are ~15
+// integer instructions.  x = (-1)^s M 2^(e-1075): the top 24 bits of M round
+// half to even by the remainder R of the low 29, and the rest R (- 2^29 if
+// rounded up) is an integer of at most 29 bits, converted to FP32 (rounded to
+// nearest) and scaled exactly.  Exponents outside [2^-70, 2^120) (zero among
+// them) take the conversions, written volatile so that they are not evaluated
+// ahead of the test.
+__device__ __forceinline__ bool split_safe(double x)
+{
+    return (((unsigned)__double2hiint(x) & 0x7fffffffu) - ((1023u - 70u) << 20)) < (190u << 20);
+}
+__device__ __forceinline__ float to_float_volatile(double x)
+{
+    float y;
+    asm volatile("cvt.rn.f32.f64 %0, %1;" : "=f"(y) : "d"(x));
+    return y;
+}
+__device__ __forceinline__ void split_ds_int(double x, float &hi, float &lo)
+{
+    if (!split_safe(x)) {
+        hi = to_float_volatile(x);
+        lo = to_float_volatile(__dsub_rn(x, (double)hi));
+        return;
+    }
+    const unsigned xh = (unsigned)__double2hiint(x), xl = (unsigned)__double2loint(x);
+    const unsigned e = (xh >> 20) & 0x7ffu;
+    const unsigned t = ((xh & 0x7fffffffu) - (896u << 20)) << 3 | xl >> 29;   // truncated to FP32
+    const unsigned R = xl & 0x1fffffffu;
+    const bool up = R + (t & 1u) > 0x10000000u;
+    hi = __uint_as_float((t + up) | (xh & 0x80000000u));
+    int r = (int)R - (up ? 0x20000000 : 0);
+    r = (int)xh < 0 ? -r : r;
+    lo = __int2float_rn(r) * __uint_as_float((e - (1075u - 127u)) << 23);
+}
+__device__ __forceinline__ float to_float_int(double x)
+{
+    if (!split_safe(x)) return to_float_volatile(x);
+    const unsigned xh = (unsigned)__double2hiint(x), xl = (unsigned)__double2loint(x);
+    const unsigned t = ((xh & 0x7fffffffu) - (896u << 20)) << 3 | xl >> 29;
+    return __uint_as_float((t + ((xl & 0x1fffffffu) + (t & 1u) > 0x10000000u)) | (xh & 0x80000000u));
 }
 
 __device__ __forceinline__ double norm3(double u0, double u1, double u2)

@@ -99,3 +99,40 @@ def test_adding_the_negation_rounds_as_the_subtraction():
             assert sub.dtype == np.float32 and add.dtype == np.float32
             same = (sub.view(np.uint32) == add.view(np.uint32)) | (np.isnan(sub) & np.isnan(add))
             assert same.all(), (x[~same][:5], y[~same][:5])
+
+
+np = pytest.importorskip("numpy")
+
+
+def _split_int(x):
+    # split_ds_int of nb_device.cuh in numpy integers: RN32(x), RN32(x - RN32(x))
+    b = x.view(np.uint64)
+    xh, xl = (b >> np.uint64(32)).astype(np.int64), (b & np.uint64(0xffffffff)).astype(np.int64)
+    e = (xh >> 20) & 0x7ff
+    t = ((((xh & 0x7fffffff) - (896 << 20)) << 3) & 0xffffffff) | (xl >> 29)
+    r = xl & 0x1fffffff
+    up = (r + (t & 1) > 0x10000000).astype(np.int64)
+    hi = ((t + up) | (xh & 0x80000000)).astype(np.uint32).view(np.float32)
+    r = r - up * 0x20000000
+    r = np.where(xh & 0x80000000, -r, r)
+    lo = r.astype(np.float32) * ((e - (1075 - 127)) << 23).astype(np.uint32).view(np.float32)
+    return hi, lo
+
+
+def test_integer_split_into_double_single():
+    # random values over the exponents that take the integer form, ties and
+    # near-ties of both roundings, and carries into the next binade
+    rng = np.random.RandomState(11)
+    e = rng.randint(1023 - 70, 1023 + 119, 200000).astype(np.uint64)
+    m = rng.randint(0, 1 << 52, 200000, dtype=np.int64).astype(np.uint64)
+    m[:20000] = (m[:20000] & ~np.uint64(0x1fffffff)) | np.uint64(0x10000000)
+    m[20000:40000] = (m[20000:40000] & ~np.uint64(0x1fffffff)) + rng.randint(0x0fffffff, 0x10000002, 20000).astype(np.uint64)
+    m[40000:41000] = np.uint64((1 << 52) - 1) - rng.randint(0, 1 << 30, 1000).astype(np.uint64)
+    m[41000:42000] = 0
+    s = rng.randint(0, 2, 200000).astype(np.uint64)
+    x = ((s << np.uint64(63)) | (e << np.uint64(52)) | m).view(np.float64)
+    hi, lo = _split_int(x)
+    want = x.astype(np.float32)
+    assert np.array_equal(hi.view(np.uint32), want.view(np.uint32))
+    rest = (x - want.astype(np.float64)).astype(np.float32)
+    assert np.array_equal(lo.view(np.uint32), rest.view(np.uint32))
