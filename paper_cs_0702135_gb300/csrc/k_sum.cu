@@ -114,13 +114,7 @@ __global__ void __launch_bounds__(NT, kFixCtas) k_force_fixed(ForceArgs fa, JDS 
         const int a = ib * NT + tid;
         const int ia = a < na ? a : -1;
         const int ii = clamp_index(fa.act[a < na ? a : 0], fa.n);
-        Side2 N;
-        {
-            const float4 p = J.pos_hi[ii], l = J.pos_lo[ii], v = J.vel[ii];
-            N.h[0] = f2(-p.x), N.h[1] = f2(-p.y), N.h[2] = f2(-p.z);
-            N.l[0] = f2(-l.x), N.l[1] = f2(-l.y), N.l[2] = f2(-l.z);
-            N.v[0] = f2(-v.x), N.v[1] = f2(-v.y), N.v[2] = f2(-v.z);
-        }
+        const Side2 N = side2_neg(J.pos_hi[ii], J.pos_lo[ii], J.vel[ii]);
         long long hi[7];
         unsigned long long lo[7];
 #pragma unroll
@@ -302,11 +296,7 @@ __device__ __forceinline__ void seq_groups(const ForceArgs &fa, const JDS &J, in
                     float *const dst = buf + (k & 1) * kSeqBufFloats;
                     for (int sub = sub0; sub < nsub; sub += kSeqTermWarps) {
                         const int jj = sub * 32 + lane, j = k * T + jj;
-                        Side2 Js;
-                        Js.h[0] = f2(np.x), Js.h[1] = f2(np.y), Js.h[2] = f2(np.z);
-                        Js.l[0] = f2(nl.x), Js.l[1] = f2(nl.y), Js.l[2] = f2(nl.z);
-                        Js.v[0] = f2(nv.x), Js.v[1] = f2(nv.y), Js.v[2] = f2(nv.z);
-                        Js.m = f2(np.w);
+                        const Side2 Js = side2(np, nl, nv, np, nl, nv);
                         const int jn = min(sub + kSeqTermWarps < nsub ? j + kSeqTermWarps * 32
                                                                       : (k + 1) * T + jlane, n - 1);
                         np = J.pos_hi[jn], nl = J.pos_lo[jn], nv = J.vel[jn];
@@ -376,26 +366,43 @@ __global__ void __launch_bounds__(kSeqNT, 1) k_force_seq(ForceArgs fa, JDS J, in
 // ---------------------------------------------------------------------------
 // FP32 running sum, smallest pair force first: one CTA per active i.
 //  1. keyed items (key bits << 32 | j) for every j into the CTA's scratch, in
-//     index order; j = i and r2 = 0 get the key 0xffffffff (sorted last).
-//  2. stable LSD radix sort on the key, four passes of 8 bits: a histogram,
-//     its exclusive scan, then tile by tile each item's rank among the equal
-//     digits of its warp (match_any) plus the counts of the earlier warps and
-//     tiles; stability keeps equal keys in index order.
-//  3. tiles of NT sorted items: every thread computes one item's terms into
-//     shared memory, then seven threads add them in order, one per component.
+//     index order, and the histograms of the key's four bytes; j = i and
+//     r2 = 0 get the key 0xffffffff (sorted last).
+//  2. stable LSD radix sort on the key, a pass per byte (a byte that all keys
+//     share is left out): tiles of 16 items a thread, each warp a contiguous
+//     run of the tile.  An item's rank is that among the equal digits of its
+//     warp (match_any and the warp's running counts in shared memory) plus
+//     the counts of the earlier warps and tiles; stability keeps equal keys in
+//     index order.  The last pass writes the indices alone.
+//  3. seven warps evaluate the sorted items' terms, two an instruction, into
+//     one of two buffers while seven lanes of the eighth add the tile before
+//     it in order, one component each.
+// The chain of additions (4 cycles an item) keeps one warp of a CTA busy and
+// nothing else, so four CTAs share an SM, each in its own phase.  1820 active
+// on 65536 bodies: 6.6 ms; before, one CTA of 1024 threads per SM ranked
+// one item a thread between five barriers and added after evaluating
+// (18.6 ms).
 
 constexpr int kSortW = kSortNT / 32;
+constexpr int kSortK = 16;                        // items per thread and tile of a pass
+constexpr int kSortTile = kSortNT * kSortK;
+constexpr int kSortSum = (kSortW - 1) * 64;       // items per tile of the sum: two per term lane
+constexpr int kSortRow = kSortSum + 4;
 
-__global__ void __launch_bounds__(kSortNT) k_force_sorted(ForceArgs fa, JDS J, SumArgs sa)
+__global__ void __launch_bounds__(kSortNT, kSortCtas) k_force_sorted(ForceArgs fa, JDS J, SumArgs sa)
 {
     constexpr int NT = kSortNT;
     const int na = read_na(fa);
     if (na <= 0) return;
-    __shared__ unsigned s_base[256], s_tot[256];
-    __shared__ unsigned short s_wc[kSortW][256];
-    __shared__ float s_t[7][NT];
+    __shared__ unsigned s_hist[4][256];
+    __shared__ unsigned s_base[256], s_scan[kSortW];
+    __shared__ union {
+        unsigned off[kSortW][256];               // pass: counts, then offsets, of a warp's digits
+        float4 t[2][7][kSortRow / 4];            // sum: two tiles of terms
+    } u;
     __shared__ float s_res[7];
     __shared__ int s_cnt;
+    static_assert(NT == 256, "a thread per digit");
     const int n = fa.n, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const unsigned lt = (1u << lane) - 1u;
     const float eps2 = (float)fa.eps2;
@@ -404,101 +411,127 @@ __global__ void __launch_bounds__(kSortNT) k_force_sorted(ForceArgs fa, JDS J, S
 
     for (int a = blockIdx.x; a < na; a += gridDim.x) {
         const int i = clamp_index(fa.act[a], n);
-        float xh[3], xl[3], vi[3];
-        load_i(J, i, xh, xl, vi);
+        const Side2 N = side2_neg(J.pos_hi[i], J.pos_lo[i], J.vel[i]);
         if (tid == 0) s_cnt = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) s_hist[q][tid] = 0;
         __syncthreads();
 
         int cnt = 0;
-        for (int j = tid; j < n; j += NT) {
-            float t[7], key;
-            const bool ok = pair_rn(J.pos_hi[j], J.pos_lo[j], J.vel[j], xh, xl, vi, eps2, 1.0f, 1.0f,
-                                    1.0f, t, &key) && j != i;
-            const unsigned kb = ok ? __float_as_uint(key) : 0xffffffffu;
-            A[j] = ((unsigned long long)kb << 32) | (unsigned)j;
-            cnt += ok;
+        for (int j = tid; j < n; j += 2 * NT) {
+            const int j1 = min(j + NT, n - 1);
+            const Side2 Js = side2(J.pos_hi[j], J.pos_lo[j], J.vel[j], J.pos_hi[j1], J.pos_lo[j1], J.vel[j1]);
+            float2 r2;
+            const float2 key = pair_key2(Js, N, eps2, r2);
+            const bool ok0 = r2.x != 0.0f && j != i, ok1 = r2.y != 0.0f && j + NT != i;
+            const unsigned k0 = ok0 ? __float_as_uint(key.x) : 0xffffffffu;
+            const unsigned k1 = ok1 ? __float_as_uint(key.y) : 0xffffffffu;
+            A[j] = ((unsigned long long)k0 << 32) | (unsigned)j;
+            cnt += ok0;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) atomicAdd(&s_hist[q][(k0 >> (8 * q)) & 255u], 1u);
+            if (j + NT < n) {
+                A[j + NT] = ((unsigned long long)k1 << 32) | (unsigned)(j + NT);
+                cnt += ok1;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) atomicAdd(&s_hist[q][(k1 >> (8 * q)) & 255u], 1u);
+            }
         }
         cnt = __reduce_add_sync(kFull, cnt);
         if (lane == 0) atomicAdd(&s_cnt, cnt);
+        __syncthreads();
 
         unsigned long long *src = A, *dst = B;
         for (int pass = 0; pass < 4; ++pass) {
-            const int shift = 32 + 8 * pass;
-            if (tid < 256) s_base[tid] = 0;
-            for (int e = tid; e < kSortW * 256; e += NT) (&s_wc[0][0])[e] = 0;
-            __syncthreads();
-            for (int t0 = 0; t0 < n; t0 += NT) {
-                const int idx = t0 + tid;
-                const bool valid = idx < n;
-                const unsigned d = valid ? (unsigned)(src[idx] >> shift) & 255u : 256u;
-                const unsigned peers = __match_any_sync(kFull, d);
-                if (valid && (peers & lt) == 0) atomicAdd(&s_base[d], (unsigned)__popc(peers));
-            }
-            __syncthreads();
-            unsigned incl = 0, cntd = 0;
-            if (tid < 256) {
-                cntd = s_base[tid];
-                incl = cntd;
+            // the digit's first place: exclusive sum of the histogram
+            const unsigned mine = s_hist[pass][tid];
+            if (__syncthreads_or(mine == (unsigned)n)) continue;   // one digit for all
+            unsigned incl = mine;
 #pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const unsigned y = __shfl_up_sync(kFull, incl, o);
-                    if (lane >= o) incl += y;
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned y = __shfl_up_sync(kFull, incl, o);
+                if (lane >= o) incl += y;
+            }
+            if (lane == 31) s_scan[warp] = incl;
+            __syncthreads();
+            unsigned before = incl - mine;
+            for (int w = 0; w < warp; ++w) before += s_scan[w];
+            s_base[tid] = before;   // read and kept by this thread only
+            const int shift = 32 + 8 * pass;
+            for (int t0 = 0; t0 < n; t0 += kSortTile) {
+                unsigned long long item[kSortK];
+                unsigned rank[kSortK];
+                const int w0 = t0 + warp * (kSortK * 32) + lane;
+#pragma unroll
+                for (int k = 0; k < kSortK; ++k)
+                    // past the end: the last digit, after every item of the tile, never stored
+                    item[k] = w0 + k * 32 < n ? src[w0 + k * 32] : ~0ULL;
+#pragma unroll
+                for (int q = 0; q < 256 / 32; ++q) u.off[warp][q * 32 + lane] = 0;
+                __syncwarp();
+#pragma unroll
+                for (int k = 0; k < kSortK; ++k) {
+                    const unsigned d = (unsigned)(item[k] >> shift) & 255u;
+                    const unsigned peers = __match_any_sync(kFull, d);
+                    const unsigned old = u.off[warp][d];
+                    rank[k] = old + __popc(peers & lt);
+                    __syncwarp();
+                    if ((peers & lt) == 0) u.off[warp][d] = old + __popc(peers);
+                    __syncwarp();
                 }
-                s_tot[tid] = incl;
+                __syncthreads();
+                unsigned run = s_base[tid];
+#pragma unroll
+                for (int w = 0; w < kSortW; ++w) {
+                    const unsigned c = u.off[w][tid];
+                    u.off[w][tid] = run;
+                    run += c;
+                }
+                s_base[tid] = run;
+                __syncthreads();
+#pragma unroll
+                for (int k = 0; k < kSortK; ++k) {
+                    const unsigned d = (unsigned)(item[k] >> shift) & 255u;
+                    if (w0 + k * 32 < n) dst[u.off[warp][d] + rank[k]] = item[k];
+                }
+                __syncwarp();   // the warp's offsets are cleared next
             }
             __syncthreads();
-            if (tid < 256) {
-                unsigned off = 0;
-                for (int w = 0; w < warp; ++w) off += s_tot[w * 32 + 31];
-                s_base[tid] = incl - cntd + off;
-            }
-            __syncthreads();
-            for (int t0 = 0; t0 < n; t0 += NT) {
-                const int idx = t0 + tid;
-                const bool valid = idx < n;
-                const unsigned long long item = valid ? src[idx] : 0ULL;
-                const unsigned d = valid ? (unsigned)(item >> shift) & 255u : 256u;
-                const unsigned peers = __match_any_sync(kFull, d);
-                const int rank = __popc(peers & lt);
-                if (valid && rank == 0) s_wc[warp][d] = (unsigned short)__popc(peers);
-                __syncthreads();
-                if (tid < 256) {
-                    unsigned run = 0;
-                    for (int w = 0; w < kSortW; ++w) {
-                        const unsigned c = s_wc[w][tid];
-                        s_wc[w][tid] = (unsigned short)run;
-                        run += c;
-                    }
-                    s_tot[tid] = run;
-                }
-                __syncthreads();
-                if (valid) dst[s_base[d] + s_wc[warp][d] + rank] = item;
-                __syncthreads();
-                if (tid < 256) s_base[tid] += s_tot[tid];
-                for (int e = tid; e < kSortW * 256; e += NT) (&s_wc[0][0])[e] = 0;
-                __syncthreads();
-            }
             unsigned long long *tmp = src;
             src = dst;
             dst = tmp;
         }
 
         const int total = s_cnt;
+        const int ntile = cdiv(total, kSortSum);
         float run = 0.0f;
-        for (int t0 = 0; t0 < total; t0 += NT) {
-            const int k = t0 + tid;
-            if (k < total) {
-                const int j = (int)(unsigned)(src[k] & 0xffffffffULL);
-                float t[7];
-                pair_rn(J.pos_hi[j], J.pos_lo[j], J.vel[j], xh, xl, vi, eps2, 1.0f, 1.0f, 1.0f, t);
+        for (int k = 0; k <= ntile; ++k) {
+            if (warp > 0) {
+                if (k < ntile) {
+                    const int q0 = (warp - 1) * 64 + lane, e0 = k * kSortSum + q0, e1 = e0 + 32;
+                    const int ja = (int)(unsigned)src[min(e0, total - 1)];
+                    const int jb = (int)(unsigned)src[min(e1, total - 1)];
+                    const Side2 Js = side2(J.pos_hi[ja], J.pos_lo[ja], J.vel[ja], J.pos_hi[jb],
+                                           J.pos_lo[jb], J.vel[jb]);
+                    float2 t[7];
+                    pair_rn2<true>(Js, N, eps2, 1.0f, 1.0f, 1.0f, t);
+                    float *const d = reinterpret_cast<float *>(u.t[k & 1]) + q0;
 #pragma unroll
-                for (int q = 0; q < 7; ++q) s_t[q][tid] = t[q];
-            }
-            __syncthreads();
-            if (tid < 7) {
-                const int m = min(NT, total - t0);
+                    for (int c = 0; c < 7; ++c) {
+                        d[c * kSortRow] = e0 < total ? t[c].x : -0.0f;   // -0 changes no sum
+                        d[c * kSortRow + 32] = e1 < total ? t[c].y : -0.0f;
+                    }
+                }
+            } else if (k > 0 && lane < 7) {
+                const float4 *s4 = u.t[(k - 1) & 1][lane];
 #pragma unroll 8
-                for (int k2 = 0; k2 < m; ++k2) run = __fadd_rn(run, s_t[tid][k2]);
+                for (int q = 0; q < kSortSum / 4; ++q) {
+                    const float4 t = s4[q];
+                    run = __fadd_rn(run, t.x);
+                    run = __fadd_rn(run, t.y);
+                    run = __fadd_rn(run, t.z);
+                    run = __fadd_rn(run, t.w);
+                }
             }
             __syncthreads();
         }

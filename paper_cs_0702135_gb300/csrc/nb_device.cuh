@@ -675,6 +675,19 @@ __device__ __forceinline__ float2 inv_sqrt_rn2(float2 x)
     return r;
 }
 
+// RN(sqrt(x)) for two x by the first of those steps.
+__device__ __forceinline__ float2 sqrt_rn2(float2 x)
+{
+    const float2 y = make_float2(rsqrt_sfu(x.x), rsqrt_sfu(x.y));
+    const float2 s0 = mul2(x, y);
+    float2 s = fma2(fma2(neg2(s0), s0, x), mul2(y, f2(0.5f)), s0);
+    if (inv_sqrt_hard(x.x) || inv_sqrt_hard(x.y)) {
+        s.x = __fsqrt_rn(x.x);
+        s.y = __fsqrt_rn(x.y);
+    }
+    return s;
+}
+
 // One side of two pairs: hi and lo position words, velocity (of the i side
 // negated), mass.
 struct Side2 {
@@ -713,6 +726,39 @@ __device__ __forceinline__ float2 pair_rn2(const Side2 &J, const Side2 &N, float
     }
     t[6] = UNIT ? neg2(mr) : mul2s(mr, f2(-sp));
     return r2;
+}
+
+// The sort keys of two pairs, min(mr3 sqrt(d2), FLT_MAX), as pair_rn's; r2 in
+// rr (a pair with r2 = 0 has no key).
+__device__ __forceinline__ float2 pair_key2(const Side2 &J, const Side2 &N, float eps2, float2 &rr)
+{
+    float2 dx[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) dx[c] = add2(add2(J.h[c], N.h[c]), add2(J.l[c], N.l[c]));
+    const float2 d2 = add2(add2(mul2s(dx[0], dx[0]), mul2s(dx[1], dx[1])), mul2s(dx[2], dx[2]));
+    rr = add2(d2, f2(eps2));
+    const float2 rinv = inv_sqrt_rn2(rr);
+    const float2 key = mul2(mul2(mul2(J.m, rinv), mul2(rinv, rinv)), sqrt_rn2(d2));
+    return make_float2(fminf(key.x, FLT_MAX), fminf(key.y, FLT_MAX));
+}
+
+// The records of two particles side by side, and one in both lanes negated.
+__device__ __forceinline__ Side2 side2(const float4 &p0, const float4 &l0, const float4 &v0,
+                                       const float4 &p1, const float4 &l1, const float4 &v1)
+{
+    Side2 s;
+    s.h[0] = make_float2(p0.x, p1.x), s.h[1] = make_float2(p0.y, p1.y), s.h[2] = make_float2(p0.z, p1.z);
+    s.l[0] = make_float2(l0.x, l1.x), s.l[1] = make_float2(l0.y, l1.y), s.l[2] = make_float2(l0.z, l1.z);
+    s.v[0] = make_float2(v0.x, v1.x), s.v[1] = make_float2(v0.y, v1.y), s.v[2] = make_float2(v0.z, v1.z);
+    s.m = make_float2(p0.w, p1.w);
+    return s;
+}
+__device__ __forceinline__ Side2 side2_neg(const float4 &p, const float4 &l, const float4 &v)
+{
+    Side2 s = side2(p, l, v, p, l, v);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) s.h[c] = neg2(s.h[c]), s.l[c] = neg2(s.l[c]), s.v[c] = neg2(s.v[c]);
+    return s;
 }
 
 __device__ __forceinline__ void load_i(const JDS &J, int i, float xh[3], float xl[3], float vi[3])

@@ -354,7 +354,8 @@ constexpr int kFixCtas = 10;
 // 13.29 ms); smaller blocks have too few j a slice for it
 constexpr int kFixWaves = 4;
 constexpr int kSeqNT = 640;         // FP32 index order: threads per CTA
-constexpr int kSortNT = 1024;       // FP32 sorted: one CTA per i
+constexpr int kSortNT = 256;        // FP32 sorted: one CTA per i
+constexpr int kSortCtas = 4;        // and at least this many per SM
 constexpr int kErrFixedScale = 64;  // device error word: fixed-point scales out of range
 constexpr int kErrInput = 65;       // device error word: a non-finite value or a negative mass
 
