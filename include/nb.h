@@ -43,10 +43,9 @@ extern "C" {
 
 #define NB_FORCE_AUTO 0  /* pick the force kernel from n_active (DS: j-parallel up to 96,
                           * then the i-parallel kernels) */
-#define NB_FORCE_IPAR 1  /* i across threads, j tiles broadcast from shared memory; DS uses
-                          * the one-i-per-thread variant wherever its 64-i blocks pad the
-                          * block by at most 3/4 of the 256-i blocks (n_active <= 192,
-                          * 257..384, 513..576), four i per thread otherwise */
+#define NB_FORCE_IPAR 1  /* i across threads, j tiles broadcast from shared memory; DS takes
+                          * one or four i per thread (blocks of 64 or 256), whichever its
+                          * time model rates faster, up to 2560 active, above that four */
 #define NB_FORCE_JPAR 2  /* j across threads, warp-shuffle tree reduction (small n_active) */
 
 /*

@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(NT) k_force_ipar_ds(ForceArgs fa, JDS J)
                         pair_ds_packed<SOFT, true>(p, l, v, I[r], eps2, ta[r], tk[r], tp[r], jt + jj, ii[r]);
                 }
             } else {
-#pragma unroll (kIparUnroll)
+#pragma unroll (R == kIparR ? kIparUnroll : kIparSmallUnroll)
                 for (int jj = 0; jj < TL; ++jj) {
                     const float4 p = s_p[jj], l = s_l[jj], v = s_v[jj];
 #pragma unroll

@@ -237,10 +237,24 @@ __global__ void k_sched_scatter(State s, Ctrl *ctrl, const long long *blockmin, 
             running += tot;
         }
     }
+    // a small problem's candidate plans are weighed by the lanes of a warp
+    int fine = -1;
+    if (blockIdx.x == nblocks - 1 && warp == 0 && pre + running > 0 && fine_applies(fa, pre + running)) {
+        static_assert(kFineCands == 32, "one candidate per lane");
+        const unsigned long long t = fine_cost(pre + running, fa.n, fa.sms, fa.part_cap, lane);
+        unsigned long long best = t;
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) {
+            const unsigned long long y = __shfl_xor_sync(0xffffffffu, best, o);
+            best = y < best ? y : best;
+        }
+        const unsigned who = __ballot_sync(0xffffffffu, t == best);   // the first, as fine_best
+        fine = best == ~0ULL ? -1 : __ffs(who) - 1;
+    }
     if (blockIdx.x == nblocks - 1 && threadIdx.x == 0) {
         const int total = pre + running;
         ctrl->n_active = total;
-        *plan_out = make_force_plan(fa, total);   // the force launches read it
+        *plan_out = make_force_plan(fa, total, fine);   // the force launches read it
         if (total > 0) {
             ctrl->t_now = tn;
             ctrl->steps += 1;

@@ -193,6 +193,7 @@ ForceArgs force_args(nb_ctx *c, const int *act, int na_host, const int *na_dev, 
     fa.slots_ipar = c->slots_ipar;
     fa.slots_jpar = c->slots_jpar;
     fa.slots_small = c->slots_small;
+    fa.sms = c->sms;
     fa.part_cap = c->part_cap;
     fa.part = c->d_part;
     fa.jcnt = c->d_jcnt;

@@ -79,9 +79,19 @@ constexpr int kJparIC = 4;     // i per pass, j-parallel kernels
 constexpr int kJparIC1Max = 2;  // DS j-parallel kernel: one i per pass up to this block size
 constexpr int kJparMaxActive = 96;     // automatic mode, DS: j-parallel up to this block size
 constexpr int kJparMaxActive64 = 32;   // automatic mode, FP64
+#ifndef NB_U1
+#define NB_U1 2
+#endif
+constexpr int kIparSmallUnroll = NB_U1;  // its j unrolling (2, 4, 8: 169, 173, 171 us for 1820 active on 65536)
 constexpr int kIparSmallR = 1;      // i per thread of the small-block DS i-parallel kernel
 constexpr int kSmallMaxActive = 1024;  // automatic mode: small-block kernel considered up to this size
 constexpr int kComp = 7;       // acc xyz, jerk xyz, pot
+// Clocks per j of an i-parallel CTA alone on its SM, and of each CTA with the SM full, for the
+// four-i and the one-i kernel, and how many are resident (see fine_cost).
+constexpr unsigned kFineAlone4 = 200, kFineEach4 = 95, kFineRes4 = 4;
+constexpr unsigned kFineAlone1 = 105, kFineEach1 = 24, kFineRes1 = 16;
+constexpr unsigned kFineItemJ = 32;
+constexpr int kFineMaxActive = 2560;
 
 struct Plan {
     int n_iblk;   // i-blocks (i-parallel) or i-chunks (j-parallel)
@@ -295,6 +305,56 @@ __host__ __device__ inline int regime_of(int na, int jpar_max, int small_max)
     return kRegIpar;
 }
 
+// DS i-parallel, up to kFineMaxActive active: kernel and slice length are
+// chosen together, by the time of the busiest SM.  Candidate c: the four-i
+// (c < 16) or the one-i kernel, with the slice length in tiles that makes
+// c % 16 + 1 waves of its resident CTAs (a single tile where that is already
+// less than a wave).  An SM given m items runs them `res` at a time; k items
+// together cost max(alone, k each) clocks per j (one CTA alone cannot hide its
+// latencies) and kFineItemJ j more per item.  Both kernels sum the same 128-j
+// tiles in the same order, so the choice does not show in the tile partials.
+//
+// The one-i kernel reaches 90% of the four-i kernel's rate on full blocks,
+// pads the block to 64 instead of 256 and cuts it four times as fine, so it
+// wins wherever the padding or a part-filled GPU costs the other more than a
+// tenth.  Force and combine, us, four-i plan before / this rule: 256 active
+// on 256 bodies 42 / 17, 1024 on 1024 44 / 19, 4096 on 4096 49 / 40, 300 on
+// 4096 25 / 19, 700 on 65536 100 / 79, 1024 on 65536 118 / 104.  Above
+// kFineMaxActive (ten blocks of the four-i kernel) the padding is below that
+// tenth and plan_ipar's search, which also runs blocks whole, is kept.
+constexpr int kFineCands = 32;
+__host__ __device__ inline unsigned fine_clocks(unsigned m, unsigned res, unsigned alone, unsigned each)
+{
+    const unsigned rem = m % res;
+    unsigned t = m / res * (res * each);
+    if (rem) t += rem * each > alone ? rem * each : alone;
+    return t;
+}
+
+// Slice length in tiles of candidate c.
+__host__ __device__ inline unsigned fine_tiles(int na, int n, int sms, int c)
+{
+    const bool one = c >= 16;
+    const unsigned tiles = ucdiv((unsigned)n, (unsigned)(kIparNT * kIparTileMult));
+    const unsigned nib = ucdiv((unsigned)na, (unsigned)(kIparNT * (one ? kIparSmallR : kIparR)));
+    const unsigned slots = (unsigned)sms * (one ? kFineRes1 : kFineRes4) * (unsigned)(c % 16 + 1);
+    return (unsigned)(((unsigned long long)tiles * nib + slots - 1) / slots);
+}
+
+// Relative time of candidate c for na active on n (~0: not possible).
+__host__ __device__ inline unsigned long long fine_cost(int na, int n, int sms, long long part_cap, int c)
+{
+    const bool one = c >= 16;
+    const unsigned tile = (unsigned)(kIparNT * kIparTileMult), L = fine_tiles(na, n, sms, c);
+    const unsigned nib = ucdiv((unsigned)na, (unsigned)(kIparNT * (one ? kIparSmallR : kIparR)));
+    const unsigned S = ucdiv(ucdiv((unsigned)n, tile), L);
+    if (S > 1 && (long long)S * kComp * na > part_cap) return ~0ULL;
+    const unsigned m = ucdiv(nib * S, (unsigned)sms);
+    return (unsigned long long)(L * tile + kFineItemJ) *
+           (one ? fine_clocks(m, kFineRes1, kFineAlone1, kFineEach1)
+                : fine_clocks(m, kFineRes4, kFineAlone4, kFineEach4));
+}
+
 // The work decomposition of one force launch: the block size, the kernel
 // that serves it and that kernel's plan.  It is computed once per launch, by
 // make_force_plan on the host when the block size is known there, else by the
@@ -323,6 +383,7 @@ struct ForceArgs {
     int small_max;
     int split;                // forced slice count for i-parallel, 0 = auto
     int slots_ipar, slots_jpar, slots_small;
+    int sms;                  // SMs of the device (0: no fine plans)
     long long part_cap;       // capacity of part in doubles
     double *part;             // slice partials: part[(s * 7 + c) * na + a]; the DS
                               // j-parallel kernel: part[(chunk * 7 ic + e) * S + s]
@@ -359,7 +420,29 @@ constexpr int kSortCtas = 4;        // and at least this many per SM
 constexpr int kErrFixedScale = 64;  // device error word: fixed-point scales out of range
 constexpr int kErrInput = 65;       // device error word: a non-finite value or a negative mass
 
-__host__ __device__ inline ForcePlan make_force_plan(const ForceArgs &fa, int na)
+// Whether a block of na is planned by fine_cost (also a larger one whose
+// four-i items of one tile are less than a wave), and its cheapest candidate.
+__host__ __device__ inline bool fine_applies(const ForceArgs &fa, int na)
+{
+    return fa.sms > 0 && fa.precision == NB_DS && fa.summation == NB_SUM_COMPENSATED && fa.split == 0 &&
+           na > fa.jpar_max &&
+           (na <= kFineMaxActive ||
+            (long long)cdiv(fa.n, kIparNT * kIparTileMult) * cdiv(na, kIparNT * kIparR) <= fa.slots_ipar);
+}
+__host__ __device__ inline int fine_best(const ForceArgs &fa, int na)
+{
+    unsigned long long best = ~0ULL;
+    int bc = -1;
+    for (int c = 0; c < kFineCands; ++c) {
+        const unsigned long long t = fine_cost(na, fa.n, fa.sms, fa.part_cap, c);
+        if (t < best) best = t, bc = c;
+    }
+    return bc;
+}
+
+// fine: the cheapest fine candidate where fine_applies, found by the caller
+// (the scheduler's warp evaluates all candidates at once); -2 = find it here.
+__host__ __device__ inline ForcePlan make_force_plan(const ForceArgs &fa, int na, int fine = -2)
 {
     ForcePlan f{};
     f.na = na;
@@ -372,6 +455,17 @@ __host__ __device__ inline ForcePlan make_force_plan(const ForceArgs &fa, int na
     }
     if (fa.summation != NB_SUM_COMPENSATED) return f;   // no slices
     const bool f64 = fa.precision == NB_FP64;
+    if (fine == -2) fine = fine_applies(fa, na) ? fine_best(fa, na) : -1;
+    if (fine >= 0) {
+        const bool one = fine >= 16;
+        f.regime = one ? kRegSmall : kRegIpar;
+        f.p.n_iblk = cdiv(na, kIparNT * (one ? kIparSmallR : kIparR));
+        f.p.jslice = (int)fine_tiles(na, fa.n, fa.sms, fine) * kIparNT * kIparTileMult;
+        f.p.S = cdiv(fa.n, f.p.jslice);
+        f.p.items = f.p.n_iblk * f.p.S;
+        f.lanes = combine_lanes(na, f.p.S);
+        return f;
+    }
     f.regime = f64 ? (use_jpar(na, fa.jpar_max) ? kRegJpar : kRegIpar)
                    : regime_of(na, fa.jpar_max, fa.small_max);
     if (f.regime == kRegJpar) {

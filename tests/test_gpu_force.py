@@ -237,3 +237,17 @@ def test_jpar_slice_counters_reset_between_calls(nb):
     ref = oracle.force(m, x, v, EPS, blocks[0], nthreads=8)
     mags = pair_magnitudes(m, x, v, EPS, blocks[0])
     assert_force_close(first[0], ref, mags, TOL_DS, "na=5 N=300000")
+
+
+@pytest.mark.parametrize("n,na", [(97, 97), (128, 100), (129, 129), (1000, 257), (3000, 2560), (3000, 2561),
+                                  (20000, 1820)])
+def test_kernel_and_slices_chosen_together(nb, n, na):
+    # one tile, one tile and a particle, blocks on both sides of a 64- and a
+    # 256-i boundary and of the largest block planned so; the slices change
+    # nothing above FP64 rounding, so a forced slice count gives the same force
+    m, x, v = plummer(n, 61 + n)
+    idx = sample_active(n, na, 7)
+    _, got = _check(nb, m, x, v, EPS, idx, 0, label="n=%d na=%d" % (n, na))
+    _, forced = _check(nb, m, x, v, EPS, idx, 0, split=3, label="split, n=%d na=%d" % (n, na))
+    for g, f in zip(got, forced):
+        assert np.allclose(g, f, rtol=1e-12, atol=1e-12 * np.abs(f).max())

@@ -283,3 +283,69 @@ def test_tail_split_plans_random(planner):
         elif S > 1:
             assert S * 7 * na <= cap, c
     assert seen > 500
+
+
+SRC_FINE = r'''
+#include <cstdio>
+#include "nb_internal.cuh"
+using namespace nbk;
+int main() {
+    int na, n, sms; long long cap;
+    while (std::scanf("%d %d %d %lld", &na, &n, &sms, &cap) == 4) {
+        ForceArgs fa{};
+        fa.n = n;
+        fa.precision = NB_DS;
+        fa.summation = NB_SUM_COMPENSATED;
+        fa.jpar_max = kJparMaxActive;
+        fa.small_max = kSmallMaxActive;
+        fa.sms = sms;
+        fa.slots_ipar = 4 * sms;
+        fa.slots_jpar = 2 * sms;
+        fa.slots_small = 16 * sms;
+        fa.part_cap = cap;
+        const ForcePlan f = make_force_plan(fa, na);
+        long long cover = 0;
+        int bad = 0;
+        for (int w = 0; w < f.p.items; ++w) {
+            int ib, sl, j0, j1;
+            ipar_item(w, f.p.n_iblk, f.p.n_whole, f.p.S, f.p.jslice, n, ib, sl, j0, j1);
+            bad += ib < 0 || ib >= f.p.n_iblk || sl >= f.p.S || (sl < 0) != (ib < f.p.n_whole || f.p.S == 1);
+            cover += j1 > j0 ? j1 - j0 : 0;
+        }
+        std::printf("%d %d %d %d %d %d %d %lld %d %d\n", f.regime, f.p.n_iblk, f.p.S, f.p.jslice, f.p.items,
+                    f.p.n_whole, f.lanes, cover, bad, fine_applies(fa, na) ? fine_best(fa, na) : -1);
+    }
+    return 0;
+}
+'''
+
+
+def test_fine_plans(tmp_path):
+    # kernel and slices chosen together: every (i-block, j) once, whole tiles,
+    # partials within the buffer, and the chosen candidate is the plan
+    cxx = shutil.which("g++")
+    cuda_inc = "/usr/local/cuda/include"
+    if not cxx or not os.path.isdir(cuda_inc):
+        pytest.skip("needs g++ and the CUDA headers")
+    src = tmp_path / "fine.cpp"
+    src.write_text(SRC_FINE)
+    exe = tmp_path / "fine"
+    subprocess.run([cxx, "-std=c++17", "-O1", "-I" + os.path.join(ROOT, "include"),
+                    "-I" + os.path.join(ROOT, "paper_cs_0702135_gb300", "csrc"), "-I" + cuda_inc,
+                    str(src), "-o", str(exe)], check=True)
+    cases = []
+    for na, n, sms in itertools.product(
+            [97, 128, 129, 256, 257, 1000, 1820, 2560, 2561, 4096, 9000],
+            [97, 128, 129, 1000, 4096, 16384, 65536, 1 << 20], [1, 152]):
+        if na <= n:
+            cases.append((na, n, sms, 7 * max(16 * 4 * sms * 256, 4 * n)))
+    for c, out in zip(cases, _run(exe, cases)):
+        na, n, sms, cap = c
+        regime, nib, S, js, items, n_whole, lanes, cover, bad, cand = out
+        assert regime in (1, 2) and bad == 0, c
+        assert nib == -(-na // (64 if regime == 1 else 256)), c
+        assert cover == nib * n and js % 128 == 0 and (S - 1) * js < n <= S * js, c
+        assert S == 1 or n_whole or S * 7 * na <= cap, c
+        assert lanes in (1, 2, 4, 8, 16, 32) and (lanes == 1 or lanes <= S), c
+        if na <= 2560:
+            assert cand >= 0 and n_whole == 0 and regime == (1 if cand >= 16 else 2), c
