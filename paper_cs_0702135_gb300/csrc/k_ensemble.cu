@@ -443,9 +443,94 @@ __global__ void __launch_bounds__(NT) k_ens_step(EnsArgs ea)
 
 // Energy of every cluster at its particles' own times (exact when the cluster
 // is synchronised): kinetic from FP64 velocities, potential as the FP64 pair
-// sum -sum_{i<j} m_i m_j / sqrt(r^2 + eps^2), per cluster in a fixed order.
+// sum -sum_{i<j} m_i m_j / sqrt(r^2 + eps^2), in a fixed order.
+//
+// The pair sum is bound by the FP64 pipe (2 lanes a clock per SM), so it is cut
+// into tiles of 128 x 128 pairs (ti <= tj) of every cluster, one CTA each, for
+// all SMs to share, and 1/sqrt takes five FP64 operations on an FP32 seed
+// instead of a square root and a division (~14): per pair 12.  256 clusters of
+// 32..4096 (2.2e8 pairs): 6.1 ms with the copies; one CTA per cluster with the square root
+// and the division waited for the largest cluster, 96 ms.
+
+constexpr int kEnTile = 128;
+
+__host__ __device__ inline long long en_items(int n)
+{
+    const long long t = (n + kEnTile - 1) / kEnTile;
+    return t * (t + 1) / 2;
+}
+
+// 1/sqrt(x): the SFU's FP32 value y0 (relative error about 2^-22), then
+// y0 + y0 e (1/2 + 3/8 e) with e = 1 - x y0^2, the series of (1 - e)^(-1/2)
+// to second order (the next term is below 2^-66).  The FP64 <-> FP32 steps are
+// bit moves: conversions run on the FP64 pipe.
+__device__ __forceinline__ double rsqrt_pair(double x)
+{
+    if (!split_safe(x)) return rsqrt(x);
+    const unsigned xh = (unsigned)__double2hiint(x), xl = (unsigned)__double2loint(x);
+    const float y = rsqrt_sfu(__uint_as_float((xh - (896u << 20)) << 3 | xl >> 29));   // truncated
+    const unsigned yb = __float_as_uint(y);
+    const double y0 = __hiloint2double((int)((yb >> 3) + (896u << 20)), (int)(yb << 29));
+    const double e = fma(-(x * y0), y0, 1.0);
+    return fma(fma(e, 0.375, 0.5), y0 * e, y0);
+}
+
+// Potential of pair tile blockIdx.x: item[] holds each cluster's first tile.
+__global__ void __launch_bounds__(kEnTile) k_ens_pairs(EnsArgs ea, const int *item, double eps2, double *part)
+{
+    __shared__ double4_32a s_j[kEnTile];
+    __shared__ double s_red[kEnTile / 32];
+    const State &S = ea.s;
+    const long long P = S.n;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int c = 0;   // the last cluster whose first tile is not past this one
+    for (int hi = ea.C - 1; c < hi;) {
+        const int mid = (c + hi + 1) / 2;
+        if (item[mid] <= (int)blockIdx.x) c = mid;
+        else hi = mid - 1;
+    }
+    const int k = blockIdx.x - item[c];
+    int tj = (int)((sqrtf(8.0f * (float)k + 1.0f) - 1.0f) * 0.5f);
+    while ((tj + 1) * (tj + 2) / 2 <= k) ++tj;
+    while (tj * (tj + 1) / 2 > k) --tj;
+    const int ti = k - tj * (tj + 1) / 2;
+    const long long o = ea.off[c];
+    const int n = (int)(ea.off[c + 1] - o);
+    const int i0 = ti * kEnTile + warp * 32, i = i0 + lane, j0 = tj * kEnTile, jc = min(kEnTile, n - j0);
+    if (tid < jc) {
+        const long long gj = o + j0 + tid;
+        s_j[tid] = make_double4_32a(S.x[gj], S.x[P + gj], S.x[2 * P + gj], S.m[gj]);
+    }
+    __syncthreads();
+    double row = 0.0, mi = 0.0;
+    if (i0 < n) {
+        const long long gi = o + min(i, n - 1);
+        const double xi = S.x[gi], yi = S.x[P + gi], zi = S.x[2 * P + gi];
+        mi = S.m[gi];
+        // on the diagonal a warp starts past its own first particle
+#pragma unroll 4
+        for (int q = ti == tj ? warp * 32 + 1 : 0; q < jc; ++q) {
+            const double4_32a p = s_j[q];
+            const double dx = p.x - xi, dy = p.y - yi, dz = p.z - zi;
+            const double r2 = fma(dx, dx, fma(dy, dy, fma(dz, dz, eps2)));
+            const double y = rsqrt_pair(r2);
+            // i < j holds off the diagonal (lanes past the end are dropped
+            // below); a pair left out may be infinite, so its term is not formed
+            if (j0 + q > i) row = fma(p.w, y, row);
+        }
+    }
+    row = i < n ? mi * row : 0.0;   // a particle past the end
+#pragma unroll
+    for (int off = 16; off >= 1; off >>= 1) row += __shfl_xor_sync(0xffffffffu, row, off);
+    if (lane == 0) s_red[warp] = row;
+    __syncthreads();
+    if (tid == 0) part[blockIdx.x] = -((s_red[0] + s_red[1]) + (s_red[2] + s_red[3]));
+}
+
+// Kinetic energies, and the sums of the clusters' tiles.
 template <int NT>
-__global__ void __launch_bounds__(NT) k_ens_energy(EnsArgs ea, double eps2, double *ekin, double *epot)
+__global__ void __launch_bounds__(NT) k_ens_energy(EnsArgs ea, const int *item, const double *part,
+                                                   double *ekin, double *epot)
 {
     __shared__ double s_red[NT / 32];
     const int tid = threadIdx.x;
@@ -459,15 +544,8 @@ __global__ void __launch_bounds__(NT) k_ens_energy(EnsArgs ea, double eps2, doub
             const long long gi = o + i;
             const double vx = S.v[gi], vy = S.v[P + gi], vz = S.v[2 * P + gi];
             ke += 0.5 * S.m[gi] * (vx * vx + vy * vy + vz * vz);
-            const double xi = S.x[gi], yi = S.x[P + gi], zi = S.x[2 * P + gi];
-            double row = 0.0;
-            for (int j = i + 1; j < n; ++j) {
-                const long long gj = o + j;
-                const double dx = S.x[gj] - xi, dy = S.x[P + gj] - yi, dz = S.x[2 * P + gj] - zi;
-                row += S.m[gj] / sqrt(dx * dx + dy * dy + dz * dz + eps2);
-            }
-            pe -= S.m[gi] * row;
         }
+        for (int q = item[c] + tid; q < item[c + 1]; q += NT) pe += part[q];
         struct Add {
             __device__ double operator()(double a, double b) const { return a + b; }
         };
@@ -529,6 +607,8 @@ struct nb_ens {
     long long qcap = 0;
     long long *d_steps = nullptr, *d_inter = nullptr;
     double *d_stage = nullptr;   // [7 P] host I/O staging
+    int *d_item = nullptr;       // [C + 1] first pair tile of each cluster (energies)
+    int items = 0;
     double *d_backup = nullptr;  // state copy for tuning
     long long *d_tbak = nullptr;
     int *d_lbak = nullptr;
@@ -708,7 +788,7 @@ void ens_release(nb_ens *e)
                     e->d_lev, e->d_work, e->d_done, e->d_err, e->d_steps, e->d_inter,
                     e->d_stage, e->d_backup, e->d_tbak, e->d_lbak, e->d_jph, e->d_jpl, e->d_jv,
                     e->d_mirror,
-                    e->d_act, e->d_na, e->d_qc, e->d_qk, e->d_tnext, e->d_pred};
+                    e->d_act, e->d_na, e->d_qc, e->d_qk, e->d_tnext, e->d_pred, e->d_item};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (e->own_stream && e->st) cudaStreamDestroy(e->st);
@@ -779,8 +859,12 @@ int ens_init_impl(nb_ens *e, int32_t C, const int64_t *off, const double *m, con
         (rc = ealloc(e, &e->d_act, P)) || (rc = ealloc(e, &e->d_na, C)) ||
         (rc = ealloc(e, &e->d_tnext, C)) || (rc = ealloc(e, &e->d_qc, P + C)) ||
         (rc = ealloc(e, &e->d_qk, P + C)) || (rc = ealloc(e, &e->d_pred, C)) ||
-        (rc = ealloc(e, &e->d_mirror, 5 * P)))
+        (rc = ealloc(e, &e->d_mirror, 5 * P)) || (rc = ealloc(e, &e->d_item, C + 1)))
         return rc;
+    // at most one tile per particle, so the tile sums fit the staging buffer
+    std::vector<int> item(C + 1, 0);
+    for (int c = 0; c < C; ++c) item[c + 1] = item[c] + (int)en_items((int)(off[c + 1] - off[c]));
+    e->items = item[C];
     e->S.x = e->d_x;
     e->S.v = e->d_v;
     e->S.a = e->d_a;
@@ -791,6 +875,7 @@ int ens_init_impl(nb_ens *e, int32_t C, const int64_t *off, const double *m, con
     e->S.n = (int)P;
     ECK(cudaMemcpyAsync(e->d_off, off, sizeof(long long) * (C + 1), cudaMemcpyHostToDevice, e->st));
     ECK(cudaMemcpyAsync(e->d_order, order.data(), sizeof(int) * C, cudaMemcpyHostToDevice, e->st));
+    ECK(cudaMemcpyAsync(e->d_item, item.data(), sizeof(int) * (C + 1), cudaMemcpyHostToDevice, e->st));
     ECK(cudaMemcpyAsync(e->d_m, m, sizeof(double) * P, cudaMemcpyHostToDevice, e->st));
     ECK(cudaMemcpyAsync(e->d_stage, x, sizeof(double) * 3 * P, cudaMemcpyHostToDevice, e->st));
     k_aos_to_soa<<<grid_of(3 * P), 256, 0, e->st>>>(e->d_stage, e->d_x, P);
@@ -1032,9 +1117,12 @@ int nb_ens_energy(nb_ens *e, double *ekin, double *epot)
     const EnsRange range_("nb_ens_energy");
     if (!e) return NB_EINVAL;
     double *d = e->d_stage;
+    double *part = d + 2LL * e->C;
+    k_ens_pairs<<<e->items, kEnTile, 0, e->st>>>(ens_args(e), e->d_item, e->eps * e->eps, part);
     k_ens_energy<256><<<std::max(1, std::min(e->C, 8 * e->sms)), 256, 0, e->st>>>(
-        ens_args(e), e->eps * e->eps, d, d + e->C);
-    e->launches += 1;
+        ens_args(e), e->d_item, part, d, d + e->C);
+    ECK(cudaGetLastError());
+    e->launches += 2;
     if (ekin) ECK(cudaMemcpyAsync(ekin, d, sizeof(double) * e->C, cudaMemcpyDeviceToHost, e->st));
     if (epot) ECK(cudaMemcpyAsync(epot, d + e->C, sizeof(double) * e->C, cudaMemcpyDeviceToHost, e->st));
     return ens_sync(e);

@@ -210,3 +210,29 @@ def test_bad_arguments(nb):
     with pytest.raises(nb.NbError) as ei:
         nb.Ensemble(np.array([0, 4097]), *big, EPS)
     assert ei.value.code == nb.NB_EINVAL
+
+
+def test_energies_of_all_cluster_sizes(nb):
+    # sizes around the warps and the 128 x 128 pair tiles, up to the largest
+    # cluster; reference: numpy's FP64 pair sums, row by row.  Every pair term
+    # has a relative error below 2^-51, sums of one sign over at most 128 terms
+    # a lane and a tree on top add at most ~2^-46: 1e-13 holds with room.
+    sizes = [1, 2, 31, 32, 33, 127, 128, 129, 257, 500, 4096]
+    rng = np.random.RandomState(19)
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    P = int(off[-1])
+    m = rng.uniform(0.5, 2.0, P) / P
+    x, v = rng.normal(size=(P, 3)), rng.normal(size=(P, 3))
+    e = nb.Ensemble(off, m, x, v, EPS)
+    try:
+        ek, ep = e.nb_ens_energy()
+    finally:
+        e.nb_ens_free()
+    for c, n in enumerate(sizes):
+        s = slice(off[c], off[c + 1])
+        mc, xc, vc = m[s], x[s], v[s]
+        rows = [0.0] + [mc[i] * np.sum(mc[:i] / np.sqrt(np.sum((xc[:i] - xc[i]) ** 2, axis=1) + EPS * EPS))
+                        for i in range(1, n)]
+        W, T = -np.sum(rows), 0.5 * np.sum(mc * np.sum(vc * vc, axis=1))
+        assert abs(ep[c] - W) <= 1e-13 * abs(W), (n, ep[c], W)
+        assert abs(ek[c] - T) <= 1e-13 * T, (n, ek[c], T)
