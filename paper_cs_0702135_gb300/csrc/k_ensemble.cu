@@ -356,10 +356,12 @@ __device__ __forceinline__ void ens_b_item(const EnsArgs &ea, int c, int k, floa
         // every lane of the group holds the sums: its first four lanes correct
         // the particle together (the same FP64 operations as one lane would);
         // the CTA's other lanes run along inactive, as the quads need
-        const int qd = lig & 3, cq = qd < 3 ? qd : 2;
+        const int qd = lig & 3;
         const bool active = valid && lig < 4;
-        const bool ok = correct_particle_quad(S, gi, P, __ldcg(&ea.tnext[c]), res[cq], res[3 + cq],
-                                              ea.eta, ea.level_min, 0, active);
+        const bool ok = correct_particle_quad(S, gi, P, __ldcg(&ea.tnext[c]),
+                                              qd == 0 ? res[0] : (qd == 1 ? res[1] : res[2]),
+                                              qd == 0 ? res[3] : (qd == 1 ? res[4] : res[5]), ea.eta,
+                                              ea.level_min, 0, active);
         __syncwarp();
         if (active && qd == 0) {
             if (!ok) atomicCAS(ea.err, 0, NB_ESTEP);

@@ -433,17 +433,16 @@ __global__ void __launch_bounds__(kRunNT) k_run(RunArgs ra)
             const int i = i0 + tid;
             // predict3's arithmetic on the state loaded above
             const double dt = ticks_to_time(tn - p_t);
-            const double dt_h = __dmul_rn(dt, 0.5), dt_q = div_by<3>(dt);
+            const double dt_h = scale2(dt, -1), dt_q = div_by<3>(dt);
             double xp[3], vp[3];
 #pragma unroll
             for (int c = 0; c < 3; ++c)
                 predict1hq(p_x[c], p_v[c], p_a[c], p_k[c], dt, dt_h, dt_q, xp[c], vp[c]);
             float h[3], l[3];
 #pragma unroll
-            for (int c = 0; c < 3; ++c) split_ds(xp[c], h[c], l[c]);
-            const float mf = __double2float_rn(S.m[i]);
-            const float4 v4 = make_float4(__double2float_rn(vp[0]), __double2float_rn(vp[1]),
-                                          __double2float_rn(vp[2]), 0.0f);
+            for (int c = 0; c < 3; ++c) split_ds_int(xp[c], h[c], l[c]);
+            const float mf = to_float_int(S.m[i]);
+            const float4 v4 = make_float4(to_float_int(vp[0]), to_float_int(vp[1]), to_float_int(vp[2]), 0.0f);
             ra.j.pos_hi[i] = make_float4(h[0], h[1], h[2], mf);
             ra.j.pos_lo[i] = make_float4(l[0], l[1], l[2], 0.0f);
             ra.j.vel[i] = v4;

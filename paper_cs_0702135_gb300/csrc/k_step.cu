@@ -39,11 +39,10 @@ __device__ __forceinline__ void predict_record(const State &s, int i, long long 
     } else {
         float hi[3], lo[3];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) split_ds(xp[c], hi[c], lo[c]);
-        jds.pos_hi[i] = make_float4(hi[0], hi[1], hi[2], __double2float_rn(m));
+        for (int c = 0; c < 3; ++c) split_ds_int(xp[c], hi[c], lo[c]);
+        jds.pos_hi[i] = make_float4(hi[0], hi[1], hi[2], to_float_int(m));
         jds.pos_lo[i] = make_float4(lo[0], lo[1], lo[2], 0.0f);
-        jds.vel[i] = make_float4(__double2float_rn(vp[0]), __double2float_rn(vp[1]),
-                                 __double2float_rn(vp[2]), 0.0f);
+        jds.vel[i] = make_float4(to_float_int(vp[0]), to_float_int(vp[1]), to_float_int(vp[2]), 0.0f);
     }
 }
 

@@ -14,9 +14,32 @@ namespace dev {
 
 constexpr double kTick = 0x1p-40;  // one tick in N-body time units
 
+// The GB300's FP64 pipe takes 2 lanes a clock per SM with 64 clocks of latency,
+// for conversions between integers, FP32 and FP64 as for arithmetic; what is
+// only a move of bits is done on the integer pipe (4 clocks) below.
+
+// d 2^-40, rounded to nearest.
 __device__ __forceinline__ double ticks_to_time(long long d)
 {
+    if (d > 0 && d < (1LL << 53)) {   // exact: the significand's bits moved into place
+        const int sh = __clzll(d) - 11;
+        const unsigned long long m = (unsigned long long)d << sh;   // leading one at bit 52
+        return __longlong_as_double((long long)(m + ((unsigned long long)(1023 + 52 - 40 - 1 - sh) << 52)));
+    }
     return __dmul_rn(__ll2double_rn(d), kTick);
+}
+
+// 2^e as FP64, -1022 <= e <= 1023.
+__device__ __forceinline__ double pow2d(int e) { return __hiloint2double((1023 + e) << 20, 0); }
+
+// x 2^e, |e| <= 130: the exponent field moved (exact), or the multiplication
+// where the field is not well inside its range (zero, tiny, huge, not finite).
+__device__ __forceinline__ double scale2(double x, int e)
+{
+    const int hi = __double2hiint(x);
+    if (((unsigned)hi & 0x7fffffffu) - (200u << 20) < (1600u << 20))
+        return __hiloint2double(hi + (e << 20), __double2loint(x));
+    return __dmul_rn(x, pow2d(e));
 }
 
 // 1/sqrt(x) on the SFU: the PTX approximate reciprocal square root with
@@ -136,7 +159,7 @@ template <bool CG = false>
 __device__ __forceinline__ void predict3(const State &s, long long i, long long n, double dt,
                                          double xp[3], double vp[3])
 {
-    const double h = __dmul_rn(dt, 0.5), q = div_by<3>(dt);
+    const double h = scale2(dt, -1), q = div_by<3>(dt);
 #pragma unroll
     for (int c = 0; c < 3; ++c)
         predict1hq(ldst<CG>(&s.x[c * n + i]), ldst<CG>(&s.v[c * n + i]), ldst<CG>(&s.a[c * n + i]),
@@ -224,7 +247,7 @@ __device__ __forceinline__ int next_level(int k_old, int k_q, long long t_new, i
     if (k_q > k_old) return k_q;
     if (k_q < k_old && k_old > kmin) {
         const long long twice_old = 1LL << (kTickBits - k_old + 1);
-        if (t_new % twice_old == 0) return k_old - 1;
+        if ((t_new & (twice_old - 1)) == 0) return k_old - 1;
     }
     return k_old;
 }
@@ -235,6 +258,81 @@ __device__ __forceinline__ double initial_dt(const double a[3], const double k[3
     const double nk = norm3(k[0], k[1], k[2]);
     return nk == 0.0 ? (double)INFINITY : __ddiv_rn(__dmul_rn(eta_init, norm3(a[0], a[1], a[2])), nk);
 }
+
+// Level of the Aarseth step
+//   dt_raw = sqrt(eta (|a| |s| + |k|^2) / (|k| |c| + |s|^2))
+// from FP32 values of the four squared norms, where they decide it: dt_raw's
+// binade is that of the FP32 estimate R of dt_raw^2 unless R lies within 2^-12
+// of a power of four, and the estimate's error, with conversions, three-term
+// sums, approximate square roots and the division, is below 2^-18.  False (the
+// caller evaluates the FP64 formulas) there, and where a norm or R is outside
+// the range in which FP32 keeps its precision (zero and non-finite included).
+// A square root or division in FP64 takes ~600 clocks, this ~100.
+__device__ __forceinline__ float sqrt_sfu(float x)
+{
+    float y;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ bool level_estimate(float na2, float nk2, float ns2, float nc2, float eta, int kmin,
+                                               int &level)
+{
+    const float lo = fminf(fminf(na2, nk2), fminf(ns2, nc2)), hi = fmaxf(fmaxf(na2, nk2), fmaxf(ns2, nc2));
+    const float num = fmaf(sqrt_sfu(na2), sqrt_sfu(ns2), nk2);
+    const float den = fmaf(sqrt_sfu(nk2), sqrt_sfu(nc2), ns2);
+    const float R = __fdividef(eta * num, den);
+    if (!(lo >= 0x1p-100f && hi <= 0x1p110f && R >= 0x1p-72f && R <= 0x1p60f) ||
+        !(na2 == na2 && nk2 == nk2 && ns2 == ns2 && nc2 == nc2))
+        return false;
+    const int b = __float_as_int(R), e = (b >> 23) - 127, m = b & 0x7fffff;
+    if ((e & 1) ? m >= 0x800000 - 0x800 : m < 0x800) return false;
+    level = max(-(e >> 1), kmin);
+    return true;
+}
+
+// The corrector's arithmetic for one axis when the step is a power of two,
+// dt = 2^e (every block step): multiplications by powers of two move the
+// exponent (scale2), dt/3 is the rounded third with its exponent moved, and
+// the other operations are those of correct_particle in its order, so the
+// results are the same bits with 27 FP64 operations instead of ~47.
+struct AxisStep {
+    double x, v, s1, c;   // new position and velocity; s1 and crackle of the step criterion
+};
+__device__ __forceinline__ AxisStep correct_axis(double x, double v, double a, double k, double ap, double kp,
+                                                 int e)
+{
+    AxisStep r;
+    const double w = __dadd_rn(a, scale2(__dmul_rn(1.0 / 3.0, k), e));
+    const double xp = __dadd_rn(x, scale2(__dadd_rn(v, scale2(w, e - 1)), e));
+    const double vp = __dadd_rn(v, scale2(__dadd_rn(a, scale2(k, e - 1)), e));
+    const double d = __dsub_rn(a, ap);
+    const double a3 = __dadd_rn(scale2(d, 1), scale2(__dadd_rn(k, kp), e));
+    const double a2 = __dsub_rn(__dmul_rn(-3.0, d), scale2(__dadd_rn(scale2(k, 1), kp), e));
+    r.x = __dadd_rn(xp, scale2(__dadd_rn(div_by<12>(a2), div_by<20>(a3)), 2 * e));
+    r.v = __dadd_rn(vp, scale2(__dadd_rn(div_by<3>(a2), scale2(a3, -2)), e));
+    r.c = scale2(__dmul_rn(6.0, a3), -3 * e);
+    r.s1 = __dadd_rn(scale2(a2, 1 - 2 * e), scale2(r.c, e));
+    return r;
+}
+
+// e of a step of `ticks` = 2^(e + 40) ticks; false for any other step.
+__device__ __forceinline__ bool step_exponent(long long ticks, int &e)
+{
+    e = 63 - kTickBits - __clzll(ticks);
+    return ticks > 0 && (ticks & (ticks - 1)) == 0 && e >= -kTickBits && e <= 0;
+}
+
+// The Aarseth step's level from the FP64 norms (false: below 2^-40).
+__device__ __forceinline__ bool level_exact(double na, double nk, double ns, double nc, double eta, int kmin,
+                                            int &level)
+{
+    const double num = __dadd_rn(__dmul_rn(na, ns), __dmul_rn(nk, nk));
+    const double den = __dadd_rn(__dmul_rn(nk, nc), __dmul_rn(ns, ns));
+    const double dt_raw = den == 0.0 ? (double)INFINITY : __dsqrt_rn(__ddiv_rn(__dmul_rn(eta, num), den));
+    return level_of(dt_raw, kmin, level);
+}
+
+__device__ __forceinline__ float norm2_f(float x, float y, float z) { return fmaf(x, x, fmaf(y, y, z * z)); }
 
 // Hermite corrector and Aarseth step for particle i of `s` (Section 2).  In
 // the paper's notation a, k are the old values (in s) and a_p, k_p the new:
@@ -250,63 +348,69 @@ __device__ __forceinline__ bool correct_particle(const State &s, long long i, lo
                                                  long long tn, const double ap[3], const double kp[3],
                                                  double eta, int level_min, int level_fixed)
 {
-    const double dt = ticks_to_time(tn - ldst<CG>(&s.t[i]));
-    const double h = __dmul_rn(dt, 0.5), q = div_by<3>(dt);
-    double a2[3], a3[3];
+    const long long ticks = tn - ldst<CG>(&s.t[i]);
+    double s1[3], cr[3];
+    int ex;
+    if (step_exponent(ticks, ex)) {
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const long long e = c * stride + i;
-        const double x = ldst<CG>(&s.x[e]), v = ldst<CG>(&s.v[e]), a = ldst<CG>(&s.a[e]),
-                     k = ldst<CG>(&s.k[e]);
-        double xp, vp;
-        predict1hq(x, v, a, k, dt, h, q, xp, vp);
-        const double d = __dsub_rn(a, ap[c]);
-        a3[c] = __dadd_rn(__dmul_rn(2.0, d), __dmul_rn(__dadd_rn(k, kp[c]), dt));
-        a2[c] = __dsub_rn(__dmul_rn(-3.0, d), __dmul_rn(__dadd_rn(__dmul_rn(2.0, k), kp[c]), dt));
-        s.x[e] = __dadd_rn(xp, __dmul_rn(__dadd_rn(div_by<12>(a2[c]), div_by<20>(a3[c])),
-                                         __dmul_rn(dt, dt)));
-        // a3 / 4 as a3 * 0.25: the same real number, so the same rounded result
-        s.v[e] = __dadd_rn(vp, __dmul_rn(__dadd_rn(div_by<3>(a2[c]), __dmul_rn(a3[c], 0.25)), dt));
-        s.a[e] = ap[c];
-        s.k[e] = kp[c];
+        for (int c = 0; c < 3; ++c) {
+            const long long e = c * stride + i;
+            const AxisStep r = correct_axis(ldst<CG>(&s.x[e]), ldst<CG>(&s.v[e]), ldst<CG>(&s.a[e]),
+                                            ldst<CG>(&s.k[e]), ap[c], kp[c], ex);
+            s.x[e] = r.x;
+            s.v[e] = r.v;
+            s.a[e] = ap[c];
+            s.k[e] = kp[c];
+            s1[c] = r.s1;
+            cr[c] = r.c;
+        }
+    } else {
+        const double dt = ticks_to_time(ticks);
+        const double h = __dmul_rn(dt, 0.5), q = div_by<3>(dt);
+        const double dt2 = __dmul_rn(dt, dt);
+        const double dt3 = __dmul_rn(dt2, dt);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const long long e = c * stride + i;
+            const double x = ldst<CG>(&s.x[e]), v = ldst<CG>(&s.v[e]), a = ldst<CG>(&s.a[e]),
+                         k = ldst<CG>(&s.k[e]);
+            double xp, vp;
+            predict1hq(x, v, a, k, dt, h, q, xp, vp);
+            const double d = __dsub_rn(a, ap[c]);
+            const double a3 = __dadd_rn(__dmul_rn(2.0, d), __dmul_rn(__dadd_rn(k, kp[c]), dt));
+            const double a2 = __dsub_rn(__dmul_rn(-3.0, d), __dmul_rn(__dadd_rn(__dmul_rn(2.0, k), kp[c]), dt));
+            s.x[e] = __dadd_rn(xp, __dmul_rn(__dadd_rn(div_by<12>(a2), div_by<20>(a3)), dt2));
+            // a3 / 4 as a3 * 0.25: the same real number, so the same rounded result
+            s.v[e] = __dadd_rn(vp, __dmul_rn(__dadd_rn(div_by<3>(a2), __dmul_rn(a3, 0.25)), dt));
+            s.a[e] = ap[c];
+            s.k[e] = kp[c];
+            const double s0 = __ddiv_rn(__dmul_rn(2.0, a2), dt2);
+            cr[c] = __ddiv_rn(__dmul_rn(6.0, a3), dt3);
+            s1[c] = __dadd_rn(s0, __dmul_rn(cr[c], dt));
+        }
     }
     s.t[i] = tn;
     if (level_fixed > 0) {
         s.lev[i] = level_fixed;
         return true;
     }
-    const double dt2 = __dmul_rn(dt, dt);
-    const double dt3 = __dmul_rn(dt2, dt);
-    // A block step is a power of two: dividing by dt^2 and dt^3 is then the
-    // same real number as multiplying by their exact reciprocals (powers of
-    // two, from the exponent field), so the rounded results are identical and
-    // four FP64 divisions per axis leave the latency chain.
-    const bool pow2 = (__double_as_longlong(dt) & 0x000FFFFFFFFFFFFFLL) == 0 && dt > 0x1p-100;
-    const double r2 = pow2 ? __longlong_as_double((2046LL << 52) - (__double_as_longlong(dt2) & 0x7FF0000000000000LL)) : 0.0;
-    const double r3 = pow2 ? __longlong_as_double((2046LL << 52) - (__double_as_longlong(dt3) & 0x7FF0000000000000LL)) : 0.0;
-    double s1[3], cr[3];
+    float f[4][3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        double s0;
-        if (pow2) {
-            s0 = __dmul_rn(__dmul_rn(2.0, a2[c]), r2);
-            cr[c] = __dmul_rn(__dmul_rn(6.0, a3[c]), r3);
-        } else {
-            s0 = __ddiv_rn(__dmul_rn(2.0, a2[c]), dt2);
-            cr[c] = __ddiv_rn(__dmul_rn(6.0, a3[c]), dt3);
-        }
-        s1[c] = __dadd_rn(s0, __dmul_rn(cr[c], dt));
+        f[0][c] = to_float_int(ap[c]);
+        f[1][c] = to_float_int(kp[c]);
+        f[2][c] = to_float_int(s1[c]);
+        f[3][c] = to_float_int(cr[c]);
     }
-    const double na = norm3(ap[0], ap[1], ap[2]);
-    const double nk = norm3(kp[0], kp[1], kp[2]);
-    const double ns = norm3(s1[0], s1[1], s1[2]);
-    const double nc = norm3(cr[0], cr[1], cr[2]);
-    const double num = __dadd_rn(__dmul_rn(na, ns), __dmul_rn(nk, nk));
-    const double den = __dadd_rn(__dmul_rn(nk, nc), __dmul_rn(ns, ns));
-    const double dt_raw = den == 0.0 ? (double)INFINITY : __dsqrt_rn(__ddiv_rn(__dmul_rn(eta, num), den));
     int kq;
-    const bool ok = level_of(dt_raw, level_min, kq);
-    if (!ok) kq = kTickBits;
+    bool ok = true;
+    if (!level_estimate(norm2_f(f[0][0], f[0][1], f[0][2]), norm2_f(f[1][0], f[1][1], f[1][2]),
+                        norm2_f(f[2][0], f[2][1], f[2][2]), norm2_f(f[3][0], f[3][1], f[3][2]),
+                        to_float_int(eta), level_min, kq)) {
+        ok = level_exact(norm3(ap[0], ap[1], ap[2]), norm3(kp[0], kp[1], kp[2]), norm3(s1[0], s1[1], s1[2]),
+                         norm3(cr[0], cr[1], cr[2]), eta, level_min, kq);
+        if (!ok) kq = kTickBits;
+    }
     s.lev[i] = next_level(ldst<CG>(&s.lev[i]), kq, tn, level_min);
     return ok;
 }
@@ -325,15 +429,15 @@ __device__ __forceinline__ void write_mirror(const State &s, const Mirror &mr, l
 {
     float hi[3], lo[3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) split_ds(ldst<CG>(&s.x[c * n + i]), hi[c], lo[c]);
-    mr.h[i] = make_float4(hi[0], hi[1], hi[2], __double2float_rn(ldst<CG>(&s.m[i])));
+    for (int c = 0; c < 3; ++c) split_ds_int(ldst<CG>(&s.x[c * n + i]), hi[c], lo[c]);
+    mr.h[i] = make_float4(hi[0], hi[1], hi[2], to_float_int(ldst<CG>(&s.m[i])));
     mr.l[i] = make_float4(lo[0], lo[1], lo[2], 0.0f);
-    mr.v[i] = make_float4(__double2float_rn(ldst<CG>(&s.v[i])), __double2float_rn(ldst<CG>(&s.v[n + i])),
-                          __double2float_rn(ldst<CG>(&s.v[2 * n + i])), 0.0f);
-    mr.a[i] = make_float4(__double2float_rn(ldst<CG>(&s.a[i])), __double2float_rn(ldst<CG>(&s.a[n + i])),
-                          __double2float_rn(ldst<CG>(&s.a[2 * n + i])), 0.0f);
-    mr.k[i] = make_float4(__double2float_rn(ldst<CG>(&s.k[i])), __double2float_rn(ldst<CG>(&s.k[n + i])),
-                          __double2float_rn(ldst<CG>(&s.k[2 * n + i])), 0.0f);
+    mr.v[i] = make_float4(to_float_int(ldst<CG>(&s.v[i])), to_float_int(ldst<CG>(&s.v[n + i])),
+                          to_float_int(ldst<CG>(&s.v[2 * n + i])), 0.0f);
+    mr.a[i] = make_float4(to_float_int(ldst<CG>(&s.a[i])), to_float_int(ldst<CG>(&s.a[n + i])),
+                          to_float_int(ldst<CG>(&s.a[2 * n + i])), 0.0f);
+    mr.k[i] = make_float4(to_float_int(ldst<CG>(&s.k[i])), to_float_int(ldst<CG>(&s.k[n + i])),
+                          to_float_int(ldst<CG>(&s.k[2 * n + i])), 0.0f);
 }
 
 // (hi, lo) + d in double-single: TwoSum of hi and d, then renormalised.
@@ -374,8 +478,8 @@ __device__ __forceinline__ void predict_j32(const Mirror &mr, long long i, long 
 // a warp), for blocks too small to fill the GPU: the corrector is a chain of
 // FP64 operations, and on the GB300 an FP64 warp instruction occupies the SM's
 // narrow FP64 pipe for many cycles however few of its lanes are active, so
-// one particle's three axes on three lanes (and its four norms on four)
-// issue about half the FP64 instructions of the one-thread form.  Each lane
+// one particle's three axes on three lanes issue a third of the one-thread
+// form's FP64 instructions.  Each lane
 // evaluates exactly the operations of correct_particle for its axis, in the
 // same order, so the results are the same bits.
 //
@@ -394,25 +498,36 @@ __device__ __forceinline__ bool correct_particle_quad(const State &s, long long 
     const int lane = threadIdx.x & 31, q = lane & 3, base = lane & ~3;
     const int c = q < 3 ? q : 2;          // lane 3 shadows axis 2 without storing
     const bool own = active && q < 3;
-    const double dt = ticks_to_time(tn - ldst<CG>(&s.t[i]));
-    const double h = __dmul_rn(dt, 0.5), q3 = div_by<3>(dt);
+    const long long ticks = tn - ldst<CG>(&s.t[i]);
     const long long e = c * stride + i;
     const double x = ldst<CG>(&s.x[e]), v = ldst<CG>(&s.v[e]), a = ldst<CG>(&s.a[e]),
                  k = ldst<CG>(&s.k[e]);
     const int lev_old = ldst<CG>(&s.lev[i]);
-    double xp, vp;
-    predict1hq(x, v, a, k, dt, h, q3, xp, vp);
-    const double d = __dsub_rn(a, apc);
-    const double a3 = __dadd_rn(__dmul_rn(2.0, d), __dmul_rn(__dadd_rn(k, kpc), dt));
-    const double a2 = __dsub_rn(__dmul_rn(-3.0, d), __dmul_rn(__dadd_rn(__dmul_rn(2.0, k), kpc), dt));
-    const double xn = __dadd_rn(xp, __dmul_rn(__dadd_rn(div_by<12>(a2), div_by<20>(a3)),
-                                            __dmul_rn(dt, dt)));
-    const double vn = __dadd_rn(vp, __dmul_rn(__dadd_rn(div_by<3>(a2), __dmul_rn(a3, 0.25)), dt));
+    AxisStep r;
+    int ex;
+    if (step_exponent(ticks, ex)) {
+        r = correct_axis(x, v, a, k, apc, kpc, ex);
+    } else {
+        const double dt = ticks_to_time(ticks);
+        const double h = __dmul_rn(dt, 0.5), q3 = div_by<3>(dt);
+        const double dt2 = __dmul_rn(dt, dt);
+        const double dt3 = __dmul_rn(dt2, dt);
+        double xp, vp;
+        predict1hq(x, v, a, k, dt, h, q3, xp, vp);
+        const double d = __dsub_rn(a, apc);
+        const double a3 = __dadd_rn(__dmul_rn(2.0, d), __dmul_rn(__dadd_rn(k, kpc), dt));
+        const double a2 = __dsub_rn(__dmul_rn(-3.0, d), __dmul_rn(__dadd_rn(__dmul_rn(2.0, k), kpc), dt));
+        r.x = __dadd_rn(xp, __dmul_rn(__dadd_rn(div_by<12>(a2), div_by<20>(a3)), dt2));
+        r.v = __dadd_rn(vp, __dmul_rn(__dadd_rn(div_by<3>(a2), __dmul_rn(a3, 0.25)), dt));
+        const double s0 = __ddiv_rn(__dmul_rn(2.0, a2), dt2);
+        r.c = __ddiv_rn(__dmul_rn(6.0, a3), dt3);
+        r.s1 = __dadd_rn(s0, __dmul_rn(r.c, dt));
+    }
     // every lane of the quad has read the old state before any lane stores
     __syncwarp();
     if (own) {
-        s.x[e] = xn;
-        s.v[e] = vn;
+        s.x[e] = r.x;
+        s.v[e] = r.v;
         s.a[e] = apc;
         s.k[e] = kpc;
     }
@@ -423,43 +538,41 @@ __device__ __forceinline__ bool correct_particle_quad(const State &s, long long 
         }
         return true;
     }
-    const double dt2 = __dmul_rn(dt, dt);
-    const double dt3 = __dmul_rn(dt2, dt);
-    const bool pow2 = (__double_as_longlong(dt) & 0x000FFFFFFFFFFFFFLL) == 0 && dt > 0x1p-100;
-    const double r2 = pow2 ? __longlong_as_double((2046LL << 52) - (__double_as_longlong(dt2) & 0x7FF0000000000000LL)) : 0.0;
-    const double r3 = pow2 ? __longlong_as_double((2046LL << 52) - (__double_as_longlong(dt3) & 0x7FF0000000000000LL)) : 0.0;
-    double s0, cr;
-    if (pow2) {
-        s0 = __dmul_rn(__dmul_rn(2.0, a2), r2);
-        cr = __dmul_rn(__dmul_rn(6.0, a3), r3);
-    } else {
-        s0 = __ddiv_rn(__dmul_rn(2.0, a2), dt2);
-        cr = __ddiv_rn(__dmul_rn(6.0, a3), dt3);
-    }
-    const double s1 = __dadd_rn(s0, __dmul_rn(cr, dt));
-    // |a_p|, |k_p|, |s1|, |c| on lanes 0..3 of the quad, each as norm3 forms it
-    const double sq0 = __dmul_rn(apc, apc), sq1 = __dmul_rn(kpc, kpc);
-    const double sq2 = __dmul_rn(s1, s1), sq3 = __dmul_rn(cr, cr);
-    double w[3];
+    // squared norms of a_p, k_p, s1, c on every lane of the quad: lane 3
+    // shadows axis 2 and adds nothing
+    float n2[4] = {to_float_int(apc), to_float_int(kpc), to_float_int(r.s1), to_float_int(r.c)};
 #pragma unroll
-    for (int cc = 0; cc < 3; ++cc) {
-        const double t0 = __shfl_sync(0xffffffffu, sq0, base + cc);
-        const double t1 = __shfl_sync(0xffffffffu, sq1, base + cc);
-        const double t2 = __shfl_sync(0xffffffffu, sq2, base + cc);
-        const double t3 = __shfl_sync(0xffffffffu, sq3, base + cc);
-        w[cc] = q == 0 ? t0 : (q == 1 ? t1 : (q == 2 ? t2 : t3));
+    for (int w = 0; w < 4; ++w) {
+        n2[w] = q < 3 ? n2[w] * n2[w] : 0.0f;
+        n2[w] += __shfl_xor_sync(0xffffffffu, n2[w], 1);
+        n2[w] += __shfl_xor_sync(0xffffffffu, n2[w], 2);
     }
-    const double nrm = __dsqrt_rn(__dadd_rn(__dadd_rn(w[0], w[1]), w[2]));
-    const double na = __shfl_sync(0xffffffffu, nrm, base + 0);
-    const double nk = __shfl_sync(0xffffffffu, nrm, base + 1);
-    const double ns = __shfl_sync(0xffffffffu, nrm, base + 2);
-    const double nc = __shfl_sync(0xffffffffu, nrm, base + 3);
-    const double num = __dadd_rn(__dmul_rn(na, ns), __dmul_rn(nk, nk));
-    const double den = __dadd_rn(__dmul_rn(nk, nc), __dmul_rn(ns, ns));
-    const double dt_raw = den == 0.0 ? (double)INFINITY : __dsqrt_rn(__ddiv_rn(__dmul_rn(eta, num), den));
-    int kq;
-    const bool ok = level_of(dt_raw, level_min, kq);
-    if (!ok) kq = kTickBits;
+    int kq = 0;
+    bool ok = true;
+    const bool known = level_estimate(n2[0], n2[1], n2[2], n2[3], to_float_int(eta), level_min, kq);
+    if (__any_sync(0xffffffffu, active && !known)) {
+        // |a_p|, |k_p|, |s1|, |c| on lanes 0..3 of the quad, each as norm3 forms it
+        const double sq0 = __dmul_rn(apc, apc), sq1 = __dmul_rn(kpc, kpc);
+        const double sq2 = __dmul_rn(r.s1, r.s1), sq3 = __dmul_rn(r.c, r.c);
+        double w[3];
+#pragma unroll
+        for (int cc = 0; cc < 3; ++cc) {
+            const double t0 = __shfl_sync(0xffffffffu, sq0, base + cc);
+            const double t1 = __shfl_sync(0xffffffffu, sq1, base + cc);
+            const double t2 = __shfl_sync(0xffffffffu, sq2, base + cc);
+            const double t3 = __shfl_sync(0xffffffffu, sq3, base + cc);
+            w[cc] = q == 0 ? t0 : (q == 1 ? t1 : (q == 2 ? t2 : t3));
+        }
+        const double nrm = __dsqrt_rn(__dadd_rn(__dadd_rn(w[0], w[1]), w[2]));
+        const double na = __shfl_sync(0xffffffffu, nrm, base + 0);
+        const double nk = __shfl_sync(0xffffffffu, nrm, base + 1);
+        const double ns = __shfl_sync(0xffffffffu, nrm, base + 2);
+        const double nc = __shfl_sync(0xffffffffu, nrm, base + 3);
+        if (!known) {
+            ok = level_exact(na, nk, ns, nc, eta, level_min, kq);
+            if (!ok) kq = kTickBits;
+        }
+    }
     if (active && q == 0) {
         s.t[i] = tn;
         s.lev[i] = next_level(lev_old, kq, tn, level_min);

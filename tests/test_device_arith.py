@@ -136,3 +136,56 @@ def test_integer_split_into_double_single():
     assert np.array_equal(hi.view(np.uint32), want.view(np.uint32))
     rest = (x - want.astype(np.float64)).astype(np.float32)
     assert np.array_equal(lo.view(np.uint32), rest.view(np.uint32))
+
+
+def _level_exact(na, nk, ns, nc, eta):
+    dt = np.sqrt(eta * (na * ns + nk * nk) / (nk * nc + ns * ns))
+    return -(np.frexp(dt)[1] - 1)
+
+
+def test_level_estimate_margin():
+    # level_estimate of nb_device.cuh in numpy float32, with every operation's
+    # result moved by up to two ulps (the device's approximate square roots and
+    # division are that good): wherever it decides, it decides as the FP64
+    # formulas do, also for norms placed so that dt_raw lies next to a power of two
+    rng = np.random.RandomState(5)
+    N = 400000
+
+    def f32(x):
+        y = np.asarray(x, dtype=np.float64).astype(np.float32)
+        return (y * (1 + rng.randint(-2, 3, y.shape) * 2.0 ** -24)).astype(np.float32)
+
+    na, nk, ns, nc = [10.0 ** rng.uniform(-6, 8, N) for _ in range(4)]
+    eta = 0.01
+    # the last half: scale the snap and crackle (dt ~ 1/scale) towards a binade edge
+    dt = np.sqrt(eta * (na * ns + nk * nk) / (nk * nc + ns * ns))
+    h = slice(N // 2, N)
+    edge = 2.0 ** np.round(np.log2(dt[h])) * (1 + rng.choice([-1, 1], N // 2) * 10.0 ** rng.uniform(-9, -2, N // 2))
+    lam = dt[h] / edge          # a, k, s, c scaled as 1, lam, lam^2, lam^3 divide dt by lam
+    nk[h] *= lam
+    ns[h] *= lam ** 2
+    nc[h] *= lam ** 3
+    n2 = [f32(f32(q) ** 2.0) for q in (na, nk, ns, nc)]
+    n2 = [f32(q * (1 + rng.uniform(-3, 3, N) * 2.0 ** -24)) for q in n2]   # three-term sums
+    root = [f32(np.sqrt(q.astype(np.float64))) for q in n2]
+    num = f32(root[0].astype(np.float64) * root[2] + n2[1])
+    den = f32(root[1].astype(np.float64) * root[3] + n2[2])
+    with np.errstate(all="ignore"):
+        R = f32(f32(eta * num.astype(np.float64)).astype(np.float64) / den)
+        lo, hi = np.min(n2, axis=0), np.max(n2, axis=0)
+        ok = (lo >= 2.0 ** -100) & (hi <= 2.0 ** 110) & (R >= 2.0 ** -72) & (R <= 2.0 ** 60)
+    b = R.view(np.int32)
+    e, m = (b >> 23) - 127, b & 0x7fffff
+    ok &= np.where(e & 1, m < 0x800000 - 0x800, m >= 0x800)
+    assert ok.mean() > 0.5 and not ok[h].all()
+    assert np.array_equal(-(e >> 1)[ok], _level_exact(na, nk, ns, nc, eta)[ok])
+
+
+def test_ticks_to_time_bits():
+    # d 2^-40 built from the integer's bits
+    rng = np.random.RandomState(6)
+    d = np.concatenate([rng.randint(1, 1 << 53, 1000), 1 << np.arange(53), [(1 << 53) - 1, 3, 5]]).astype(np.int64)
+    for q in d.tolist():
+        sh = (64 - q.bit_length()) - 11
+        bits = (q << sh) + ((1023 + 52 - 40 - 1 - sh) << 52)
+        assert np.array([bits], dtype=np.uint64).view(np.float64)[0] == q * 2.0 ** -40
