@@ -59,10 +59,7 @@ struct nb_ctx {
     SumArgs sum{};                  // summation variant (NB_SUM_COMPENSATED: unused)
     // persistent nb_run (k_run.cu), allocated on first use
     double *d_run_part = nullptr;
-    long long *d_run_mins = nullptr;
-    int *d_run_counts = nullptr;
-    unsigned *d_run_maxs = nullptr;
-    unsigned long long *d_run_bar = nullptr;
+    ulonglong2 *d_run_sync = nullptr;   // records and flags, zeroed before each launch
     int run_ncta = 0, run_per = 0;
     unsigned *d_bounds = nullptr;   // fixed point: mass and velocity bounds
     unsigned long long *d_sort = nullptr;  // sorted: keyed items, 2n per resident CTA
@@ -320,7 +317,7 @@ void release(nb_ctx *c)
                     c->d_blockcnt, c->d_epart, c->d_stage, c->d_ck, c->d_seg, c->d_fin, c->d_tfin,
                     c->d_jcnt, c->d_plan, c->d_cot, c->vrec.ph, c->vrec.pl, c->vrec.v, c->vrec.ab, c->vrec.kb,
                     c->vrec64.x, c->vrec64.v, c->vrec64.ab, c->vrec64.kb, c->d_bounds, c->d_sort,
-                    c->d_run_part, c->d_run_mins, c->d_run_counts, c->d_run_maxs, c->d_run_bar};
+                    c->d_run_part, c->d_run_sync};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     for (cudaEvent_t e : c->ev_free) cudaEventDestroy(e);
@@ -412,25 +409,21 @@ int run_persistent(nb_ctx *c, long long te, long long max_steps)
     if (c->n > kRunMaxN || c->o.precision != NB_DS || (c->o.flags & NB_RUN_GRAPH) ||
         (c->o.summation != NB_SUM_COMPENSATED && c->o.summation != NB_SUM_FIXED))
         return kRunNotUsed;
-    if (!c->d_run_bar) {
+    // records of 16 bytes: 2 C end times, 2 C bounds, C flags (half used), 3 n block records
+    const auto sync_count = [&]() { return 5LL * c->run_ncta + 3LL * c->n; };
+    if (!c->d_run_sync) {
         int bps = 0;
         if (occupancy_run(c->o.summation, &bps) ||
             run_layout(c->n, c->sms, bps, &c->run_ncta, &c->run_per))
             return kRunNotUsed;
         const long long C = c->run_ncta, N = c->n;
+        const int vals = c->o.summation == NB_SUM_FIXED ? 16 : 8;
         int rc;
-        if ((rc = dalloc(c, &c->d_run_part, C * N * 2 * kComp)) || (rc = dalloc(c, &c->d_run_mins, C)) ||
-            (rc = dalloc(c, &c->d_run_counts, C)) || (rc = dalloc(c, &c->d_run_maxs, 2 * C)) ||
-            (rc = dalloc(c, &c->d_run_bar, 1))) {
+        if ((rc = dalloc(c, &c->d_run_part, C * N * vals)) || (rc = dalloc(c, &c->d_run_sync, sync_count()))) {
             // all or nothing: a later call starts again from scratch
-            void *ps[] = {c->d_run_part, c->d_run_mins, c->d_run_counts, c->d_run_maxs, c->d_run_bar};
-            for (void *q : ps)
-                if (q) cudaFree(q);
+            if (c->d_run_part) cudaFree(c->d_run_part);
             c->d_run_part = nullptr;
-            c->d_run_mins = nullptr;
-            c->d_run_counts = nullptr;
-            c->d_run_maxs = nullptr;
-            c->d_run_bar = nullptr;
+            c->d_run_sync = nullptr;
             return rc;
         }
     }
@@ -446,23 +439,29 @@ int run_persistent(nb_ctx *c, long long te, long long max_steps)
     ra.level_min = c->o.level_min;
     ra.level_fixed = c->o.level_fixed;
     ra.t_end = te;
-    ra.max_steps = max_steps;
     ra.act = c->d_act;
-    ra.mins = c->d_run_mins;
-    ra.counts = c->d_run_counts;
-    ra.maxs = c->d_run_maxs;
     ra.part = c->d_run_part;
-    ra.bar = c->d_run_bar;
-    CK(cudaMemsetAsync(c->d_run_bar, 0, sizeof(unsigned long long), c->st));
-    const cudaError_t e = launch_run(ra, c->o.summation, c->st);
-    if (e == cudaErrorCooperativeLaunchTooLarge) {
-        // not every CTA can be resident now (a shared GPU): use the graph
-        cudaGetLastError();
-        return kRunNotUsed;
+    ra.minrec = c->d_run_sync;
+    ra.maxrec = ra.minrec + 2 * ra.ncta;
+    ra.flag = reinterpret_cast<unsigned long long *>(ra.maxrec + 2 * ra.ncta);
+    ra.blk = reinterpret_cast<float4 *>(c->d_run_sync + 5LL * ra.ncta);
+    for (;;) {
+        ra.max_steps = max_steps < kRunMaxSteps ? max_steps : kRunMaxSteps;
+        const long long steps0 = c->h_ctrl->steps;   // as of the caller's, or the last launch's, sync
+        CK(cudaMemsetAsync(c->d_run_sync, 0, sizeof(ulonglong2) * (size_t)sync_count(), c->st));
+        const cudaError_t e = launch_run(ra, c->o.summation, c->st);
+        if (e == cudaErrorCooperativeLaunchTooLarge) {
+            // not every CTA can be resident now (a shared GPU): use the graph
+            cudaGetLastError();
+            return kRunNotUsed;
+        }
+        if (e != cudaSuccess) return fail(c, NB_ECUDA, "persistent run launch: %s", cudaGetErrorString(e));
+        c->launches += 1;
+        const int rc = sync_ctrl(c);
+        const long long done = c->h_ctrl->steps - steps0;
+        max_steps -= done;
+        if (rc || done < ra.max_steps || max_steps <= 0 || c->h_ctrl->n_active == 0) return rc;
     }
-    if (e != cudaSuccess) return fail(c, NB_ECUDA, "persistent run launch: %s", cudaGetErrorString(e));
-    c->launches += 1;
-    return sync_ctrl(c);
 }
 
 }  // namespace

@@ -496,6 +496,11 @@ constexpr int kRunNT = 256;
 // a CTA corrects up to this many particles of a step with four lanes each
 constexpr int kRunQuadMax = 16;
 constexpr int kRunMaxN = 16384;   // above it the per-stage graph, using every SM for the force, is faster
+constexpr int kRunIndexBits = 14;   // particle index in a block record's tag, below the step
+constexpr int kRunPerLane = 8;      // CTAs at most: 32 times this
+// steps per launch at most: a tag's step number must not come round again
+constexpr long long kRunMaxSteps = 1LL << 17;
+static_assert(kRunMaxN == 1 << kRunIndexBits && kRunMaxSteps < 1LL << (32 - kRunIndexBits), "tags");
 struct RunArgs {
     State s;
     JDS j;
@@ -505,12 +510,13 @@ struct RunArgs {
     double eta;
     int level_min, level_fixed;
     long long t_end, max_steps;  // stop before a block time past t_end, or after max_steps steps
-    int *act;                    // [n] block list
-    long long *mins;             // [ncta] per-CTA minimum end time
-    int *counts;                 // [ncta] per-CTA block count
-    unsigned *maxs;              // [2 ncta] fixed point: per-CTA mass and |v|_1 bounds (float bits)
-    double *part;                // [ncta][n][7] partials (fixed point: pairs of int64)
-    unsigned long long *bar;     // grid-barrier arrivals (zero at launch)
+    int *act;                    // [n] block list (written at the end)
+    // exchanged between CTAs, all zero at launch:
+    ulonglong2 *minrec;          // [2][ncta] least end time; count, error bit and step
+    ulonglong2 *maxrec;          // [2][ncta] fixed point: mass and |v|_1 bounds (float bits), step
+    unsigned long long *flag;    // [ncta] steps whose partials are written
+    float4 *blk;                 // [n][3] block records: hi, lo, velocity, each with its tag
+    double *part;                // [n][ncta][8] partials (fixed point: pairs of int64, [16])
 };
 
 // Reverse mode (k_adjoint.cu).  Force-VJP records: DS (x_hi, y_hi, z_hi, m),
