@@ -468,7 +468,7 @@ __host__ __device__ inline long long en_items(int n)
 // bit moves: conversions run on the FP64 pipe.
 __device__ __forceinline__ double rsqrt_pair(double x)
 {
-    if (!split_safe(x)) return rsqrt(x);
+    if (!exponent_in<-70, 190>(x)) return rsqrt(x);
     const unsigned xh = (unsigned)__double2hiint(x), xl = (unsigned)__double2loint(x);
     const float y = rsqrt_sfu(__uint_as_float((xh - (896u << 20)) << 3 | xl >> 29));   // truncated
     const unsigned yb = __float_as_uint(y);

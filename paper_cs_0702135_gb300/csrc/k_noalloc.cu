@@ -51,7 +51,7 @@ static __device__ __align__(256) double g_scratch[kScratchDoubles];
 
 using nbk::dev::ds_add;
 using nbk::dev::rsqrt_sfu;
-using nbk::dev::split_ds_int;
+using nbk::dev::split_record;
 using nbk::dev::to_float_int;
 using nbk::dev::warp_reduce_scatter;
 
@@ -63,11 +63,8 @@ __device__ __forceinline__ DSPoint load_point(const double *m, const double *x, 
                                               long long j)
 {
     DSPoint p;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        split_ds_int(x[3 * j + c], p.xh[c], p.xl[c]);
-        p.v[c] = to_float_int(v[3 * j + c]);
-    }
+    const double xj[3] = {x[3 * j], x[3 * j + 1], x[3 * j + 2]}, vj[3] = {v[3 * j], v[3 * j + 1], v[3 * j + 2]};
+    split_record(xj, vj, p.xh, p.xl, p.v);
     p.m = to_float_int(m[j]);
     return p;
 }

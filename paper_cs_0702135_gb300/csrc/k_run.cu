@@ -98,6 +98,14 @@ __device__ __forceinline__ bool wait_counter(const unsigned long long *p, unsign
     return true;
 }
 
+// The least of the lanes' non-negative values, by its two halves.
+__device__ __forceinline__ long long warp_min(long long v)
+{
+    const unsigned hi = (unsigned)(v >> 32), mh = __reduce_min_sync(kFullR, hi);
+    const unsigned ml = __reduce_min_sync(kFullR, hi == mh ? (unsigned)v : 0xffffffffu);
+    return (long long)((unsigned long long)mh << 32 | ml);
+}
+
 // The limit of a wait that polls records or flags: false once it has run out.
 struct Patience {
     long long t0 = 0;
@@ -299,7 +307,7 @@ __device__ __forceinline__ bool force_phase(const RunArgs &ra, int r, int na, in
 }
 
 // Bytes of shared memory per particle of a CTA (see k_run).
-constexpr int kRunBytesPer = 12 * 8 + 8 + 8 + 8 * 8 + 3 * 16 + 4 + 4 + 4;
+constexpr int kRunBytesPer = 12 * 8 + 8 + 8 + 8 * 8 + 3 * 16 + 4 + 4;
 
 template <int MODE>
 __global__ void __launch_bounds__(kRunNT) k_run(RunArgs ra)
@@ -316,7 +324,6 @@ __global__ void __launch_bounds__(kRunNT) k_run(RunArgs ra)
     long long *const s_et = s_t + per;                              // t_i + 2^-lev_i
     int *const s_lev = reinterpret_cast<int *>(s_et + per);
     int *const s_blk = s_lev + per;                                 // block members (local indices)
-    float *const s_m = reinterpret_cast<float *>(s_blk + per);
     __shared__ long long s_tn;
     __shared__ int s_na, s_off, s_stop, s_err, s_late;
     __shared__ unsigned s_max[2][kRunNT / 32];
@@ -340,7 +347,8 @@ __global__ void __launch_bounds__(kRunNT) k_run(RunArgs ra)
         s_t[tid] = ra.s.t[i];
         s_lev[tid] = ra.s.lev[i];
         s_et[tid] = s_t[tid] + (1LL << (kTickBits - s_lev[tid]));
-        s_m[tid] = to_float_int(ra.s.m[i]);
+        s_p[tid] = make_float4(0.0f, 0.0f, 0.0f, to_float_int(ra.s.m[i]));
+        s_l[tid] = s_v[tid] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     }
     if (tid == 0) {
         s_err = ra.ctrl->err != 0;
@@ -453,8 +461,7 @@ __global__ void __launch_bounds__(kRunNT) k_run(RunArgs ra)
         if (warp == 0) {
             long long mn = LLONG_MAX;
             for (int q = lane; q < m; q += 32) mn = min(mn, s_et[q]);
-#pragma unroll
-            for (int o = 16; o >= 1; o >>= 1) mn = min(mn, __shfl_xor_sync(kFullR, mn, o));
+            mn = warp_min(mn);
             unsigned cnt = 0;
             for (int q = lane; q < m; q += 32) cnt += s_et[q] == mn;
             cnt = __reduce_add_sync(kFullR, cnt);
@@ -484,8 +491,7 @@ __global__ void __launch_bounds__(kRunNT) k_run(RunArgs ra)
                     tn = min(tn, (long long)rec[u].x);
                     err |= (unsigned)rec[u].y & 0x80000000u;
                 }
-#pragma unroll
-            for (int o = 16; o >= 1; o >>= 1) tn = min(tn, __shfl_xor_sync(kFullR, tn, o));
+            tn = warp_min(tn);
             unsigned na = 0, off = 0;
 #pragma unroll
             for (int u = 0; u < kRunPerLane; ++u)
@@ -527,48 +533,55 @@ __global__ void __launch_bounds__(kRunNT) k_run(RunArgs ra)
         cnt_b = cnt_own;
         na_b = na;
         tn_b = tn;
+        // Prediction, a warp to one axis of 32 particles: a warp has one FP64
+        // instruction in flight, whatever its lanes.
+        const bool member = tid < m && s_et[tid] == tn;
+        if (member) s_blk[before] = tid;
+        for (int task = warp; task < 3 * ((m + 31) / 32); task += kRunNT / 32) {
+            const int c = task % 3, q = task / 3 * 32 + lane;
+            if (q < m) {
+                const double dt = ticks_to_time(tn - s_t[q]);
+                const int e = c * per + q;
+                double xp, vp;
+                predict1hq(L.x[e], L.v[e], L.a[e], L.k[e], dt, half_dt(dt), div_core<3>(dt), xp, vp);
+                float h, l, u;
+                bool bad = false;
+                split_ds_int(xp, h, l, bad);
+                u = to_float_int(vp, bad);
+                if (bad) {
+                    h = to_float_volatile(xp);
+                    l = to_float_volatile(__dsub_rn(xp, (double)h));
+                    u = to_float_volatile(vp);
+                }
+                reinterpret_cast<float *>(&s_p[q])[c] = h;
+                reinterpret_cast<float *>(&s_l[q])[c] = l;
+                reinterpret_cast<float *>(&s_v[q])[c] = u;
+            }
+        }
+        __syncthreads();
         unsigned mb = 0, vb = 0;
-        if (tid < m) {
-            // predict3's arithmetic
-            const double dt = ticks_to_time(tn - s_t[tid]);
-            const double dt_h = scale2(dt, -1), dt_q = div_by<3>(dt);
-            double xp[3], vp[3];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                const int e = c * per + tid;
-                predict1hq(L.x[e], L.v[e], L.a[e], L.k[e], dt, dt_h, dt_q, xp[c], vp[c]);
-            }
-            float h[3], l[3];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) split_ds_int(xp[c], h[c], l[c]);
-            const float4 v4 = make_float4(to_float_int(vp[0]), to_float_int(vp[1]), to_float_int(vp[2]), 0.0f);
-            if (s_et[tid] == tn) {
-                s_blk[before] = tid;
-                float4 *const dst = ra.blk + 3 * (long long)(off_b + before);
-                const unsigned tag = epoch << kRunIndexBits | (unsigned)(i0 + tid);
-                auto put = [&](int q, float x, float y, float z) {
-                    store128(dst + q, {(unsigned long long)__float_as_uint(x) | (unsigned long long)__float_as_uint(y) << 32,
-                                       (unsigned long long)__float_as_uint(z) | (unsigned long long)tag << 32});
-                };
-                put(0, h[0], h[1], h[2]);
-                put(1, l[0], l[1], l[2]);
-                put(2, v4.x, v4.y, v4.z);
-            }
-            s_p[tid] = make_float4(h[0], h[1], h[2], s_m[tid]);
-            s_l[tid] = make_float4(l[0], l[1], l[2], 0.0f);
-            s_v[tid] = v4;
-            if (MODE == NB_SUM_FIXED) {
-                mb = __float_as_uint(s_m[tid]);
-                vb = __float_as_uint(__fadd_rn(__fadd_rn(fabsf(v4.x), fabsf(v4.y)), fabsf(v4.z)));
-            }
+        if (member) {
+            const float4 h = s_p[tid], l = s_l[tid], v = s_v[tid];
+            float4 *const dst = ra.blk + 3 * (long long)(off_b + before);
+            const unsigned long long tag = (unsigned long long)(epoch << kRunIndexBits | (unsigned)(i0 + tid)) << 32;
+            auto put = [&](int q, float x, float y, float z) {
+                store128(dst + q, {(unsigned long long)__float_as_uint(x) | (unsigned long long)__float_as_uint(y) << 32,
+                                   (unsigned long long)__float_as_uint(z) | tag});
+            };
+            put(0, h.x, h.y, h.z);
+            put(1, l.x, l.y, l.z);
+            put(2, v.x, v.y, v.z);
+        }
+        if (MODE == NB_SUM_FIXED && tid < m) {
+            const float4 v = s_v[tid];
+            mb = __float_as_uint(s_p[tid].w);
+            vb = __float_as_uint(__fadd_rn(__fadd_rn(fabsf(v.x), fabsf(v.y)), fabsf(v.z)));
         }
         if (MODE == NB_SUM_FIXED) {
             mb = __reduce_max_sync(kFullR, mb);
             vb = __reduce_max_sync(kFullR, vb);
             if (lane == 0) s_max[0][warp] = mb, s_max[1][warp] = vb;
-        }
-        __syncthreads();
-        if (MODE == NB_SUM_FIXED) {
+            __syncthreads();
             // the bounds over all particles: published and read like the end times
             if (warp == 0) {
                 mb = lane < kRunNT / 32 ? s_max[0][lane] : 0u;

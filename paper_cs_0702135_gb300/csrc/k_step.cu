@@ -37,12 +37,11 @@ __device__ __forceinline__ void predict_record(const State &s, int i, long long 
         jf.pos[i] = make_double4_32a(xp[0], xp[1], xp[2], m);
         jf.vel[i] = make_double4_32a(vp[0], vp[1], vp[2], 0.0);
     } else {
-        float hi[3], lo[3];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) split_ds_int(xp[c], hi[c], lo[c]);
+        float hi[3], lo[3], u[3];
+        split_record(xp, vp, hi, lo, u);
         jds.pos_hi[i] = make_float4(hi[0], hi[1], hi[2], to_float_int(m));
         jds.pos_lo[i] = make_float4(lo[0], lo[1], lo[2], 0.0f);
-        jds.vel[i] = make_float4(to_float_int(vp[0]), to_float_int(vp[1]), to_float_int(vp[2]), 0.0f);
+        jds.vel[i] = make_float4(u[0], u[1], u[2], 0.0f);
     }
 }
 

@@ -14,32 +14,55 @@ namespace dev {
 
 constexpr double kTick = 0x1p-40;  // one tick in N-body time units
 
-// The GB300's FP64 pipe takes 2 lanes a clock per SM with 64 clocks of latency,
-// for conversions between integers, FP32 and FP64 as for arithmetic; what is
-// only a move of bits is done on the integer pipe (4 clocks) below.
+// The GB300's FP64 pipe serves an SM one warp instruction in 20 clocks, a warp
+// one in 66 however many lanes are active and however independent they are,
+// and conversions between integers, FP32 and FP64 are such instructions too
+// (measured; a division or square root takes ~600 clocks).  What is only a
+// move of bits is therefore done on the integer pipe, without branches: a
+// function that works on a range of exponents sets `bad` outside it, and the
+// caller redoes the whole expression with the FP64 operations once at its end
+// (written volatile, or in a function of its own, so that the compiler does
+// not evaluate them ahead of that test).
+__device__ __forceinline__ double mul_volatile(double x, double y)
+{
+    double r;
+    asm volatile("mul.rn.f64 %0, %1, %2;" : "=d"(r) : "d"(x), "d"(y));
+    return r;
+}
 
-// d 2^-40, rounded to nearest.
+// d 2^-40, rounded to nearest.  Up to 2^52 ticks the integer goes into the
+// significand of 2^12, whose last place is 2^-40, and 2^12 is subtracted: exact.
 __device__ __forceinline__ double ticks_to_time(long long d)
 {
-    if (d > 0 && d < (1LL << 53)) {   // exact: the significand's bits moved into place
-        const int sh = __clzll(d) - 11;
-        const unsigned long long m = (unsigned long long)d << sh;   // leading one at bit 52
-        return __longlong_as_double((long long)(m + ((unsigned long long)(1023 + 52 - 40 - 1 - sh) << 52)));
-    }
-    return __dmul_rn(__ll2double_rn(d), kTick);
+    if ((unsigned long long)d < (1ULL << 52))
+        return __dsub_rn(__longlong_as_double(d | 0x40B0000000000000LL), 4096.0);
+    double r;
+    asm volatile("cvt.rn.f64.s64 %0, %1;" : "=d"(r) : "l"(d));
+    return mul_volatile(r, kTick);
 }
 
 // 2^e as FP64, -1022 <= e <= 1023.
 __device__ __forceinline__ double pow2d(int e) { return __hiloint2double((1023 + e) << 20, 0); }
 
-// x 2^e, |e| <= 130: the exponent field moved (exact), or the multiplication
-// where the field is not well inside its range (zero, tiny, huge, not finite).
-__device__ __forceinline__ double scale2(double x, int e)
+// Whether x's exponent lies in [2^(lo), 2^(lo + n)) (not zero, not finite: no).
+template <int LO, int N>
+__device__ __forceinline__ bool exponent_in(double x)
 {
-    const int hi = __double2hiint(x);
-    if (((unsigned)hi & 0x7fffffffu) - (200u << 20) < (1600u << 20))
-        return __hiloint2double(hi + (e << 20), __double2loint(x));
-    return __dmul_rn(x, pow2d(e));
+    return ((unsigned)__double2hiint(x) & 0x7fffffffu) - ((unsigned)(1023 + LO) << 20) < ((unsigned)N << 20);
+}
+
+// x 2^e, |e| <= 130, by moving the exponent field (exact).
+__device__ __forceinline__ double scale2(double x, int e, bool &bad)
+{
+    bad = bad || !exponent_in<-823, 1600>(x);
+    return __hiloint2double(__double2hiint(x) + (e << 20), __double2loint(x));
+}
+
+// dt / 2 for dt >= 0 from ticks_to_time.
+__device__ __forceinline__ double half_dt(double dt)
+{
+    const int hi = __double2hiint(dt);
+    return __hiloint2double(hi != 0 ? hi - (1 << 20) : 0, __double2loint(dt));
 }
 
 // 1/sqrt(x) on the SFU: the PTX approximate reciprocal square root with
@@ -114,17 +137,29 @@ __device__ __forceinline__ void warp_reduce_scatter(float (&h)[P], float (&lo)[P
 // 2^-900 < |a| < 2^1000 (zero with its sign, huge, not finite) take the plain
 // division; the range test reads the exponent bits on the integer pipe.
 template <int C>
-__device__ __forceinline__ double div_by(double a)
+__device__ __forceinline__ double div_core(double a)
 {
     static_assert(C == 3 || C == 12 || C == 20, "reciprocal error checked for 3, 12, 20 only");
+    constexpr double y = 1.0 / C;
+    const double q0 = __dmul_rn(a, y);
+    const double r = __fma_rn(-q0, (double)C, a);
+    return __fma_rn(r, y, q0);
+}
+
+template <int C>
+__device__ __forceinline__ double div_by(double a)
+{
     const unsigned hi = (unsigned)__double2hiint(a) & 0x7FFFFFFFu;
-    if (hi >= (123u << 20) && hi < (2023u << 20)) {
-        constexpr double y = 1.0 / C;
-        const double q0 = __dmul_rn(a, y);
-        const double r = __fma_rn(-q0, (double)C, a);
-        return __fma_rn(r, y, q0);
-    }
+    if (hi >= (123u << 20) && hi < (2023u << 20)) return div_core<C>(a);
     return __ddiv_rn(a, (double)C);
+}
+
+// The same without the branch: `bad` outside the range.
+template <int C>
+__device__ __forceinline__ double div_by(double a, bool &bad)
+{
+    bad = bad || !exponent_in<123 - 1023, 1900>(a);
+    return div_core<C>(a);
 }
 
 // Hermite predictor (Section 2), round-to-nearest in the formula's order:
@@ -159,7 +194,8 @@ template <bool CG = false>
 __device__ __forceinline__ void predict3(const State &s, long long i, long long n, double dt,
                                          double xp[3], double vp[3])
 {
-    const double h = scale2(dt, -1), q = div_by<3>(dt);
+    // a time step needs no range test: 0 (exact) or 2^-40 .. 2^22
+    const double h = half_dt(dt), q = div_core<3>(dt);
 #pragma unroll
     for (int c = 0; c < 3; ++c)
         predict1hq(ldst<CG>(&s.x[c * n + i]), ldst<CG>(&s.v[c * n + i]), ldst<CG>(&s.a[c * n + i]),
@@ -173,32 +209,14 @@ __device__ __forceinline__ void split_ds(double x, float &hi, float &lo)
     lo = __double2float_rn(__dsub_rn(x, (double)hi));
 }
 
-// RN32(x) and RN32(x - RN32(x)) on the integer pipe.  A conversion between
-// FP64 and FP32 runs on the GB300's FP64 pipe like an FP64 operation (2 lanes
-// a clock per SM, 64 cycles), so a split costs four of those; these are ~15
-// integer instructions.  x = (-1)^s M 2^(e-1075): the top 24 bits of M round
-// half to even by the remainder R of the low 29, and the rest R (- 2^29 if
-// rounded up) is an integer of at most 29 bits, converted to FP32 (rounded to
-// nearest) and scaled exactly.  Exponents outside [2^-70, 2^120) (zero among
-// them) take the conversions, written volatile so that they are not evaluated
-// ahead of the test.
-__device__ __forceinline__ bool split_safe(double x)
+// RN32(x) and RN32(x - RN32(x)) on the integer pipe (~15 instructions; a split
+// by conversions is four FP64 instructions).  x = (-1)^s M 2^(e-1075): the top
+// 24 bits of M round half to even by the remainder R of the low 29, and the
+// rest R (- 2^29 if rounded up) is an integer of at most 29 bits, converted to
+// FP32 (rounded to nearest) and scaled exactly.  `bad` outside [2^-70, 2^120).
+__device__ __forceinline__ void split_ds_int(double x, float &hi, float &lo, bool &bad)
 {
-    return (((unsigned)__double2hiint(x) & 0x7fffffffu) - ((1023u - 70u) << 20)) < (190u << 20);
-}
-__device__ __forceinline__ float to_float_volatile(double x)
-{
-    float y;
-    asm volatile("cvt.rn.f32.f64 %0, %1;" : "=f"(y) : "d"(x));
-    return y;
-}
-__device__ __forceinline__ void split_ds_int(double x, float &hi, float &lo)
-{
-    if (!split_safe(x)) {
-        hi = to_float_volatile(x);
-        lo = to_float_volatile(__dsub_rn(x, (double)hi));
-        return;
-    }
+    bad = bad || !exponent_in<-70, 190>(x);
     const unsigned xh = (unsigned)__double2hiint(x), xl = (unsigned)__double2loint(x);
     const unsigned e = (xh >> 20) & 0x7ffu;
     const unsigned t = ((xh & 0x7fffffffu) - (896u << 20)) << 3 | xl >> 29;   // truncated to FP32
@@ -209,12 +227,43 @@ __device__ __forceinline__ void split_ds_int(double x, float &hi, float &lo)
     r = (int)xh < 0 ? -r : r;
     lo = __int2float_rn(r) * __uint_as_float((e - (1075u - 127u)) << 23);
 }
-__device__ __forceinline__ float to_float_int(double x)
+__device__ __forceinline__ float to_float_int(double x, bool &bad)
 {
-    if (!split_safe(x)) return to_float_volatile(x);
+    bad = bad || !exponent_in<-70, 190>(x);
     const unsigned xh = (unsigned)__double2hiint(x), xl = (unsigned)__double2loint(x);
     const unsigned t = ((xh & 0x7fffffffu) - (896u << 20)) << 3 | xl >> 29;
     return __uint_as_float((t + ((xl & 0x1fffffffu) + (t & 1u) > 0x10000000u)) | (xh & 0x80000000u));
+}
+__device__ __forceinline__ float to_float_volatile(double x)
+{
+    float y;
+    asm volatile("cvt.rn.f32.f64 %0, %1;" : "=f"(y) : "d"(x));
+    return y;
+}
+__device__ __forceinline__ float to_float_int(double x)
+{
+    bool bad = false;
+    const float y = to_float_int(x, bad);
+    return bad ? to_float_volatile(x) : y;
+}
+
+// A position split into double-single and a velocity in FP32, all axes.
+__device__ __forceinline__ void split_record(const double x[3], const double v[3], float hi[3], float lo[3],
+                                             float u[3])
+{
+    bool bad = false;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        split_ds_int(x[c], hi[c], lo[c], bad);
+        u[c] = to_float_int(v[c], bad);
+    }
+    if (bad)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            hi[c] = to_float_volatile(x[c]);
+            lo[c] = to_float_volatile(__dsub_rn(x[c], (double)hi[c]));
+            u[c] = to_float_volatile(v[c]);
+        }
 }
 
 __device__ __forceinline__ double norm3(double u0, double u1, double u2)
@@ -293,25 +342,49 @@ __device__ __forceinline__ bool level_estimate(float na2, float nk2, float ns2, 
 // The corrector's arithmetic for one axis when the step is a power of two,
 // dt = 2^e (every block step): multiplications by powers of two move the
 // exponent (scale2), dt/3 is the rounded third with its exponent moved, and
-// the other operations are those of correct_particle in its order, so the
-// results are the same bits with 27 FP64 operations instead of ~47.
+// the other operations are those of correct_axis_any in its order, so the
+// results are the same bits with 24 FP64 operations instead of ~47.
 struct AxisStep {
     double x, v, s1, c;   // new position and velocity; s1 and crackle of the step criterion
 };
 __device__ __forceinline__ AxisStep correct_axis(double x, double v, double a, double k, double ap, double kp,
-                                                 int e)
+                                                 int e, bool &bad)
 {
     AxisStep r;
-    const double w = __dadd_rn(a, scale2(__dmul_rn(1.0 / 3.0, k), e));
-    const double xp = __dadd_rn(x, scale2(__dadd_rn(v, scale2(w, e - 1)), e));
-    const double vp = __dadd_rn(v, scale2(__dadd_rn(a, scale2(k, e - 1)), e));
     const double d = __dsub_rn(a, ap);
-    const double a3 = __dadd_rn(scale2(d, 1), scale2(__dadd_rn(k, kp), e));
-    const double a2 = __dsub_rn(__dmul_rn(-3.0, d), scale2(__dadd_rn(scale2(k, 1), kp), e));
-    r.x = __dadd_rn(xp, scale2(__dadd_rn(div_by<12>(a2), div_by<20>(a3)), 2 * e));
-    r.v = __dadd_rn(vp, scale2(__dadd_rn(div_by<3>(a2), scale2(a3, -2)), e));
-    r.c = scale2(__dmul_rn(6.0, a3), -3 * e);
-    r.s1 = __dadd_rn(scale2(a2, 1 - 2 * e), scale2(r.c, e));
+    const double a3 = __dadd_rn(scale2(d, 1, bad), scale2(__dadd_rn(k, kp), e, bad));
+    const double a2 = __dsub_rn(__dmul_rn(-3.0, d), scale2(__dadd_rn(scale2(k, 1, bad), kp), e, bad));
+    const double w = __dadd_rn(a, scale2(__dmul_rn(1.0 / 3.0, k), e, bad));
+    const double xp = __dadd_rn(x, scale2(__dadd_rn(v, scale2(w, e - 1, bad)), e, bad));
+    const double vp = __dadd_rn(v, scale2(__dadd_rn(a, scale2(k, e - 1, bad)), e, bad));
+    const double a2_3 = div_by<3>(a2, bad);   // a2 / 12 is a quarter of it
+    r.x = __dadd_rn(xp, scale2(__dadd_rn(scale2(a2_3, -2, bad), div_by<20>(a3, bad)), 2 * e, bad));
+    r.v = __dadd_rn(vp, scale2(__dadd_rn(a2_3, scale2(a3, -2, bad)), e, bad));
+    r.c = scale2(__dmul_rn(6.0, a3), -3 * e, bad);
+    r.s1 = __dadd_rn(scale2(a2, 1 - 2 * e, bad), scale2(r.c, e, bad));
+    return r;
+}
+
+// The same for any step and any values.
+static __device__ __noinline__ AxisStep correct_axis_any(double x, double v, double a, double k, double ap, double kp,
+                                                  long long ticks)
+{
+    AxisStep r;
+    const double dt = ticks_to_time(ticks);
+    const double h = __dmul_rn(dt, 0.5), q3 = div_by<3>(dt);
+    const double dt2 = __dmul_rn(dt, dt);
+    const double dt3 = __dmul_rn(dt2, dt);
+    double xp, vp;
+    predict1hq(x, v, a, k, dt, h, q3, xp, vp);
+    const double d = __dsub_rn(a, ap);
+    const double a3 = __dadd_rn(__dmul_rn(2.0, d), __dmul_rn(__dadd_rn(k, kp), dt));
+    const double a2 = __dsub_rn(__dmul_rn(-3.0, d), __dmul_rn(__dadd_rn(__dmul_rn(2.0, k), kp), dt));
+    r.x = __dadd_rn(xp, __dmul_rn(__dadd_rn(div_by<12>(a2), div_by<20>(a3)), dt2));
+    // a3 / 4 as a3 * 0.25: the same real number, so the same rounded result
+    r.v = __dadd_rn(vp, __dmul_rn(__dadd_rn(div_by<3>(a2), __dmul_rn(a3, 0.25)), dt));
+    const double s0 = __ddiv_rn(__dmul_rn(2.0, a2), dt2);
+    r.c = __ddiv_rn(__dmul_rn(6.0, a3), dt3);
+    r.s1 = __dadd_rn(s0, __dmul_rn(r.c, dt));
     return r;
 }
 
@@ -323,7 +396,7 @@ __device__ __forceinline__ bool step_exponent(long long ticks, int &e)
 }
 
 // The Aarseth step's level from the FP64 norms (false: below 2^-40).
-__device__ __forceinline__ bool level_exact(double na, double nk, double ns, double nc, double eta, int kmin,
+static __device__ __noinline__ bool level_exact(double na, double nk, double ns, double nc, double eta, int kmin,
                                             int &level)
 {
     const double num = __dadd_rn(__dmul_rn(na, ns), __dmul_rn(nk, nk));
@@ -351,43 +424,21 @@ __device__ __forceinline__ bool correct_particle(const State &s, long long i, lo
     const long long ticks = tn - ldst<CG>(&s.t[i]);
     double s1[3], cr[3];
     int ex;
-    if (step_exponent(ticks, ex)) {
+    const bool block_step = step_exponent(ticks, ex);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const long long e = c * stride + i;
-            const AxisStep r = correct_axis(ldst<CG>(&s.x[e]), ldst<CG>(&s.v[e]), ldst<CG>(&s.a[e]),
-                                            ldst<CG>(&s.k[e]), ap[c], kp[c], ex);
-            s.x[e] = r.x;
-            s.v[e] = r.v;
-            s.a[e] = ap[c];
-            s.k[e] = kp[c];
-            s1[c] = r.s1;
-            cr[c] = r.c;
-        }
-    } else {
-        const double dt = ticks_to_time(ticks);
-        const double h = __dmul_rn(dt, 0.5), q = div_by<3>(dt);
-        const double dt2 = __dmul_rn(dt, dt);
-        const double dt3 = __dmul_rn(dt2, dt);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const long long e = c * stride + i;
-            const double x = ldst<CG>(&s.x[e]), v = ldst<CG>(&s.v[e]), a = ldst<CG>(&s.a[e]),
-                         k = ldst<CG>(&s.k[e]);
-            double xp, vp;
-            predict1hq(x, v, a, k, dt, h, q, xp, vp);
-            const double d = __dsub_rn(a, ap[c]);
-            const double a3 = __dadd_rn(__dmul_rn(2.0, d), __dmul_rn(__dadd_rn(k, kp[c]), dt));
-            const double a2 = __dsub_rn(__dmul_rn(-3.0, d), __dmul_rn(__dadd_rn(__dmul_rn(2.0, k), kp[c]), dt));
-            s.x[e] = __dadd_rn(xp, __dmul_rn(__dadd_rn(div_by<12>(a2), div_by<20>(a3)), dt2));
-            // a3 / 4 as a3 * 0.25: the same real number, so the same rounded result
-            s.v[e] = __dadd_rn(vp, __dmul_rn(__dadd_rn(div_by<3>(a2), __dmul_rn(a3, 0.25)), dt));
-            s.a[e] = ap[c];
-            s.k[e] = kp[c];
-            const double s0 = __ddiv_rn(__dmul_rn(2.0, a2), dt2);
-            cr[c] = __ddiv_rn(__dmul_rn(6.0, a3), dt3);
-            s1[c] = __dadd_rn(s0, __dmul_rn(cr[c], dt));
-        }
+    for (int c = 0; c < 3; ++c) {
+        const long long e = c * stride + i;
+        const double x = ldst<CG>(&s.x[e]), v = ldst<CG>(&s.v[e]), a = ldst<CG>(&s.a[e]),
+                     k = ldst<CG>(&s.k[e]);
+        bool bad = !block_step;
+        AxisStep r = correct_axis(x, v, a, k, ap[c], kp[c], ex, bad);
+        if (bad) r = correct_axis_any(x, v, a, k, ap[c], kp[c], ticks);
+        s.x[e] = r.x;
+        s.v[e] = r.v;
+        s.a[e] = ap[c];
+        s.k[e] = kp[c];
+        s1[c] = r.s1;
+        cr[c] = r.c;
     }
     s.t[i] = tn;
     if (level_fixed > 0) {
@@ -427,13 +478,14 @@ struct Mirror {
 template <bool CG = false>
 __device__ __forceinline__ void write_mirror(const State &s, const Mirror &mr, long long i, long long n)
 {
-    float hi[3], lo[3];
+    double x[3], v[3];
+    float hi[3], lo[3], u[3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) split_ds_int(ldst<CG>(&s.x[c * n + i]), hi[c], lo[c]);
+    for (int c = 0; c < 3; ++c) x[c] = ldst<CG>(&s.x[c * n + i]), v[c] = ldst<CG>(&s.v[c * n + i]);
+    split_record(x, v, hi, lo, u);
     mr.h[i] = make_float4(hi[0], hi[1], hi[2], to_float_int(ldst<CG>(&s.m[i])));
     mr.l[i] = make_float4(lo[0], lo[1], lo[2], 0.0f);
-    mr.v[i] = make_float4(to_float_int(ldst<CG>(&s.v[i])), to_float_int(ldst<CG>(&s.v[n + i])),
-                          to_float_int(ldst<CG>(&s.v[2 * n + i])), 0.0f);
+    mr.v[i] = make_float4(u[0], u[1], u[2], 0.0f);
     mr.a[i] = make_float4(to_float_int(ldst<CG>(&s.a[i])), to_float_int(ldst<CG>(&s.a[n + i])),
                           to_float_int(ldst<CG>(&s.a[2 * n + i])), 0.0f);
     mr.k[i] = make_float4(to_float_int(ldst<CG>(&s.k[i])), to_float_int(ldst<CG>(&s.k[n + i])),
@@ -503,26 +555,10 @@ __device__ __forceinline__ bool correct_particle_quad(const State &s, long long 
     const double x = ldst<CG>(&s.x[e]), v = ldst<CG>(&s.v[e]), a = ldst<CG>(&s.a[e]),
                  k = ldst<CG>(&s.k[e]);
     const int lev_old = ldst<CG>(&s.lev[i]);
-    AxisStep r;
     int ex;
-    if (step_exponent(ticks, ex)) {
-        r = correct_axis(x, v, a, k, apc, kpc, ex);
-    } else {
-        const double dt = ticks_to_time(ticks);
-        const double h = __dmul_rn(dt, 0.5), q3 = div_by<3>(dt);
-        const double dt2 = __dmul_rn(dt, dt);
-        const double dt3 = __dmul_rn(dt2, dt);
-        double xp, vp;
-        predict1hq(x, v, a, k, dt, h, q3, xp, vp);
-        const double d = __dsub_rn(a, apc);
-        const double a3 = __dadd_rn(__dmul_rn(2.0, d), __dmul_rn(__dadd_rn(k, kpc), dt));
-        const double a2 = __dsub_rn(__dmul_rn(-3.0, d), __dmul_rn(__dadd_rn(__dmul_rn(2.0, k), kpc), dt));
-        r.x = __dadd_rn(xp, __dmul_rn(__dadd_rn(div_by<12>(a2), div_by<20>(a3)), dt2));
-        r.v = __dadd_rn(vp, __dmul_rn(__dadd_rn(div_by<3>(a2), __dmul_rn(a3, 0.25)), dt));
-        const double s0 = __ddiv_rn(__dmul_rn(2.0, a2), dt2);
-        r.c = __ddiv_rn(__dmul_rn(6.0, a3), dt3);
-        r.s1 = __dadd_rn(s0, __dmul_rn(r.c, dt));
-    }
+    bool bad = !step_exponent(ticks, ex);
+    AxisStep r = correct_axis(x, v, a, k, apc, kpc, ex, bad);
+    if (bad) r = correct_axis_any(x, v, a, k, apc, kpc, ticks);
     // every lane of the quad has read the old state before any lane stores
     __syncwarp();
     if (own) {
