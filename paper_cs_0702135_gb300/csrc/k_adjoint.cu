@@ -28,15 +28,14 @@ namespace {
 
 using namespace dev;
 
-constexpr int kVNT = 128;  // threads per CTA = partners per tile
-#ifndef NB_VJP_R
-#define NB_VJP_R 2
+constexpr int kVNT = 128;  // partners per tile; FP64: threads per CTA
+constexpr int kVDsNT = 64; // DS: threads per CTA
+#ifndef NB_VJP_U2
+#define NB_VJP_U2 4
 #endif
-#ifndef NB_VJP_UNROLL
-#define NB_VJP_UNROLL 4
+#ifndef NB_VJP_U1
+#define NB_VJP_U1 4
 #endif
-constexpr int kVKR = NB_VJP_R;          // DS: particles k per thread
-constexpr int kVUnroll = NB_VJP_UNROLL; // DS: partner unrolling
 
 // One particle's VJP record: (predicted) position and velocity, mass and the
 // cotangents of its acc and jerk, in the layout of the context's precision.
@@ -65,16 +64,24 @@ __device__ __forceinline__ void write_vjp_record(int i, const double x[3], const
 }
 
 
+// The k side of a pair: the x and y components of position and velocity
+// negated and paired for the packed differences (see pair_ds_packed).
+struct VjpK {
+    IDS q;
+    float m, ab[3], kb[3];
+};
+
 // One (k, p) pair in FP32 on double-single positions; acc[0..2] xbar,
 // acc[3..5] vbar, acc[6] mbar.
 template <bool SOFT, bool GUARD>
-__device__ __forceinline__ void vjp_pair_ds(const VjpRec &P, const VjpRec &Kp, float eps2,
+__device__ __forceinline__ void vjp_pair_ds(const VjpRec &P, const VjpK &Kp, float eps2,
                                             float acc[7], int p = 0, int k = 1)
 {
-    const float dx = (P.ph.x - Kp.ph.x) + (P.pl.x - Kp.pl.x);
-    const float dy = (P.ph.y - Kp.ph.y) + (P.pl.y - Kp.pl.y);
-    const float dz = (P.ph.z - Kp.ph.z) + (P.pl.z - Kp.pl.z);
-    const float wx = P.v.x - Kp.v.x, wy = P.v.y - Kp.v.y, wz = P.v.z - Kp.v.z;
+    const float2 dxy = __fadd2_rn(__fadd2_rn(make_float2(P.ph.x, P.ph.y), Kp.q.nh),
+                                  __fadd2_rn(make_float2(P.pl.x, P.pl.y), Kp.q.nl));
+    const float2 wxy = __fadd2_rn(make_float2(P.v.x, P.v.y), Kp.q.nv);
+    const float dx = dxy.x, dy = dxy.y, dz = (P.ph.z - Kp.q.zh) + (P.pl.z - Kp.q.zl);
+    const float wx = wxy.x, wy = wxy.y, wz = P.v.z - Kp.q.vz;
     const float r2 = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, eps2)));
     float rinv = rsqrt_sfu(r2);
     if (!SOFT) rinv = (r2 > 0.0f) ? rinv : 0.0f;
@@ -84,13 +91,13 @@ __device__ __forceinline__ void vjp_pair_ds(const VjpRec &P, const VjpRec &Kp, f
     const float r5 = r3 * rinv2;
     const float r7 = r5 * rinv2;
     const float s = fmaf(dx, wx, fmaf(dy, wy, dz * wz));
-    const float mk = Kp.ph.w, mp = P.ph.w;
-    const float Ax = fmaf(mk, P.ab.x, -mp * Kp.ab.x);
-    const float Ay = fmaf(mk, P.ab.y, -mp * Kp.ab.y);
-    const float Az = fmaf(mk, P.ab.z, -mp * Kp.ab.z);
-    const float Kx = fmaf(mk, P.kb.x, -mp * Kp.kb.x);
-    const float Ky = fmaf(mk, P.kb.y, -mp * Kp.kb.y);
-    const float Kz = fmaf(mk, P.kb.z, -mp * Kp.kb.z);
+    const float mk = Kp.m, mp = P.ph.w;
+    const float Ax = fmaf(mk, P.ab.x, -mp * Kp.ab[0]);
+    const float Ay = fmaf(mk, P.ab.y, -mp * Kp.ab[1]);
+    const float Az = fmaf(mk, P.ab.z, -mp * Kp.ab[2]);
+    const float Kx = fmaf(mk, P.kb.x, -mp * Kp.kb[0]);
+    const float Ky = fmaf(mk, P.kb.y, -mp * Kp.kb[1]);
+    const float Kz = fmaf(mk, P.kb.z, -mp * Kp.kb[2]);
     const float Ad = fmaf(Ax, dx, fmaf(Ay, dy, Az * dz));
     const float Kd = fmaf(Kx, dx, fmaf(Ky, dy, Kz * dz));
     const float Kw = fmaf(Kx, wx, fmaf(Ky, wy, Kz * wz));
@@ -110,10 +117,11 @@ __device__ __forceinline__ void vjp_pair_ds(const VjpRec &P, const VjpRec &Kp, f
     acc[6] += fmaf(-r3, apd + kpw, 3.0f * s * kpd * r5);
 }
 
-template <bool SOFT>
-__global__ void __launch_bounds__(kVNT) k_force_vjp_ds(VjpArgs va)
+// R particles k per thread, tiles of kVNT partners.
+template <int R, bool SOFT>
+__global__ void __launch_bounds__(kVDsNT) k_force_vjp_ds(VjpArgs va)
 {
-    constexpr int R = kVKR;
+    constexpr int NT = kVDsNT;
     const Plan P = va.plan;
     __shared__ float4 s_ph[kVNT], s_pl[kVNT], s_v[kVNT], s_ab[kVNT], s_kb[kVNT];
     const float eps2 = (float)va.eps2;
@@ -123,26 +131,32 @@ __global__ void __launch_bounds__(kVNT) k_force_vjp_ds(VjpArgs va)
         const int j0 = sl * P.jslice;
         const int j1 = min(va.n, j0 + P.jslice);
         int kk[R], k[R];
-        VjpRec K[R];
+        VjpK K[R];
         float hi[R][7], lo[R][7];
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            kk[r] = ib * kVNT * R + r * kVNT + tid;
+            kk[r] = ib * NT * R + r * NT + tid;
             k[r] = clamp_index(kk[r], va.n);
-            K[r].ph = va.rec.ph[k[r]]; K[r].pl = va.rec.pl[k[r]]; K[r].v = va.rec.v[k[r]];
-            K[r].ab = va.rec.ab[k[r]]; K[r].kb = va.rec.kb[k[r]];
+            const float4 ph = va.rec.ph[k[r]], ab = va.rec.ab[k[r]], kb = va.rec.kb[k[r]];
+            K[r].q = make_ids(ph, va.rec.pl[k[r]], va.rec.v[k[r]]);
+            K[r].m = ph.w;
+            K[r].ab[0] = ab.x, K[r].ab[1] = ab.y, K[r].ab[2] = ab.z;
+            K[r].kb[0] = kb.x, K[r].kb[1] = kb.y, K[r].kb[2] = kb.z;
 #pragma unroll
             for (int c = 0; c < 7; ++c) hi[r][c] = lo[r][c] = 0.0f;
         }
         for (int jt = j0; jt < j1; jt += kVNT) {
             __syncthreads();
-            const int j = jt + tid;
-            const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-            s_ph[tid] = j < j1 ? va.rec.ph[j] : z;
-            s_pl[tid] = j < j1 ? va.rec.pl[j] : z;
-            s_v[tid] = j < j1 ? va.rec.v[j] : z;
-            s_ab[tid] = j < j1 ? va.rec.ab[j] : z;
-            s_kb[tid] = j < j1 ? va.rec.kb[j] : z;
+#pragma unroll
+            for (int u = 0; u < kVNT / NT; ++u) {
+                const int t = tid + u * NT, j = jt + t;
+                const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+                s_ph[t] = j < j1 ? va.rec.ph[j] : z;
+                s_pl[t] = j < j1 ? va.rec.pl[j] : z;
+                s_v[t] = j < j1 ? va.rec.v[j] : z;
+                s_ab[t] = j < j1 ? va.rec.ab[j] : z;
+                s_kb[t] = j < j1 ? va.rec.kb[j] : z;
+            }
             __syncthreads();
             float t[R][7];
 #pragma unroll
@@ -160,7 +174,8 @@ __global__ void __launch_bounds__(kVNT) k_force_vjp_ds(VjpArgs va)
                     for (int r = 0; r < R; ++r) vjp_pair_ds<SOFT, true>(Pq, K[r], eps2, t[r], jt + jj, k[r]);
                 }
             } else {
-#pragma unroll (kVUnroll)
+                constexpr int U = R == 1 ? NB_VJP_U1 : NB_VJP_U2;
+#pragma unroll (U)
                 for (int jj = 0; jj < kVNT; ++jj) {
                     VjpRec Pq;
                     Pq.ph = s_ph[jj]; Pq.pl = s_pl[jj]; Pq.v = s_v[jj]; Pq.ab = s_ab[jj]; Pq.kb = s_kb[jj];
@@ -192,6 +207,29 @@ __global__ void __launch_bounds__(kVNT) k_force_vjp_ds(VjpArgs va)
             }
         }
     }
+}
+
+// The DS sweep's particles per thread and slices.  Up to kVOneMax particles one
+// k per thread and slices of one tile: the sweep is then short of CTAs (4096:
+// 59 us, two k a thread 66, and 70 with 128-thread CTAs and slices of two tiles;
+// 1024: 15 against 23 us).  Above, two k per thread, each partner record
+// read from shared memory serving two pairs, and slices that make about
+// kVWaves waves of the resident CTAs, dealt out as CTAs end (65536: 12.4 ms,
+// 12.9 ms with one k; one wave 14.8 ms, three 12.7 ms).
+constexpr int kVOneMax = 8192, kVWaves = 8;
+
+Plan plan_vjp_ds(int n, int slots, long long part_cap, int &R)
+{
+    Plan p{};
+    R = n <= kVOneMax ? 1 : 2;
+    p.n_iblk = cdiv(n, kVDsNT * R);
+    const long long tiles = cdiv(n, kVNT);
+    long long L = R == 1 ? 1 : cdiv(tiles * p.n_iblk, (long long)kVWaves * slots);
+    while (L < tiles && cdiv(tiles, L) * (long long)kComp * n > part_cap) ++L;
+    p.jslice = (int)(L * kVNT);
+    p.S = cdiv(n, p.jslice);
+    p.items = p.n_iblk * p.S;
+    return p;
 }
 
 // FP64 twin, one k per thread, partners through shared memory.
@@ -298,8 +336,8 @@ __global__ void k_adj_pre(State st, double dt, const double *xb, const double *v
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             const long long q = 3LL * i + c;
-            const double a2b = xb[q] * dt * dt / 12.0 + vb[q] * dt / 3.0;
-            const double a3b = xb[q] * dt * dt / 20.0 + vb[q] * dt / 4.0;
+            const double a2b = div_by<12>(xb[q] * dt * dt) + div_by<3>(vb[q] * dt);
+            const double a3b = div_by<20>(xb[q] * dt * dt) + vb[q] * dt * 0.25;
             const double Db = 2.0 * a3b - 3.0 * a2b;
             a1b[c] = ab[q] - Db;
             k1b[c] = kb[q] + (a3b - a2b) * dt;
@@ -375,6 +413,172 @@ __global__ void k_set_ak(State st, const double *acc, const double *jerk)
         }
 }
 
+// ---------------------------------------------------------------------------
+// Trajectories with a shared power-of-two step dt: every particle is active in
+// every step and all are at one time, so the host knows each block and no
+// scheduler runs.  A step is the force sweep and one kernel that adds its
+// slices, corrects (or takes the force as it is, at the start), writes the new
+// state where the caller wants it (and to a checkpoint), and predicts the next
+// step's j records.  32 particles a CTA: a warp per force component adds the
+// slices, then a warp per axis does the FP64 chain, because a warp has one
+// FP64 instruction in flight whatever its lanes.  (The device-driven step's
+// seven launches and the copies took 95 us a step at 4096 bodies beside a
+// force of 38 us.)
+
+constexpr int kShNT = 256, kShP = 32;
+
+// Value c of particle a: the sum of its slices in order, or the result itself.
+__device__ __forceinline__ double sum_slices(const double *part, int S, int c, long long nb, long long a)
+{
+    double s = 0.0;
+#pragma unroll 8
+    for (int q = 0; q < S; ++q) s += part[((long long)q * kComp + c) * nb + a];
+    return s;
+}
+
+__global__ void __launch_bounds__(kShNT) k_shared_step(SharedStep q)
+{
+    __shared__ double s_f[6][kShP];
+    __shared__ double s_r[6][kShP];   // predicted x, v
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int n = q.src.n, i = blockIdx.x * kShP + lane;
+    if (q.mode != kShPredict && warp < 6 && i < n) {
+        const double *out = warp < 3 ? q.out.acc : q.out.jerk;
+        s_f[warp][lane] = q.S > 1 && i >= q.a0 ? sum_slices(q.part, q.S, warp, n - q.a0, i - q.a0)
+                                               : out[3LL * i + warp % 3];
+    }
+    __syncthreads();
+    const double dt = pow2d(-q.level);
+    if (warp < 3 && i < n) {
+        const long long e = (long long)warp * n + i;
+        double x = q.src.x[e], v = q.src.v[e], a = q.src.a[e], k = q.src.k[e];
+        if (q.mode != kShPredict) {
+            const double ap = s_f[warp][lane], kp = s_f[3 + warp][lane];
+            if (q.mode == kShCorrect) {
+                bool bad = false;
+                AxisStep r = correct_axis(x, v, a, k, ap, kp, -q.level, bad);
+                if (bad) r = correct_axis_any(x, v, a, k, ap, kp, 1LL << (kTickBits - q.level));
+                x = r.x, v = r.v;
+            }
+            a = ap, k = kp;
+            q.dst.x[e] = x, q.dst.v[e] = v, q.dst.a[e] = a, q.dst.k[e] = k;
+            if (q.copy.x) q.copy.x[e] = x, q.copy.v[e] = v, q.copy.a[e] = a, q.copy.k[e] = k;
+        }
+        if (q.predict) predict1hq(x, v, a, k, dt, half_dt(dt), div_core<3>(dt), s_r[warp][lane], s_r[3 + warp][lane]);
+    }
+    if (!q.predict) return;
+    __syncthreads();
+    if (warp >= 3 || i >= n) return;
+    const double m = q.src.m[i];
+    if (q.precision == NB_FP64) {
+        if (warp == 0) q.jf.pos[i] = make_double4_32a(s_r[0][lane], s_r[1][lane], s_r[2][lane], m);
+        if (warp == 1) q.jf.vel[i] = make_double4_32a(s_r[3][lane], s_r[4][lane], s_r[5][lane], 0.0);
+        return;
+    }
+    const double xp[3] = {s_r[0][lane], s_r[1][lane], s_r[2][lane]}, vp[3] = {s_r[3][lane], s_r[4][lane], s_r[5][lane]};
+    float hi[3], lo[3], u[3];
+    split_record(xp, vp, hi, lo, u);
+    if (warp == 0) q.jds.pos_hi[i] = make_float4(hi[0], hi[1], hi[2], to_float_int(m));
+    else if (warp == 1) q.jds.pos_lo[i] = make_float4(lo[0], lo[1], lo[2], 0.0f);
+    else q.jds.vel[i] = make_float4(u[0], u[1], u[2], 0.0f);
+}
+
+// After the last of `steps` shared steps: particle times, the block list and
+// the counters as the device-driven steps leave them.
+__global__ void k_shared_done(State s, Ctrl *ctrl, int *act, long long steps, int level)
+{
+    const int n = s.n;
+    const long long t = ctrl->t_now + steps * (1LL << (kTickBits - level));
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        s.t[i] = t;
+        act[i] = i;
+    }
+}
+__global__ void k_shared_ctrl(Ctrl *ctrl, int n, long long steps, int level)
+{
+    ctrl->t_now += steps * (1LL << (kTickBits - level));
+    ctrl->t_next = ctrl->t_now;
+    ctrl->n_active = n;
+    ctrl->steps += steps;
+    ctrl->interactions += steps * (long long)n * (long long)(n - 1);
+}
+
+// The reverse pass between two force VJPs, fused the same way: the slices of
+// the last VJP added; its second half (k_adj_post's formulas) or the final
+// accumulation; then the first half of the step before it (k_adj_pre's
+// formulas) or the record of the initial state, as the next VJP's records.
+// Every operation is written out, so the results do not depend on which parts
+// share a launch.
+__global__ void __launch_bounds__(kShNT) k_adj_step(AdjStep q)
+{
+    __shared__ double s_g[7][kShP];
+    __shared__ double s_r[12][kShP];   // x, v, and the cotangents of acc and jerk
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int n = q.st.n, i = blockIdx.x * kShP + lane;
+    if ((q.post || q.add) && warp < 7 && i < n) {
+        if (q.S > 1) s_g[warp][lane] = sum_slices(q.part, q.S, warp, n, i);
+        else s_g[warp][lane] = warp < 3 ? q.xg[3LL * i + warp] : (warp < 6 ? q.vg[3LL * i + warp - 3] : q.mg[i]);
+    }
+    __syncthreads();
+    const double dt = pow2d(-q.level), h = half_dt(dt), third = div_core<3>(dt);
+    if (warp < 3 && i < n) {
+        const long long e = 3LL * i + warp;
+        double xb = q.xb[e], vb = q.vb[e], ab = q.ab[e], kb = q.kb[e];
+        if (q.post) {
+            //   xp = x + v dt + a h dt + k q h dt,   vp = v + a dt + k h dt
+            const double xpb = __dadd_rn(xb, s_g[warp][lane]), vpb = __dadd_rn(vb, s_g[3 + warp][lane]);
+            xb = xpb;
+            vb = __fma_rn(xpb, dt, vpb);
+            ab = __dadd_rn(ab, __fma_rn(xpb, __dmul_rn(h, dt), __dmul_rn(vpb, dt)));
+            kb = __dadd_rn(kb, __fma_rn(__dmul_rn(xpb, third), __dmul_rn(h, dt), __dmul_rn(vpb, __dmul_rn(h, dt))));
+        } else if (q.add) {
+            xb = __dadd_rn(xb, s_g[warp][lane]);
+            vb = __dadd_rn(vb, s_g[3 + warp][lane]);
+        }
+        if (q.pre != kAdjNone) {
+            const long long c = (long long)warp * n + i;
+            const double x = q.st.x[c], v = q.st.v[c];
+            if (q.pre == kAdjPre) {
+                //   a2b = xb dt^2/12 + vb dt/3,  a3b = xb dt^2/20 + vb dt/4,  Db = 2 a3b - 3 a2b
+                const double xd = __dmul_rn(xb, __dmul_rn(dt, dt)), vd = __dmul_rn(vb, dt);
+                const double a2b = __dadd_rn(div_by<12>(xd), div_by<3>(vd));
+                const double a3b = __dadd_rn(div_by<20>(xd), __dmul_rn(vd, 0.25));
+                const double Db = __fma_rn(-3.0, a2b, __dmul_rn(2.0, a3b));
+                s_r[6 + warp][lane] = __dsub_rn(ab, Db);
+                s_r[9 + warp][lane] = __fma_rn(__dsub_rn(a3b, a2b), dt, kb);
+                ab = Db;
+                kb = __dmul_rn(__fma_rn(-2.0, a2b, a3b), dt);
+                predict1hq(x, v, q.st.a[c], q.st.k[c], dt, h, third, s_r[warp][lane], s_r[3 + warp][lane]);
+            } else {
+                s_r[warp][lane] = x;
+                s_r[3 + warp][lane] = v;
+                s_r[6 + warp][lane] = ab;
+                s_r[9 + warp][lane] = kb;
+            }
+        }
+        q.xb[e] = xb, q.vb[e] = vb, q.ab[e] = ab, q.kb[e] = kb;
+    }
+    if (warp == 3 && i < n && (q.post || q.add)) q.mb[i] = __dadd_rn(q.mb[i], s_g[6][lane]);
+    if (q.pre == kAdjNone) return;
+    __syncthreads();
+    // four warps share the record: position, velocity, two cotangents
+    if (warp >= 4 || i >= n) return;
+    const double r[3] = {s_r[3 * warp][lane], s_r[3 * warp + 1][lane], s_r[3 * warp + 2][lane]};
+    const double m = q.st.m[i];
+    if (q.precision == NB_FP64) {
+        double4_32a *const dst[4] = {q.rec64.x, q.rec64.v, q.rec64.ab, q.rec64.kb};
+        dst[warp][i] = make_double4_32a(r[0], r[1], r[2], warp == 0 ? m : 0.0);
+    } else if (warp == 0) {
+        float hi[3], lo[3], u[3];
+        split_record(r, r, hi, lo, u);
+        q.rec.ph[i] = make_float4(hi[0], hi[1], hi[2], to_float_int(m));
+        q.rec.pl[i] = make_float4(lo[0], lo[1], lo[2], 0.0f);
+    } else {
+        float4 *const dst = warp == 1 ? q.rec.v : (warp == 2 ? q.rec.ab : q.rec.kb);
+        dst[i] = make_float4(to_float_int(r[0]), to_float_int(r[1]), to_float_int(r[2]), 0.0f);
+    }
+}
+
 // Copies of the FP64 state (checkpoints).
 __global__ void k_copy_state(State dst, State src)
 {
@@ -401,33 +605,58 @@ int vjp_slots(int precision, int sms)
     int b = 0;
     cudaError_t e = precision == NB_FP64
                         ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_force_vjp_f64<true>, kVNT, 0)
-                        : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_force_vjp_ds<true>, kVNT, 0);
+                        : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_force_vjp_ds<2, true>, kVDsNT, 0);
     return e == cudaSuccess ? sms * (b > 0 ? b : 1) : sms;
 }
 
 int vjp_tile() { return kVNT; }
 
-int launch_force_vjp(const VjpArgs &va_in, int precision, bool softened, cudaStream_t st)
+int launch_force_vjp(const VjpArgs &va_in, int precision, bool softened, bool combine, int *slices,
+                     cudaStream_t st)
 {
     VjpArgs va = va_in;
-    // once, on the host; the DS kernel owns kVKR particles per thread
-    va.plan = plan_ipar(va.n, va.n, kVNT * (precision == NB_FP64 ? 1 : kVKR), kVNT, va.slots, 0,
-                        va.part_cap);
-    const Plan P = va.plan;
-    const int g = P.items < va.slots ? P.items : va.slots;
     if (precision == NB_FP64) {
+        va.plan = plan_ipar(va.n, va.n, kVNT, kVNT, va.slots, 0, va.part_cap);
+        const int g = va.plan.items < va.slots ? va.plan.items : va.slots;
         if (softened) k_force_vjp_f64<true><<<g, kVNT, 0, st>>>(va);
         else k_force_vjp_f64<false><<<g, kVNT, 0, st>>>(va);
     } else {
-        if (softened) k_force_vjp_ds<true><<<g, kVNT, 0, st>>>(va);
-        else k_force_vjp_ds<false><<<g, kVNT, 0, st>>>(va);
+        int R = 2;
+        va.plan = plan_vjp_ds(va.n, va.slots, va.part_cap, R);
+        const int g = va.plan.items;
+        if (R == 1) {
+            if (softened) k_force_vjp_ds<1, true><<<g, kVDsNT, 0, st>>>(va);
+            else k_force_vjp_ds<1, false><<<g, kVDsNT, 0, st>>>(va);
+        } else {
+            if (softened) k_force_vjp_ds<2, true><<<g, kVDsNT, 0, st>>>(va);
+            else k_force_vjp_ds<2, false><<<g, kVDsNT, 0, st>>>(va);
+        }
     }
+    const Plan P = va.plan;
     int launches = 1;
-    if (P.S > 1) {
+    // without the combine the caller adds the slices, in slice order
+    if (slices) *slices = combine ? 1 : P.S;
+    if (P.S > 1 && combine) {
         k_vjp_combine<<<grid_for(7LL * va.n, 256), 256, 0, st>>>(va, P.S);
         ++launches;
     }
     return launches;
+}
+
+void launch_shared_step(const SharedStep &q, cudaStream_t st)
+{
+    k_shared_step<<<cdiv(q.src.n, kShP), kShNT, 0, st>>>(q);
+}
+
+void launch_shared_done(const State &s, Ctrl *ctrl, int *act, long long steps, int level, cudaStream_t st)
+{
+    k_shared_done<<<grid_for(s.n, 256), 256, 0, st>>>(s, ctrl, act, steps, level);
+    k_shared_ctrl<<<1, 1, 0, st>>>(ctrl, s.n, steps, level);
+}
+
+void launch_adj_step(const AdjStep &q, cudaStream_t st)
+{
+    k_adj_step<<<cdiv(q.st.n, kShP), kShNT, 0, st>>>(q);
 }
 
 void launch_adj_pre(const State &s, double dt, const double *xb, const double *vb, double *ab,

@@ -509,7 +509,7 @@ int combine_grid(const ForceArgs &fa)
 }  // namespace
 
 int launch_force_ds(const ForceArgs &fa, const JDS &j, bool softened, int grid_ipar,
-                    int grid_jpar, int grid_small, cudaStream_t st)
+                    int grid_jpar, int grid_small, bool combine, cudaStream_t st)
 {
     if (softened) {
         if (grid_ipar > 0)
@@ -526,7 +526,7 @@ int launch_force_ds(const ForceArgs &fa, const JDS &j, bool softened, int grid_i
     }
     int launches = (grid_ipar > 0) + (grid_small > 0) + (grid_jpar > 0);
     // a host-sized j-parallel launch combines its own slices
-    if (fa.na_dev || grid_ipar > 0 || grid_small > 0) {
+    if (combine && (fa.na_dev || grid_ipar > 0 || grid_small > 0)) {
         k_force_combine<<<combine_grid(fa), 256, 0, st>>>(fa, NB_DS);
         ++launches;
     }

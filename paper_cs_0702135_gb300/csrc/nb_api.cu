@@ -84,6 +84,9 @@ struct nb_ctx {
     VjpRec64 vrec64{};
     int slots_vjp = 0;
     bool traj_valid = false;
+    bool traj_shared = false;       // made by the shared-step kernels
+    // every particle at one time with level_fixed (else the scheduler picks blocks)
+    bool synchronous = false;
     long long traj_steps = 0, traj_ckpt = 0;
 
     // measurement counters (nb_get_stats)
@@ -219,13 +222,15 @@ ForceOut res_out(nb_ctx *c)
 // precision is launched with a persistent grid and all but the one serving the
 // block exit at once.  Otherwise the host plans, and only the kernel that
 // serves na_host is launched, sized to its work.
-void enqueue_force(nb_ctx *c, const int *act, int na_host, const int *na_dev, ForceOut out)
+// combine = false (host-sized, DS, compensated sums): the slices of an
+// i-parallel launch are left to the caller, as the returned plan says.
+Plan enqueue_force(nb_ctx *c, const int *act, int na_host, const int *na_dev, ForceOut out, bool combine = true)
 {
     const ForceArgs fa = force_args(c, act, na_host, na_dev, out);
     const bool f64 = c->o.precision == NB_FP64;
     int gi = c->slots_ipar, gj = c->slots_jpar, gs = f64 ? 0 : c->slots_small;
     if (!na_dev) {
-        if (na_host <= 0) return;
+        if (na_host <= 0) return fa.plan.p;
         const Plan &p = fa.plan.p;
         gi = gj = gs = 0;
         if (fa.plan.regime == kRegJpar) gj = p.items < c->slots_jpar ? p.items : c->slots_jpar;
@@ -234,7 +239,7 @@ void enqueue_force(nb_ctx *c, const int *act, int na_host, const int *na_dev, Fo
     }
     const bool summed = c->o.summation != NB_SUM_COMPENSATED;
     const int gsum = summed ? grid_summed(fa, c->sum) : 0;
-    if (summed && gsum <= 0) return;
+    if (summed && gsum <= 0) return fa.plan.p;
     cudaEvent_t ev[2] = {nullptr, nullptr};
     const bool timed = c->profiling && !c->capturing;
     if (timed) {
@@ -254,7 +259,7 @@ void enqueue_force(nb_ctx *c, const int *act, int na_host, const int *na_dev, Fo
         launch_force_f64(fa, c->jf, c->eps > 0.0, gi, gj, c->st);
         c->launches += (gi > 0) + (gj > 0) + 1;
     } else {
-        c->launches += launch_force_ds(fa, c->jds, c->eps > 0.0, gi, gj, gs, c->st);
+        c->launches += launch_force_ds(fa, c->jds, c->eps > 0.0, gi, gj, gs, combine, c->st);
     }
     if (timed) {
         if (ev[0] && ev[1]) {
@@ -266,6 +271,9 @@ void enqueue_force(nb_ctx *c, const int *act, int na_host, const int *na_dev, Fo
                 if (e) c->ev_free.push_back(e);
         }
     }
+    Plan left = fa.plan.p;
+    if (summed || f64 || combine || fa.plan.regime == kRegJpar) left.S = 1;   // results are whole
+    return left;
 }
 
 // The device-driven block step: schedule, predict all, force, correct.
@@ -372,7 +380,8 @@ double *cot(nb_ctx *c, int which)  // 0 xb, 1 vb, 2 ab, 3 kb, 4 mb, 5 xg, 6 vg, 
 
 // VJP of every particle's acc and jerk at the records in c->vrec / vrec64,
 // results into xg, vg, mg.
-void enqueue_vjp(nb_ctx *c)
+// combine = false: the slices (their count is returned) are left in d_part.
+int enqueue_vjp(nb_ctx *c, bool combine = true)
 {
     VjpArgs va{};
     va.n = c->n;
@@ -386,7 +395,9 @@ void enqueue_vjp(nb_ctx *c)
     va.xbar = cot(c, 5);
     va.vbar = cot(c, 6);
     va.mbar = cot(c, 7);
-    c->launches += launch_force_vjp(va, c->o.precision, c->eps > 0.0, c->st);
+    int slices = 1;
+    c->launches += launch_force_vjp(va, c->o.precision, c->eps > 0.0, combine, &slices, c->st);
+    return slices;
 }
 
 int copy_results_out(nb_ctx *c, int na, double *acc, double *jerk, double *pot, cudaMemcpyKind k)
@@ -397,6 +408,51 @@ int copy_results_out(nb_ctx *c, int na, double *acc, double *jerk, double *pot, 
         CK(cudaMemcpyAsync(jerk, c->d_res + 3LL * c->n, sizeof(double) * 3 * (size_t)na, k, c->st));
     if (pot) CK(cudaMemcpyAsync(pot, c->d_res + 6LL * c->n, sizeof(double) * (size_t)na, k, c->st));
     return NB_OK;
+}
+
+// The force on all particles from the j records, then one shared step's kernel.
+// src = dst in place; copy: a second place for the new state (or none).
+void enqueue_shared(nb_ctx *c, int mode, const State &src, const State &dst, const State *copy, bool predict)
+{
+    SharedStep q{};
+    q.mode = mode;
+    q.predict = predict;
+    q.src = src;
+    q.dst = dst;
+    if (copy) q.copy = *copy;
+    q.level = c->o.level_fixed;
+    q.precision = c->o.precision;
+    q.out = res_out(c);
+    if (mode != kShPredict) {
+        const Plan p = enqueue_force(c, c->d_all, c->n, nullptr, q.out, false);
+        q.part = c->d_part;
+        q.S = p.S;
+        q.a0 = p.a0;
+    }
+    q.jds = c->jds;
+    q.jf = c->jf;
+    launch_shared_step(q, c->st);
+    c->launches += 1;
+}
+
+// One kernel of the reverse pass; slices: of the VJP before it (post or add).
+void enqueue_adj(nb_ctx *c, bool post, bool add, int slices, int pre, const State &st)
+{
+    AdjStep q{};
+    q.post = post;
+    q.add = add;
+    q.pre = pre;
+    q.st = st;
+    q.level = c->o.level_fixed;
+    q.precision = c->o.precision;
+    q.S = slices;
+    q.part = c->d_part;
+    q.xg = cot(c, 5), q.vg = cot(c, 6), q.mg = cot(c, 7);
+    q.xb = cot(c, 0), q.vb = cot(c, 1), q.ab = cot(c, 2), q.kb = cot(c, 3), q.mb = cot(c, 4);
+    q.rec = c->vrec;
+    q.rec64 = c->vrec64;
+    launch_adj_step(q, c->st);
+    c->launches += 1;
 }
 
 // nb_run in one persistent launch (k_run.cu) when the system is small enough:
@@ -655,6 +711,7 @@ static int init_impl(nb_ctx *c, int64_t n, const double *m, const double *x, con
     CK(cudaGetLastError());
     c->t_pred = 0;
     c->force_valid = false;
+    c->synchronous = o.level_fixed > 0;
     return sync_ctrl(c);
 }
 
@@ -795,6 +852,7 @@ int nb_correct(nb_ctx *c, const int32_t *idx, int32_t na, double t, const double
         kn = c->d_stage + 3 * N;
     }
     CK(cudaMemcpyAsync(c->d_idx, idx, sizeof(int) * (size_t)na, cudaMemcpyHostToDevice, c->st));
+    c->synchronous = false;   // the caller chose the particles and the time
     launch_correct(c->S, c->d_idx, na, nullptr, ticks, nullptr, an, kn, c->o.eta, c->o.level_min,
                    c->o.level_fixed, &c->d_ctrl->err, c->sms, c->st);
     CK(cudaGetLastError());
@@ -842,7 +900,10 @@ int nb_run(nb_ctx *c, double t_end, int64_t max_steps, int64_t *steps_out, int64
     c->force_valid = false;
     rc = run_persistent(c, te, max_steps);
     if (rc != kRunNotUsed) {
-        if (rc) return rc;
+        if (rc) {
+            c->synchronous = false;
+            return rc;
+        }
         if (steps_out) *steps_out = c->h_ctrl->steps - steps0;
         if (inter_out) *inter_out = c->h_ctrl->interactions - inter0;
         return set_t_end(c, LLONG_MAX);
@@ -972,6 +1033,7 @@ int nb_set_state(nb_ctx *c, const double *x, const double *v, const double *a, c
         !finite_all(k, 3 * N))
         return fail(c, NB_EINVAL, "non-finite state");
     long long t_max = 0;
+    bool synchronous = c->o.level_fixed > 0;
     for (long long i = 0; i < N; ++i) {
         if (lev[i] < c->o.level_min || lev[i] > kTickBits)
             return fail(c, NB_EINVAL, "level[%lld]=%d outside [%d, 40]", i, lev[i], c->o.level_min);
@@ -979,8 +1041,10 @@ int nb_set_state(nb_ctx *c, const double *x, const double *v, const double *a, c
         if (t[i] < 0 || t[i] % dt != 0 || t[i] > (1LL << 62))
             return fail(c, NB_EINVAL, "t_ticks[%lld] is not a multiple of its step", i);
         if (t[i] > t_max) t_max = t[i];
+        synchronous = synchronous && t[i] == t[0] && lev[i] == c->o.level_fixed;
     }
     CK(cudaStreamSynchronize(c->st));
+    c->synchronous = false;   // until the whole state is in
     CK(cudaMemcpyAsync(c->d_stage, x, sizeof(double) * 3 * N, cudaMemcpyHostToDevice, c->st));
     CK(cudaMemcpyAsync(c->d_stage + 3 * N, v, sizeof(double) * 3 * N, cudaMemcpyHostToDevice, c->st));
     launch_scatter_state(c->S, c->d_stage, c->d_stage + 3 * N, nullptr, nullptr, c->st);
@@ -997,6 +1061,7 @@ int nb_set_state(nb_ctx *c, const double *x, const double *v, const double *a, c
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(c->st));
     c->force_valid = false;
+    c->synchronous = synchronous;
     return NB_OK;
 }
 
@@ -1070,6 +1135,28 @@ int nb_traj_forward(nb_ctx *c, int64_t steps, int64_t checkpoint_every)
     if ((rc = set_t_end(c, LLONG_MAX))) return rc;
     // the initial acceleration and jerk are the force of the initial state
     launch_predict(c->S, 0, &c->d_ctrl->t_now, nullptr, c->o.precision, c->jds, c->jf, c->st);
+    c->traj_valid = false;
+    c->traj_shared = c->synchronous;
+    if (c->traj_shared) {
+        const State ck0 = state_view(c, c->d_ck);
+        enqueue_shared(c, kShStart, c->S, c->S, &ck0, true);
+        for (long long s = 0; s < steps; ++s) {
+            const bool last = s + 1 == steps;
+            const State keep = state_view(c, last ? c->d_fin : c->d_ck + (s + 1) / checkpoint_every * per);
+            enqueue_shared(c, kShCorrect, c->S, c->S,
+                           last || (s + 1) % checkpoint_every == 0 ? &keep : nullptr, !last);
+        }
+        launch_shared_done(c->S, c->d_ctrl, c->d_act, steps, c->o.level_fixed, c->st);
+        c->launches += 3;
+        CK(cudaMemcpyAsync(c->d_tfin, c->d_t, sizeof(long long) * N, cudaMemcpyDeviceToDevice, c->st));
+        CK(cudaGetLastError());
+        c->force_valid = false;
+        if ((rc = sync_ctrl(c))) return rc;
+        c->traj_valid = true;
+        c->traj_steps = steps;
+        c->traj_ckpt = checkpoint_every;
+        return NB_OK;
+    }
     enqueue_full_sweep(c);
     launch_set_ak(c->S, c->d_res, c->d_res + 3 * N, c->st);
     c->launches += 2;
@@ -1120,7 +1207,29 @@ static int traj_backward_impl(nb_ctx *c, const double *xbar_T, const double *vba
     CK(cudaMemsetAsync(cot(c, 2), 0, sizeof(double) * (6 * N + N), c->st));  // ab, kb, mb
     const long long steps = c->traj_steps, ck = c->traj_ckpt;
     const long long nseg = (steps + ck - 1) / ck;
-    for (long long seg = nseg - 1; seg >= 0; --seg) {
+    if (c->traj_shared) {
+        // state q of a segment: its checkpoint, then d_seg; the state after the
+        // segment's last step is not needed again
+        int slices = 0;   // of the VJP that the next kernel takes in
+        for (long long seg = nseg - 1; seg >= 0; --seg) {
+            const long long s0 = seg * ck, len = (s0 + ck < steps ? ck : steps - s0);
+            auto at = [&](long long q) { return state_view(c, q ? c->d_seg + q * per : c->d_ck + seg * per); };
+            // the VJP of the step after this segment goes first: d_part is the force's too
+            if (slices) enqueue_adj(c, true, false, slices, kAdjNone, at(0));
+            if (len > 1) enqueue_shared(c, kShPredict, at(0), at(0), nullptr, true);
+            for (long long q = 0; q + 1 < len; ++q)
+                enqueue_shared(c, kShCorrect, at(q), at(q + 1), nullptr, q + 2 < len);
+            for (long long q = len - 1; q >= 0; --q) {
+                if (q == len - 1) enqueue_adj(c, false, false, 0, kAdjPre, at(q));
+                else enqueue_adj(c, true, false, slices, kAdjPre, at(q));
+                slices = enqueue_vjp(c, false);
+            }
+        }
+        enqueue_adj(c, true, false, slices, kAdjInitial, state_view(c, c->d_ck));
+        slices = enqueue_vjp(c, false);
+        enqueue_adj(c, false, true, slices, kAdjNone, state_view(c, c->d_ck));
+    }
+    for (long long seg = nseg - 1; seg >= 0 && !c->traj_shared; --seg) {
         const long long s0 = seg * ck, len = (s0 + ck < steps ? ck : steps - s0);
         // recompute the segment's step states from its checkpoint
         launch_copy_state(c->S, state_view(c, c->d_ck + seg * per), c->st);
@@ -1139,12 +1248,14 @@ static int traj_backward_impl(nb_ctx *c, const double *xbar_T, const double *vba
             c->launches += 2;
         }
     }
-    // the initial acceleration and jerk were the force of the initial state
-    launch_adj_initial_rec(state_view(c, c->d_ck), cot(c, 2), cot(c, 3), c->o.precision, c->vrec,
-                           c->vrec64, c->st);
-    enqueue_vjp(c);
-    launch_add3(c->n, cot(c, 0), cot(c, 5), cot(c, 1), cot(c, 6), cot(c, 4), cot(c, 7), c->st);
-    c->launches += 2;
+    if (!c->traj_shared) {
+        // the initial acceleration and jerk were the force of the initial state
+        launch_adj_initial_rec(state_view(c, c->d_ck), cot(c, 2), cot(c, 3), c->o.precision, c->vrec,
+                               c->vrec64, c->st);
+        enqueue_vjp(c);
+        launch_add3(c->n, cot(c, 0), cot(c, 5), cot(c, 1), cot(c, 6), cot(c, 4), cot(c, 7), c->st);
+        c->launches += 2;
+    }
     CK(cudaGetLastError());
     if (xbar0) CK(cudaMemcpyAsync(xbar0, cot(c, 0), sizeof(double) * 3 * N, kout, c->st));
     if (vbar0) CK(cudaMemcpyAsync(vbar0, cot(c, 1), sizeof(double) * 3 * N, kout, c->st));

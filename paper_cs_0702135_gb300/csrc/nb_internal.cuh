@@ -536,7 +536,7 @@ struct VjpArgs {
     double eps2;
     int slots;
     long long part_cap;
-    Plan plan;             // plan_ipar over all n particles (set by the launcher)
+    Plan plan;             // over all n particles (set by the launcher)
     double *part;          // slice partials part[(s * 7 + c) * n + k]
     VjpRecDS rec;
     VjpRec64 rec64;
@@ -544,13 +544,44 @@ struct VjpArgs {
     double *xbar, *vbar, *mbar;  // outputs [n][3], [n][3], [n] (overwritten)
 };
 
+// One kernel of a trajectory with a shared step 2^-level (k_shared_step).
+enum ShMode { kShPredict = 0, kShStart = 1, kShCorrect = 2 };
+struct SharedStep {
+    int mode;              // predict only; take the force as acc and jerk; correct with it
+    bool predict;          // then write the next step's j records
+    State src, dst, copy;  // state before and after the step; copy.x may be null
+    int level, precision;
+    // the force: slices part[(s * 7 + c) * (n - a0) + (a - a0)] from particle a0 on
+    // when S > 1, the results themselves otherwise
+    const double *part;
+    int S, a0;
+    ForceOut out;
+    JDS jds;
+    JF64 jf;
+};
+
+// One kernel of its reverse pass (k_adj_step).
+enum AdjMode { kAdjNone = 0, kAdjPre = 1, kAdjInitial = 2 };
+struct AdjStep {
+    bool post, add;        // take the VJP through the predictor, or just add it
+    int pre;               // then the records of the next VJP
+    State st;              // the state those start from
+    int level, precision, S;
+    const double *part;    // S > 1: the VJP's slices, else xg, vg, mg
+    const double *xg, *vg, *mg;
+    double *xb, *vb, *ab, *kb, *mb;
+    VjpRecDS rec;
+    VjpRec64 rec64;
+};
+
 // ---------------------------------------------------------------------------
 // Launchers (defined in the .cu files).
 
 // k_force.cu
 // Returns the number of kernels launched.
+// combine: add the slices of an i-parallel launch (else the caller does).
 int launch_force_ds(const ForceArgs &fa, const JDS &j, bool softened, int grid_ipar, int grid_jpar,
-                    int grid_small, cudaStream_t st);
+                    int grid_small, bool combine, cudaStream_t st);
 void launch_force_f64(const ForceArgs &fa, const JF64 &j, bool softened, int grid_ipar,
                       int grid_jpar, cudaStream_t st);
 int occupancy_force(int precision, int regime, int *blocks_per_sm);
@@ -604,7 +635,11 @@ void launch_check_input(const double *p, long long cnt, bool nonneg, int *err, c
 // k_adjoint.cu
 int vjp_slots(int precision, int sms);
 int vjp_tile();
-int launch_force_vjp(const VjpArgs &va, int precision, bool softened, cudaStream_t st);
+int launch_force_vjp(const VjpArgs &va, int precision, bool softened, bool combine, int *slices,
+                     cudaStream_t st);
+void launch_shared_step(const SharedStep &q, cudaStream_t st);
+void launch_shared_done(const State &s, Ctrl *ctrl, int *act, long long steps, int level, cudaStream_t st);
+void launch_adj_step(const AdjStep &q, cudaStream_t st);
 void launch_adj_pre(const State &s, double dt, const double *xb, const double *vb, double *ab,
                     double *kb, int precision, const VjpRecDS &rec, const VjpRec64 &rec64,
                     cudaStream_t st);

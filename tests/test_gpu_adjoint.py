@@ -225,3 +225,41 @@ def test_traj_backward_dev_matches_host(nb):
         assert ei.value.code == nb.NB_EINVAL
     finally:
         c.nb_free()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("n", [31, 96, 130, 700])
+def test_shared_steps_match_scheduled_steps(nb, n, precision):
+    # A synchronous context runs the fused shared-step kernels; after a
+    # host-driven correction the context no longer knows that its particles
+    # are at one time and lets the scheduler pick the blocks.  Same state, same
+    # steps: the sums of slices differ in order alone (2^-53 each, amplified
+    # little over six steps), 1e-11 of the largest component.
+    m, x, v = plummer(n, 300 + n)
+    rng = np.random.RandomState(n)
+    gx, gv = rng.normal(size=(n, 3)), rng.normal(size=(n, 3))
+    idx = np.arange(n, dtype=np.int32)
+    out = []
+    for shared in (True, False):
+        ctx = nb.Context(m, x, v, 1.0 / 64, level_fixed=9, precision=precision)
+        try:
+            if shared:
+                ctx.nb_step()
+            else:
+                ctx.nb_predict(2.0 ** -9)
+                ctx.nb_force(idx)
+                ctx.nb_correct(idx, 2.0 ** -9)
+            ctx.nb_traj_forward(6, 4)
+            st = ctx.nb_get_state()
+            act, ticks = ctx.nb_get_active()
+            assert np.array_equal(act, idx) and ticks == 7 << 31
+            grads = ctx.nb_traj_backward(gx, gv)
+            after = ctx.nb_get_state()
+            assert all(np.array_equal(st[k], after[k]) for k in st)
+            out.append((st, grads))
+        finally:
+            ctx.nb_free()
+    (sa, ga), (sb, gb) = out
+    assert np.array_equal(sa["t"], sb["t"]) and np.array_equal(sa["level"], sb["level"])
+    for a, b in [(sa[k], sb[k]) for k in ("x", "v", "a", "k")] + list(zip(ga, gb)):
+        assert np.abs(a - b).max() <= 1e-11 * np.abs(b).max()
