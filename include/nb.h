@@ -163,7 +163,7 @@ int nb_force(nb_ctx *ctx, const int32_t *active_idx, int32_t n_active, double *a
  * kernels clamp every index into [0, n), so a bad index only wastes work); the
  * call then synchronises the context's stream once and returns NB_EINVAL for
  * a bad or repeated index, leaving the outputs untouched.  On success the
- * copies into the outputs are enqueued on the context's stream.
+ * outputs have been written.
  */
 int nb_force_dev(nb_ctx *ctx, const int32_t *d_active_idx, int32_t n_active, double *d_acc,
                  double *d_jerk, double *d_pot);

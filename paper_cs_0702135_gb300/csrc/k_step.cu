@@ -327,6 +327,57 @@ __global__ void k_validate(const int *idx, int na, int n, unsigned int *bitmap, 
     }
 }
 
+// Force results from the context into the caller's arrays (device memory, or
+// pinned host memory), unless an error is set, and the control block into its
+// pinned mirror, so that the call needs no copies of its own.  With `validate`
+// (one CTA, na <= kPublishCheckMax) the indices are checked first, by a hash
+// table in shared memory: a block of a few particles spares the bitmap's
+// clearing and the separate check.
+constexpr int kPubNT = 512, kPubSlots = 2048;
+static_assert(2 * kPublishCheckMax <= kPubSlots, "the table stays half empty");
+
+__global__ void __launch_bounds__(kPubNT) k_publish(PublishArgs p)
+{
+    __shared__ int s_tab[kPubSlots];
+    __shared__ int s_err;
+    const int tid = threadIdx.x;
+    if (tid == 0) s_err = p.ctrl->err;
+    if (p.validate)
+        for (int q = tid; q < kPubSlots; q += kPubNT) s_tab[q] = -1;
+    __syncthreads();
+    if (p.validate) {
+        for (int a = tid; a < p.na; a += kPubNT) {
+            const int i = p.idx[a];
+            bool bad = i < 0 || i >= p.n;
+            unsigned h = ((unsigned)i * 2654435761u) >> 21;
+            while (!bad) {   // at most na of the slots are taken, so a free one is met
+                const int old = atomicCAS(&s_tab[h], -1, i);
+                if (old == -1) break;
+                bad = old == i;
+                h = (h + 1) & (kPubSlots - 1);
+            }
+            if (bad) {
+                raise_err(&p.ctrl->err, NB_EINVAL);
+                s_err = NB_EINVAL;
+            }
+        }
+        __syncthreads();
+    }
+    if (s_err == 0) {
+        const long long n3 = 3LL * p.na, step = (long long)gridDim.x * kPubNT;
+        for (long long e = blockIdx.x * (long long)kPubNT + tid; e < n3; e += step) {
+            if (p.out.acc) p.out.acc[e] = p.res.acc[e];
+            if (p.out.jerk) p.out.jerk[e] = p.res.jerk[e];
+            if (p.out.pot && e < p.na) p.out.pot[e] = p.res.pot[e];
+        }
+    }
+    if (blockIdx.x == 0 && tid < (int)(sizeof(Ctrl) / 8)) {
+        static_assert(sizeof(Ctrl) % 8 == 0, "copied by 8-byte words");
+        __threadfence();
+        reinterpret_cast<volatile long long *>(p.host)[tid] = reinterpret_cast<volatile long long *>(p.ctrl)[tid];
+    }
+}
+
 __global__ void k_check_input(const double *p, long long cnt, bool nonneg, int *err)
 {
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < cnt;
@@ -434,6 +485,12 @@ void launch_validate(const int *idx, int na, int n, unsigned int *bitmap, int *e
 {
     if (na <= 0) return;
     k_validate<<<grid_for(na, 256), 256, 0, st>>>(idx, na, n, bitmap, err);
+}
+
+void launch_publish(const PublishArgs &p, cudaStream_t st)
+{
+    const long long g = p.validate ? 1 : (3LL * p.na + kPubNT - 1) / kPubNT;
+    k_publish<<<(int)std::max(1LL, std::min(g, 1024LL)), kPubNT, 0, st>>>(p);
 }
 
 void launch_gather_state(const State &s, double *x, double *v, double *a, double *k, cudaStream_t st)

@@ -49,6 +49,9 @@ struct nb_ctx {
     unsigned *d_bitmap = nullptr;   // index validation
     Ctrl *d_ctrl = nullptr;
     Ctrl *h_ctrl = nullptr;         // pinned mirror
+    double *h_stage = nullptr;      // pinned, behind it: results [7] and index of stage_na particles
+    int stage_na = 0;
+    std::vector<uint64_t> seen;     // index check on the host: a bit per particle, clear between calls
     long long *d_blockmin = nullptr;
     int *d_blockcnt = nullptr;
     int nsched = 0;
@@ -100,6 +103,10 @@ struct nb_ctx {
 
 namespace {
 
+// Blocks of host arrays go through pinned staging up to this size (16384 made
+// nb_init 0.27 ms longer, and above a few thousand the force hides the copies).
+constexpr int kStageMax = 4096;
+
 const char *const kNoCtx = "null context";
 thread_local std::string g_init_err;  // message of the last failed nb_init on this thread
 
@@ -145,14 +152,26 @@ int check_indices_host(nb_ctx *c, const int32_t *idx, int32_t na)
 {
     if (na < 0 || na > c->n) return fail(c, NB_EINVAL, "n_active=%d outside [0, %d]", na, c->n);
     if (na > 0 && !idx) return fail(c, NB_EINVAL, "active_idx is NULL");
-    std::vector<unsigned char> seen((size_t)c->n, 0);
-    for (int32_t a = 0; a < na; ++a) {
-        const int32_t i = idx[a];
-        if (i < 0 || i >= c->n) return fail(c, NB_EINVAL, "active_idx[%d]=%d out of range", a, i);
-        if (seen[(size_t)i]) return fail(c, NB_EINVAL, "active_idx[%d]=%d repeated", a, i);
-        seen[(size_t)i] = 1;
+    // the bits are set and cleared again: a call costs its own indices, not n
+    if (c->seen.empty()) c->seen.assign(((size_t)c->n + 63) / 64, 0);
+    int rc = NB_OK;
+    int32_t marked = 0;
+    for (; marked < na; ++marked) {
+        const int32_t i = idx[marked];
+        if (i < 0 || i >= c->n) {
+            rc = fail(c, NB_EINVAL, "active_idx[%d]=%d out of range", marked, i);
+            break;
+        }
+        uint64_t &w = c->seen[(size_t)i >> 6];
+        const uint64_t bit = 1ULL << (i & 63);
+        if (w & bit) {
+            rc = fail(c, NB_EINVAL, "active_idx[%d]=%d repeated", marked, i);
+            break;
+        }
+        w |= bit;
     }
-    return NB_OK;
+    for (int32_t a = 0; a < marked; ++a) c->seen[(size_t)idx[a] >> 6] &= ~(1ULL << (idx[a] & 63));
+    return rc;
 }
 
 // Pulls the control block to the host and turns a kernel-raised error into a
@@ -410,6 +429,27 @@ int copy_results_out(nb_ctx *c, int na, double *acc, double *jerk, double *pot, 
     return NB_OK;
 }
 
+// The last force's results to `out` and the control block to its mirror in one
+// kernel, then the wait; a device-raised error as sync_ctrl returns it.
+int publish(nb_ctx *c, const ForceOut &out, int na, const int *idx, bool validate)
+{
+    PublishArgs p{};
+    p.res = res_out(c);
+    p.out = out;
+    p.na = na;
+    p.n = c->n;
+    p.idx = idx;
+    p.validate = validate;
+    p.ctrl = c->d_ctrl;
+    p.host = c->h_ctrl;
+    launch_publish(p, c->st);
+    CK(cudaGetLastError());
+    c->launches += 1;
+    CK(cudaStreamSynchronize(c->st));
+    CK(cudaGetLastError());
+    return c->h_ctrl->err != 0 ? sync_ctrl(c) : NB_OK;
+}
+
 // The force on all particles from the j records, then one shared step's kernel.
 // src = dst in place; copy: a second place for the new state (or none).
 void enqueue_shared(nb_ctx *c, int mode, const State &src, const State &dst, const State *copy, bool predict)
@@ -665,12 +705,17 @@ static int init_impl(nb_ctx *c, int64_t n, const double *m, const double *x, con
             (rc = dalloc(c, &c->jds.vel, N)))
             return rc;
     }
-    cudaError_t he = cudaMallocHost((void **)&c->h_ctrl, sizeof(Ctrl));
+    // pinned: the control block's mirror and, up to kStageMax particles, host
+    // callers' indices and results
+    c->stage_na = c->n < kStageMax ? c->n : kStageMax;
+    static_assert(sizeof(Ctrl) % 8 == 0, "the staging follows it");
+    cudaError_t he = cudaMallocHost((void **)&c->h_ctrl, sizeof(Ctrl) + (size_t)c->stage_na * (7 * 8 + 4));
     if (he != cudaSuccess) {
         c->h_ctrl = nullptr;
         return fail(c, NB_ENOMEM, "cudaMallocHost failed: %s", cudaGetErrorString(he));
     }
     std::memset(c->h_ctrl, 0, sizeof(Ctrl));
+    c->h_stage = reinterpret_cast<double *>(c->h_ctrl + 1);
     c->h_ctrl->t_end = LLONG_MAX;
     c->t_end_dev = LLONG_MAX;
 
@@ -785,13 +830,28 @@ int nb_force(nb_ctx *c, const int32_t *idx, int32_t na, double *acc, double *jer
     if (!c) return NB_EINVAL;
     int rc = check_indices_host(c, idx, na);
     if (rc) return rc;
-    if (na > 0) {
-        CK(cudaMemcpyAsync(c->d_idx, idx, sizeof(int) * (size_t)na, cudaMemcpyHostToDevice, c->st));
+    if (na > 0 && na <= c->stage_na) {
+        // one transfer each way, through pinned memory
+        double *const h = c->h_stage;
+        int *const h_idx = reinterpret_cast<int *>(h + 7LL * c->stage_na);
+        std::memcpy(h_idx, idx, sizeof(int) * (size_t)na);
+        CK(cudaMemcpyAsync(c->d_idx, h_idx, sizeof(int) * (size_t)na, cudaMemcpyHostToDevice, c->st));
         enqueue_force(c, c->d_idx, na, nullptr, res_out(c));
         CK(cudaGetLastError());
-        if ((rc = copy_results_out(c, na, acc, jerk, pot, cudaMemcpyDeviceToHost))) return rc;
+        const ForceOut o = {acc ? h : nullptr, jerk ? h + 3LL * na : nullptr, pot ? h + 6LL * na : nullptr};
+        if ((rc = publish(c, o, na, nullptr, false))) return rc;
+        if (acc) std::memcpy(acc, o.acc, sizeof(double) * 3 * (size_t)na);
+        if (jerk) std::memcpy(jerk, o.jerk, sizeof(double) * 3 * (size_t)na);
+        if (pot) std::memcpy(pot, o.pot, sizeof(double) * (size_t)na);
+    } else {
+        if (na > 0) {
+            CK(cudaMemcpyAsync(c->d_idx, idx, sizeof(int) * (size_t)na, cudaMemcpyHostToDevice, c->st));
+            enqueue_force(c, c->d_idx, na, nullptr, res_out(c));
+            CK(cudaGetLastError());
+            if ((rc = copy_results_out(c, na, acc, jerk, pot, cudaMemcpyDeviceToHost))) return rc;
+        }
+        if ((rc = sync_ctrl(c))) return rc;
     }
-    if ((rc = sync_ctrl(c))) return rc;
     c->force_valid = true;
     c->force_na = na;
     c->force_t = c->t_pred;
@@ -807,17 +867,19 @@ int nb_force_dev(nb_ctx *c, const int32_t *d_idx, int32_t na, double *d_acc, dou
     if (na > 0 && !d_idx) return fail(c, NB_EINVAL, "active_idx is NULL");
     if (na > 0) {
         // Validation and force (on the caller's indices) go out together, and
-        // the one synchronisation follows the force: the force kernels clamp every
+        // the one synchronisation follows both: the force kernels clamp every
         // index into [0, n), so a bad index costs only wasted work, and the
         // caller's outputs are written only once the indices proved valid.
-        CK(cudaMemsetAsync(c->d_bitmap, 0, sizeof(unsigned) * (size_t)((c->n + 31) / 32), c->st));
-        launch_validate(d_idx, na, c->n, c->d_bitmap, &c->d_ctrl->err, c->st);
-        c->launches += 1;
+        const bool few = na <= kPublishCheckMax;
+        if (!few) {
+            CK(cudaMemsetAsync(c->d_bitmap, 0, sizeof(unsigned) * (size_t)((c->n + 31) / 32), c->st));
+            launch_validate(d_idx, na, c->n, c->d_bitmap, &c->d_ctrl->err, c->st);
+            c->launches += 1;
+        }
         enqueue_force(c, d_idx, na, nullptr, res_out(c));
         CK(cudaGetLastError());
-        int rc = sync_ctrl(c);
+        const int rc = publish(c, {d_acc, d_jerk, d_pot}, na, d_idx, few);
         if (rc) return rc;
-        if ((rc = copy_results_out(c, na, d_acc, d_jerk, d_pot, cudaMemcpyDeviceToDevice))) return rc;
     }
     c->force_valid = true;
     c->force_na = na;

@@ -623,6 +623,16 @@ void launch_energy(const State &s, const long long *t_ptr, const double *pot, do
 int energy_blocks(int n);
 void launch_validate(const int *idx, int na, int n, unsigned int *bitmap, int *err,
                      cudaStream_t st);
+// na > 0 results from res to out (see k_publish); validate: check idx[na] first.
+constexpr int kPublishCheckMax = 1024;
+struct PublishArgs {
+    ForceOut res, out;
+    int na, n;
+    const int *idx;
+    bool validate;
+    Ctrl *ctrl, *host;
+};
+void launch_publish(const PublishArgs &p, cudaStream_t st);
 void launch_gather_state(const State &s, double *x, double *v, double *a, double *k,
                          cudaStream_t st);
 void launch_scatter_state(const State &s, const double *x, const double *v, const double *a,

@@ -134,6 +134,16 @@ def _dptr(t):
     return ctypes.c_void_p(t.data_ptr())
 
 
+_DTYPE_NAMES = {}   # torch dtype -> its name without "torch."
+
+
+def _dtype_name(t, dt):
+    if dt is None:
+        return type(t).__name__
+    _DTYPE_NAMES[dt] = str(dt).replace("torch.", "")
+    return _DTYPE_NAMES[dt]
+
+
 def _dev(t, dtype, count, name, required=True):
     """Device address of a torch CUDA tensor after checking that it is a
     contiguous CUDA tensor of `dtype` ("float64" or "int32") holding at least
@@ -146,7 +156,8 @@ def _dev(t, dtype, count, name, required=True):
         return None
     if isinstance(t, int):
         return ctypes.c_void_p(t)
-    dt = str(getattr(t, "dtype", type(t).__name__)).replace("torch.", "")
+    dt = getattr(t, "dtype", None)
+    dt = _DTYPE_NAMES.get(dt) or _dtype_name(t, dt)
     if dt != dtype:
         raise ValueError("%s must be a %s tensor, got %s" % (name, dtype, dt))
     if not getattr(t, "is_cuda", False):

@@ -251,3 +251,37 @@ def test_kernel_and_slices_chosen_together(nb, n, na):
     _, forced = _check(nb, m, x, v, EPS, idx, 0, split=3, label="split, n=%d na=%d" % (n, na))
     for g, f in zip(got, forced):
         assert np.allclose(g, f, rtol=1e-12, atol=1e-12 * np.abs(f).max())
+
+
+@pytest.mark.parametrize("na", [1, 6, 512, 1024, 1025, 4096, 4097])
+def test_index_checks_and_untouched_outputs(nb, na):
+    # the device check by hash table (up to 1024) and by bitmap, and the host
+    # path through staging (up to 4096) and without: the same forces, and a
+    # repeated or out-of-range index refused with the outputs as they were
+    torch = pytest.importorskip("torch")
+    n = 5000
+    m, x, v = plummer(n, 71)
+    idx = sample_active(n, na, 3)[::-1].copy()   # descending: any order is allowed
+    ctx = nb.Context(m, x, v, EPS, flags=nb.NB_INIT_NO_FORCE)
+    try:
+        host = ctx.nb_force(idx)
+        d_idx = torch.from_numpy(idx).cuda()
+        outs = [torch.full((na, 3), 7.0, dtype=torch.float64, device="cuda") for _ in range(2)]
+        outs.append(torch.full((na,), 7.0, dtype=torch.float64, device="cuda"))
+        for bad in ([n, -1, 1 << 30, -(1 << 31)] if na == 1 else [n, -1, int(idx[0]), int(idx[na // 2])]):
+            wrong = idx.copy()
+            wrong[-1] = bad
+            with pytest.raises(nb.NbError) as ei:
+                ctx.nb_force_dev(torch.from_numpy(wrong).cuda(), na, *outs)
+            assert ei.value.code == nb.NB_EINVAL
+            torch.cuda.synchronize()
+            assert all(bool((o == 7.0).all()) for o in outs)
+            with pytest.raises(nb.NbError) as ei:
+                ctx.nb_force(wrong)
+            assert ei.value.code == nb.NB_EINVAL
+        ctx.nb_force_dev(d_idx, na, *outs)
+        torch.cuda.synchronize()
+        assert all(np.array_equal(o.cpu().numpy(), h) for o, h in zip(outs, host))
+        assert all(np.array_equal(a, b) for a, b in zip(ctx.nb_force(idx), host))
+    finally:
+        ctx.nb_free()
