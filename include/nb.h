@@ -45,7 +45,7 @@ extern "C" {
                           * then the i-parallel kernels) */
 #define NB_FORCE_IPAR 1  /* i across threads, j tiles broadcast from shared memory; DS takes
                           * one or four i per thread (blocks of 64 or 256), whichever its
-                          * time model rates faster, up to 2560 active, above that four */
+                          * time model rates faster, up to 20000 active, above that four */
 #define NB_FORCE_JPAR 2  /* j across threads, warp-shuffle tree reduction (small n_active) */
 
 /*

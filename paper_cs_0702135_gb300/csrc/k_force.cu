@@ -101,7 +101,12 @@ __global__ void __launch_bounds__(NT) k_force_ipar_ds(ForceArgs fa, JDS J)
     const float eps2 = (float)fa.eps2;
     const int tid = threadIdx.x;
 
-    for (int w = blockIdx.x; w < P.items; w += gridDim.x) {
+    // one-i items of a device-sized launch: the next item is drawn from a
+    // counter while the present one runs (host-sized launches have a CTA each)
+    __shared__ int s_next;
+    constexpr bool kDraw = REG == kRegSmall;
+    for (int w = blockIdx.x; w < P.items;) {
+        if (kDraw && tid == 0) s_next = fa.na_dev ? (int)gridDim.x + atomicAdd(fa.work, 1) : P.items;
         int ib, sl, j0, j1;
         ipar_item(w, P.n_iblk, P.n_whole, P.S, P.jslice, fa.n, ib, sl, j0, j1);
 
@@ -190,6 +195,10 @@ __global__ void __launch_bounds__(NT) k_force_ipar_ds(ForceArgs fa, JDS J)
                 for (int c = 0; c < kComp; ++c) dst[(long long)c * nb] = res[c];
             }
         }
+        // s_next was written before the tile loop's barriers; the next item's
+        // first barrier follows this read
+        w = kDraw ? *(volatile int *)&s_next : w + (int)gridDim.x;
+        if (kDraw) __syncthreads();
     }
 }
 

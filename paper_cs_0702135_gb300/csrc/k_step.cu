@@ -253,6 +253,7 @@ __global__ void k_sched_scatter(State s, Ctrl *ctrl, const long long *blockmin, 
         const int total = pre + running;
         ctrl->n_active = total;
         *plan_out = make_force_plan(fa, total, fine);   // the force launches read it
+        *fa.work = 0;
         if (total > 0) {
             ctrl->t_now = tn;
             ctrl->steps += 1;

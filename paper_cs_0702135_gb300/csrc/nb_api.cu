@@ -41,6 +41,7 @@ struct nb_ctx {
     double *d_res = nullptr;        // force results: acc [n][3], jerk [n][3], pot [n]
     double *d_part = nullptr;       // slice partials
     ForcePlan *d_plan = nullptr;    // plan of the device-sized force (written by the scheduler)
+    int *d_work = nullptr;          // item counter of the device-sized force
     int *d_jcnt = nullptr;          // [n] slice arrival counters of the DS j-parallel kernel
     long long part_cap = 0;
     int *d_act = nullptr;           // block of the device-driven step
@@ -216,6 +217,7 @@ ForceArgs force_args(nb_ctx *c, const int *act, int na_host, const int *na_dev, 
     fa.part_cap = c->part_cap;
     fa.part = c->d_part;
     fa.jcnt = c->d_jcnt;
+    fa.work = c->d_work;
     fa.out = out;
     fa.eps2 = c->eps * c->eps;
     fa.err = &c->d_ctrl->err;
@@ -253,7 +255,7 @@ Plan enqueue_force(nb_ctx *c, const int *act, int na_host, const int *na_dev, Fo
         const Plan &p = fa.plan.p;
         gi = gj = gs = 0;
         if (fa.plan.regime == kRegJpar) gj = p.items < c->slots_jpar ? p.items : c->slots_jpar;
-        else if (fa.plan.regime == kRegSmall) gs = p.items < c->slots_small ? p.items : c->slots_small;
+        else if (fa.plan.regime == kRegSmall) gs = p.items;   // dealt out as CTAs end
         else gi = p.items < c->slots_ipar ? p.items : c->slots_ipar;
     }
     const bool summed = c->o.summation != NB_SUM_COMPENSATED;
@@ -342,7 +344,7 @@ void release(nb_ctx *c)
                     c->jds.pos_lo, c->jds.vel, c->jf.pos, c->jf.vel, c->d_res, c->d_part,
                     c->d_act, c->d_idx, c->d_all, c->d_bitmap, c->d_ctrl, c->d_blockmin,
                     c->d_blockcnt, c->d_epart, c->d_stage, c->d_ck, c->d_seg, c->d_fin, c->d_tfin,
-                    c->d_jcnt, c->d_plan, c->d_cot, c->vrec.ph, c->vrec.pl, c->vrec.v, c->vrec.ab, c->vrec.kb,
+                    c->d_jcnt, c->d_plan, c->d_work, c->d_cot, c->vrec.ph, c->vrec.pl, c->vrec.v, c->vrec.ab, c->vrec.kb,
                     c->vrec64.x, c->vrec64.v, c->vrec64.ab, c->vrec64.kb, c->d_bounds, c->d_sort,
                     c->d_run_part, c->d_run_sync};
     for (void *p : ptrs)
@@ -689,7 +691,7 @@ static int init_impl(nb_ctx *c, int64_t n, const double *m, const double *x, con
         (rc = dalloc(c, &c->d_blockmin, c->nsched)) || (rc = dalloc(c, &c->d_blockcnt, c->nsched)) ||
         (rc = dalloc(c, &c->d_epart, 2LL * energy_blocks(c->n))) ||
         (rc = dalloc(c, &c->d_stage, 7 * N)) || (rc = dalloc(c, &c->d_jcnt, N)) ||
-        (rc = dalloc(c, &c->d_plan, 1)))
+        (rc = dalloc(c, &c->d_plan, 1)) || (rc = dalloc(c, &c->d_work, 1)))
         return rc;
     if (o.summation == NB_SUM_FIXED) {
         if ((rc = dalloc(c, &c->d_bounds, 2))) return rc;

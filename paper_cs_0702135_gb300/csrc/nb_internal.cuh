@@ -89,9 +89,9 @@ constexpr int kComp = 7;       // acc xyz, jerk xyz, pot
 // Clocks per j of an i-parallel CTA alone on its SM, and of each CTA with the SM full, for the
 // four-i and the one-i kernel, and how many are resident (see fine_cost).
 constexpr unsigned kFineAlone4 = 200, kFineEach4 = 95, kFineRes4 = 4;
-constexpr unsigned kFineAlone1 = 105, kFineEach1 = 24, kFineRes1 = 16;
+constexpr unsigned kFineAlone1 = 105, kFineEach1 = 22, kFineTail1 = 50, kFineRes1 = 16;
 constexpr unsigned kFineItemJ = 32;
-constexpr int kFineMaxActive = 2560;
+constexpr int kFineMaxActive = 20000;
 
 struct Plan {
     int n_iblk;   // i-blocks (i-parallel) or i-chunks (j-parallel)
@@ -309,19 +309,22 @@ __host__ __device__ inline int regime_of(int na, int jpar_max, int small_max)
 // chosen together, by the time of the busiest SM.  Candidate c: the four-i
 // (c < 16) or the one-i kernel, with the slice length in tiles that makes
 // c % 16 + 1 waves of its resident CTAs (a single tile where that is already
-// less than a wave).  An SM given m items runs them `res` at a time; k items
-// together cost max(alone, k each) clocks per j (one CTA alone cannot hide its
-// latencies) and kFineItemJ j more per item.  Both kernels sum the same 128-j
-// tiles in the same order, so the choice does not show in the tile partials.
+// less than a wave).  Four-i items go to the CTAs in turn: an SM given m items
+// runs `res` at a time, k together at max(alone, k each) clocks per j (one
+// CTA alone cannot hide its latencies).  One-i items are taken as CTAs end
+// (with four warps a scheduler, CTAs progress unevenly): each clocks per j and
+// item on average, and a tail.  Every item costs kFineItemJ j more.  Both
+// kernels sum the same 128-j tiles in the same order, so the choice does not
+// show in the tile partials.
 //
 // The one-i kernel reaches 90% of the four-i kernel's rate on full blocks,
 // pads the block to 64 instead of 256 and cuts it four times as fine, so it
 // wins wherever the padding or a part-filled GPU costs the other more than a
 // tenth.  Force and combine, us, four-i plan before / this rule: 256 active
-// on 256 bodies 42 / 17, 1024 on 1024 44 / 19, 4096 on 4096 49 / 40, 300 on
-// 4096 25 / 19, 700 on 65536 100 / 79, 1024 on 65536 118 / 104.  Above
-// kFineMaxActive (ten blocks of the four-i kernel) the padding is below that
-// tenth and plan_ipar's search, which also runs blocks whole, is kept.
+// on 256 bodies 42 / 17, 1024 on 1024 44 / 17, 4096 on 4096 49 / 40, 300 on
+// 4096 25 / 19; on 65536: 700 100 / 79, 1820 208 / 165, 4096 347 / 330, 8192
+// 654 / 625, 20000 1579 / 1475.  Above kFineMaxActive the two are within 2%
+// and plan_ipar's search, which also runs blocks whole, is kept.
 constexpr int kFineCands = 32;
 __host__ __device__ inline unsigned fine_clocks(unsigned m, unsigned res, unsigned alone, unsigned each)
 {
@@ -349,10 +352,15 @@ __host__ __device__ inline unsigned long long fine_cost(int na, int n, int sms, 
     const unsigned nib = ucdiv((unsigned)na, (unsigned)(kIparNT * (one ? kIparSmallR : kIparR)));
     const unsigned S = ucdiv(ucdiv((unsigned)n, tile), L);
     if (S > 1 && (long long)S * kComp * na > part_cap) return ~0ULL;
-    const unsigned m = ucdiv(nib * S, (unsigned)sms);
-    return (unsigned long long)(L * tile + kFineItemJ) *
-           (one ? fine_clocks(m, kFineRes1, kFineAlone1, kFineEach1)
-                : fine_clocks(m, kFineRes4, kFineAlone4, kFineEach4));
+    const unsigned items = nib * S;
+    unsigned t;
+    if (one) {
+        t = (unsigned)((unsigned long long)items * kFineEach1 / (unsigned)sms) + kFineTail1;
+        if (t < kFineAlone1) t = kFineAlone1;
+    } else {
+        t = fine_clocks(ucdiv(items, (unsigned)sms), kFineRes4, kFineAlone4, kFineEach4);
+    }
+    return (unsigned long long)(L * tile + kFineItemJ) * t;
 }
 
 // The work decomposition of one force launch: the block size, the kernel
@@ -387,6 +395,8 @@ struct ForceArgs {
     long long part_cap;       // capacity of part in doubles
     double *part;             // slice partials: part[(s * 7 + c) * na + a]; the DS
                               // j-parallel kernel: part[(chunk * 7 ic + e) * S + s]
+    int *work;                // device-sized launches: items taken by the one-i kernel's CTAs
+                              // beyond their first (zeroed by the scheduler)
     int *jcnt;                // per-chunk slice arrival counters (zero between launches)
     ForceOut out;
     double eps2;

@@ -239,12 +239,11 @@ def test_jpar_slice_counters_reset_between_calls(nb):
     assert_force_close(first[0], ref, mags, TOL_DS, "na=5 N=300000")
 
 
-@pytest.mark.parametrize("n,na", [(97, 97), (128, 100), (129, 129), (1000, 257), (3000, 2560), (3000, 2561),
-                                  (20000, 1820)])
+@pytest.mark.parametrize("n,na", [(97, 97), (128, 100), (129, 129), (1000, 257), (3000, 2561), (20000, 1820)])
 def test_kernel_and_slices_chosen_together(nb, n, na):
     # one tile, one tile and a particle, blocks on both sides of a 64- and a
-    # 256-i boundary and of the largest block planned so; the slices change
-    # nothing above FP64 rounding, so a forced slice count gives the same force
+    # 256-i boundary; the slices change nothing above FP64 rounding, so a
+    # forced slice count gives the same force
     m, x, v = plummer(n, 61 + n)
     idx = sample_active(n, na, 7)
     _, got = _check(nb, m, x, v, EPS, idx, 0, label="n=%d na=%d" % (n, na))
@@ -285,3 +284,25 @@ def test_index_checks_and_untouched_outputs(nb, na):
         assert all(np.array_equal(a, b) for a, b in zip(ctx.nb_force(idx), host))
     finally:
         ctx.nb_free()
+
+
+def test_device_sized_blocks_draw_the_same_items(nb):
+    # the one-i kernel draws its items from a counter when the block size is
+    # known on the device only: the same force as the host-sized launch
+    m, x, v = plummer(6000, 77)
+    a, b = (nb.Context(m, x, v, EPS, level_min=6) for _ in range(2))
+    try:
+        seen = set()
+        for _ in range(12):
+            t, na = a.nb_step()
+            idx, _ = a.nb_get_active()
+            b.nb_predict(t)
+            b.nb_force(idx)
+            b.nb_correct(idx, t)
+            seen.add(na)
+            sa, sb = a.nb_get_state(), b.nb_get_state()
+            assert all(np.array_equal(sa[k], sb[k]) for k in sa), na
+        assert max(seen) > 96
+    finally:
+        a.nb_free()
+        b.nb_free()

@@ -335,7 +335,7 @@ def test_fine_plans(tmp_path):
                     str(src), "-o", str(exe)], check=True)
     cases = []
     for na, n, sms in itertools.product(
-            [97, 128, 129, 256, 257, 1000, 1820, 2560, 2561, 4096, 9000],
+            [97, 128, 129, 256, 257, 1000, 1820, 4096, 9000, 20000, 20001, 40000],
             [97, 128, 129, 1000, 4096, 16384, 65536, 1 << 20], [1, 152]):
         if na <= n:
             cases.append((na, n, sms, 7 * max(16 * 4 * sms * 256, 4 * n)))
@@ -347,5 +347,5 @@ def test_fine_plans(tmp_path):
         assert cover == nib * n and js % 128 == 0 and (S - 1) * js < n <= S * js, c
         assert S == 1 or n_whole or S * 7 * na <= cap, c
         assert lanes in (1, 2, 4, 8, 16, 32) and (lanes == 1 or lanes <= S), c
-        if na <= 2560:
+        if na <= 20000:
             assert cand >= 0 and n_whole == 0 and regime == (1 if cand >= 16 else 2), c
