@@ -210,6 +210,43 @@ __global__ void k_fixed_combine(ForceArgs fa, SumArgs sa)
     }
 }
 
+// Adds 4 N4 values of s to run in order.  Four reads are in flight while the
+// sixteen values before them are added (64 clocks, a read takes about 30);
+// left to the compiler the reads end up just ahead of their additions, 10
+// clocks a value instead of 4.  The reads are volatile to stay where they are.
+__device__ __forceinline__ float4 read_early(const float4 *p)
+{
+    float4 v;
+    const unsigned a = (unsigned)__cvta_generic_to_shared(p);
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "r"(a));
+    return v;
+}
+__device__ __forceinline__ float add4(float run, const float4 &t)
+{
+    return __fadd_rn(__fadd_rn(__fadd_rn(__fadd_rn(run, t.x), t.y), t.z), t.w);
+}
+template <int N4>
+__device__ __forceinline__ float add_in_order(const float4 *s, float run)
+{
+    static_assert(N4 % 4 == 0, "whole groups of reads");
+    float4 a[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) a[u] = read_early(s + u);
+#pragma unroll 2
+    for (int q = 4; q < N4; q += 4) {
+        float4 b[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) b[u] = read_early(s + q + u);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) run = add4(run, a[u]), a[u] = b[u];
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) run = add4(run, a[u]);
+    return run;
+}
+
 // ---------------------------------------------------------------------------
 // FP32 running sum in index order.  The order fixes one chain of additions per
 // output (4 cycles a term), but nothing fixes who evaluates the terms: a CTA
@@ -328,16 +365,8 @@ __device__ __forceinline__ void seq_groups(const ForceArgs &fa, const JDS &J, in
                     }
                 }
             } else if (k > 0 && chain < cnt * kComp) {
-                const float4 *src = reinterpret_cast<const float4 *>(buf + ((k - 1) & 1) * kSeqBufFloats +
-                                                                     chain * row);
-#pragma unroll 8
-                for (int q = 0; q < T / 4; ++q) {
-                    const float4 t = src[q];
-                    sum = __fadd_rn(sum, t.x);
-                    sum = __fadd_rn(sum, t.y);
-                    sum = __fadd_rn(sum, t.z);
-                    sum = __fadd_rn(sum, t.w);
-                }
+                sum = add_in_order<T / 4>(reinterpret_cast<const float4 *>(buf + ((k - 1) & 1) * kSeqBufFloats +
+                                                                           chain * row), sum);
             }
             __syncthreads();
         }
@@ -364,176 +393,359 @@ __global__ void __launch_bounds__(kSeqNT, 1) k_force_seq(ForceArgs fa, JDS J, in
 }
 
 // ---------------------------------------------------------------------------
-// FP32 running sum, smallest pair force first: one CTA per active i.
-//  1. keyed items (key bits << 32 | j) for every j into the CTA's scratch, in
-//     index order, and the histograms of the key's four bytes; j = i and
-//     r2 = 0 get the key 0xffffffff (sorted last).
-//  2. stable LSD radix sort on the key, a pass per byte (a byte that all keys
-//     share is left out): tiles of 16 items a thread, each warp a contiguous
-//     run of the tile.  An item's rank is that among the equal digits of its
-//     warp (match_any and the warp's running counts in shared memory) plus
-//     the counts of the earlier warps and tiles; stability keeps equal keys in
-//     index order.  The last pass writes the indices alone.
-//  3. seven warps evaluate the sorted items' terms, two an instruction, into
-//     one of two buffers while seven lanes of the eighth add the tile before
-//     it in order, one component each.
-// The chain of additions (4 cycles an item) keeps one warp of a CTA busy and
-// nothing else, so four CTAs share an SM, each in its own phase.  1820 active
-// on 65536 bodies: 6.6 ms; before, one CTA of 1024 threads per SM ranked
-// one item a thread between five barriers and added after evaluating
-// (18.6 ms).
+// FP32 running sum, smallest pair force first: one CTA per active i.  The keys
+// |mj dx/r^3| are sorted stably by j and the terms added in that order.
+//  1. a histogram of the keys over bins of 1/32 octave;
+//  2. consecutive bins make chunks of up to 4096 items (about 2048 each); the
+//     items (key bits << 32 | j) go to their chunk in the CTA's scratch, keys
+//     evaluated again rather than stored and read: 8 bytes written and read
+//     per item in all;
+//  3. chunk by chunk, in increasing key: a bucket sort of (key, j) in shared
+//     memory, then the terms.
+// While seven warps evaluate a tile's terms, seven lanes of the eighth add the
+// tile before it in order, one component each (4 clocks an item), so four CTAs
+// share an SM, each in its own phase.
+//
+// Where a bin holds more than 2048 items (many equal keys) or there are more
+// than 255 chunks, all items are sorted in the scratch instead, by a stable LSD
+// radix sort with a pass per key byte (a byte that all keys share is left
+// out).  An item's rank within a pass is that among the equal digits of its
+// warp (match_any and the warp's running counts in shared memory) plus the
+// counts of the earlier warps and tiles; stability keeps equal keys in index
+// order.  Its scattered 8-byte stores to a footprint beyond the L2 are what
+// that waits for.
+//
+// 1820 active on 65536 bodies: 5.3 ms (a radix sort of the chunks 6.1 ms, the
+// scratch sort 6.6 ms); one CTA
+// of 1024 threads per SM, ranking one item a thread between five barriers and
+// adding after evaluating, 18.6 ms.
 
 constexpr int kSortW = kSortNT / 32;
-constexpr int kSortK = 16;                        // items per thread and tile of a pass
+constexpr int kSortK = 16;                        // items per thread of a chunk or tile
 constexpr int kSortTile = kSortNT * kSortK;
-constexpr int kSortSum = (kSortW - 1) * 64;       // items per tile of the sum: two per term lane
+constexpr int kBinShift = 18, kBins = 8192;       // bins of the key's upper bits
+constexpr int kChunk = 2048, kChunks = 255;       // aim of a chunk, and how many at most
+static_assert((0x7f7fffff >> kBinShift) < kBins && 2 * kChunk <= kSortTile, "keys have a bin, chunks fit");
+constexpr int kSortSum = (kSortW - 1) * 32;       // items per tile of the sum: one per term lane
 constexpr int kSortRow = kSortSum + 4;
+
+struct SortShared {
+    union {
+        unsigned hist[kBins];                    // 1: histogram; the scratch sort's [4][256]
+        unsigned long long item[kSortTile];      // 3: the chunk
+    } a;
+    unsigned char id[kBins];                     // chunk of a bin
+    union {
+        unsigned off[kSortW][256];               // counts, then offsets, of a warp's digits
+        unsigned bucket[2048];                   // chunk: items per bucket, then places
+        float4 t[2][7][kSortRow / 4];            // two tiles of terms
+    } u;
+    unsigned start[kChunks + 2];                 // first item of a chunk
+    unsigned next[kChunks + 1];                  // place of its next item
+    unsigned base[256];
+    unsigned scan[kSortW], lo[kSortW], hi[kSortW];
+    int cnt;
+};
+
+// Exclusive sum over the CTA's threads (a barrier before and after use of s).
+__device__ __forceinline__ unsigned cta_exclusive(unsigned v, unsigned *s, int lane, int warp)
+{
+    unsigned incl = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned y = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += y;
+    }
+    if (lane == 31) s[warp] = incl;
+    __syncthreads();
+    unsigned before = incl - v;
+    for (int w = 0; w < warp; ++w) before += s[w];
+    return before;
+}
+
+// Ranks of a warp's K rows of 32 items (digit(k), or -1: none) among the equal
+// digits of its rows so far, two 16-bit ranks a register; cnt[256] ends with
+// the warp's counts.
+template <int K, typename Digit>
+__device__ __forceinline__ void warp_ranks(Digit digit, unsigned (&rank)[K / 2], unsigned *cnt, int lane, int rows)
+{
+    const unsigned lt = (1u << lane) - 1u;
+#pragma unroll
+    for (int q = 0; q < 256 / 32; ++q) cnt[q * 32 + lane] = 0;
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        if (k % 2 == 0) rank[k / 2] = 0;
+        if (k < rows) {
+            const int d = digit(k);
+            const unsigned peers = __match_any_sync(kFull, d);
+            const unsigned old = d >= 0 ? cnt[d] : 0u;
+            rank[k / 2] |= (old + __popc(peers & lt)) << (16 * (k % 2));
+            __syncwarp();
+            if (d >= 0 && (peers & lt) == 0) cnt[d] = old + __popc(peers);
+            __syncwarp();
+        }
+    }
+}
+template <int H>
+__device__ __forceinline__ unsigned rank_of(const unsigned (&rank)[H], int k)
+{
+    return (rank[k / 2] >> (16 * (k % 2))) & 0xffffu;
+}
+
+// Two j's keys, ~0 for a pair that is left out.
+__device__ __forceinline__ uint2 sort_keys(const JDS &J, int j0, int j1, int n, int i, const Side2 &N, float eps2)
+{
+    const int c0 = min(j0, n - 1), c1 = min(j1, n - 1);
+    const Side2 Js = side2(J.pos_hi[c0], J.pos_lo[c0], J.vel[c0], J.pos_hi[c1], J.pos_lo[c1], J.vel[c1]);
+    float2 r2;
+    const float2 key = pair_key2(Js, N, eps2, r2);
+    return make_uint2(j0 < n && j0 != i && r2.x != 0.0f ? __float_as_uint(key.x) : ~0u,
+                      j1 < n && j1 != i && r2.y != 0.0f ? __float_as_uint(key.y) : ~0u);
+}
+
+// Adds the terms of sorted items 0 .. total - 1 (index by `at`) to run, which
+// lane c of warp 0 holds for component c.
+template <typename At>
+__device__ __forceinline__ void sum_sorted(SortShared &sh, const JDS &J, int i, float eps2, int total, At at, float &run)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    float xh[3], xl[3], vi[3];
+    load_i(J, i, xh, xl, vi);
+    const int ntile = cdiv(total, kSortSum), q0 = (warp - 1) * 32 + lane;
+    // a lane's next source record is loaded while it works on the present one
+    float4 p, l, v;
+    if (warp > 0 && ntile > 0) {
+        const int j = at(min(q0, total - 1));
+        p = J.pos_hi[j], l = J.pos_lo[j], v = J.vel[j];
+    }
+    for (int k = 0; k <= ntile; ++k) {
+        if (warp > 0) {
+            if (k < ntile) {
+                const int e = k * kSortSum + q0;
+                const int j = at(min(e + kSortSum, total - 1));
+                const float4 np = J.pos_hi[j], nl = J.pos_lo[j], nv = J.vel[j];
+                float t[7];
+                pair_rn(p, l, v, xh, xl, vi, eps2, 1.0f, 1.0f, 1.0f, t);
+                p = np, l = nl, v = nv;
+                float *const d = reinterpret_cast<float *>(sh.u.t[k & 1]) + q0;
+#pragma unroll
+                for (int c = 0; c < 7; ++c) d[c * kSortRow] = e < total ? t[c] : -0.0f;   // -0 changes no sum
+            }
+        } else if (k > 0 && lane < 7) {
+            run = add_in_order<kSortSum / 4>(sh.u.t[(k - 1) & 1][lane], run);
+        }
+        __syncthreads();
+    }
+}
+
+// The scratch sort: all n items by four passes between A and B; the sorted array.
+__device__ __noinline__ const unsigned long long *sort_scratch(SortShared &sh, const JDS &J, int i, int n, float eps2,
+                                                               unsigned long long *A, unsigned long long *B)
+{
+    constexpr int NT = kSortNT;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const Side2 N = side2_neg(J.pos_hi[i], J.pos_lo[i], J.vel[i]);
+    unsigned(*hist)[256] = reinterpret_cast<unsigned(*)[256]>(sh.a.hist);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) hist[q][tid] = 0;
+    __syncthreads();
+    for (int j = tid; j < n; j += 2 * NT) {
+        const uint2 key = sort_keys(J, j, j + NT, n, i, N, eps2);
+        A[j] = ((unsigned long long)key.x << 32) | (unsigned)j;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) atomicAdd(&hist[q][(key.x >> (8 * q)) & 255u], 1u);
+        if (j + NT < n) {
+            A[j + NT] = ((unsigned long long)key.y << 32) | (unsigned)(j + NT);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) atomicAdd(&hist[q][(key.y >> (8 * q)) & 255u], 1u);
+        }
+    }
+    __syncthreads();
+    unsigned long long *src = A, *dst = B;
+    for (int pass = 0; pass < 4; ++pass) {
+        const unsigned mine = hist[pass][tid];
+        if (__syncthreads_or(mine == (unsigned)n)) continue;   // one digit for all
+        sh.base[tid] = cta_exclusive(mine, sh.scan, lane, warp);   // kept by this thread only
+        const int shift = 32 + 8 * pass;
+        for (int t0 = 0; t0 < n; t0 += kSortTile) {
+            unsigned long long item[kSortK];
+            unsigned rank[kSortK / 2];
+            const int w0 = t0 + warp * (kSortK * 32) + lane;
+#pragma unroll
+            for (int k = 0; k < kSortK; ++k) item[k] = w0 + k * 32 < n ? src[w0 + k * 32] : 0ULL;
+            auto digit = [&](int k) { return w0 + k * 32 < n ? (int)(item[k] >> shift) & 255 : -1; };
+            warp_ranks<kSortK>(digit, rank, sh.u.off[warp], lane, kSortK);
+            __syncthreads();
+            unsigned run = sh.base[tid];
+#pragma unroll
+            for (int w = 0; w < kSortW; ++w) {
+                const unsigned c = sh.u.off[w][tid];
+                sh.u.off[w][tid] = run;
+                run += c;
+            }
+            sh.base[tid] = run;
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < kSortK; ++k)
+                if (w0 + k * 32 < n) dst[sh.u.off[warp][digit(k)] + rank_of(rank, k)] = item[k];
+            __syncwarp();   // the warp's offsets are cleared next
+        }
+        __syncthreads();
+        unsigned long long *tmp = src;
+        src = dst;
+        dst = tmp;
+    }
+    return src;
+}
+
+// Chunk of cnt <= kSortTile items from src sorted into sh.a.item, by buckets:
+// the chunk's key range over 2048 buckets, a place in its bucket for every
+// item in any order (an atomic counter), then its rank among the bucket's items,
+// which are compared as (key, j).  A bucket holds one or two items where the
+// keys are spread; many equal keys cost their square.
+constexpr int kBuckets = 2048;
+__device__ __forceinline__ void sort_chunk(SortShared &sh, const unsigned long long *src, int cnt)
+{
+    constexpr int NT = kSortNT, kOwn = kBuckets / NT;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    unsigned long long v[kSortK];
+    unsigned lo = ~0u, hi = 0u;
+#pragma unroll
+    for (int k = 0; k < kSortK; ++k) {
+        const int q = k * NT + tid;
+        v[k] = q < cnt ? src[q] : ~0ULL;
+        if (q < cnt) {
+            lo = min(lo, (unsigned)(v[k] >> 32));
+            hi = max(hi, (unsigned)(v[k] >> 32));
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < kOwn; ++q) sh.u.bucket[q * NT + tid] = 0;
+    lo = __reduce_min_sync(kFull, lo);
+    hi = __reduce_max_sync(kFull, hi);
+    if (lane == 0) sh.lo[warp] = lo, sh.hi[warp] = hi;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < kSortW; ++w) lo = min(lo, sh.lo[w]), hi = max(hi, sh.hi[w]);
+    const int shift = max(0, 21 - __clz(hi - lo));   // (hi - lo) >> shift < 2048
+    auto bucket = [&](unsigned long long x) { return ((unsigned)(x >> 32) - lo) >> shift; };
+#pragma unroll
+    for (int k = 0; k < kSortK; ++k)
+        if (k * NT + tid < cnt) atomicAdd(&sh.u.bucket[bucket(v[k])], 1u);
+    __syncthreads();
+    unsigned c[kOwn], sum = 0;
+#pragma unroll
+    for (int q = 0; q < kOwn; ++q) c[q] = sh.u.bucket[tid * kOwn + q], sum += c[q];
+    unsigned at = cta_exclusive(sum, sh.scan, lane, warp);
+#pragma unroll
+    for (int q = 0; q < kOwn; ++q) {
+        sh.u.bucket[tid * kOwn + q] = at;
+        at += c[q];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kSortK; ++k)
+        if (k * NT + tid < cnt) sh.a.item[atomicAdd(&sh.u.bucket[bucket(v[k])], 1u)] = v[k];
+    __syncthreads();
+    // a bucket's counter now stands at its end, the start of the next
+    unsigned place[kSortK / 2];
+#pragma unroll
+    for (int k = 0; k < kSortK; ++k) {
+        if (k % 2 == 0) place[k / 2] = 0;
+        if (k * NT + tid < cnt) {
+            const unsigned d = bucket(v[k]), e = sh.u.bucket[d];
+            unsigned q = d ? sh.u.bucket[d - 1] : 0u, r = q;
+            for (; q < e; ++q) r += sh.a.item[q] < v[k];
+            place[k / 2] |= r << (16 * (k % 2));
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kSortK; ++k)
+        if (k * NT + tid < cnt) sh.a.item[rank_of(place, k)] = v[k];
+    __syncthreads();
+}
 
 __global__ void __launch_bounds__(kSortNT, kSortCtas) k_force_sorted(ForceArgs fa, JDS J, SumArgs sa)
 {
     constexpr int NT = kSortNT;
+    static_assert(NT == 256, "a thread per digit and per 32 bins");
     const int na = read_na(fa);
     if (na <= 0) return;
-    __shared__ unsigned s_hist[4][256];
-    __shared__ unsigned s_base[256], s_scan[kSortW];
-    __shared__ union {
-        unsigned off[kSortW][256];               // pass: counts, then offsets, of a warp's digits
-        float4 t[2][7][kSortRow / 4];            // sum: two tiles of terms
-    } u;
+    extern __shared__ float4 s_sorted[];
+    SortShared &sh = *reinterpret_cast<SortShared *>(s_sorted);
     __shared__ float s_res[7];
-    __shared__ int s_cnt;
-    static_assert(NT == 256, "a thread per digit");
     const int n = fa.n, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const unsigned lt = (1u << lane) - 1u;
     const float eps2 = (float)fa.eps2;
     unsigned long long *const A = sa.scratch + (size_t)blockIdx.x * 2 * (size_t)n;
-    unsigned long long *const B = A + n;
 
     for (int a = blockIdx.x; a < na; a += gridDim.x) {
         const int i = clamp_index(fa.act[a], n);
         const Side2 N = side2_neg(J.pos_hi[i], J.pos_lo[i], J.vel[i]);
-        if (tid == 0) s_cnt = 0;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) s_hist[q][tid] = 0;
+        // 1. histogram
+        if (tid == 0) sh.cnt = 0;
+        for (int q = tid; q < kBins; q += NT) sh.a.hist[q] = 0;
         __syncthreads();
-
         int cnt = 0;
         for (int j = tid; j < n; j += 2 * NT) {
-            const int j1 = min(j + NT, n - 1);
-            const Side2 Js = side2(J.pos_hi[j], J.pos_lo[j], J.vel[j], J.pos_hi[j1], J.pos_lo[j1], J.vel[j1]);
-            float2 r2;
-            const float2 key = pair_key2(Js, N, eps2, r2);
-            const bool ok0 = r2.x != 0.0f && j != i, ok1 = r2.y != 0.0f && j + NT != i;
-            const unsigned k0 = ok0 ? __float_as_uint(key.x) : 0xffffffffu;
-            const unsigned k1 = ok1 ? __float_as_uint(key.y) : 0xffffffffu;
-            A[j] = ((unsigned long long)k0 << 32) | (unsigned)j;
-            cnt += ok0;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) atomicAdd(&s_hist[q][(k0 >> (8 * q)) & 255u], 1u);
-            if (j + NT < n) {
-                A[j + NT] = ((unsigned long long)k1 << 32) | (unsigned)(j + NT);
-                cnt += ok1;
-#pragma unroll
-                for (int q = 0; q < 4; ++q) atomicAdd(&s_hist[q][(k1 >> (8 * q)) & 255u], 1u);
-            }
+            const uint2 key = sort_keys(J, j, j + NT, n, i, N, eps2);
+            if (key.x != ~0u) atomicAdd(&sh.a.hist[key.x >> kBinShift], 1u), ++cnt;
+            if (key.y != ~0u) atomicAdd(&sh.a.hist[key.y >> kBinShift], 1u), ++cnt;
         }
         cnt = __reduce_add_sync(kFull, cnt);
-        if (lane == 0) atomicAdd(&s_cnt, cnt);
+        if (lane == 0) atomicAdd(&sh.cnt, cnt);
         __syncthreads();
-
-        unsigned long long *src = A, *dst = B;
-        for (int pass = 0; pass < 4; ++pass) {
-            // the digit's first place: exclusive sum of the histogram
-            const unsigned mine = s_hist[pass][tid];
-            if (__syncthreads_or(mine == (unsigned)n)) continue;   // one digit for all
-            unsigned incl = mine;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned y = __shfl_up_sync(kFull, incl, o);
-                if (lane >= o) incl += y;
-            }
-            if (lane == 31) s_scan[warp] = incl;
-            __syncthreads();
-            unsigned before = incl - mine;
-            for (int w = 0; w < warp; ++w) before += s_scan[w];
-            s_base[tid] = before;   // read and kept by this thread only
-            const int shift = 32 + 8 * pass;
-            for (int t0 = 0; t0 < n; t0 += kSortTile) {
-                unsigned long long item[kSortK];
-                unsigned rank[kSortK];
-                const int w0 = t0 + warp * (kSortK * 32) + lane;
-#pragma unroll
-                for (int k = 0; k < kSortK; ++k)
-                    // past the end: the last digit, after every item of the tile, never stored
-                    item[k] = w0 + k * 32 < n ? src[w0 + k * 32] : ~0ULL;
-#pragma unroll
-                for (int q = 0; q < 256 / 32; ++q) u.off[warp][q * 32 + lane] = 0;
-                __syncwarp();
-#pragma unroll
-                for (int k = 0; k < kSortK; ++k) {
-                    const unsigned d = (unsigned)(item[k] >> shift) & 255u;
-                    const unsigned peers = __match_any_sync(kFull, d);
-                    const unsigned old = u.off[warp][d];
-                    rank[k] = old + __popc(peers & lt);
-                    __syncwarp();
-                    if ((peers & lt) == 0) u.off[warp][d] = old + __popc(peers);
-                    __syncwarp();
-                }
-                __syncthreads();
-                unsigned run = s_base[tid];
-#pragma unroll
-                for (int w = 0; w < kSortW; ++w) {
-                    const unsigned c = u.off[w][tid];
-                    u.off[w][tid] = run;
-                    run += c;
-                }
-                s_base[tid] = run;
-                __syncthreads();
-#pragma unroll
-                for (int k = 0; k < kSortK; ++k) {
-                    const unsigned d = (unsigned)(item[k] >> shift) & 255u;
-                    if (w0 + k * 32 < n) dst[u.off[warp][d] + rank[k]] = item[k];
-                }
-                __syncwarp();   // the warp's offsets are cleared next
-            }
-            __syncthreads();
-            unsigned long long *tmp = src;
-            src = dst;
-            dst = tmp;
-        }
-
-        const int total = s_cnt;
-        const int ntile = cdiv(total, kSortSum);
+        const int total = sh.cnt;
         float run = 0.0f;
-        for (int k = 0; k <= ntile; ++k) {
-            if (warp > 0) {
-                if (k < ntile) {
-                    const int q0 = (warp - 1) * 64 + lane, e0 = k * kSortSum + q0, e1 = e0 + 32;
-                    const int ja = (int)(unsigned)src[min(e0, total - 1)];
-                    const int jb = (int)(unsigned)src[min(e1, total - 1)];
-                    const Side2 Js = side2(J.pos_hi[ja], J.pos_lo[ja], J.vel[ja], J.pos_hi[jb],
-                                           J.pos_lo[jb], J.vel[jb]);
-                    float2 t[7];
-                    pair_rn2<true>(Js, N, eps2, 1.0f, 1.0f, 1.0f, t);
-                    float *const d = reinterpret_cast<float *>(u.t[k & 1]) + q0;
-#pragma unroll
-                    for (int c = 0; c < 7; ++c) {
-                        d[c * kSortRow] = e0 < total ? t[c].x : -0.0f;   // -0 changes no sum
-                        d[c * kSortRow + 32] = e1 < total ? t[c].y : -0.0f;
-                    }
-                }
-            } else if (k > 0 && lane < 7) {
-                const float4 *s4 = u.t[(k - 1) & 1][lane];
-#pragma unroll 8
-                for (int q = 0; q < kSortSum / 4; ++q) {
-                    const float4 t = s4[q];
-                    run = __fadd_rn(run, t.x);
-                    run = __fadd_rn(run, t.y);
-                    run = __fadd_rn(run, t.z);
-                    run = __fadd_rn(run, t.w);
-                }
+
+        // 2. chunks: this thread's 32 bins
+        constexpr int kOwn = kBins / NT;
+        unsigned sum = 0, most = 0;
+        for (int q = 0; q < kOwn; ++q) {
+            const unsigned c = sh.a.hist[tid * kOwn + q];
+            sum += c;
+            most = max(most, c);
+        }
+        unsigned place = cta_exclusive(sum, sh.scan, lane, warp);
+        if (__syncthreads_or(most > kChunk || total > kChunks * kChunk)) {
+            const unsigned long long *sorted = sort_scratch(sh, J, i, n, eps2, A, A + n);
+            sum_sorted(sh, J, i, eps2, total, [&](int q) { return (int)(unsigned)sorted[q]; }, run);
+        } else {
+            for (int q = tid; q < kChunks + 2; q += NT) sh.start[q] = total;
+            __syncthreads();
+            // a chunk starts at the first bin that starts at or past a multiple of kChunk
+            int prev = tid == 0 ? -1 : (int)((place - sh.a.hist[tid * kOwn - 1]) / kChunk);
+            for (int q = 0; q < kOwn; ++q) {
+                const int c = (int)(place / kChunk);   // past the last item: kChunks at most
+                sh.id[tid * kOwn + q] = (unsigned char)c;
+                if (c != prev && c <= kChunks) sh.start[c] = place;
+                prev = c;
+                place += sh.a.hist[tid * kOwn + q];
             }
             __syncthreads();
+            // items to their chunk, in any order within it (the chunk's sort
+            // compares j too)
+            for (int q = tid; q < kChunks + 1; q += NT) sh.next[q] = sh.start[q];
+            __syncthreads();
+            for (int j = tid; j < n; j += 2 * NT) {
+                const uint2 key = sort_keys(J, j, j + NT, n, i, N, eps2);
+                if (key.x != ~0u)
+                    A[atomicAdd(&sh.next[sh.id[key.x >> kBinShift]], 1u)] =
+                        (unsigned long long)key.x << 32 | (unsigned)j;
+                if (key.y != ~0u)
+                    A[atomicAdd(&sh.next[sh.id[key.y >> kBinShift]], 1u)] =
+                        (unsigned long long)key.y << 32 | (unsigned)(j + NT);
+            }
+            __syncthreads();
+            // 3. chunk by chunk
+            for (int c = 0; c <= kChunks; ++c) {
+                const int first = (int)sh.start[c], len = (int)sh.start[c + 1] - first;
+                if (first >= total) break;
+                if (len <= 0) continue;
+                sort_chunk(sh, A + first, len);
+                sum_sorted(sh, J, i, eps2, len, [&](int q) { return (int)(unsigned)sh.a.item[q]; }, run);
+            }
         }
         if (tid < 7) s_res[tid] = run;
         __syncthreads();
@@ -561,8 +773,11 @@ int occupancy_sum(int mode, int *blocks_per_sm)
         if (e == cudaSuccess)
             e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_force_seq, kSeqNT, kSeqSmem);
     }
-    else
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_force_sorted, kSortNT, 0);
+    else {
+        e = cudaFuncSetAttribute(k_force_sorted, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortShared));
+        if (e == cudaSuccess)
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_force_sorted, kSortNT, sizeof(SortShared));
+    }
     return e == cudaSuccess ? 0 : -1;
 }
 
@@ -604,7 +819,7 @@ int launch_force_summed(const ForceArgs &fa, const JDS &j, const SumArgs &sa, in
         k_force_seq<<<grid, kSeqNT, kSeqSmem, st>>>(fa, j, sa.slots);
         return 1;
     }
-    k_force_sorted<<<grid, kSortNT, 0, st>>>(fa, j, sa);
+    k_force_sorted<<<grid, kSortNT, sizeof(SortShared), st>>>(fa, j, sa);
     return 1;
 }
 

@@ -260,3 +260,37 @@ def test_square_root_exceptions_bit_exact(nb, mode, case):
     got = _gpu_force(nb, m, x, v, eps, idx, MODES[mode][0], no_force=True)
     ref = oracle.force_summed(m, x, v, eps, idx, mode=MODES[mode][1], nthreads=8)
     _assert_same(got, ref, "%s %s" % (mode, case))
+
+
+@pytest.mark.parametrize("n", [255, 256, 257, 2047, 2049, 4096, 4097, 9000])
+def test_sorted_chunks_bit_exact(nb, n):
+    # sizes around a row, a chunk and a tile; the sums have a fixed order
+    m, x, v = plummer(n, 41)
+    idx = sample_active(n, 12, n)
+    got = _gpu_force(nb, m, x, v, EPS, idx, nb.NB_SUM_FP32_SORTED, no_force=True)
+    ref = oracle.force_summed(m, x, v, EPS, idx, mode=oracle.SUM_FP32_SORTED, nthreads=8)
+    _assert_same(got, ref, "sorted n=%d" % n)
+
+
+@pytest.mark.parametrize("case", ["lattice", "one_bin", "wide", "massless"])
+def test_sorted_key_distributions_bit_exact(nb, case):
+    # many equal keys, one bin above a chunk's size (both sorted in the
+    # scratch), keys over most of the single-precision range, and zero keys
+    rng = np.random.RandomState(8)
+    n = 5000
+    m = np.full(n, 1.0 / n)
+    v = rng.normal(size=(n, 3))
+    if case == "lattice":
+        x = np.stack(np.meshgrid(*[np.arange(18.0)] * 3, indexing="ij"), -1).reshape(-1, 3)[:n] / 4
+    elif case == "one_bin":
+        u = rng.normal(size=(n, 3))
+        x = u / np.linalg.norm(u, axis=1)[:, None] * (1 + 1e-3 * rng.uniform(size=(n, 1)))
+        x[0] = 0.0
+    else:
+        x = rng.normal(size=(n, 3)) * 10.0 ** rng.uniform(-3, 8, (n, 1))
+        if case == "massless":
+            m[rng.permutation(n)[:3000]] = 0.0
+    idx = np.array([0, 1, 77, n - 1], dtype=np.int32)
+    got = _gpu_force(nb, m, x, v, EPS, idx, nb.NB_SUM_FP32_SORTED, no_force=True)
+    ref = oracle.force_summed(m, x, v, EPS, idx, mode=oracle.SUM_FP32_SORTED, nthreads=8)
+    _assert_same(got, ref, "sorted %s" % case)
