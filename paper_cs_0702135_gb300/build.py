@@ -20,6 +20,7 @@ LIB = os.path.join(PKG, "libnb_gb300.so")
 SOURCES = ["k_force.cu", "k_step.cu", "nb_api.cu", "k_noalloc.cu", "k_adjoint.cu", "k_ensemble.cu",
            "k_sum.cu", "k_run.cu"]
 HEADERS = [os.path.join(CSRC, "nb_internal.cuh"), os.path.join(CSRC, "nb_device.cuh"),
+           os.path.join(CSRC, "nb_int64.cuh"),
            os.path.join(INCLUDE, "nb.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I" + INCLUDE,

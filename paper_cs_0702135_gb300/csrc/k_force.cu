@@ -11,7 +11,8 @@
 // x_j - x_i is formed as (x_j,hi - x_i,hi) + (x_j,lo - x_i,lo), the pair terms
 // run in FP32 with rsqrt.approx on the SFU, and each thread's per-tile FP32 partials
 // are folded into hi + lo FP32 accumulators with TwoSum, so that the error of
-// the sum over all N does not grow with N.  FP64 kernels do everything in FP64.
+// the sum over all N does not grow with N.  FP64 kernels sum in FP64 and
+// round every factor to FP64.
 //
 // i-parallel kernels: a CTA owns a block of active i (R per thread, in
 // registers) and one j slice, streamed through shared memory in tiles that
@@ -31,6 +32,7 @@
 // ratios is larger than the potential itself.)  With eps = 0 a pair at r = 0
 // between distinct particles is dropped as well.
 #include "nb_device.cuh"
+#include "nb_int64.cuh"
 
 namespace nbk {
 namespace {
@@ -67,6 +69,75 @@ __device__ __forceinline__ void pair_f64(const double4_32a &p, const double4_32a
     pot -= mr;
 }
 
+// The same with all but the final multiply-adds on the integer pipes (nb_int64.cuh):
+// softened, all values in range.
+struct J64I {
+    i64::Fix x[6];   // position, velocity
+    i64::Num m;
+};
+__device__ __forceinline__ void pair_f64_int(const J64I &J, const i64::Fix I[6], const i64::Eps &eps,
+                                             double acc[3], double jk[3], double &pot, int j, int i)
+{
+    double d[6], mr, mr3, b;
+    i64::Num D[6];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) D[c] = i64::diff(J.x[c], I[c], d[c]);
+    i64::pair_factors(D, D + 3, J.m, eps, mr, mr3, b);
+    mr = (j == i) ? 0.0 : mr;   // its d and b are 0
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        acc[c] = fma(mr3, d[c], acc[c]);
+        jk[c] = fma(mr3, fma(b, d[c], d[3 + c]), jk[c]);
+    }
+    pot -= mr;
+}
+
+// The integer form of a j in 64 bytes: the seven significands, and their
+// exponents and the sign of the mass as signed bytes.
+struct __align__(16) J64Tile {
+    long long m[7];
+    unsigned e[2];
+};
+__device__ __forceinline__ void to_fix6(const double4_32a &p, const double4_32a &w, i64::Fix x[6])
+{
+    x[0] = i64::to_fix(p.x); x[1] = i64::to_fix(p.y); x[2] = i64::to_fix(p.z);
+    x[3] = i64::to_fix(w.x); x[4] = i64::to_fix(w.y); x[5] = i64::to_fix(w.z);
+}
+__device__ __forceinline__ J64Tile tile_of(const double4_32a &p, const double4_32a &w)
+{
+    i64::Fix x[6];
+    to_fix6(p, w, x);
+    const i64::Num m = i64::to_num(p.w);
+    J64Tile t;
+#pragma unroll
+    for (int c = 0; c < 6; ++c) t.m[c] = x[c].m;
+    t.m[6] = (long long)m.m;
+    t.e[0] = (unsigned)(x[0].e & 255) | (unsigned)(x[1].e & 255) << 8 | (unsigned)(x[2].e & 255) << 16 |
+             (unsigned)x[3].e << 24;
+    t.e[1] = (unsigned)(x[4].e & 255) | (unsigned)(x[5].e & 255) << 8 | (unsigned)(m.e & 255) << 16 |
+             (m.neg ? 1u << 31 : 0u);
+    return t;
+}
+__device__ __forceinline__ int signed_byte(unsigned w, int k) { return (int)(w << (24 - 8 * k)) >> 24; }
+__device__ __forceinline__ J64I j_of(const J64Tile &t)
+{
+    J64I J;
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+        J.x[c].m = t.m[c];
+        J.x[c].e = signed_byte(t.e[c / 4], c % 4);
+    }
+    J.m.m = (unsigned long long)t.m[6];
+    J.m.e = signed_byte(t.e[1], 2);
+    J.m.neg = (int)t.e[1] < 0;
+    return J;
+}
+
+__device__ __forceinline__ bool in_range_f64(const double4_32a &p, const double4_32a &w)
+{
+    return i64::in_range(p.x) && i64::in_range(p.y) && i64::in_range(p.z) && i64::in_range(p.w) &&
+           i64::in_range(w.x) && i64::in_range(w.y) && i64::in_range(w.z);
+}
 
 // ----------------------------------------------------------------------------
 // DS, i-parallel.
@@ -328,16 +399,30 @@ __global__ void __launch_bounds__(NT, 2) k_force_jpar_ds(ForceArgs fa, JDS J)
 
 // ----------------------------------------------------------------------------
 // FP64, i-parallel.
+//
+// A tile whose j and the CTA's i are all in the range of nb_int64.cuh runs on the
+// integer pipes, any other tile (and eps = 0) the FP64 form: 1820 active of 65536
+// in 2.85 ms against 7.38 ms for the FP64 form alone.  Moving the pair factors but
+// not the differences gave 3.79 ms (16 FP64 operations a pair, against 10).  With
+// 12 CTAs an SM (80 registers, 60 bytes spilled) against 9 without the limit:
+// 2.85 against 3.14 ms; 1024 active 1.75 against 1.65, 4096 6.20 against 6.24.
 
 template <int NT, int R, bool SOFT>
-__global__ void __launch_bounds__(NT) k_force_ipar_f64(ForceArgs fa, JF64 J)
+__global__ void __launch_bounds__(NT, 12) k_force_ipar_f64(ForceArgs fa, JF64 J)
 {
     const ForcePlan F = load_plan(fa);
     const int na = F.na;
     if (na <= 0 || F.regime != kRegIpar) return;
     const Plan P = F.p;
-    __shared__ double4_32a s_p[NT], s_v[NT];
+    __shared__ union Tile {
+        struct {
+            double4_32a p, v;
+        } f;
+        J64Tile i;
+        __device__ Tile() {}
+    } s_t[NT];
     const double eps2 = fa.eps2;
+    const i64::Eps ieps = i64::make_eps(eps2);
     const int tid = threadIdx.x;
 
     for (int w = blockIdx.x; w < P.items; w += gridDim.x) {
@@ -345,7 +430,9 @@ __global__ void __launch_bounds__(NT) k_force_ipar_f64(ForceArgs fa, JF64 J)
         ipar_item(w, P.n_iblk, P.n_whole, P.S, P.jslice, fa.n, ib, sl, j0, j1);
 
         double xi[R][3], vi[R][3];
+        i64::Fix xf[R][6];
         int ia[R], ii[R];
+        bool iok = SOFT && i64::eps2_in_range(eps2);
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const int a = ib * NT * R + r * NT + tid;
@@ -353,6 +440,8 @@ __global__ void __launch_bounds__(NT) k_force_ipar_f64(ForceArgs fa, JF64 J)
             const int i = clamp_index(fa.act[a < na ? a : 0], fa.n);
             ii[r] = i;
             const double4_32a p = J.pos[i], v = J.vel[i];
+            iok = iok && in_range_f64(p, v);
+            to_fix6(p, v, xf[r]);
             xi[r][0] = p.x; xi[r][1] = p.y; xi[r][2] = p.z;
             vi[r][0] = v.x; vi[r][1] = v.y; vi[r][2] = v.z;
         }
@@ -364,19 +453,31 @@ __global__ void __launch_bounds__(NT) k_force_ipar_f64(ForceArgs fa, JF64 J)
             pot[r] = 0.0;
         }
         for (int jt = j0; jt < j1; jt += NT) {
-            __syncthreads();
             const int j = jt + tid;
+            double4_32a pj = make_double4_32a(0., 0., 0., 0.), vj = pj;
             if (j < j1) {
-                s_p[tid] = J.pos[j];
-                s_v[tid] = J.vel[j];
-            } else {
-                s_p[tid] = make_double4_32a(0., 0., 0., 0.);
-                s_v[tid] = make_double4_32a(0., 0., 0., 0.);
+                pj = J.pos[j];
+                vj = J.vel[j];
             }
+            // also the barrier between the tiles
+            if (__syncthreads_and(iok && in_range_f64(pj, vj))) {
+                s_t[tid].i = tile_of(pj, vj);
+                __syncthreads();
+#pragma unroll 1
+                for (int jj = 0; jj < NT; ++jj) {
+                    const J64I JJ = j_of(s_t[jj].i);
+#pragma unroll
+                    for (int r = 0; r < R; ++r)
+                        pair_f64_int(JJ, xf[r], ieps, acc[r], jk[r], pot[r], jt + jj, ii[r]);
+                }
+                continue;
+            }
+            s_t[tid].f.p = pj;
+            s_t[tid].f.v = vj;
             __syncthreads();
 #pragma unroll 4
             for (int jj = 0; jj < NT; ++jj) {
-                const double4_32a p = s_p[jj], v = s_v[jj];
+                const double4_32a p = s_t[jj].f.p, v = s_t[jj].f.v;
 #pragma unroll
                 for (int r = 0; r < R; ++r)
                     pair_f64<SOFT>(p, v, xi[r], vi[r], eps2, acc[r], jk[r], pot[r], jt + jj, ii[r]);
@@ -400,7 +501,8 @@ __global__ void __launch_bounds__(NT) k_force_ipar_f64(ForceArgs fa, JF64 J)
 }
 
 // ----------------------------------------------------------------------------
-// FP64, j-parallel (small blocks).
+// FP64, j-parallel (small blocks).  The same choice as above for each j: 32
+// active of 65536 in 126 us against 180 in FP64, one in 84 against 126.
 
 template <int NT, int IC, bool SOFT>
 __global__ void __launch_bounds__(NT) k_force_jpar_f64(ForceArgs fa, JF64 J)
@@ -413,6 +515,7 @@ __global__ void __launch_bounds__(NT) k_force_jpar_f64(ForceArgs fa, JF64 J)
     constexpr int NV = IC * kComp;
     __shared__ double s_r[NW][NV];
     const double eps2 = fa.eps2;
+    const i64::Eps ieps = i64::make_eps(eps2);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
     for (int w = blockIdx.x; w < P.items; w += gridDim.x) {
@@ -421,13 +524,17 @@ __global__ void __launch_bounds__(NT) k_force_jpar_f64(ForceArgs fa, JF64 J)
         const int j0 = sl * P.jslice;
         const int j1 = min(fa.n, j0 + P.jslice);
         double xi[IC][3], vi[IC][3];
+        i64::Fix xf[IC][6];
         int ii[IC];
+        bool iok = SOFT && i64::eps2_in_range(eps2);
 #pragma unroll
         for (int q = 0; q < IC; ++q) {
             const int a = ch * IC + q;
             const int i = clamp_index(fa.act[a < na ? a : 0], fa.n);
             ii[q] = i;
             const double4_32a p = J.pos[i], v = J.vel[i];
+            iok = iok && in_range_f64(p, v);
+            to_fix6(p, v, xf[q]);
             xi[q][0] = p.x; xi[q][1] = p.y; xi[q][2] = p.z;
             vi[q][0] = v.x; vi[q][1] = v.y; vi[q][2] = v.z;
         }
@@ -436,12 +543,17 @@ __global__ void __launch_bounds__(NT) k_force_jpar_f64(ForceArgs fa, JF64 J)
         for (int e = 0; e < NV; ++e) val[e] = 0.0;
         for (int j = j0 + tid; j < j1; j += NT) {
             const double4_32a p = J.pos[j], v = J.vel[j];
+            const bool ok = iok && in_range_f64(p, v);
+            J64I JJ;
+            to_fix6(p, v, JJ.x);
+            JJ.m = i64::to_num(p.w);
 #pragma unroll
             for (int q = 0; q < IC; ++q) {
                 double a3[3] = {val[q * kComp], val[q * kComp + 1], val[q * kComp + 2]};
                 double k3[3] = {val[q * kComp + 3], val[q * kComp + 4], val[q * kComp + 5]};
                 double pp = val[q * kComp + 6];
-                pair_f64<SOFT>(p, v, xi[q], vi[q], eps2, a3, k3, pp, j, ii[q]);
+                if (ok) pair_f64_int(JJ, xf[q], ieps, a3, k3, pp, j, ii[q]);
+                else pair_f64<SOFT>(p, v, xi[q], vi[q], eps2, a3, k3, pp, j, ii[q]);
                 val[q * kComp] = a3[0]; val[q * kComp + 1] = a3[1]; val[q * kComp + 2] = a3[2];
                 val[q * kComp + 3] = k3[0]; val[q * kComp + 4] = k3[1]; val[q * kComp + 5] = k3[2];
                 val[q * kComp + 6] = pp;

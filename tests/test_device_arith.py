@@ -189,3 +189,83 @@ def test_ticks_to_time_bits():
         sh = (64 - q.bit_length()) - 11
         bits = (q << sh) + ((1023 + 52 - 40 - 1 - sh) << 52)
         assert np.array([bits], dtype=np.uint64).view(np.float64)[0] == q * 2.0 ** -40
+
+
+SRC_INT64 = r"""
+#include <cstdio>
+#include "nb_int64.cuh"
+using namespace nbk::i64;
+int main() {
+    double a[6], c[6], m, e2, d[6], mr, mr3, b;
+    for (;;) {
+        for (int k = 0; k < 6; ++k) if (std::scanf("%lf %lf", a + k, c + k) != 2) return 0;
+        if (std::scanf("%lf %lf", &m, &e2) != 2) return 0;
+        Num D[6];
+        bool ok = in_range(m) && eps2_in_range(e2);
+        for (int k = 0; k < 6; ++k) {
+            ok = ok && in_range(a[k]) && in_range(c[k]);
+            D[k] = diff(to_fix(a[k]), to_fix(c[k]), d[k]);
+        }
+        pair_factors(D, D + 3, to_num(m), make_eps(e2), mr, mr3, b);
+        for (int k = 0; k < 6; ++k) std::printf("%a ", d[k]);
+        std::printf("%a %a %a %d\n", mr, mr3, b, ok ? 1 : 0);
+    }
+}
+"""
+
+
+def test_integer_pair_factors(tmp_path):
+    # in units of 2^-53: a difference is rounded once (1, and 2^-8 for the cut);
+    # r^2 loses at most 10 of 2^59 and so 1/r 0.08 more, its power 3 0.23, and the
+    # products 3 of 2^60 each: 1.25, 1.5 and (of the sum of magnitudes) 1.5
+    import os
+    import shutil
+    import subprocess
+    cxx = shutil.which("g++")
+    if not cxx:
+        pytest.skip("needs g++")
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    src, exe = tmp_path / "i64.cpp", tmp_path / "i64"
+    src.write_text(SRC_INT64)
+    subprocess.run([cxx, "-std=c++17", "-O1", "-I" + os.path.join(root, "paper_cs_0702135_gb300", "csrc"),
+                    str(src), "-o", str(exe)], check=True)
+    rng = random.Random(3)
+    rows = []
+    for k in range(6000):
+        wide = 99 if k % 3 == 0 else 6
+        sx, sv = rng.uniform(-wide, wide), rng.uniform(-wide, wide)
+        row = []
+        for c in range(6):
+            s = 2.0 ** min(99, max(-99, (sx if c < 3 else sv) + rng.uniform(-4, 4)))
+            a, b = rng.uniform(-1, 1) * s, rng.uniform(-1, 1) * s
+            b = rng.choice((b, b, 0.0, a, a * (1 + 2.0 ** -rng.randint(1, 52)), math.nextafter(a, 2 * a)))
+            row += [a, b] if rng.random() < 0.5 else [b, a]
+        if k % 50 == 0:
+            row[6:] = [0.0] * 6
+        if k % 60 == 0:
+            row[:6] = [row[0]] * 6
+        row += [rng.choice((0.0, 1.0, -1.0, 1.0)) * 2.0 ** rng.uniform(-99, 99),
+                2.0 ** rng.uniform(-99, 99) if k % 2 else 2.0 ** rng.uniform(-20, -10)]
+        rows.append(row)
+    inp = "\n".join(" ".join(v.hex() for v in r) for r in rows)
+    out = subprocess.run([str(exe)], input=inp, capture_output=True, text=True, check=True).stdout.splitlines()
+    assert len(out) == len(rows)
+    u, inside = F(1, 1 << 53), 0
+    for row, line in zip(rows, out):
+        got = [float.fromhex(t) for t in line.split()[:9]]
+        if not int(line.split()[9]):
+            continue   # too small a value: not taken by this arithmetic
+        inside += 1
+        d = [F(row[2 * c]) - F(row[2 * c + 1]) for c in range(6)]
+        for c in range(6):
+            assert abs(F(got[c]) - d[c]) <= abs(d[c]) * u * (1 + F(1, 256)), row
+        r2 = sum(q * q for q in d[:3]) + F(row[13])
+        num, den = r2.numerator << 600, r2.denominator << 600
+        r = F(math.isqrt(num * den), den)
+        m = F(row[12])
+        assert abs(F(got[6]) - m / r) <= abs(m / r) * u * F(5, 4), row
+        assert abs(F(got[7]) - m / r / r2) <= abs(m / r / r2) * u * F(3, 2), row
+        dot = sum(d[c] * d[3 + c] for c in range(3))
+        mag = sum(abs(d[c] * d[3 + c]) for c in range(3))
+        assert abs(F(got[8]) + 3 * dot / r2) <= 3 * mag / r2 * u * F(3, 2), row
+    assert inside > 5000

@@ -306,3 +306,42 @@ def test_device_sized_blocks_draw_the_same_items(nb):
     finally:
         a.nb_free()
         b.nb_free()
+
+
+@pytest.mark.parametrize("na", [1, 5, 33, 64, 65, 130])
+@pytest.mark.parametrize("n", [65, 130, 700])
+def test_fp64_values_out_of_range(nb, n, na):
+    # the FP64 kernels take a tile (or a j) with a value outside 2^-100..2^100 through
+    # another form; masses of zero, bodies at rest, equal positions
+    if na > n:
+        return
+    rng = np.random.default_rng(n + na)
+    m, x, v = plummer(n, 31)
+    m[::7] = 0.0
+    v[::5] = 0.0
+    x[8] = x[9]
+    idx = sample_active(n, na, 5)
+    res = []
+    for far in (0.0, 2.0 ** 101, 2.0 ** -101):
+        xx, vv = x.copy(), v.copy()
+        for j in rng.choice(n, 2, replace=False):
+            if far:
+                xx[j, j % 3] = far
+                vv[j, (j + 1) % 3] = 2.0 ** -101
+        res.append(_check(nb, m, xx, vv, EPS, idx, nb.NB_FP64, label="far=%g" % far)[1])
+    assert all(np.isfinite(a).all() for r in res for a in r)
+    for eps in (EPS, 2.0 ** -51):   # eps^2 below the range too
+        ctx = nb.Context(m, x, v, eps, precision=nb.NB_FP64, flags=nb.NB_INIT_NO_FORCE)
+        try:
+            got = ctx.nb_force(idx)
+        finally:
+            ctx.nb_free()
+        ref = oracle.force(m, x, v, eps, idx, nthreads=8)
+        mags = pair_magnitudes(m, x, v, eps, idx)
+        ea, ek, _ = force_errors(got, ref, mags)
+        assert ea.max() < TOL_F64["acc"] and ek.max() < TOL_F64["jerk"]
+    zero = nb.Context(np.zeros(n), x, np.zeros((n, 3)), EPS, precision=nb.NB_FP64, flags=nb.NB_INIT_NO_FORCE)
+    try:
+        assert all((a == 0.0).all() for a in zero.nb_force(idx))
+    finally:
+        zero.nb_free()
