@@ -1,33 +1,31 @@
 // k_ensemble.cu -- many independent clusters advanced together: every
 // ensemble block step advances every unfinished cluster by its own next block
-// step (Section 2 step loop: select the block, predict, force, correct) in one
-// persistent cooperative launch, replayed from a CUDA graph.  Its CTAs work in
-// two phases:
-//   A. clusters, largest first, from a work counter: block time t_next = min
-//      over the cluster of t_i + dt_i, the block compacted in ascending order
-//      (ballot + prefix sums), every particle predicted to t_next (FP64, the
-//      single-system predictor's arithmetic) into global double-single j
-//      records, and one work item per chunk of up to threads / gmax active
-//      particles published to a queue (the item's cluster index is written
-//      last and marks it ready).  A cluster above 512 particles is not
-//      predicted here: its prediction goes to the queue as chunks of 512,
-//      ahead of its force items, so several CTAs share the FP64 work;
-//   B. once every cluster is claimed, queue items in order: prediction chunks;
-//      force items (which first wait for their cluster's prediction): the j
-//      records stream through shared-memory tiles, g consecutive lanes share one
-//      active particle and split its j loop when the chunk is small (g = the
-//      largest power of two with g * chunk <= threads, capped at gmax), FP32
-//      pair arithmetic on double-single positions with TwoSum-promoted partials
-//      and a shuffle reduction in the lane group; the group's first lane
-//      corrects its particle (FP64 corrector and Aarseth step, the
-//      single-system corrector's arithmetic).  The force reads only the j
-//      records, so correcting while other items still sum is safe.
-// An item waits only for its own cluster's phase A, so the large clusters'
-// items run while small clusters are still being predicted.  A CTA waiting for
-// an item spins with a time limit (error NB_ETIMEOUT past it); the cooperative
-// launch keeps every CTA resident, and every cluster is claimed before any CTA
-// waits, so the wait always ends.  Every item is computed by one CTA in a fixed
-// order, so results do not depend on which CTA takes it.
+// step (Section 2 step loop: select the block, predict, force, correct) in
+// three launches, replayed from CUDA graphs:
+//   k_ens_sched, a CTA per cluster, largest first: block time t_next = min over
+//      the cluster of t_i + dt_i, the block compacted in ascending order, a
+//      force item per chunk of active particles queued by size class, and up to
+//      512 particles predicted to t_next (predict_j32: FP32 increments on a
+//      single-precision mirror, into double-single j records);
+//   k_ens_predict: the prediction of larger clusters, a CTA per 512 particles;
+//   k_ens_force: the force items, the largest clusters' first, drawn by CTAs
+//      that fill the GPU: g lanes share one or two active particles and split
+//      the j (FP32 pair arithmetic on double-single positions, TwoSum-promoted
+//      sums), then four lanes correct a particle (FP64 corrector and Aarseth
+//      step).  The force reads only the j records, so correcting while other
+//      items still sum is safe.
+// Nothing waits inside a launch, and every particle's sums are formed in an order
+// that only (threads, gmax) fix, so results do not depend on which CTA takes an item.
+//
+// 256 clusters of 32..4096, a mean of 2e7 pairs a step: 70 us a step (start-up
+// of a graph included: 73 with one step a graph), of which k_ens_sched 6.3,
+// k_ens_predict 4, k_ens_force 37-45, the gaps between launches 2.3 each.  One
+// cooperative launch with queues between the phases took 125 us: its items
+// computed all of the CTA's lane groups, active or not, and their CTAs waited for
+// the correction; with lone particles' warps leaving early and the j of a large
+// cluster shared by ways 80, as three launches 76.  All particles active, the force
+// runs at 7e11 pairs/s, bound by instruction issue (44 a pair and lane) and by shared
+// memory (6.4 wavefronts; one particle a lane: 5.5e11, 52 and 12.9).
 #include <algorithm>
 #include <climits>
 #include <cmath>
@@ -49,6 +47,19 @@ using namespace dev;
 
 constexpr int kEnsMaxN = 4096;       // largest cluster
 constexpr int kEnsPredChunk = 512;   // larger clusters are predicted in chunks by several CTAs
+constexpr int kEnsClasses = 4;       // force items by cluster size, the longest first
+
+__host__ __device__ inline int ens_class(int n) { return n > 2048 ? 0 : (n > 1024 ? 1 : (n > 512 ? 2 : 3)); }
+
+constexpr int kEnsANT = 256;         // threads of a scheduling CTA
+constexpr int kEnsPNT = 128;         // ... of a prediction CTA
+constexpr int kEnsFNT = 128;         // ... of a force CTA
+constexpr int kEnsR = 2;             // active particles of a lane group, large blocks
+constexpr int kEnsMaxWays = 2;       // sum blocks that a force CTA works on at once (see ens_sums)
+constexpr int kEnsChain = 2048;      // a cluster above this many j has its force items cut for two ways
+constexpr int kEnsStageJ = 256;      // j of a stage
+constexpr int kEnsStages = 2;
+constexpr int kEnsGraphSteps = 8;    // steps of the longer graph
 
 struct EnsArgs {
     int C;                    // clusters
@@ -59,16 +70,13 @@ struct EnsArgs {
     double eta, eta_init;
     int level_min;
     long long t_end;
-    int gmax;                 // largest lane group per active particle
-    int chunk;                // active particles per work item (threads / gmax)
-    int *work;                // phase A: cluster counter
-    int *work_b;              // phase B: item counter
-    int *qlen;                // queue length (items reserved in phase A)
-    int *a_done;              // clusters whose phase A finished
-    int *qc, *qk;             // queue: cluster (-1 = not ready); force chunk k >= 0 or
-                              // prediction chunk -1 - k of each item
-    int qcap;                 // queue capacity: P + C (at most n_c + 1 items per cluster)
-    int *pred_left;           // [C] prediction chunks of the cluster not yet done
+    int g;                    // lanes per active particle
+    int sb;                   // j of a sum block
+    int *work;                // counters: force items claimed, force CTAs done, and the queue
+                              // lengths [kEnsClasses]; all 0 between launches
+    const int2 *pitem;        // prediction items: cluster, chunk
+    int2 *queue;              // force items: cluster, chunk; [P] in size classes
+    int qbase[kEnsClasses];   // first slot of each class
     float4 *jph, *jpl, *jv;   // [P] predicted double-single records
     Mirror mir;               // [P] single-precision mirror of the FP64 state for the j predictor
     int *act;                 // [P] active particles of each cluster (local indices)
@@ -80,6 +88,17 @@ struct EnsArgs {
     int *err;
     double *out_acc, *out_jerk, *out_pot;  // force-only mode: [P][3], [P][3], [P]
 };
+
+// Ways and particles of a full force item of a cluster.  Two ways above 2048 j:
+// 512 launches of 256 clusters of 32..4096 take 37.9 ms with the line there, 38.6
+// at 1024 or 512, 42.6 without it, 41.9 with four ways above 1024 (the items
+// read their j from the L2 cache, so smaller ones read more).
+__device__ __forceinline__ int ens_ways(int n) { return n > kEnsChain ? kEnsMaxWays : 1; }
+__device__ __forceinline__ int ens_chunk(int n, int na, int g)
+{
+    const int one = kEnsFNT / g / ens_ways(n);
+    return na > one ? kEnsR * one : one;
+}
 
 template <typename T, typename Op>
 __device__ __forceinline__ T cta_reduce(T v, Op op, T *smem)
@@ -126,320 +145,367 @@ __global__ void k_ens_mirror(EnsArgs ea)
         ens_write_mirror(ea, gi);
 }
 
-// Phase A for the cluster of rank q: schedule, predict, compact, publish.
-template <int NT, int MODE>
-__device__ __forceinline__ void ens_a_cluster(const EnsArgs &ea, int q, long long *s_red, int *s_wtot)
+// The j record of the stored state itself (start-up and force-only passes: dt = 0).
+__device__ __forceinline__ void ens_record(const EnsArgs &ea, long long gi)
 {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const State &S = ea.s;
     const long long P = S.n;
-    const int c = ea.order[q];
+    float hi[3], lo[3];
+#pragma unroll
+    for (int cc = 0; cc < 3; ++cc) split_ds(S.x[cc * P + gi], hi[cc], lo[cc]);
+    ea.jph[gi] = make_float4(hi[0], hi[1], hi[2], __double2float_rn(S.m[gi]));
+    ea.jpl[gi] = make_float4(lo[0], lo[1], lo[2], 0.0f);
+    ea.jv[gi] = make_float4(__double2float_rn(S.v[gi]), __double2float_rn(S.v[P + gi]),
+                            __double2float_rn(S.v[2 * P + gi]), 0.0f);
+}
+
+struct AShared {
+    long long red[16];
+    unsigned bal[kEnsMaxN / 32];
+    int off[kEnsMaxN / 32];
+    int base;
+};
+
+// Schedules the cluster of rank blockIdx.x: block time, block, force items; a small
+// cluster is predicted as well.  The
+// next times are read once, into shared memory, and the block is compacted with
+// one ballot word per 32 particles and one scan of the words.
+template <int MODE>
+__global__ void __launch_bounds__(kEnsANT) k_ens_sched(EnsArgs ea)
+{
+    constexpr int NT = kEnsANT;
+    __shared__ AShared A;
+    __shared__ long long s_next[kEnsMaxN];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const State &S = ea.s;
+    const int c = ea.order[blockIdx.x];
     const long long o = ea.off[c];
     const int n = (int)(ea.off[c + 1] - o);
     if (MODE == kEnsStep && ea.done[c]) return;
     long long tn = 0;
     if (MODE == kEnsStep) {
         long long mn = LLONG_MAX;
-        for (int i = tid; i < n; i += NT)
-            mn = min(mn, S.t[o + i] + (1LL << (kTickBits - S.lev[o + i])));
-        tn = cta_reduce(mn, MinLL(), s_red);
+#pragma unroll 4
+        for (int i = tid; i < n; i += NT) {
+            const long long nx = S.t[o + i] + (1LL << (kTickBits - S.lev[o + i]));
+            s_next[i] = nx;
+            mn = min(mn, nx);
+        }
+        tn = cta_reduce(mn, MinLL(), A.red);
         if (tn > ea.t_end) {
             if (tid == 0) ea.done[c] = 1;
             return;
         }
     }
-    const bool split = n > kEnsPredChunk;  // prediction left to queue items
-    int running = 0;
-    for (int base = 0; base < n; base += NT) {
-        const int i = base + tid;
-        bool f = false;
-        if (i < n && !split) {
-            const long long gi = o + i;
-            if (MODE == kEnsStep) {
-                ens_predict_j32(ea, gi, tn);
-            } else {
-                // start-up and force-only passes: the stored state itself (dt = 0)
-                float hi[3], lo[3];
+    const int words = (n + 31) >> 5;
+    for (int w = warp; w < words; w += NT / 32) {
+        const int i = 32 * w + lane;
+        const unsigned bal = __ballot_sync(0xffffffffu, i < n && (MODE != kEnsStep || s_next[i] == tn));
+        if (lane == 0) A.bal[w] = bal;
+    }
+    const bool split = n > kEnsPredChunk;  // prediction left to items of its own
+    if (!split)
+        for (int i = tid; i < n; i += NT) {
+            if (MODE == kEnsStep) ens_predict_j32(ea, o + i, tn);
+            else ens_record(ea, o + i);
+        }
+    __syncthreads();
+    if (warp == 0) {
+        constexpr int kPer = kEnsMaxN / 32 / 32;
+        int cw[kPer], sum = 0;
 #pragma unroll
-                for (int cc = 0; cc < 3; ++cc) split_ds(S.x[cc * P + gi], hi[cc], lo[cc]);
-                ea.jph[gi] = make_float4(hi[0], hi[1], hi[2], __double2float_rn(S.m[gi]));
-                ea.jpl[gi] = make_float4(lo[0], lo[1], lo[2], 0.0f);
-                ea.jv[gi] = make_float4(__double2float_rn(S.v[gi]), __double2float_rn(S.v[P + gi]),
-                                        __double2float_rn(S.v[2 * P + gi]), 0.0f);
+        for (int u = 0; u < kPer; ++u) {
+            const int w = kPer * lane + u;
+            cw[u] = w < words ? __popc(A.bal[w]) : 0;
+            sum += cw[u];
+        }
+        int inc = sum;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int up = __shfl_up_sync(0xffffffffu, inc, d);
+            inc += lane >= d ? up : 0;
+        }
+        int at = inc - sum;
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) {
+            A.off[kPer * lane + u] = at;
+            at += cw[u];
+        }
+        const int na = __shfl_sync(0xffffffffu, inc, 31);
+        if (lane == 0) {
+            ea.na[c] = na;
+            ea.tnext[c] = tn;
+            if (MODE == kEnsStep) {
+                ea.steps[c] += 1;
+                ea.inter[c] += (long long)na * (n - 1);
             }
         }
-        if (i < n) {
-            const long long gi = o + i;
-            f = MODE == kEnsStep ? (S.t[gi] + (1LL << (kTickBits - S.lev[gi])) == tn) : true;
-        }
-        const unsigned bal = __ballot_sync(0xffffffffu, f);
-        if (lane == 0) s_wtot[warp] = __popc(bal);
-        __syncthreads();
-        int woff = 0, tot = 0;
-        for (int w = 0; w < NT / 32; ++w) {
-            woff += w < warp ? s_wtot[w] : 0;
-            tot += s_wtot[w];
-        }
-        if (f) ea.act[o + running + woff + __popc(bal & ((1u << lane) - 1u))] = i;
-        running += tot;
-        __syncthreads();
+        const int chunk = ens_chunk(n, na, ea.g), cls = ens_class(n), nforce = (na + chunk - 1) / chunk;
+        int base = lane == 0 ? atomicAdd(&ea.work[2 + cls], nforce) : 0;
+        base = ea.qbase[cls] + __shfl_sync(0xffffffffu, base, 0);
+        for (int k = lane; k < nforce; k += 32) ea.queue[base + k] = make_int2(c, k);
     }
-    // every thread's records and active indices are written before tid 0 publishes
-    __threadfence();
     __syncthreads();
-    if (tid == 0) {
-        const int na = running;
-        ea.na[c] = na;
-        ea.tnext[c] = tn;
-        if (MODE == kEnsStep) {
-            ea.steps[c] += 1;
-            ea.inter[c] += (long long)na * (n - 1);
-        }
-        const int npred = split ? (n + kEnsPredChunk - 1) / kEnsPredChunk : 0;
-        const int nforce = (na + ea.chunk - 1) / ea.chunk;
-        ea.pred_left[c] = npred;
-        const int base = atomicAdd(ea.qlen, npred + nforce);
-        for (int k = 0; k < npred; ++k) ea.qk[base + k] = -1 - k;  // ahead of the force items
-        for (int k = 0; k < nforce; ++k) ea.qk[base + npred + k] = k;
-        __threadfence();
-        for (int k = 0; k < npred + nforce; ++k) atomicExch(&ea.qc[base + k], c);
+    for (int w = warp; w < words; w += NT / 32) {
+        const unsigned bal = A.bal[w];
+        if (bal >> lane & 1) ea.act[o + A.off[w] + __popc(bal & ((1u << lane) - 1u))] = 32 * w + lane;
     }
 }
 
-// Queue item `it` for phase B: true with (c, k) once it is published; false
-// when there is no such item (every cluster's phase A finished and the queue
-// is shorter) or the wait ran past its limit (error NB_ETIMEOUT).  Consuming
-// an item marks it not ready again for the next launch.
-constexpr long long kEnsSpinCycles = 4000000000LL;  // about 2 s at 2 GHz
-
-__device__ __forceinline__ bool ens_take_item(const EnsArgs &ea, int it, int &c, int &k)
+// Predicts one chunk of 512 particles of a larger cluster to its block time.
+template <int MODE>
+__global__ void __launch_bounds__(kEnsPNT) k_ens_predict(EnsArgs ea)
 {
-    // Every CTA takes one index past the last item before it stops, so indices
-    // run up to (items + CTAs - 1): those at or past the capacity hold no item.
-    if (it >= ea.qcap) return false;
-    volatile int *qc = ea.qc;
-    volatile int *adone = ea.a_done;
-    volatile int *qlen = ea.qlen;
-    const long long t0 = clock64();
-    for (;;) {
-        const int cc = qc[it];
-        if (cc >= 0) {
-            __threadfence();
-            c = cc;
-            k = __ldcg(&ea.qk[it]);
-            qc[it] = -1;
-            return true;
-        }
-        if (*adone >= ea.C) {
-            __threadfence();
-            if (it >= *qlen) return false;
-            continue;  // published before the last cluster finished: visible next read
-        }
-        if (clock64() - t0 > kEnsSpinCycles) {
-            atomicCAS(ea.err, 0, NB_ETIMEOUT);
-            return false;
-        }
-        __nanosleep(64);
+    const int2 it = ea.pitem[blockIdx.x];
+    if (MODE == kEnsStep && ea.done[it.x]) return;
+    const long long o = ea.off[it.x];
+    const int n = (int)(ea.off[it.x + 1] - o);
+    const long long tn = ea.tnext[it.x];
+    const int i1 = min(n, (it.y + 1) * kEnsPredChunk);
+    for (int i = it.y * kEnsPredChunk + threadIdx.x; i < i1; i += kEnsPNT) {
+        if (MODE == kEnsStep) ens_predict_j32(ea, o + i, tn);
+        else ens_record(ea, o + i);
     }
 }
 
-// Phase B, prediction item: particles [512 p, 512 (p + 1)) of cluster c to its
-// block time; the last CTA to finish a cluster's chunks releases its force items.
-template <int NT, int MODE>
-__device__ __forceinline__ void ens_predict_chunk(const EnsArgs &ea, int c, int p)
+__device__ __forceinline__ void copy16(float4 *dst, const float4 *src)
 {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+
+struct FShared {
+    union {
+        float4 j[kEnsStages][3][kEnsStageJ];
+        float res[kEnsR * kEnsFNT][14];
+    };
+    float part[kEnsR][7][kEnsFNT];
+    int it;
+};
+
+// Sums of the particles act[0 .. cnt) of a cluster (R to a lane group) into sh.res.
+//
+// A particle's sums are fixed by (g, sb): lane q of its g lanes adds the j
+// = q, q + g, ... of a sum block of sb j in FP32, and the blocks are promoted in
+// order.  So the blocks can be shared out: the CTA's lanes make up several ways,
+// each takes every ways-th block, and the first way's lanes promote all of them.
+// The j come in stages of one tile a way, kEnsStages - 1 stages ahead.
+template <int R, bool SOFT>
+__device__ __forceinline__ void ens_sums(const EnsArgs &ea, long long o, int n, const int *act, int cnt, FShared &sh)
+{
+    constexpr int NT = kEnsFNT;
     const int tid = threadIdx.x;
-    const State &S = ea.s;
-    const long long P = S.n;
-    const long long o = ea.off[c];
-    const int n = (int)(ea.off[c + 1] - o);
-    const long long tn = __ldcg(&ea.tnext[c]);
-    const int i1 = min(n, (p + 1) * kEnsPredChunk);
-    for (int i = p * kEnsPredChunk + tid; i < i1; i += NT) {
-        const long long gi = o + i;
-        if (MODE == kEnsStep) {
-            ens_predict_j32(ea, gi, tn);
-        } else {
-            float hi[3], lo[3];
+    const int g = ea.g, sb = ea.sb;
+    int per = g;   // lanes of a way
+    while (R * per < cnt * g) per <<= 1;
+    const int ways = min(min(kEnsMaxWays, NT / per), n <= sb ? 1 : 2);
+    const int T = min(sb, kEnsStageJ / ways);   // j of a tile, a divisor of sb
+    const int lgT = 31 - __clz(T);
+    const float4 *jph = ea.jph + o, *jpl = ea.jpl + o, *jv = ea.jv + o;
+    int fb = 0, fr = 0, fs = 0;   // next fetch: first block, tile within it, stage
+    auto fetch = [&]() {
+        for (int t = tid; t < ways * T; t += NT) {
+            const int j = fb + (t >> lgT) * sb + fr + (t & (T - 1));
+            if (j < n) {
+                copy16(&sh.j[fs][0][t], jph + j);
+                copy16(&sh.j[fs][1][t], jpl + j);
+                copy16(&sh.j[fs][2][t], jv + j);
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        fs = fs == kEnsStages - 1 ? 0 : fs + 1;
+        fr += T;
+        if (fr == sb) {
+            fr = 0;
+            fb += ways * sb;
+        }
+    };
 #pragma unroll
-            for (int cc = 0; cc < 3; ++cc) split_ds(S.x[cc * P + gi], hi[cc], lo[cc]);
-            ea.jph[gi] = make_float4(hi[0], hi[1], hi[2], __double2float_rn(S.m[gi]));
-            ea.jpl[gi] = make_float4(lo[0], lo[1], lo[2], 0.0f);
-            ea.jv[gi] = make_float4(__double2float_rn(S.v[gi]), __double2float_rn(S.v[P + gi]),
-                                    __double2float_rn(S.v[2 * P + gi]), 0.0f);
+    for (int q = 1; q < kEnsStages; ++q) fetch();
+    const int way = tid / per, grp = tid % per / g, lig = tid % g, slots = per / g;
+    const bool work = way < ways && grp < cnt, valid = work && way == 0;
+    const bool warp_work = __any_sync(0xffffffffu, work), warp_valid = __any_sync(0xffffffffu, valid);
+    int i[R];
+    IDS I[R];
+    float hi[R][7], lo[R][7];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int a = grp + r * slots;
+        i[r] = act[a < cnt ? a : 0];
+        I[r] = make_ids(jph[i[r]], jpl[i[r]], jv[i[r]]);
+#pragma unroll
+        for (int cc = 0; cc < 7; ++cc) hi[r][cc] = lo[r][cc] = 0.0f;
+    }
+    int buf = 0;
+    for (int jb = 0; jb < n; jb += ways * sb) {
+        float ta[R][3], tk[R][3], tp[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            ta[r][0] = ta[r][1] = ta[r][2] = tk[r][0] = tk[r][1] = tk[r][2] = tp[r] = 0.0f;
+        for (int q = 0; q < sb && jb + q < n; q += T) {
+            asm volatile("cp.async.wait_group %0;" ::"n"(kEnsStages - 2) : "memory");
+            __syncthreads();
+            fetch();
+            const int jt = jb + way * sb + q, jn = work ? min(n - jt, T) : 0;
+            if (warp_work) {
+                const float4 *ph = sh.j[buf][0] + way * T, *pl = sh.j[buf][1] + way * T, *pv = sh.j[buf][2] + way * T;
+                bool mine = false;
+#pragma unroll
+                for (int r = 0; r < R; ++r) mine |= (unsigned)(i[r] - jt) < (unsigned)T;
+                if (__any_sync(0xffffffffu, mine)) {
+#pragma unroll 1
+                    for (int jj = lig; jj < jn; jj += g)
+#pragma unroll
+                        for (int r = 0; r < R; ++r)
+                            pair_ds_packed<SOFT, true>(ph[jj], pl[jj], pv[jj], I[r], ea.eps2, ta[r], tk[r], tp[r],
+                                                       jt + jj, i[r]);
+                } else {
+#pragma unroll (R == 1 ? 4 : 2)
+                    for (int jj = lig; jj < jn; jj += g) {
+                        const float4 h = ph[jj], l = pl[jj], v = pv[jj];
+#pragma unroll
+                        for (int r = 0; r < R; ++r)
+                            pair_ds_packed<SOFT, false>(h, l, v, I[r], ea.eps2, ta[r], tk[r], tp[r]);
+                    }
+                }
+            }
+            buf = buf == kEnsStages - 1 ? 0 : buf + 1;
+        }
+        if (ways > 1) {
+            if (work && way > 0)
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+#pragma unroll
+                    for (int cc = 0; cc < 7; ++cc)
+                        sh.part[r][cc][tid] = cc < 3 ? ta[r][cc] : (cc < 6 ? tk[r][cc - 3] : tp[r]);
+            __syncthreads();
+        }
+        if (valid)
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+#pragma unroll
+                for (int cc = 0; cc < 7; ++cc)
+                    two_sum_acc(hi[r][cc], lo[r][cc], cc < 3 ? ta[r][cc] : (cc < 6 ? tk[r][cc - 3] : tp[r]));
+                for (int w = 1; w < ways && jb + w * sb < n; ++w)
+#pragma unroll
+                    for (int cc = 0; cc < 7; ++cc)
+                        two_sum_acc(hi[r][cc], lo[r][cc], sh.part[r][cc][w * per + tid]);
+            }
+    }
+    __syncthreads();   // the j tiles are done with: their space takes the sums
+    if (warp_valid) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            for (int d = 1; d < g; d <<= 1) {
+#pragma unroll
+                for (int cc = 0; cc < 7; ++cc) {
+                    const float h2 = __shfl_xor_sync(0xffffffffu, hi[r][cc], d);
+                    const float l2 = __shfl_xor_sync(0xffffffffu, lo[r][cc], d);
+                    ds_add(hi[r][cc], lo[r][cc], h2, l2);
+                }
+            }
+            if (valid && lig == 0 && grp + r * slots < cnt)
+#pragma unroll
+                for (int cc = 0; cc < 7; ++cc) {
+                    sh.res[grp + r * slots][cc] = hi[r][cc];
+                    sh.res[grp + r * slots][7 + cc] = lo[r][cc];
+                }
         }
     }
-    __threadfence();
     __syncthreads();
-    if (tid == 0) atomicSub(&ea.pred_left[c], 1);
 }
 
-// Waits (thread 0) until cluster c's prediction chunks are done; false past
-// the time limit (error NB_ETIMEOUT).  The chunks precede the cluster's force
-// items in the queue, so CTAs already hold them and finish them without waiting.
-__device__ __forceinline__ bool ens_wait_predicted(const EnsArgs &ea, int c)
-{
-    volatile int *left = ea.pred_left;
-    const long long t0 = clock64();
-    while (left[c] > 0) {
-        if (clock64() - t0 > kEnsSpinCycles) {
-            atomicCAS(ea.err, 0, NB_ETIMEOUT);
-            return false;
-        }
-        __nanosleep(64);
-    }
-    __threadfence();
-    return true;
-}
-
-// Phase B, force item (c, k): force on one chunk of the cluster's block, then the
+// Force item (c, k): force on one chunk of the cluster's block, then the
 // correction (or the start-up levels, or plain output).
-template <int NT, int MODE>
-__device__ __forceinline__ void ens_b_item(const EnsArgs &ea, int c, int k, float4 *s_ph, float4 *s_pl,
-                                           float4 *s_v, int *s_ok)
+template <int MODE, bool SOFT>
+__device__ __forceinline__ void ens_b_item(const EnsArgs &ea, int c, int k, FShared &sh)
 {
+    constexpr int NT = kEnsFNT;
     const int tid = threadIdx.x;
     const State &S = ea.s;
     const long long P = S.n;
     const long long o = ea.off[c];
-    const int n = (int)(ea.off[c + 1] - o);
-    if (tid == 0) *s_ok = ens_wait_predicted(ea, c);
-    __syncthreads();
-    if (!*s_ok) return;
-    // Everything phase A wrote in this launch is read past L1 (__ldcg): L1 is
-    // not coherent across SMs, and a line read earlier for a neighbouring
-    // cluster could hold this cluster's records from before they were written.
-    const int s0 = k * ea.chunk;
-    const int cnt = min(ea.chunk, __ldcg(&ea.na[c]) - s0);
-    int g = 1;
-    while (g < ea.gmax && g * 2 * cnt <= NT) g <<= 1;
-    const int grp = tid / g, lig = tid % g;
-    const bool valid = grp < cnt;
-    const int i = __ldcg(&ea.act[o + s0 + (valid ? grp : 0)]);
-    const float4 ip = __ldcg(&ea.jph[o + i]), il = __ldcg(&ea.jpl[o + i]), iv = __ldcg(&ea.jv[o + i]);
-    const IDS I = make_ids(ip, il, iv);
-    float hi[7] = {0, 0, 0, 0, 0, 0, 0}, lo[7] = {0, 0, 0, 0, 0, 0, 0};
-    for (int jt = 0; jt < n; jt += NT) {
-        __syncthreads();
-        const int j = jt + tid;
-        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-        s_ph[tid] = j < n ? __ldcg(&ea.jph[o + j]) : z;
-        s_pl[tid] = j < n ? __ldcg(&ea.jpl[o + j]) : z;
-        s_v[tid] = j < n ? __ldcg(&ea.jv[o + j]) : z;
-        __syncthreads();
-        const int jc = min(NT, n - jt);
-        // FP32 partials over at most 64 pairs per lane, then TwoSum promotion
-        for (int jb = 0; jb < jc; jb += 64 * g) {
-            const int je = min(jc, jb + 64 * g);
-            float ta[3] = {0, 0, 0}, tk[3] = {0, 0, 0}, tp = 0.0f;
-            for (int jj = jb + lig; jj < je; jj += g)
-                pair_ds_packed<false, true>(s_ph[jj], s_pl[jj], s_v[jj], I, ea.eps2, ta, tk, tp,
-                                            jt + jj, i);
-            const float t7[7] = {ta[0], ta[1], ta[2], tk[0], tk[1], tk[2], tp};
+    const int n = (int)(ea.off[c + 1] - o), na = ea.na[c];
+    const int chunk = ens_chunk(n, na, ea.g), s0 = k * chunk, cnt = min(chunk, na - s0);
+    if (cnt > kEnsFNT / ea.g / ens_ways(n)) ens_sums<kEnsR, SOFT>(ea, o, n, ea.act + o + s0, cnt, sh);
+    else ens_sums<1, SOFT>(ea, o, n, ea.act + o + s0, cnt, sh);
+    if constexpr (MODE == kEnsStep) {
+        // four lanes correct a particle, one axis each; whole warps of particles
+        const int q = tid & 3, ax = q < 3 ? q : 2;
+        const long long tn = ea.tnext[c];
+        for (int u0 = 0; u0 + (tid >> 5) * 8 < cnt; u0 += NT / 4) {
+            const int u = u0 + (tid >> 2), uu = min(u, cnt - 1);
+            const long long gi = o + ea.act[o + s0 + uu];
+            const bool ok = correct_particle_quad(S, gi, P, tn, (double)sh.res[uu][ax] + (double)sh.res[uu][7 + ax],
+                                                  (double)sh.res[uu][3 + ax] + (double)sh.res[uu][10 + ax], ea.eta,
+                                                  ea.level_min, 0, u < cnt);
+            __syncwarp();
+            if (u < cnt && q == 0) {
+                if (!ok) atomicCAS(ea.err, 0, NB_ESTEP);
+                ens_write_mirror(ea, gi);
+            }
+        }
+    } else for (int u = tid; u < cnt; u += NT) {
+        const long long gi = o + ea.act[o + s0 + u];
+        double res[7];
 #pragma unroll
-            for (int cc = 0; cc < 7; ++cc) two_sum_acc(hi[cc], lo[cc], t7[cc]);
+        for (int cc = 0; cc < 7; ++cc) res[cc] = (double)sh.res[u][cc] + (double)sh.res[u][7 + cc];
+        if constexpr (MODE == kEnsForce) {
+#pragma unroll
+            for (int cc = 0; cc < 3; ++cc) {
+                ea.out_acc[3 * gi + cc] = res[cc];
+                ea.out_jerk[3 * gi + cc] = res[3 + cc];
+            }
+            ea.out_pot[gi] = res[6];
+        } else {
+#pragma unroll
+            for (int cc = 0; cc < 3; ++cc) {
+                S.a[cc * P + gi] = res[cc];
+                S.k[cc * P + gi] = res[3 + cc];
+            }
+            S.t[gi] = 0;
+            int lv;
+            if (!level_of(initial_dt(res, res + 3, ea.eta_init), ea.level_min, lv)) {
+                atomicCAS(ea.err, 0, NB_ESTEP);
+                lv = kTickBits;
+            }
+            S.lev[gi] = lv;
         }
     }
-    for (int sh = 1; sh < g; sh <<= 1) {
-#pragma unroll
-        for (int cc = 0; cc < 7; ++cc) {
-            const float h2 = __shfl_xor_sync(0xffffffffu, hi[cc], sh);
-            const float l2 = __shfl_xor_sync(0xffffffffu, lo[cc], sh);
-            ds_add(hi[cc], lo[cc], h2, l2);
-        }
-    }
-    double res[7];
-#pragma unroll
-    for (int cc = 0; cc < 7; ++cc) res[cc] = (double)hi[cc] + (double)lo[cc];
-    const long long gi = o + i;
-    if (MODE == kEnsStep && g >= 4) {
-        // every lane of the group holds the sums: its first four lanes correct
-        // the particle together (the same FP64 operations as one lane would);
-        // the CTA's other lanes run along inactive, as the quads need
-        const int qd = lig & 3;
-        const bool active = valid && lig < 4;
-        const bool ok = correct_particle_quad(S, gi, P, __ldcg(&ea.tnext[c]),
-                                              qd == 0 ? res[0] : (qd == 1 ? res[1] : res[2]),
-                                              qd == 0 ? res[3] : (qd == 1 ? res[4] : res[5]), ea.eta,
-                                              ea.level_min, 0, active);
-        __syncwarp();
-        if (active && qd == 0) {
-            if (!ok) atomicCAS(ea.err, 0, NB_ESTEP);
-            ens_write_mirror(ea, gi);
-        }
-        return;
-    }
-    if (!valid || lig != 0) return;
-    if (MODE == kEnsForce) {
-#pragma unroll
-        for (int cc = 0; cc < 3; ++cc) {
-            ea.out_acc[3 * gi + cc] = res[cc];
-            ea.out_jerk[3 * gi + cc] = res[3 + cc];
-        }
-        ea.out_pot[gi] = res[6];
-        return;
-    }
-    if (MODE == kEnsInit) {
-#pragma unroll
-        for (int cc = 0; cc < 3; ++cc) {
-            S.a[cc * P + gi] = res[cc];
-            S.k[cc * P + gi] = res[3 + cc];
-        }
-        S.t[gi] = 0;
-        int lv;
-        if (!level_of(initial_dt(res, res + 3, ea.eta_init), ea.level_min, lv)) {
-            atomicCAS(ea.err, 0, NB_ESTEP);
-            lv = kTickBits;
-        }
-        S.lev[gi] = lv;
-        return;
-    }
-    // corrector and new step (the single-system corrector's arithmetic)
-    const double ap[3] = {res[0], res[1], res[2]}, kp[3] = {res[3], res[4], res[5]};
-    if (!correct_particle(S, gi, P, __ldcg(&ea.tnext[c]), ap, kp, ea.eta, ea.level_min, 0))
-        atomicCAS(ea.err, 0, NB_ESTEP);
-    ens_write_mirror(ea, gi);
 }
 
-// One ensemble block step (or start-up, or force-only pass): phase A over the
-// clusters, then phase B over the queue.
-template <int NT, int MODE>
-__global__ void __launch_bounds__(NT) k_ens_step(EnsArgs ea)
+// The force items, the longest clusters' first.
+template <int MODE, bool SOFT>
+__global__ void __launch_bounds__(kEnsFNT, 4) k_ens_force(EnsArgs ea)
 {
-    __shared__ long long s_red[NT / 32];
-    __shared__ int s_wtot[NT / 32];
-    __shared__ float4 s_ph[NT], s_pl[NT], s_v[NT];
-    __shared__ int s_q, s_c, s_k, s_ok;
-    const int tid = threadIdx.x;
+    __shared__ FShared s;
+    int len[kEnsClasses];
+#pragma unroll
+    for (int cls = 0; cls < kEnsClasses; ++cls) len[cls] = ea.work[2 + cls];
+    int it = blockIdx.x;
     for (;;) {
-        if (tid == 0) s_q = atomicAdd(ea.work, 1);
-        __syncthreads();
-        const int q = s_q;
-        __syncthreads();
-        if (q >= ea.C) break;
-        ens_a_cluster<NT, MODE>(ea, q, s_red, s_wtot);
-        __syncthreads();
-        if (tid == 0) {
-            __threadfence();
-            atomicAdd(ea.a_done, 1);
+        int at = it, slot = -1;
+#pragma unroll
+        for (int cls = 0; cls < kEnsClasses; ++cls) {
+            if (slot < 0 && at < len[cls]) slot = ea.qbase[cls] + at;
+            at -= len[cls];
         }
+        if (slot < 0) break;
+        if (threadIdx.x == 0) s.it = (int)gridDim.x + atomicAdd(&ea.work[0], 1);
+        const int2 f = ea.queue[slot];
+        ens_b_item<MODE, SOFT>(ea, f.x, f.y, s);
+        __syncthreads();
+        it = s.it;
+        __syncthreads();
     }
-    for (;;) {
-        if (tid == 0) {
-            int c = -1, k = 0;
-            const int it = atomicAdd(ea.work_b, 1);
-            if (!ens_take_item(ea, it, c, k)) c = -1;
-            s_c = c;
-            s_k = k;
+    // the last CTA leaves the counters at 0
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(&ea.work[1], 1) == (int)gridDim.x - 1) {
+            __threadfence();
+            for (int q = 0; q < 2 + kEnsClasses; ++q) ea.work[q] = 0;
         }
-        __syncthreads();
-        const int c = s_c, k = s_k;
-        __syncthreads();
-        if (c < 0) break;
-        if (k < 0)
-            ens_predict_chunk<NT, MODE>(ea, c, -1 - k);
-        else
-            ens_b_item<NT, MODE>(ea, c, k, s_ph, s_pl, s_v, &s_ok);
     }
 }
 
@@ -601,12 +667,13 @@ struct nb_ens {
     double *d_x = nullptr, *d_v = nullptr, *d_a = nullptr, *d_k = nullptr, *d_m = nullptr;
     long long *d_t = nullptr;
     int *d_lev = nullptr;
-    int *d_work = nullptr, *d_done = nullptr, *d_err = nullptr;  // d_work: [4] counters A, B, queue, A done
+    int *d_work = nullptr, *d_done = nullptr, *d_err = nullptr;  // d_work: [2 + kEnsClasses] counters
     float4 *d_jph = nullptr, *d_jpl = nullptr, *d_jv = nullptr;
     float4 *d_mirror = nullptr;  // [5 P]: x_hi + m, x_lo, v, a, k in single precision
-    int *d_act = nullptr, *d_na = nullptr, *d_qc = nullptr, *d_qk = nullptr, *d_pred = nullptr;
+    int *d_act = nullptr, *d_na = nullptr;
+    int2 *d_queue = nullptr, *d_pitem = nullptr;
+    int npitem = 0, qbase[kEnsClasses] = {};
     long long *d_tnext = nullptr;
-    long long qcap = 0;
     long long *d_steps = nullptr, *d_inter = nullptr;
     double *d_stage = nullptr;   // [7 P] host I/O staging
     int *d_item = nullptr;       // [C + 1] first pair tile of each cluster (energies)
@@ -614,9 +681,9 @@ struct nb_ens {
     double *d_backup = nullptr;  // state copy for tuning
     long long *d_tbak = nullptr;
     int *d_lbak = nullptr;
-    int nt = 256, gmax = 8;      // threads per CTA and lane-group cap (tunable); items of nt / gmax
+    int nt = 256, gmax = 8;      // order of the sums (tunable): gmax lanes, blocks of min(64 gmax, nt) j
     long long t_end = LLONG_MAX;
-    cudaGraphExec_t graph = nullptr;
+    cudaGraphExec_t graph = nullptr, graph_n = nullptr;   // one step, kEnsGraphSteps of them
     int graph_nt = 0, graph_gmax = 0;
     long long graph_tend = -1;
     long long launches = 0;
@@ -666,16 +733,12 @@ EnsArgs ens_args(nb_ens *e)
     a.eta_init = e->o.eta_init;
     a.level_min = e->o.level_min;
     a.t_end = e->t_end;
-    a.gmax = e->gmax;
-    a.chunk = e->nt / e->gmax;  // every full item uses gmax lanes per particle
+    a.g = e->gmax;
+    a.sb = std::min(64 * e->gmax, e->nt);
     a.work = e->d_work;
-    a.work_b = e->d_work + 1;
-    a.qlen = e->d_work + 2;
-    a.a_done = e->d_work + 3;
-    a.pred_left = e->d_pred;
-    a.qc = e->d_qc;
-    a.qcap = (int)(e->P + e->C);
-    a.qk = e->d_qk;
+    a.queue = e->d_queue;
+    a.pitem = e->d_pitem;
+    for (int k = 0; k < kEnsClasses; ++k) a.qbase[k] = e->qbase[k];
     a.jph = e->d_jph;
     a.jpl = e->d_jpl;
     a.jv = e->d_jv;
@@ -694,47 +757,18 @@ EnsArgs ens_args(nb_ens *e)
     return a;
 }
 
-// Resident CTAs per SM of the fused kernel for this configuration.
-template <int NT, int MODE>
-int ens_blocks_per_sm()
-{
-    static int bps = 0;
-    if (bps == 0 &&
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_ens_step<NT, MODE>, NT, 0) != cudaSuccess)
-        bps = 1;
-    return bps > 0 ? bps : 1;
-}
-
-// One cooperative launch over all resident CTAs (CTAs wait on each other's
-// phase A, so they must all be resident).
-template <int NT, int MODE>
-cudaError_t launch_step_t(nb_ens *e, const EnsArgs &a)
-{
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    cfg.gridDim = dim3(e->sms * ens_blocks_per_sm<NT, MODE>());
-    cfg.blockDim = dim3(NT);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = e->st;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_ens_step<NT, MODE>, a);
-}
-
-// One pass: counters zeroed, then the fused launch.
+// One pass: schedule (with the small clusters' prediction), prediction of the
+// larger ones, force and correction.
 template <int MODE>
 int enqueue_ens(nb_ens *e, const EnsArgs &a)
 {
-    ECK(cudaMemsetAsync(e->d_work, 0, 4 * sizeof(int), e->st));
-    cudaError_t ce;
-    switch (e->nt) {
-    case 128: ce = launch_step_t<128, MODE>(e, a); break;
-    case 512: ce = launch_step_t<512, MODE>(e, a); break;
-    default: ce = launch_step_t<256, MODE>(e, a); break;
-    }
-    if (ce != cudaSuccess) return efail(e, NB_ECUDA, "ensemble launch: %s", cudaGetErrorString(ce));
+    int bps = 0;
+    const auto force = a.eps2 > 0.0f ? k_ens_force<MODE, true> : k_ens_force<MODE, false>;
+    ECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, force, kEnsFNT, 0));
+    k_ens_sched<MODE><<<e->C, kEnsANT, 0, e->st>>>(a);
+    if (e->npitem) k_ens_predict<MODE><<<e->npitem, kEnsPNT, 0, e->st>>>(a);
+    force<<<e->sms * std::max(1, bps), kEnsFNT, 0, e->st>>>(a);
+    ECK(cudaGetLastError());
     e->launches += 1;
     return NB_OK;
 }
@@ -759,12 +793,8 @@ int ens_sync(nb_ens *e)
     ECK(cudaStreamSynchronize(e->st));
     ECK(cudaGetLastError());
     if (h_err) {
-        // an aborted launch may leave items unconsumed: mark every item not ready
-        ECK(cudaMemsetAsync(e->d_qc, 0xff, sizeof(int) * (e->P + e->C), e->st));
         ECK(cudaMemsetAsync(e->d_err, 0, sizeof(int), e->st));
         ECK(cudaStreamSynchronize(e->st));
-        if (h_err == NB_ETIMEOUT)
-            return efail(e, NB_ETIMEOUT, "an ensemble launch waited too long for a cluster's block");
         return efail(e, h_err, "a new time step fell below 2^-40 in some cluster");
     }
     return NB_OK;
@@ -782,15 +812,46 @@ int ealloc(nb_ens *e, T **p, long long count)
     return NB_OK;
 }
 
+void drop_graphs(nb_ens *e)
+{
+    if (e->graph) cudaGraphExecDestroy(e->graph);
+    if (e->graph_n) cudaGraphExecDestroy(e->graph_n);
+    e->graph = e->graph_n = nullptr;
+}
+
+// `steps` ensemble steps as one graph.
+int capture_steps(nb_ens *e, int steps, cudaGraphExec_t *out)
+{
+    cudaGraph_t g;
+    const long long l0 = e->launches;
+    ECK(cudaStreamBeginCapture(e->st, cudaStreamCaptureModeThreadLocal));
+    int rc = NB_OK;
+    for (int q = 0; q < steps && !rc; ++q) rc = enqueue_ens_step(e);
+    e->launches = l0;
+    cudaError_t ce = cudaStreamEndCapture(e->st, &g);
+    if (rc) {
+        if (ce == cudaSuccess && g) cudaGraphDestroy(g);
+        return rc;
+    }
+    if (ce != cudaSuccess) return efail(e, NB_ECUDA, "graph capture: %s", cudaGetErrorString(ce));
+    ce = cudaGraphInstantiate(out, g, 0);
+    cudaGraphDestroy(g);
+    if (ce != cudaSuccess) {
+        *out = nullptr;
+        return efail(e, NB_ECUDA, "graph instantiate: %s", cudaGetErrorString(ce));
+    }
+    return NB_OK;
+}
+
 void ens_release(nb_ens *e)
 {
     if (e->st) cudaStreamSynchronize(e->st);
-    if (e->graph) cudaGraphExecDestroy(e->graph);
+    drop_graphs(e);
     void *ptrs[] = {e->d_off, e->d_order, e->d_x, e->d_v, e->d_a, e->d_k, e->d_m, e->d_t,
                     e->d_lev, e->d_work, e->d_done, e->d_err, e->d_steps, e->d_inter,
                     e->d_stage, e->d_backup, e->d_tbak, e->d_lbak, e->d_jph, e->d_jpl, e->d_jv,
                     e->d_mirror,
-                    e->d_act, e->d_na, e->d_qc, e->d_qk, e->d_tnext, e->d_pred, e->d_item};
+                    e->d_act, e->d_na, e->d_queue, e->d_pitem, e->d_tnext, e->d_item};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (e->own_stream && e->st) cudaStreamDestroy(e->st);
@@ -834,7 +895,15 @@ int ens_init_impl(nb_ens *e, int32_t C, const int64_t *off, const double *m, con
         if (m[i] < 0.0) return efail(e, NB_EINVAL, "negative mass");
     std::stable_sort(sizes.begin(), sizes.end());
     std::vector<int> order(C);
-    for (int q = 0; q < C; ++q) order[q] = sizes[q].second;
+    // a cluster has at most n force items: the classes' parts of the queue
+    std::vector<int2> pitem;
+    for (int q = 0; q < C; ++q) {
+        const int c = order[q] = sizes[q].second, nc = (int)-sizes[q].first;
+        for (int k = ens_class(nc) + 1; k < kEnsClasses; ++k) e->qbase[k] += nc;
+        if (nc > kEnsPredChunk)
+            for (int p = 0; p * kEnsPredChunk < nc; ++p) pitem.push_back(make_int2(c, p));
+    }
+    e->npitem = (int)pitem.size();
 
     e->C = C;
     e->P = P;
@@ -854,13 +923,13 @@ int ens_init_impl(nb_ens *e, int32_t C, const int64_t *off, const double *m, con
         (rc = ealloc(e, &e->d_x, 3 * P)) || (rc = ealloc(e, &e->d_v, 3 * P)) ||
         (rc = ealloc(e, &e->d_a, 3 * P)) || (rc = ealloc(e, &e->d_k, 3 * P)) ||
         (rc = ealloc(e, &e->d_m, P)) || (rc = ealloc(e, &e->d_t, P)) || (rc = ealloc(e, &e->d_lev, P)) ||
-        (rc = ealloc(e, &e->d_work, 4)) || (rc = ealloc(e, &e->d_done, C)) || (rc = ealloc(e, &e->d_err, 1)) ||
+        (rc = ealloc(e, &e->d_work, 2 + kEnsClasses)) || (rc = ealloc(e, &e->d_done, C)) || (rc = ealloc(e, &e->d_err, 1)) ||
         (rc = ealloc(e, &e->d_steps, C)) || (rc = ealloc(e, &e->d_inter, C)) ||
         (rc = ealloc(e, &e->d_stage, 7 * P)) || (rc = ealloc(e, &e->d_jph, P)) ||
         (rc = ealloc(e, &e->d_jpl, P)) || (rc = ealloc(e, &e->d_jv, P)) ||
         (rc = ealloc(e, &e->d_act, P)) || (rc = ealloc(e, &e->d_na, C)) ||
-        (rc = ealloc(e, &e->d_tnext, C)) || (rc = ealloc(e, &e->d_qc, P + C)) ||
-        (rc = ealloc(e, &e->d_qk, P + C)) || (rc = ealloc(e, &e->d_pred, C)) ||
+        (rc = ealloc(e, &e->d_tnext, C)) || (rc = ealloc(e, &e->d_queue, P)) ||
+        (rc = ealloc(e, &e->d_pitem, std::max<long long>(1, (long long)pitem.size()))) ||
         (rc = ealloc(e, &e->d_mirror, 5 * P)) || (rc = ealloc(e, &e->d_item, C + 1)))
         return rc;
     // at most one tile per particle, so the tile sums fit the staging buffer
@@ -891,8 +960,9 @@ int ens_init_impl(nb_ens *e, int32_t C, const int64_t *off, const double *m, con
     ECK(cudaMemsetAsync(e->d_err, 0, sizeof(int), e->st));
     ECK(cudaMemsetAsync(e->d_steps, 0, sizeof(long long) * C, e->st));
     ECK(cudaMemsetAsync(e->d_inter, 0, sizeof(long long) * C, e->st));
-    ECK(cudaMemsetAsync(e->d_qc, 0xff, sizeof(int) * (P + C), e->st));  // no item ready
-    ECK(cudaMemsetAsync(e->d_pred, 0, sizeof(int) * C, e->st));
+    if (!pitem.empty())
+        ECK(cudaMemcpyAsync(e->d_pitem, pitem.data(), sizeof(int2) * pitem.size(), cudaMemcpyHostToDevice, e->st));
+    ECK(cudaMemsetAsync(e->d_work, 0, sizeof(int) * (2 + kEnsClasses), e->st));
     // start-up: force on every particle of every cluster, initial steps
     if ((rc = enqueue_ens<kEnsInit>(e, ens_args(e)))) return rc;
     ECK(cudaGetLastError());
@@ -964,29 +1034,14 @@ int nb_ens_run(nb_ens *e, double t_end, int64_t max_launches, int64_t *launches_
         ECK(cudaMemsetAsync(e->d_done, 0, sizeof(int) * e->C, e->st));
         e->t_end = te;
     }
-    // capture one ensemble step (memset + persistent launch) into a graph
+    // one ensemble step, and a stretch of them (a graph's start costs about 5 us), as graphs
     if (!e->graph || e->graph_nt != e->nt || e->graph_gmax != e->gmax || e->graph_tend != te) {
-        if (e->graph) cudaGraphExecDestroy(e->graph);
-        e->graph = nullptr;
-        int rc0 = 0;
-        // a first launch of this configuration outside capture (occupancy query)
-        EnsArgs probe = ens_args(e);
-        probe.C = 0;
-        if ((rc0 = enqueue_ens<kEnsStep>(e, probe))) return rc0;
-        ECK(cudaStreamSynchronize(e->st));
-        cudaGraph_t g;
-        ECK(cudaStreamBeginCapture(e->st, cudaStreamCaptureModeThreadLocal));
-        const long long l0 = e->launches;
-        const int rc = enqueue_ens_step(e);
-        e->launches = l0;
-        cudaError_t ce = cudaStreamEndCapture(e->st, &g);
-        if (rc) return rc;
-        if (ce != cudaSuccess) return efail(e, NB_ECUDA, "graph capture: %s", cudaGetErrorString(ce));
-        ce = cudaGraphInstantiate(&e->graph, g, 0);
-        cudaGraphDestroy(g);
-        if (ce != cudaSuccess) {
-            e->graph = nullptr;
-            return efail(e, NB_ECUDA, "graph instantiate: %s", cudaGetErrorString(ce));
+        drop_graphs(e);
+        int rc = capture_steps(e, 1, &e->graph);
+        if (!rc) rc = capture_steps(e, kEnsGraphSteps, &e->graph_n);
+        if (rc) {
+            drop_graphs(e);
+            return rc;
         }
         e->graph_nt = e->nt;
         e->graph_gmax = e->gmax;
@@ -998,7 +1053,9 @@ int nb_ens_run(nb_ens *e, double t_end, int64_t max_launches, int64_t *launches_
     ECK(cudaMemcpyAsync(inter0.data(), e->d_inter, sizeof(long long) * e->C, cudaMemcpyDeviceToHost, e->st));
     while (n < max_launches) {
         const long long k = std::min<long long>(32, max_launches - n);
-        for (long long q = 0; q < k; ++q) ECK(cudaGraphLaunch(e->graph, e->st));
+        long long q = 0;
+        for (; q + kEnsGraphSteps <= k; q += kEnsGraphSteps) ECK(cudaGraphLaunch(e->graph_n, e->st));
+        for (; q < k; ++q) ECK(cudaGraphLaunch(e->graph, e->st));
         n += k;
         e->launches += k;
         ECK(cudaMemcpyAsync(done.data(), e->d_done, sizeof(int) * e->C, cudaMemcpyDeviceToHost, e->st));
@@ -1062,7 +1119,7 @@ int nb_ens_tune(nb_ens *e, int launches_per_candidate, int *threads_out, int *gm
             e->nt = cand_nt[a];
             e->gmax = cand_g[b];
             if ((rc = save(true))) return rc;
-            if ((rc = enqueue_ens_step(e))) return rc;  // warm-up (and shared-memory set-up)
+            if ((rc = enqueue_ens_step(e))) return rc;  // warm-up
             ECK(cudaEventRecord(e0, e->st));
             for (int q = 0; q < launches_per_candidate; ++q)
                 if ((rc = enqueue_ens_step(e))) return rc;

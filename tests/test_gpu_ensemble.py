@@ -236,3 +236,35 @@ def test_energies_of_all_cluster_sizes(nb):
         W, T = -np.sum(rows), 0.5 * np.sum(mc * np.sum(vc * vc, axis=1))
         assert abs(ep[c] - W) <= 1e-13 * abs(W), (n, ep[c], W)
         assert abs(ek[c] - T) <= 1e-13 * T, (n, ek[c], T)
+
+
+@pytest.mark.parametrize("eps", [EPS, 0.0])
+@pytest.mark.parametrize("threads,gmax", [(256, 8), (128, 1), (256, 4), (512, 32)])
+def test_item_shapes(nb, threads, gmax, eps):
+    # sizes at the edges of tiles, sum blocks, prediction chunks and of the two-way
+    # items; force against the oracle, and a cluster alone steps as among the others
+    cl = [plummer(n, 900 + n, exact_virial_max=0)
+          for n in (2, 17, 64, 65, 127, 129, 256, 257, 511, 513, 1023, 2047, 2048, 2049, 2305, 4095)]
+    off, m, x, v = _flatten(cl)
+
+    def steps(args, count):
+        e = nb.Ensemble(*args, eps)
+        try:
+            e.nb_ens_configure(threads, gmax)
+            f = e.nb_ens_force()
+            for _ in range(count):
+                e.nb_ens_step()
+            return f, e.nb_ens_get_state()
+        finally:
+            e.nb_ens_free()
+
+    f, st = steps((off, m, x, v), 12)
+    for c, (mc, xc, vc) in enumerate(cl):
+        s, t = off[c], off[c + 1]
+        ref = oracle.force(mc, xc, vc, eps, nthreads=8)
+        mags = pair_magnitudes(mc, xc, vc, eps, np.arange(t - s))
+        assert_force_close([a[s:t] for a in f], ref, mags, TOL_DS, "n=%d" % (t - s))
+        if t - s in (65, 513, 2049):
+            f1, s1 = steps((np.array([0, t - s]), mc, xc, vc), 12)
+            assert all(np.array_equal(a, b[s:t]) for a, b in zip(f1, f))
+            assert all(np.array_equal(s1[k], st[k][s:t]) for k in ("x", "v", "a", "k", "t", "level"))
