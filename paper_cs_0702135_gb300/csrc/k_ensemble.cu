@@ -1037,12 +1037,8 @@ int nb_ens_run(nb_ens *e, double t_end, int64_t max_launches, int64_t *launches_
     // one ensemble step, and a stretch of them (a graph's start costs about 5 us), as graphs
     if (!e->graph || e->graph_nt != e->nt || e->graph_gmax != e->gmax || e->graph_tend != te) {
         drop_graphs(e);
-        int rc = capture_steps(e, 1, &e->graph);
-        if (!rc) rc = capture_steps(e, kEnsGraphSteps, &e->graph_n);
-        if (rc) {
-            drop_graphs(e);
-            return rc;
-        }
+        const int rc = capture_steps(e, 1, &e->graph);
+        if (rc) return rc;
         e->graph_nt = e->nt;
         e->graph_gmax = e->gmax;
         e->graph_tend = te;
@@ -1054,7 +1050,11 @@ int nb_ens_run(nb_ens *e, double t_end, int64_t max_launches, int64_t *launches_
     while (n < max_launches) {
         const long long k = std::min<long long>(32, max_launches - n);
         long long q = 0;
-        for (; q + kEnsGraphSteps <= k; q += kEnsGraphSteps) ECK(cudaGraphLaunch(e->graph_n, e->st));
+        if (k == 32) {   // a longer graph only where its capture pays
+            const int rc = e->graph_n ? NB_OK : capture_steps(e, kEnsGraphSteps, &e->graph_n);
+            if (rc) return rc;
+            for (; q < k; q += kEnsGraphSteps) ECK(cudaGraphLaunch(e->graph_n, e->st));
+        }
         for (; q < k; ++q) ECK(cudaGraphLaunch(e->graph, e->st));
         n += k;
         e->launches += k;
