@@ -66,11 +66,12 @@ extern "C" {
  *                       largest mass, the largest |vx|+|vy|+|vz| and eps, so
  *                       that no term or sum can overflow; requires eps^2 to be
  *                       a normal single-precision number (eps >~ 1.1e-19).
- *   NB_SUM_FP32         FP32 running sum over j in index order, one thread per
- *                       active particle (a single-precision GPU summation).
+ *   NB_SUM_FP32         FP32 running sum over j in index order (a single-precision
+ *                       GPU's summation).
  *   NB_SUM_FP32_SORTED  FP32 running sum with the smallest pair force
  *                       |m_j dx / r^3| first (ties in index order), after a
- *                       per-particle sort; memory: 16 n bytes per resident CTA.
+ *                       per-particle sort (in shared memory unless thousands of
+ *                       keys share a bin); memory: 16 n bytes per resident CTA.
  * force_mode and split_j only apply to NB_SUM_COMPENSATED and NB_SUM_FIXED
  * (whose results split_j does not change).
  */
@@ -196,22 +197,22 @@ int nb_step(nb_ctx *ctx, double *t_out, int32_t *n_active_out);
  * Block steps until every particle has reached t_end (which must be a multiple
  * of the largest step so that all particles meet there), or max_steps steps.
  * For n <= 16384 with precision NB_DS and summation NB_SUM_COMPENSATED or
- * NB_SUM_FIXED the whole loop runs in one persistent launch (up to 128 CTAs
- * of 32 to 128 particles, grid barriers between the stages of a step, no host
- * synchronisation); otherwise, or with nb_opts.flags & NB_RUN_GRAPH, each step
- * is replayed from a captured CUDA graph of the per-stage kernels.  The two
+ * NB_SUM_FIXED the whole loop runs in one persistent launch per 131072 steps
+ * (CTAs of at least 32 particles that pass tagged records to each other, no host
+ * synchronisation); otherwise, or with nb_opts.flags & NB_RUN_GRAPH, the steps
+ * are replayed from captured CUDA graphs of the per-stage kernels.  The two
  * forms take the same steps with the same arithmetic except the order in
  * which the compensated sums add their partials (fixed-point sums are exact:
  * both forms give the same bits).  Outputs (may be NULL): steps taken,
  * interactions (sum of n_active (n - 1)).  Errors: NB_EINVAL, NB_ESTEP,
- * NB_ETIMEOUT (a grid barrier of the persistent launch waited ~2 s), NB_ECUDA.
+ * NB_ETIMEOUT (a CTA of the persistent launch waited ~2 s for another), NB_ECUDA.
  */
 int nb_run(nb_ctx *ctx, double t_end, int64_t max_steps, int64_t *steps_out,
            int64_t *interactions_out);
 
 /*
  * Self-test of failure detection (the paper has no counterpart): one device
- * thread runs the bounded wait that the persistent nb_run's grid barriers use,
+ * thread runs the bounded wait of the persistent nb_run's step flags,
  * on a counter that nothing increments, with a limit of about `ms`
  * milliseconds of SM clock.  The wait runs out, the kernel raises NB_ETIMEOUT
  * in the context's error word and returns, and the call reports it; the

@@ -84,7 +84,7 @@ constexpr int kJparMaxActive64 = 32;   // automatic mode, FP64
 #endif
 constexpr int kIparSmallUnroll = NB_U1;  // its j unrolling (2, 4, 8: 169, 173, 171 us for 1820 active on 65536)
 constexpr int kIparSmallR = 1;      // i per thread of the small-block DS i-parallel kernel
-constexpr int kSmallMaxActive = 1024;  // automatic mode: small-block kernel considered up to this size
+constexpr int kSmallMaxActive = 1024;  // with a forced slice count: small-block kernel considered up to this size
 constexpr int kComp = 7;       // acc xyz, jerk xyz, pot
 // Clocks per j of an i-parallel CTA alone on its SM, and of each CTA with the SM full, for the
 // four-i and the one-i kernel, and how many are resident (see fine_cost).
@@ -285,11 +285,10 @@ __host__ __device__ inline bool use_jpar(int na, int jpar_max) { return na <= jp
 
 // Force kernels by block size: j-parallel, small-block i-parallel (one i per
 // thread, blocks of kIparNT i), i-parallel (kIparR i per thread, blocks of
-// kIparNT * kIparR i).  The small-block kernel runs at about three quarters of
-// the other's rate on full blocks, so it serves a block when its padded i
-// count is at most 3/4 of the other's: up to 192, 257..384 and 513..576 active
-// with 64-i and 256-i blocks (measured crossings on 2^16 and 2^20 bodies).
-// small_max <= jpar_max disables it.
+// kIparNT * kIparR i).  Where the rule below on fine plans does not apply (a
+// forced slice count), the small-block kernel serves a block when its padded
+// i count is at most 3/4 of the other's: up to 192, 257..384 and 513..576
+// active with 64-i and 256-i blocks.  small_max <= jpar_max disables it.
 __host__ __device__ inline bool small_pays(int na)
 {
     const long long s = (long long)cdiv(na, kIparNT) * kIparNT;
