@@ -39,6 +39,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "nb_device.cuh"
+#include "nb_int64.cuh"
 
 namespace nbk {
 namespace {
@@ -513,12 +514,12 @@ __global__ void __launch_bounds__(kEnsFNT, 4) k_ens_force(EnsArgs ea)
 // is synchronised): kinetic from FP64 velocities, potential as the FP64 pair
 // sum -sum_{i<j} m_i m_j / sqrt(r^2 + eps^2), in a fixed order.
 //
-// The pair sum is bound by the FP64 pipe (2 lanes a clock per SM), so it is cut
-// into tiles of 128 x 128 pairs (ti <= tj) of every cluster, one CTA each, for
-// all SMs to share, and 1/sqrt takes five FP64 operations on an FP32 seed
-// instead of a square root and a division (~14): per pair 12.  256 clusters of
-// 32..4096 (2.2e8 pairs): 6.1 ms with the copies; one CTA per cluster with the square root
-// and the division waited for the largest cluster, 96 ms.
+// The pair sum is cut into tiles of 128 x 128 pairs (ti <= tj) of every cluster,
+// one CTA each, for all SMs to share.  A pair's m_j / r is formed on the integer
+// pipes (nb_int64.cuh) with one FP64 addition; a tile with a value out of that
+// range takes 12 FP64 operations a pair, 1/sqrt being five on an FP32 seed.
+// 256 clusters of 32..4096 (2.7e8 pairs), with the copies: 1.3 ms; 6.1 with every
+// tile in FP64; 96 with one CTA per cluster, a square root and a division.
 
 constexpr int kEnTile = 128;
 
@@ -546,7 +547,14 @@ __device__ __forceinline__ double rsqrt_pair(double x)
 // Potential of pair tile blockIdx.x: item[] holds each cluster's first tile.
 __global__ void __launch_bounds__(kEnTile) k_ens_pairs(EnsArgs ea, const int *item, double eps2, double *part)
 {
-    __shared__ double4_32a s_j[kEnTile];
+    __shared__ union JTile {
+        double4_32a f;
+        struct {
+            long long m[4];
+            unsigned e;
+        } i;
+        __device__ JTile() {}
+    } s_j[kEnTile];
     __shared__ double s_red[kEnTile / 32];
     const State &S = ea.s;
     const long long P = S.n;
@@ -565,29 +573,67 @@ __global__ void __launch_bounds__(kEnTile) k_ens_pairs(EnsArgs ea, const int *it
     const long long o = ea.off[c];
     const int n = (int)(ea.off[c + 1] - o);
     const int i0 = ti * kEnTile + warp * 32, i = i0 + lane, j0 = tj * kEnTile, jc = min(kEnTile, n - j0);
+    double4_32a pj = make_double4_32a(0., 0., 0., 0.), pi = pj;
     if (tid < jc) {
         const long long gj = o + j0 + tid;
-        s_j[tid] = make_double4_32a(S.x[gj], S.x[P + gj], S.x[2 * P + gj], S.m[gj]);
+        pj = make_double4_32a(S.x[gj], S.x[P + gj], S.x[2 * P + gj], S.m[gj]);
     }
-    __syncthreads();
-    double row = 0.0, mi = 0.0;
     if (i0 < n) {
         const long long gi = o + min(i, n - 1);
-        const double xi = S.x[gi], yi = S.x[P + gi], zi = S.x[2 * P + gi];
-        mi = S.m[gi];
-        // on the diagonal a warp starts past its own first particle
-#pragma unroll 4
-        for (int q = ti == tj ? warp * 32 + 1 : 0; q < jc; ++q) {
-            const double4_32a p = s_j[q];
-            const double dx = p.x - xi, dy = p.y - yi, dz = p.z - zi;
-            const double r2 = fma(dx, dx, fma(dy, dy, fma(dz, dz, eps2)));
-            const double y = rsqrt_pair(r2);
-            // i < j holds off the diagonal (lanes past the end are dropped
-            // below); a pair left out may be infinite, so its term is not formed
-            if (j0 + q > i) row = fma(p.w, y, row);
-        }
+        pi = make_double4_32a(S.x[gi], S.x[P + gi], S.x[2 * P + gi], S.m[gi]);
     }
-    row = i < n ? mi * row : 0.0;   // a particle past the end
+    const auto in_range = [](const double4_32a &p) {
+        return i64::in_range(p.x) && i64::in_range(p.y) && i64::in_range(p.z) && i64::in_range(p.w);
+    };
+    double row = 0.0;
+    // on the diagonal a warp starts past its own first particle
+    const int q0 = ti == tj ? warp * 32 + 1 : 0;
+    if (__syncthreads_and(i64::eps2_in_range(eps2) && in_range(pi) && in_range(pj))) {
+        const i64::Fix x = i64::to_fix(pj.x), y = i64::to_fix(pj.y), z = i64::to_fix(pj.z);
+        const i64::Num m = i64::to_num(pj.w);
+        s_j[tid].i.m[0] = x.m;
+        s_j[tid].i.m[1] = y.m;
+        s_j[tid].i.m[2] = z.m;
+        s_j[tid].i.m[3] = (long long)m.m;
+        s_j[tid].i.e = (unsigned)(x.e & 255) | (unsigned)(y.e & 255) << 8 | (unsigned)(z.e & 255) << 16 |
+                       (unsigned)m.e << 24;
+        __syncthreads();
+        const i64::Eps eps = i64::make_eps(eps2);
+        const i64::Fix I[3] = {i64::to_fix(pi.x), i64::to_fix(pi.y), i64::to_fix(pi.z)};
+        if (i0 < n)
+#pragma unroll 1
+            for (int q = q0; q < jc; ++q) {
+                const unsigned e = s_j[q].i.e;
+                i64::Num D[3], mj;
+#pragma unroll
+                for (int cc = 0; cc < 3; ++cc) {
+                    i64::Fix X;
+                    X.m = s_j[q].i.m[cc];
+                    X.e = i64::signed_byte(e, cc);
+                    double d;
+                    D[cc] = i64::diff(X, I[cc], d);
+                }
+                mj.m = (unsigned long long)s_j[q].i.m[3];
+                mj.e = i64::signed_byte(e, 3);
+                mj.neg = false;
+                const double v = i64::pair_potential(D, mj, eps);
+                row += j0 + q > i ? v : 0.0;
+            }
+    } else {
+        s_j[tid].f = pj;
+        __syncthreads();
+        if (i0 < n)
+#pragma unroll 4
+            for (int q = q0; q < jc; ++q) {
+                const double4_32a p = s_j[q].f;
+                const double dx = p.x - pi.x, dy = p.y - pi.y, dz = p.z - pi.z;
+                const double y = rsqrt_pair(fma(dx, dx, fma(dy, dy, fma(dz, dz, eps2))));
+                // i < j holds off the diagonal (lanes past the end are dropped
+                // below); a pair left out may be infinite, so its term is not formed
+                if (j0 + q > i) row = fma(p.w, y, row);
+            }
+    }
+    row = i < n ? pi.w * row : 0.0;   // a particle past the end
 #pragma unroll
     for (int off = 16; off >= 1; off >>= 1) row += __shfl_xor_sync(0xffffffffu, row, off);
     if (lane == 0) s_red[warp] = row;

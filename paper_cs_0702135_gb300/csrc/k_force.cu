@@ -118,17 +118,16 @@ __device__ __forceinline__ J64Tile tile_of(const double4_32a &p, const double4_3
              (m.neg ? 1u << 31 : 0u);
     return t;
 }
-__device__ __forceinline__ int signed_byte(unsigned w, int k) { return (int)(w << (24 - 8 * k)) >> 24; }
 __device__ __forceinline__ J64I j_of(const J64Tile &t)
 {
     J64I J;
 #pragma unroll
     for (int c = 0; c < 6; ++c) {
         J.x[c].m = t.m[c];
-        J.x[c].e = signed_byte(t.e[c / 4], c % 4);
+        J.x[c].e = i64::signed_byte(t.e[c / 4], c % 4);
     }
     J.m.m = (unsigned long long)t.m[6];
-    J.m.e = signed_byte(t.e[1], 2);
+    J.m.e = i64::signed_byte(t.e[1], 2);
     J.m.neg = (int)t.e[1] < 0;
     return J;
 }

@@ -81,6 +81,8 @@ struct Num {
     bool neg;
 };
 constexpr int kZeroExp = -128;   // exponent kept for a value that is 0
+// Byte k of w as a signed number: exponents in range fit one.
+NB_HD int signed_byte(unsigned w, int k) { return (int)(w << (24 - 8 * k)) >> 24; }
 
 // The values that this arithmetic takes: 0 and 2^-100 <= |x| < 2^100 (a
 // difference of two such values that is not 0 is at least 2^-152, and no
@@ -168,9 +170,8 @@ NB_HD float rsqrt_seed(float f)
 #endif
 }
 
-// m / r, m / r^3 and b = -3 (x . u) / r^2 with r^2 = |x|^2 + eps^2.
-NB_HD void pair_factors(const Num x[3], const Num u[3], const Num &m, const Eps &eps, double &mr, double &mr3,
-                        double &b)
+// 1/r = Y 2^(-63 - h) with r^2 = |x|^2 + eps^2.
+NB_HD u64 inv_dist(const Num x[3], const Eps &eps, int &h)
 {
     // r^2 = S 2^(E - 59), four terms below 2^61 each
     const int E = imax(imax(2 * x[0].e, 2 * x[1].e), imax(2 * x[2].e, eps.e));
@@ -180,15 +181,32 @@ NB_HD void pair_factors(const Num x[3], const Num u[3], const Num &m, const Eps 
     // = f 2^(2 h), F = f 2^61 in [2^61, 2^63): E is even and S at least 2^59
     const bool low = S < (1ULL << 61);
     const u64 F = low ? S << 2 : S;
-    const int h = (E >> 1) + (low ? 0 : 1);
+    h = (E >> 1) + (low ? 0 : 1);
     // y0 = Yi 2^-24 from the SFU, pulled below 1, then y0 (1 + e/2 + 3/8 e^2)
     // with e = 1 - f y0^2 (below 2^-20; the next term is below 2^-62)
     const unsigned Yi = (unsigned)(rsqrt_seed((float)(unsigned)(F >> 31)) * 0x1.fffffcp38f);
     const s64 e = (s64)((1ULL << 60) - mulhi(F, ((u64)Yi * Yi) << 15));   // in 2^-60
     const int e10 = (int)(e >> 10);
     const s64 c = (e >> 1) + ((((s64)e10 * e10) >> 40) * 3 >> 3);
-    const u64 Y = ((u64)Yi << 39) + (u64)(((s64)Yi * c) >> 21);   // 1/sqrt(f) in 2^-63
-    const u64 Z = mulhi(Y, Y) << 1;                               // 1/f in 2^-63
+    return ((u64)Yi << 39) + (u64)(((s64)Yi * c) >> 21);   // 1/sqrt(f) in 2^-63
+}
+
+// m / r.
+NB_HD double pair_potential(const Num x[3], const Num &m, const Eps &eps)
+{
+    int h;
+    const u64 H = mulhi(m.m, inv_dist(x, eps, h)) << 1;
+    const double mr = pack(H, clz32((unsigned)(H >> 32)), m.e - 62 - h, m.neg);
+    return m.m == 0 ? 0.0 : mr;
+}
+
+// m / r, m / r^3 and b = -3 (x . u) / r^2 with r^2 = |x|^2 + eps^2.
+NB_HD void pair_factors(const Num x[3], const Num u[3], const Num &m, const Eps &eps, double &mr, double &mr3,
+                        double &b)
+{
+    int h;
+    const u64 Y = inv_dist(x, eps, h);
+    const u64 Z = mulhi(Y, Y) << 1;   // 1/f in 2^-63, r^2 = f 2^(2 h)
     const u64 H = mulhi(m.m, Y) << 1, T = mulhi(H, Z);
     mr = pack(H, clz32((unsigned)(H >> 32)), m.e - 62 - h, m.neg);
     mr3 = pack(T, clz32((unsigned)(T >> 32)), m.e - 61 - 3 * h, m.neg);

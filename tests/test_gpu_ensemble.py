@@ -268,3 +268,25 @@ def test_item_shapes(nb, threads, gmax, eps):
             f1, s1 = steps((np.array([0, t - s]), mc, xc, vc), 12)
             assert all(np.array_equal(a, b[s:t]) for a, b in zip(f1, f))
             assert all(np.array_equal(s1[k], st[k][s:t]) for k in ("x", "v", "a", "k", "t", "level"))
+
+
+@pytest.mark.parametrize("eps", [EPS, 0.0, 2.0 ** -60])
+@pytest.mark.parametrize("far", [0.0, 2.0 ** 101])
+def test_energies_out_of_range(nb, far, eps):
+    # a tile with a value outside 2^-100..2^100, or such an eps^2, is summed in
+    # FP64, the others on the integer pipes: the bound of the test above for both
+    n = 300
+    rng = np.random.RandomState(23)
+    m, x = rng.uniform(0.5, 2.0, n) / n, rng.normal(size=(n, 3))
+    m[::9] = 0.0
+    x[7, 1] = 0.0
+    if far:
+        x[200, 0] = far
+    v = np.zeros((n, 3))
+    e = nb.Ensemble(np.array([0, n]), m, x, v, eps)
+    try:
+        ek, ep = e.nb_ens_energy()
+    finally:
+        e.nb_ens_free()
+    W = -np.sum([m[i] * np.sum(m[:i] / np.sqrt(np.sum((x[:i] - x[i]) ** 2, axis=1) + eps * eps)) for i in range(1, n)])
+    assert ek[0] == 0.0 and abs(ep[0] - W) <= 1e-13 * abs(W)
