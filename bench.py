@@ -944,8 +944,8 @@ def run_ensemble(args):
     """Batched ensemble: independent Plummer clusters (N log-uniform in
     [32, 4096], Salpeter masses on [0.1, 100], virial ratio uniform in
     [0.3, 0.7], seed 5), eps = 1/256, eta = 0.01, each to t = 1 with its own
-    block steps; one graph-replayed launch per ensemble step, launch
-    configuration from the autotuner.  Compared with per-cluster launches: the
+    block steps; graph-replayed launches, three per ensemble step, sum
+    order from the autotuner.  Compared with per-cluster launches: the
     single-system path (nb_run per cluster), timed on a seeded sample of
     clusters and scaled to all of them."""
     import torch
@@ -1172,7 +1172,7 @@ def run_summation(args):
                           "reduction and combine around it)",
                 "peak_note": "FP32 FMA peak 2 x 128 lanes x %d SMs x 2070 MHz (max SM clock); "
                              "achieved counts 60 flop per interaction although the variant issues "
-                             "about 130 instructions per pair" % sms}
+                             "about 79 instructions per pair" % sms}
     if clocks.get("sm_mhz"):
         roofline["frac_at_measured_clock"] = achieved / fp32_peak_tflops(sms, clocks["sm_mhz"])
 
