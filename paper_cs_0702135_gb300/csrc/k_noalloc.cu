@@ -20,14 +20,19 @@
 // loads its eight j of a group straight from the FP64 arrays and splits them
 // into double-single form once, in registers, then walks the active particles
 // (in shared memory): eight pairs, and a warp reduce-scatter into the warp's
-// double-single totals.  The CTA adds its warps and writes one FP64 partial
-// per value; a second kernel adds the ranges, a warp per value.  Every partial
-// is written before it is read in the same call, so nothing in the scratch
-// array needs clearing between calls.
+// double-single totals (k_few_partials).  Where the particles fill the lanes of a
+// warp, they take the lanes and the runs the warps instead (k_few_lanes), without
+// the reductions (27 of the 63 instructions a pair).  Both are bound by issue.
+// The CTA adds its warps and writes one FP64 partial per value; a second kernel
+// adds the ranges, a warp per value.  Every partial is written before it is
+// read in the same call, so nothing in the scratch array needs clearing between
+// calls.
 //
 // The first form held four active particles per CTA and split every j again
 // for each four, on the FP64 pipe: 16 conversions a j at 2 lanes a clock per
-// SM were nearly all of its time (64 active on 2^18 + 37 bodies: 148 us).
+// SM were nearly all of its time (64 active on 2^18 + 37 bodies: 148 us; 49 with
+// the split once a CTA, 41 with the particles over the lanes).
+#include <algorithm>
 #include <climits>
 #include <cmath>
 #include <mutex>
@@ -50,9 +55,13 @@ constexpr int kMaxDevices = 64;
 static __device__ __align__(256) double g_scratch[kScratchDoubles];
 
 using nbk::dev::ds_add;
+using nbk::dev::IDS;
+using nbk::dev::make_ids;
+using nbk::dev::pair_ds_packed;
 using nbk::dev::rsqrt_sfu;
 using nbk::dev::split_record;
 using nbk::dev::to_float_int;
+using nbk::dev::two_sum_acc;
 using nbk::dev::warp_reduce_scatter;
 
 struct DSPoint {
@@ -166,6 +175,124 @@ __global__ void __launch_bounds__(kNT, 2) k_few_partials(long long n, const doub
     }
 }
 
+// The same with the active particles over the lanes (R a lane) and
+// the runs over the warps: a run's sum is added to its lane's totals by one TwoSum
+// a value, where the form above needs a warp reduction of every run.  A CTA takes
+// the items [b W / B, (b + 1) W / B) of W = 16 G: the runs t0 .. t0 + 15 of a group,
+// 128 j, split once into shared memory (the next item's are on their way from
+// memory meanwhile) and read by broadcast.
+constexpr int kItemRuns = 16;               // runs of an item
+constexpr int kItemJ = kItemRuns * kRun;    // its j
+constexpr int kGroupItems = kNT / kItemRuns;
+
+template <int R>
+__global__ void __launch_bounds__(kNT, 2) k_few_lanes(long long n, const double *m, const double *x, const double *v,
+                                                      float eps2, const int *act, int na, long long jslice, int gps,
+                                                      long long G, double *part)
+{
+    constexpr int NW = kNT / 32, NV = 32 * R * kComp;
+    __shared__ float4 s_j[2][3][kItemJ];
+    __shared__ float s_h[NW][NV], s_l[NW][NV];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, b = blockIdx.x, B = gridDim.x;
+    long long ii[R];
+    IDS I[R];
+    float hi[R][kComp], lo[R][kComp];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int a = 32 * r + lane;
+        const long long i = act[a < na ? a : 0];
+        ii[r] = i < 0 ? 0 : (i >= n ? n - 1 : i);
+        const DSPoint p = load_point(m, x, v, ii[r]);
+        I[r] = make_ids(make_float4(p.xh[0], p.xh[1], p.xh[2], p.m), make_float4(p.xl[0], p.xl[1], p.xl[2], 0.0f),
+                        make_float4(p.v[0], p.v[1], p.v[2], 0.0f));
+#pragma unroll
+        for (int c = 0; c < kComp; ++c) hi[r][c] = lo[r][c] = 0.0f;
+    }
+    const long long w1 = (b + 1) * G * kGroupItems / B;
+    double xj[3], vj[3], mj = 0.0;
+    // this thread's j of item w (past the end: the last one, whose pairs are not formed)
+    const auto fetch = [&](long long w) {
+        const long long g = w / kGroupItems, sl = g / gps;
+        const long long j1 = (sl + 1) * jslice < n ? (sl + 1) * jslice : n;
+        long long j = sl * jslice + (g - sl * gps) * kGroup + (w % kGroupItems) * kItemRuns +
+                      (tid / kItemRuns) * kNT + tid % kItemRuns;
+        j = j < j1 ? j : j1 - 1;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) xj[c] = x[3 * j + c], vj[c] = v[3 * j + c];
+        mj = m[j];
+    };
+    long long w = b * G * kGroupItems / B;
+    if (tid < kItemJ && w < w1) fetch(w);
+    for (int buf = 0; w < w1; ++w, buf ^= 1) {
+        if (tid < kItemJ) {
+            float h[3], l[3], u[3];
+            split_record(xj, vj, h, l, u);
+            s_j[buf][0][tid] = make_float4(h[0], h[1], h[2], to_float_int(mj));
+            s_j[buf][1][tid] = make_float4(l[0], l[1], l[2], 0.0f);
+            s_j[buf][2][tid] = make_float4(u[0], u[1], u[2], 0.0f);
+        }
+        __syncthreads();
+        if (tid < kItemJ && w + 1 < w1) fetch(w + 1);
+        const long long g = w / kGroupItems, sl = g / gps;
+        const long long j0 = sl * jslice + (g - sl * gps) * kGroup;
+        const long long j1 = (sl + 1) * jslice < n ? (sl + 1) * jslice : n;
+        const int left = (int)(j1 - j0 < kGroup ? j1 - j0 : kGroup);   // at most 0 past a short slice
+        int own[R];   // the particle's position in the group
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            own[r] = (unsigned long long)(ii[r] - j0) < (unsigned long long)kGroup ? (int)(ii[r] - j0) : -1;
+#pragma unroll 1
+        for (int q = 0; q < kItemRuns / NW; ++q) {
+            const int tt = warp * (kItemRuns / NW) + q, t = (int)(w % kGroupItems) * kItemRuns + tt;
+            float a3[R][3], k3[R][3], pp[R];
+            bool mine = false;
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                a3[r][0] = a3[r][1] = a3[r][2] = k3[r][0] = k3[r][1] = k3[r][2] = pp[r] = 0.0f;
+                mine |= own[r] >= 0 && ((own[r] - t) & (kNT - 1)) == 0;
+            }
+            if (t + (kRun - 1) * kNT >= left || __any_sync(0xffffffffu, mine)) {
+#pragma unroll 1
+                for (int u = 0; u < kRun && t + u * kNT < left; ++u) {
+                    const int e = u * kItemRuns + tt;
+#pragma unroll
+                    for (int r = 0; r < R; ++r)
+                        pair_ds_packed<false, true>(s_j[buf][0][e], s_j[buf][1][e], s_j[buf][2][e], I[r], eps2, a3[r],
+                                                    k3[r], pp[r], t + u * kNT, own[r]);
+                }
+            } else {
+#pragma unroll
+                for (int u = 0; u < kRun; ++u) {
+                    const int e = u * kItemRuns + tt;
+                    const float4 p = s_j[buf][0][e], l = s_j[buf][1][e], d = s_j[buf][2][e];
+#pragma unroll
+                    for (int r = 0; r < R; ++r)
+                        pair_ds_packed<false, false>(p, l, d, I[r], eps2, a3[r], k3[r], pp[r]);
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int c = 0; c < kComp; ++c)
+                    two_sum_acc(hi[r][c], lo[r][c], c < 3 ? a3[r][c] : (c < 6 ? k3[r][c - 3] : pp[r]));
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int c = 0; c < kComp; ++c) {
+            s_h[warp][(32 * r + lane) * kComp + c] = hi[r][c];
+            s_l[warp][(32 * r + lane) * kComp + c] = lo[r][c];
+        }
+    __syncthreads();
+    for (int t = tid; t < na * kComp; t += kNT) {
+        float th = s_h[0][t], tl = s_l[0][t];
+#pragma unroll
+        for (int ww = 1; ww < NW; ++ww) ds_add(th, tl, s_h[ww][t], s_l[ww][t]);
+        part[((long long)b * kComp + t % kComp) * na + t / kComp] = (double)th + (double)tl;
+    }
+}
+
 // One warp per value: lanes over the ranges in a fixed stride, then a fixed
 // tree (one thread per value, adding the ranges in turn, waited for its loads
 // four at a time: ~15 us for one active particle on 2^18 bodies).
@@ -261,15 +388,29 @@ extern "C" int nb_force_few_noalloc(int64_t n, const double *d_m, const double *
     const int gps = (int)((jslice + kGroup - 1) / kGroup);
     const long long G = S * gps, slots = 2LL * s.sms;
     const long long rounds = (G + slots - 1) / slots;
-    const int B = (int)((G + rounds - 1) / rounds);
+    int B = (int)((G + rounds - 1) / rounds);
     int parts = (int)(slots / B < n_active ? slots / B : n_active);
     if (parts < 1) parts = 1;
     const int IC = (n_active + parts - 1) / parts;
     const int ichunks = (n_active + IC - 1) / IC;
 
     cudaStream_t st = (cudaStream_t)stream;
-    k_few_partials<<<B * ichunks, kNT, 0, st>>>(n, d_m, d_x, d_v, (float)(eps * eps), d_active_idx,
-                                                n_active, jslice, gps, G, B, IC, ichunks, s.scratch);
+    // Particles over the lanes where nearly all lanes have one.  This form / the one
+    // with the runs over the lanes, us, on 2^18 + 37 bodies: 24 active 31.2 / 27.1,
+    // 32 31.2 / 31.2, 48 41.5 / 39.4, 64 41.5 / 48.7; on 2^20: 24 82.5 / 70.1,
+    // 32 78.4 / 86.5, 48 123.5 / 119.3, 64 119.5 / 150.0.
+    const int R = (n_active + 31) / 32;
+    const bool lanes = 16 * n_active >= 15 * 32 * R;
+    if (lanes) {
+        const long long W = G * kGroupItems;
+        B = (int)std::min<long long>(W, std::min<long long>(slots, kMaxSlices));
+        const auto kernel = R == 1 ? k_few_lanes<1> : k_few_lanes<2>;
+        kernel<<<B, kNT, 0, st>>>(n, d_m, d_x, d_v, (float)(eps * eps), d_active_idx, n_active, jslice, gps, G,
+                                  s.scratch);
+    } else {
+        k_few_partials<<<B * ichunks, kNT, 0, st>>>(n, d_m, d_x, d_v, (float)(eps * eps), d_active_idx,
+                                                    n_active, jslice, gps, G, B, IC, ichunks, s.scratch);
+    }
     if (cudaGetLastError() != cudaSuccess) return NB_ECUDA;
     k_few_combine<<<(n_active * kComp * 32 + 255) / 256, 256, 0, st>>>(n_active, B, s.scratch, d_acc,
                                                                        d_jerk, d_pot);

@@ -108,3 +108,18 @@ def test_noalloc_rejects_sizes_beyond_the_maximum(nb):
         nb.nb_force_few_noalloc(n, d_m, d_x, d_v, EPS, d_idx.long(), 3, out, None, None)
     with pytest.raises(ValueError):
         nb.nb_force_few_noalloc(n, d_m, d_x[:50], d_v, EPS, d_idx, 3, out, None, None)
+
+
+@pytest.mark.parametrize("na", [23, 29, 30, 32, 33, 48, 60, 63])
+@pytest.mark.parametrize("n,eps", [(64, EPS), (2047, 0.0), (2049, EPS), (70001, EPS)])
+def test_noalloc_particles_over_lanes(nb, n, na, eps):
+    # both sides of the rule that puts the particles over a warp's lanes, with
+    # short groups and slices
+    torch = pytest.importorskip("torch")
+    m, x, v = plummer(n, 29)
+    idx = sample_active(n, na, 57 + na)
+    d_m, d_x, d_v = (torch.from_numpy(a).cuda() for a in (m, x, v))
+    got = _noalloc(nb, torch, n, d_m, d_x, d_v, eps, idx, calls=2)
+    ref = oracle.force(m, x, v, eps, idx, nthreads=os.cpu_count() or 1)
+    mags = pair_magnitudes(m, x, v, eps, idx, chunk=8)
+    assert_force_close(got, ref, mags, TOL_DS, "no-alloc n=%d n_active=%d eps=%g" % (n, na, eps))
