@@ -401,10 +401,14 @@ __global__ void __launch_bounds__(NT, 2) k_force_jpar_ds(ForceArgs fa, JDS J)
 //
 // A tile whose j and the CTA's i are all in the range of nb_int64.cuh runs on the
 // integer pipes, any other tile (and eps = 0) the FP64 form: 1820 active of 65536
-// in 2.85 ms against 7.38 ms for the FP64 form alone.  Moving the pair factors but
+// in 2.93 ms against 7.38 ms for the FP64 form alone.  Moving the pair factors but
 // not the differences gave 3.79 ms (16 FP64 operations a pair, against 10).  With
-// 12 CTAs an SM (80 registers, 60 bytes spilled) against 9 without the limit:
-// 2.85 against 3.14 ms; 1024 active 1.75 against 1.65, 4096 6.20 against 6.24.
+// 12 CTAs an SM (80 registers, some spilled) against 9 without the limit: 2.85
+// against 3.14 ms; 1024 active 1.75 against 1.65, 4096 6.20 against 6.24 (before
+// the tiles had sums of their own, which cost 2.7% and take the error, against
+// quadruple precision, of 400 active of 256..65536 from 1.4e-16 to 1.0e-16 in acc,
+// 4.4e-16 to 3.4e-16 in jerk, 0.92e-16 to 0.81e-16 in pot; the FP64 form has 1.4,
+// 5.2 and 0.91e-16).
 
 template <int NT, int R, bool SOFT>
 __global__ void __launch_bounds__(NT, 12) k_force_ipar_f64(ForceArgs fa, JF64 J)
@@ -462,12 +466,25 @@ __global__ void __launch_bounds__(NT, 12) k_force_ipar_f64(ForceArgs fa, JF64 J)
             if (__syncthreads_and(iok && in_range_f64(pj, vj))) {
                 s_t[tid].i = tile_of(pj, vj);
                 __syncthreads();
+                // a sum of the tile first: fewer roundings at the size of the total
+                double ta[R][3], tk[R][3], tp[R];
+#pragma unroll
+                for (int r = 0; r < R; ++r) ta[r][0] = ta[r][1] = ta[r][2] = tk[r][0] = tk[r][1] = tk[r][2] = tp[r] = 0.0;
 #pragma unroll 1
                 for (int jj = 0; jj < NT; ++jj) {
                     const J64I JJ = j_of(s_t[jj].i);
 #pragma unroll
                     for (int r = 0; r < R; ++r)
-                        pair_f64_int(JJ, xf[r], ieps, acc[r], jk[r], pot[r], jt + jj, ii[r]);
+                        pair_f64_int(JJ, xf[r], ieps, ta[r], tk[r], tp[r], jt + jj, ii[r]);
+                }
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) {
+                        acc[r][c] += ta[r][c];
+                        jk[r][c] += tk[r][c];
+                    }
+                    pot[r] += tp[r];
                 }
                 continue;
             }
