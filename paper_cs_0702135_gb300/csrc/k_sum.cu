@@ -493,15 +493,17 @@ __device__ __forceinline__ unsigned rank_of(const unsigned (&rank)[H], int k)
     return (rank[k / 2] >> (16 * (k % 2))) & 0xffffu;
 }
 
-// Two j's keys, ~0 for a pair that is left out.
+// Two j's keys, ~0 for a pair that is left out.  The sign is cleared: a mass of
+// -0.0 has the key -0.0, whose bits lie past the last bin (its terms are zeros,
+// which change no running sum wherever they stand).
 __device__ __forceinline__ uint2 sort_keys(const JDS &J, int j0, int j1, int n, int i, const Side2 &N, float eps2)
 {
     const int c0 = min(j0, n - 1), c1 = min(j1, n - 1);
     const Side2 Js = side2(J.pos_hi[c0], J.pos_lo[c0], J.vel[c0], J.pos_hi[c1], J.pos_lo[c1], J.vel[c1]);
     float2 r2;
     const float2 key = pair_key2(Js, N, eps2, r2);
-    return make_uint2(j0 < n && j0 != i && r2.x != 0.0f ? __float_as_uint(key.x) : ~0u,
-                      j1 < n && j1 != i && r2.y != 0.0f ? __float_as_uint(key.y) : ~0u);
+    return make_uint2(j0 < n && j0 != i && r2.x != 0.0f ? __float_as_uint(fabsf(key.x)) : ~0u,
+                      j1 < n && j1 != i && r2.y != 0.0f ? __float_as_uint(fabsf(key.y)) : ~0u);
 }
 
 // Adds the terms of sorted items 0 .. total - 1 (index by `at`) to run, which

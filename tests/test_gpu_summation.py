@@ -294,3 +294,21 @@ def test_sorted_key_distributions_bit_exact(nb, case):
     got = _gpu_force(nb, m, x, v, EPS, idx, nb.NB_SUM_FP32_SORTED, no_force=True)
     ref = oracle.force_summed(m, x, v, EPS, idx, mode=oracle.SUM_FP32_SORTED, nthreads=8)
     _assert_same(got, ref, "sorted %s" % case)
+
+
+@pytest.mark.parametrize("n", [300, 3000, 9000])
+@pytest.mark.parametrize("share", ["one", "half", "all"])
+def test_sorted_masses_of_negative_zero_bit_exact(nb, n, share):
+    # -0.0 is a mass of zero: its key has to fall into a bin, and its terms
+    # change no sum.  Sizes of one and of several chunks.
+    m, x, v = plummer(n, 43)
+    where = np.random.RandomState(4).permutation(n)[:{"one": 1, "half": n // 2, "all": n}[share]]
+    m = m.copy()
+    m[where] = -0.0
+    idx = np.unique(np.concatenate([where[:3], sample_active(n, 9, n)])).astype(np.int32)
+    got = _gpu_force(nb, m, x, v, EPS, idx, nb.NB_SUM_FP32_SORTED, no_force=True)
+    ref = oracle.force_summed(m, x, v, EPS, idx, mode=oracle.SUM_FP32_SORTED, nthreads=8)
+    _assert_same(got, ref, "sorted n=%d" % n)
+    pos = np.where(m == 0.0, 0.0, m)
+    same = _gpu_force(nb, pos, x, v, EPS, idx, nb.NB_SUM_FP32_SORTED, no_force=True)
+    _assert_same(got, same, "masses of +0.0, n=%d" % n)
