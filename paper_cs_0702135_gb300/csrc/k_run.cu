@@ -574,7 +574,7 @@ __global__ void __launch_bounds__(kRunNT) k_run(RunArgs ra)
         }
         if (MODE == NB_SUM_FIXED && tid < m) {
             const float4 v = s_v[tid];
-            mb = __float_as_uint(s_p[tid].w);
+            mb = __float_as_uint(fabsf(s_p[tid].w));   // a mass may be -0.0
             vb = __float_as_uint(__fadd_rn(__fadd_rn(fabsf(v.x), fabsf(v.y)), fabsf(v.z)));
         }
         if (MODE == NB_SUM_FIXED) {

@@ -42,15 +42,15 @@ using namespace dev;
 constexpr unsigned kFull = 0xffffffffu;
 
 // The largest single-precision mass and |vx| + |vy| + |vz| over all j, as
-// float bits (non-negative floats order like their bits); bounds[] must be
-// zero on entry.
+// float bits (non-negative floats order like their bits; the sign of a mass of
+// -0.0 is cleared); bounds[] must be zero on entry.
 __global__ void k_fixed_bounds(JDS J, int n, unsigned *bounds)
 {
     unsigned mb = 0, vb = 0;
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
         const float4 v = J.vel[j];
         const float v1 = __fadd_rn(__fadd_rn(fabsf(v.x), fabsf(v.y)), fabsf(v.z));
-        mb = max(mb, __float_as_uint(J.pos_hi[j].w));
+        mb = max(mb, __float_as_uint(fabsf(J.pos_hi[j].w)));
         vb = max(vb, __float_as_uint(v1));
     }
     mb = __reduce_max_sync(kFull, mb);

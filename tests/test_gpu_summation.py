@@ -312,3 +312,26 @@ def test_sorted_masses_of_negative_zero_bit_exact(nb, n, share):
     pos = np.where(m == 0.0, 0.0, m)
     same = _gpu_force(nb, pos, x, v, EPS, idx, nb.NB_SUM_FP32_SORTED, no_force=True)
     _assert_same(got, same, "masses of +0.0, n=%d" % n)
+
+
+@pytest.mark.parametrize("n", [64, 3000])
+def test_fixed_masses_of_negative_zero_bit_exact(nb, n):
+    # the units follow the largest mass; -0.0 is not it.  Force, persistent
+    # run and graph run.
+    m, x, v = plummer(n, 47)
+    m = m.copy()
+    m[1::3] = -0.0
+    idx = sample_active(n, 20, n)
+    got = _gpu_force(nb, m, x, v, EPS, idx, nb.NB_SUM_FIXED)
+    ref = oracle.force_summed(m, x, v, EPS, idx, mode=oracle.SUM_FIXED, nthreads=8)
+    _assert_same(got, ref, "fixed n=%d" % n)
+    for flags in (0, nb.NB_RUN_GRAPH):
+        orc = oracle.Integrator(m, x, v, EPS, summation=oracle.SUM_FIXED, nthreads=8)
+        ctx = nb.Context(m, x, v, EPS, summation=nb.NB_SUM_FIXED, flags=flags)
+        try:
+            assert ctx.nb_run(1.0, 12)[0] == 12
+            for _ in range(12):
+                orc.step()
+            _assert_state_equal(ctx.nb_get_state(), orc, "flags=%d" % flags)
+        finally:
+            ctx.nb_free()
