@@ -335,3 +335,22 @@ def test_fixed_masses_of_negative_zero_bit_exact(nb, n):
             _assert_state_equal(ctx.nb_get_state(), orc, "flags=%d" % flags)
         finally:
             ctx.nb_free()
+
+
+@pytest.mark.parametrize("size", [127, 128, 129, 140, 500, 1000])
+def test_sorted_equal_keys_in_a_chunk_bit_exact(nb, size):
+    # clumps of `size` coincident particles: equal keys that differ in their jerk,
+    # so that the order by index shows, around the largest bucket that is ranked
+    # by comparisons, in short and in full chunks
+    rng = np.random.RandomState(size)
+    c = rng.normal(size=(max(2, 6000 // size), 3))
+    x = np.repeat(c, size, axis=0)[rng.permutation(len(c) * size)]
+    n = len(x)
+    m = np.full(n, 1.0 / n)
+    v = rng.normal(size=(n, 3))
+    idx = sample_active(n, 6, size)
+    for k in (n, 3 * size):       # the first particles alone: one short chunk
+        few = idx[idx < k] if (idx < k).any() else np.array([0], dtype=np.int32)
+        got = _gpu_force(nb, m[:k], x[:k], v[:k], EPS, few, nb.NB_SUM_FP32_SORTED, no_force=True)
+        ref = oracle.force_summed(m[:k], x[:k], v[:k], EPS, few, mode=oracle.SUM_FP32_SORTED, nthreads=8)
+        _assert_same(got, ref, "n=%d" % k)
