@@ -71,7 +71,11 @@ extern "C" {
  *   NB_SUM_FP32_SORTED  FP32 running sum with the smallest pair force
  *                       |m_j dx / r^3| first (ties in index order), after a
  *                       per-particle sort (in shared memory unless thousands of
- *                       keys share a bin); memory: 16 n bytes per resident CTA.
+ *                       keys share a bin).  Memory: 8 n bytes for each of four
+ *                       CTAs per SM (above 522240 particles 16 n, and at most
+ *                       4 GiB in all): 0.32 GB at 65536 particles on 152 SMs.
+ *                       Where that is more than a 32nd of the free device
+ *                       memory, fewer CTAs run, of 16 n bytes per SM in all.
  * force_mode and split_j only apply to NB_SUM_COMPENSATED and NB_SUM_FIXED
  * (whose results split_j does not change).
  */

@@ -395,7 +395,9 @@ __global__ void __launch_bounds__(kSeqNT, 1) k_force_seq(ForceArgs fa, JDS J, in
 // ---------------------------------------------------------------------------
 // FP32 running sum, smallest pair force first: one CTA per active i.  The keys
 // |mj dx/r^3| are sorted stably by j and the terms added in that order.
-//  1. a histogram of the keys over bins of 1/32 octave;
+//  1. a histogram of the keys over bins of 1/32 octave, and where a bin holds
+//     more than 2048 items (a particle far out sees all others at one distance)
+//     a second one of finer bins over the keys' own range;
 //  2. consecutive bins make chunks of up to 4096 items (about 2048 each); the
 //     items (key bits << 32 | j) go to their chunk in the CTA's scratch, keys
 //     evaluated again rather than stored and read: 8 bytes written and read
@@ -406,25 +408,27 @@ __global__ void __launch_bounds__(kSeqNT, 1) k_force_seq(ForceArgs fa, JDS J, in
 // tile before it in order, one component each (4 clocks an item), so four CTAs
 // share an SM, each in its own phase.
 //
-// Where a bin holds more than 2048 items (many equal keys) or there are more
-// than 255 chunks, all items are sorted in the scratch instead, by a stable LSD
-// radix sort with a pass per key byte (a byte that all keys share is left
+// Where a bin still holds more than 2048 items (many equal keys) or there are
+// more than 255 chunks, all items are sorted in the scratch instead, by a stable
+// LSD radix sort with a pass per key byte (a byte that all keys share is left
 // out).  An item's rank within a pass is that among the equal digits of its
 // warp (match_any and the warp's running counts in shared memory) plus the
 // counts of the earlier warps and tiles; stability keeps equal keys in index
-// order.  Its scattered 8-byte stores to a footprint beyond the L2 are what
-// that waits for.
+// order.  Its scattered stores to a footprint beyond the L2 are what that waits
+// for.  Up to kChunks kChunk particles, where it is the exception, it moves
+// indices alone and evaluates their keys again in every pass, so that a CTA's
+// scratch is n words (sort_scratch_size); above, keyed items in two arrays.
 //
-// 1820 active on 65536 bodies: 5.3 ms (a radix sort of the chunks 6.1 ms, the
-// scratch sort 6.6 ms); one CTA
-// of 1024 threads per SM, ranking one item a thread between five barriers and
-// adding after evaluating, 18.6 ms.
+// 1820 active on 65536 bodies: 5.1 ms (5.4 with the scratch sort in place of the
+// finer bins, by keyed items, and 6.8 by indices; a radix sort of the chunks 6.1,
+// the scratch sort alone 6.6); one CTA of 1024 threads per SM, ranking one item a
+// thread between five barriers and adding after evaluating, 18.6 ms.
 
 constexpr int kSortW = kSortNT / 32;
 constexpr int kSortK = 16;                        // items per thread of a chunk or tile
 constexpr int kSortTile = kSortNT * kSortK;
-constexpr int kBinShift = 18, kBins = 8192;       // bins of the key's upper bits
-constexpr int kChunk = 2048, kChunks = 255;       // aim of a chunk, and how many at most
+constexpr int kBinBits = 13, kBins = 1 << kBinBits;   // bins of the key's upper bits
+constexpr int kBinShift = 18;
 static_assert((0x7f7fffff >> kBinShift) < kBins && 2 * kChunk <= kSortTile, "keys have a bin, chunks fit");
 constexpr int kSortSum = (kSortW - 1) * 32;       // items per tile of the sum: one per term lane
 constexpr int kSortRow = kSortSum + 4;
@@ -446,6 +450,13 @@ struct SortShared {
     unsigned scan[kSortW], lo[kSortW], hi[kSortW];
     int cnt;
 };
+
+// (Functions that are not inlined take it from here, to know that it is shared memory.)
+__device__ __forceinline__ SortShared &sort_shared()
+{
+    extern __shared__ float4 s_sorted[];
+    return *reinterpret_cast<SortShared *>(s_sorted);
+}
 
 // Exclusive sum over the CTA's threads (a barrier before and after use of s).
 __device__ __forceinline__ unsigned cta_exclusive(unsigned v, unsigned *s, int lane, int warp)
@@ -541,42 +552,72 @@ __device__ __forceinline__ void sum_sorted(SortShared &sh, const JDS &J, int i, 
     }
 }
 
-// The scratch sort: all n items by four passes between A and B; the sorted array.
-__device__ __noinline__ const unsigned long long *sort_scratch(SortShared &sh, const JDS &J, int i, int n, float eps2,
-                                                               unsigned long long *A, unsigned long long *B)
+// An item of the scratch sort: key and index where the scratch has room for two
+// arrays of them; else the index alone, its key evaluated again for every pass.
+template <typename Item>
+struct SortItem {
+    static constexpr bool kKeyed = sizeof(Item) == 8;
+    static __device__ __forceinline__ Item make(unsigned key, int j)
+    {
+        return kKeyed ? (Item)((unsigned long long)key << 32 | (unsigned)j) : (Item)j;
+    }
+};
+
+// The scratch sort: all n items by four passes between A and B; the sorted array,
+// and in sh.cnt how many of its items are pairs to add.
+template <typename Item>
+__device__ __forceinline__ const Item *sort_scratch(SortShared &sh, const JDS &J, int i, int n, float eps2, Item *A,
+                                                 Item *B)
 {
     constexpr int NT = kSortNT;
+    using It = SortItem<Item>;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const Side2 N = side2_neg(J.pos_hi[i], J.pos_lo[i], J.vel[i]);
     unsigned(*hist)[256] = reinterpret_cast<unsigned(*)[256]>(sh.a.hist);
 #pragma unroll
     for (int q = 0; q < 4; ++q) hist[q][tid] = 0;
+    if (tid == 0) sh.cnt = 0;
     __syncthreads();
+    int cnt = 0;
     for (int j = tid; j < n; j += 2 * NT) {
         const uint2 key = sort_keys(J, j, j + NT, n, i, N, eps2);
-        A[j] = ((unsigned long long)key.x << 32) | (unsigned)j;
+        cnt += (key.x != ~0u) + (key.y != ~0u);
+        A[j] = It::make(key.x, j);
 #pragma unroll
         for (int q = 0; q < 4; ++q) atomicAdd(&hist[q][(key.x >> (8 * q)) & 255u], 1u);
         if (j + NT < n) {
-            A[j + NT] = ((unsigned long long)key.y << 32) | (unsigned)(j + NT);
+            A[j + NT] = It::make(key.y, j + NT);
 #pragma unroll
             for (int q = 0; q < 4; ++q) atomicAdd(&hist[q][(key.y >> (8 * q)) & 255u], 1u);
         }
     }
+    cnt = __reduce_add_sync(kFull, cnt);
+    if (lane == 0) atomicAdd(&sh.cnt, cnt);
     __syncthreads();
-    unsigned long long *src = A, *dst = B;
+    Item *src = A, *dst = B;
     for (int pass = 0; pass < 4; ++pass) {
         const unsigned mine = hist[pass][tid];
         if (__syncthreads_or(mine == (unsigned)n)) continue;   // one digit for all
         sh.base[tid] = cta_exclusive(mine, sh.scan, lane, warp);   // kept by this thread only
-        const int shift = 32 + 8 * pass;
         for (int t0 = 0; t0 < n; t0 += kSortTile) {
-            unsigned long long item[kSortK];
-            unsigned rank[kSortK / 2];
+            Item item[kSortK];
+            unsigned rank[kSortK / 2], dig[kSortK / 4];   // dig: four digits a register
             const int w0 = t0 + warp * (kSortK * 32) + lane;
 #pragma unroll
-            for (int k = 0; k < kSortK; ++k) item[k] = w0 + k * 32 < n ? src[w0 + k * 32] : 0ULL;
-            auto digit = [&](int k) { return w0 + k * 32 < n ? (int)(item[k] >> shift) & 255 : -1; };
+            for (int k = 0; k < kSortK; ++k) item[k] = w0 + k * 32 < n ? src[w0 + k * 32] : (Item)0;
+            if (!It::kKeyed) {
+#pragma unroll
+                for (int k = 0; k < kSortK; k += 2) {
+                    const uint2 key = sort_keys(J, (int)item[k], (int)item[k + 1], n, i, N, eps2);
+                    const unsigned two = ((key.x >> (8 * pass)) & 255u) | ((key.y >> (8 * pass)) & 255u) << 8;
+                    dig[k / 4] = k % 4 == 0 ? two : dig[k / 4] | two << 16;
+                }
+            }
+            auto digit = [&](int k) {
+                const unsigned d = It::kKeyed ? (unsigned)((unsigned long long)item[k] >> (32 + 8 * pass))
+                                              : dig[k / 4] >> (8 * (k % 4));
+                return w0 + k * 32 < n ? (int)(d & 255u) : -1;
+            };
             warp_ranks<kSortK>(digit, rank, sh.u.off[warp], lane, kSortK);
             __syncthreads();
             unsigned run = sh.base[tid];
@@ -594,11 +635,22 @@ __device__ __noinline__ const unsigned long long *sort_scratch(SortShared &sh, c
             __syncwarp();   // the warp's offsets are cleared next
         }
         __syncthreads();
-        unsigned long long *tmp = src;
+        Item *tmp = src;
         src = dst;
         dst = tmp;
     }
     return src;
+}
+
+// All terms of particle i by the scratch sort.
+template <typename Item>
+__device__ __noinline__ float sum_in_scratch(const JDS J, int i, int n, float eps2, Item *A)
+{
+    SortShared &sh = sort_shared();
+    const Item *sorted = sort_scratch(sh, J, i, n, eps2, A, A + n);
+    float run = 0.0f;
+    sum_sorted(sh, J, i, eps2, sh.cnt, [&](int q) { return (int)(unsigned)sorted[q]; }, run);
+    return run;
 }
 
 // Chunk of cnt <= kSortTile items from src sorted into sh.a.item, by buckets:
@@ -715,77 +767,104 @@ __device__ __forceinline__ void sort_chunk(SortShared &sh, const unsigned long l
     __syncthreads();
 }
 
-__global__ void __launch_bounds__(kSortNT, kSortCtas) k_force_sorted(ForceArgs fa, JDS J, SumArgs sa)
+// Steps 1 and 2 for particle i: the number of items, in chunks from sh.start[c] on
+// in A, or -1 where a bin stays overfull.  (A function of its own:
+// its registers are then not held, or spilled, through the chunks' sorts.)
+__device__ __noinline__ int sort_into_chunks(const JDS J, int i, int n, float eps2, unsigned long long *A)
 {
-    constexpr int NT = kSortNT;
-    static_assert(NT == 256, "a thread per digit and per 32 bins");
-    const int na = read_na(fa);
-    if (na <= 0) return;
-    extern __shared__ float4 s_sorted[];
-    SortShared &sh = *reinterpret_cast<SortShared *>(s_sorted);
-    __shared__ float s_res[7];
-    const int n = fa.n, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const float eps2 = (float)fa.eps2;
-    unsigned long long *const A = sa.scratch + (size_t)blockIdx.x * 2 * (size_t)n;
-
-    for (int a = blockIdx.x; a < na; a += gridDim.x) {
-        const int i = clamp_index(fa.act[a], n);
-        const Side2 N = side2_neg(J.pos_hi[i], J.pos_lo[i], J.vel[i]);
-        // 1. histogram
-        if (tid == 0) sh.cnt = 0;
+    SortShared &sh = sort_shared();
+    constexpr int NT = kSortNT, kOwn = kBins / NT;   // this thread's bins
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const Side2 N = side2_neg(J.pos_hi[i], J.pos_lo[i], J.vel[i]);
+    if (tid == 0) sh.cnt = 0;
+    unsigned key0 = 0, place = 0;
+    int shift = kBinShift, total = 0;
+    auto histogram = [&](auto bin, bool first) {
         for (int q = tid; q < kBins; q += NT) sh.a.hist[q] = 0;
         __syncthreads();
         int cnt = 0;
         for (int j = tid; j < n; j += 2 * NT) {
             const uint2 key = sort_keys(J, j, j + NT, n, i, N, eps2);
-            if (key.x != ~0u) atomicAdd(&sh.a.hist[key.x >> kBinShift], 1u), ++cnt;
-            if (key.y != ~0u) atomicAdd(&sh.a.hist[key.y >> kBinShift], 1u), ++cnt;
+            if (key.x != ~0u) atomicAdd(&sh.a.hist[bin(key.x)], 1u), ++cnt;
+            if (key.y != ~0u) atomicAdd(&sh.a.hist[bin(key.y)], 1u), ++cnt;
         }
         cnt = __reduce_add_sync(kFull, cnt);
-        if (lane == 0) atomicAdd(&sh.cnt, cnt);
+        if (lane == 0 && first) atomicAdd(&sh.cnt, cnt);
         __syncthreads();
-        const int total = sh.cnt;
-        float run = 0.0f;
-
-        // 2. chunks: this thread's 32 bins
-        constexpr int kOwn = kBins / NT;
+        total = sh.cnt;
+    };
+    auto bin = [&](unsigned key) { return (key - key0) >> shift; };
+    histogram([](unsigned key) { return key >> kBinShift; }, true);
+    for (;;) {
         unsigned sum = 0, most = 0;
         for (int q = 0; q < kOwn; ++q) {
             const unsigned c = sh.a.hist[tid * kOwn + q];
             sum += c;
             most = max(most, c);
         }
-        unsigned place = cta_exclusive(sum, sh.scan, lane, warp);
-        if (__syncthreads_or(most > kChunk || total > kChunks * kChunk)) {
-            const unsigned long long *sorted = sort_scratch(sh, J, i, n, eps2, A, A + n);
-            sum_sorted(sh, J, i, eps2, total, [&](int q) { return (int)(unsigned)sorted[q]; }, run);
+        place = cta_exclusive(sum, sh.scan, lane, warp);
+        if (!__syncthreads_or(most > kChunk)) break;
+        // once more, over the keys' own range, if that makes the bins finer
+        if (shift != kBinShift) return -1;
+        unsigned lo = kBins, hi = 0;
+        for (int q = tid * kOwn; q < (tid + 1) * kOwn; ++q)
+            if (sh.a.hist[q]) lo = min(lo, (unsigned)q), hi = q;
+        lo = __reduce_min_sync(kFull, lo);
+        hi = __reduce_max_sync(kFull, hi);
+        if (lane == 0) sh.lo[warp] = lo, sh.hi[warp] = hi;
+        __syncthreads();
+        for (int w = 0; w < kSortW; ++w) lo = min(lo, sh.lo[w]), hi = max(hi, sh.hi[w]);
+        const int finer = __clz(hi - lo) - (32 - kBinBits);   // doublings of the bins
+        if (finer <= 0) return -1;
+        key0 = lo << kBinShift;
+        shift = kBinShift - finer;
+        histogram(bin, false);
+    }
+    for (int q = tid; q < kChunks + 2; q += NT) sh.start[q] = total;
+    __syncthreads();
+    // a chunk starts at the first bin that starts at or past a multiple of kChunk
+    int prev = tid == 0 ? -1 : (int)((place - sh.a.hist[tid * kOwn - 1]) / kChunk);
+    for (int q = 0; q < kOwn; ++q) {
+        const int c = (int)(place / kChunk);   // past the last item: kChunks at most
+        sh.id[tid * kOwn + q] = (unsigned char)c;
+        if (c != prev && c <= kChunks) sh.start[c] = place;
+        prev = c;
+        place += sh.a.hist[tid * kOwn + q];
+    }
+    __syncthreads();
+    // items to their chunk, in any order within it (the chunk's sort compares j too)
+    for (int q = tid; q < kChunks + 1; q += NT) sh.next[q] = sh.start[q];
+    __syncthreads();
+    for (int j = tid; j < n; j += 2 * NT) {
+        const uint2 key = sort_keys(J, j, j + NT, n, i, N, eps2);
+        if (key.x != ~0u)
+            A[atomicAdd(&sh.next[sh.id[bin(key.x)]], 1u)] = (unsigned long long)key.x << 32 | (unsigned)j;
+        if (key.y != ~0u)
+            A[atomicAdd(&sh.next[sh.id[bin(key.y)]], 1u)] = (unsigned long long)key.y << 32 | (unsigned)(j + NT);
+    }
+    __syncthreads();
+    return total;
+}
+
+__global__ void __launch_bounds__(kSortNT, kSortCtas) k_force_sorted(ForceArgs fa, JDS J, SumArgs sa)
+{
+    static_assert(kSortNT == 256, "a thread per digit and per 32 bins");
+    const int na = read_na(fa);
+    if (na <= 0) return;
+    SortShared &sh = sort_shared();
+    __shared__ float s_res[7];
+    const int n = fa.n, tid = threadIdx.x;
+    const float eps2 = (float)fa.eps2;
+    unsigned long long *const A = sa.scratch + (size_t)blockIdx.x * (size_t)sa.words;
+
+    for (int a = blockIdx.x; a < na; a += gridDim.x) {
+        const int i = clamp_index(fa.act[a], n);
+        const int total = n <= kChunks * kChunk ? sort_into_chunks(J, i, n, eps2, A) : -1;
+        float run = 0.0f;
+        if (total < 0) {
+            run = sa.words >= 2LL * n ? sum_in_scratch(J, i, n, eps2, A)
+                                      : sum_in_scratch(J, i, n, eps2, reinterpret_cast<unsigned *>(A));
         } else {
-            for (int q = tid; q < kChunks + 2; q += NT) sh.start[q] = total;
-            __syncthreads();
-            // a chunk starts at the first bin that starts at or past a multiple of kChunk
-            int prev = tid == 0 ? -1 : (int)((place - sh.a.hist[tid * kOwn - 1]) / kChunk);
-            for (int q = 0; q < kOwn; ++q) {
-                const int c = (int)(place / kChunk);   // past the last item: kChunks at most
-                sh.id[tid * kOwn + q] = (unsigned char)c;
-                if (c != prev && c <= kChunks) sh.start[c] = place;
-                prev = c;
-                place += sh.a.hist[tid * kOwn + q];
-            }
-            __syncthreads();
-            // items to their chunk, in any order within it (the chunk's sort
-            // compares j too)
-            for (int q = tid; q < kChunks + 1; q += NT) sh.next[q] = sh.start[q];
-            __syncthreads();
-            for (int j = tid; j < n; j += 2 * NT) {
-                const uint2 key = sort_keys(J, j, j + NT, n, i, N, eps2);
-                if (key.x != ~0u)
-                    A[atomicAdd(&sh.next[sh.id[key.x >> kBinShift]], 1u)] =
-                        (unsigned long long)key.x << 32 | (unsigned)j;
-                if (key.y != ~0u)
-                    A[atomicAdd(&sh.next[sh.id[key.y >> kBinShift]], 1u)] =
-                        (unsigned long long)key.y << 32 | (unsigned)(j + NT);
-            }
-            __syncthreads();
             // 3. chunk by chunk
             for (int c = 0; c <= kChunks; ++c) {
                 const int first = (int)sh.start[c], len = (int)sh.start[c + 1] - first;

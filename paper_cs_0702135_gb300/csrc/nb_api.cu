@@ -66,7 +66,7 @@ struct nb_ctx {
     ulonglong2 *d_run_sync = nullptr;   // records and flags, zeroed before each launch
     int run_ncta = 0, run_per = 0;
     unsigned *d_bounds = nullptr;   // fixed point: mass and velocity bounds
-    unsigned long long *d_sort = nullptr;  // sorted: keyed items, 2n per resident CTA
+    unsigned long long *d_sort = nullptr;  // sorted: scratch of the resident CTAs
     long long t_pred = 0;           // ticks of the last host-driven prediction
     bool force_valid = false;       // results in d_res usable by nb_correct
     int force_na = 0;
@@ -667,9 +667,11 @@ static int init_impl(nb_ctx *c, int64_t n, const double *m, const double *x, con
         c->sum.mode = o.summation;
         c->sum.slots = c->sms * (bsum > 0 ? bsum : 1);
         if (o.summation == NB_SUM_FP32_SORTED) {
-            // keyed items: 16 n bytes per resident CTA, at most 4 GiB in all
-            const long long per = 16LL * n, cap = (4LL << 30) / per;
-            if (cap < c->sum.slots) c->sum.slots = (int)(cap > 0 ? cap : 1);
+            size_t free_bytes = 0, total_bytes = 0;
+            CK(cudaMemGetInfo(&free_bytes, &total_bytes));
+            const SortScratch sc = sort_scratch_size(n, c->sms, bsum > 0 ? bsum : 1, free_bytes);
+            c->sum.words = sc.words;
+            c->sum.slots = sc.slots;
         }
     }
     const long long iblk = kIparNT * (f64 ? kIparR64 : kIparR);
@@ -698,7 +700,7 @@ static int init_impl(nb_ctx *c, int64_t n, const double *m, const double *x, con
         if ((rc = dalloc(c, &c->d_bounds, 2))) return rc;
         c->sum.bounds = c->d_bounds;
     } else if (o.summation == NB_SUM_FP32_SORTED) {
-        if ((rc = dalloc(c, &c->d_sort, 2LL * N * c->sum.slots))) return rc;
+        if ((rc = dalloc(c, &c->d_sort, c->sum.words * c->sum.slots))) return rc;
         c->sum.scratch = c->d_sort;
     }
     if (f64) {

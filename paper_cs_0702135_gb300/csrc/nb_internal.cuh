@@ -409,7 +409,8 @@ struct ForceArgs {
 struct SumArgs {
     int mode;                       // NB_SUM_FIXED, NB_SUM_FP32 or NB_SUM_FP32_SORTED
     unsigned *bounds;               // [2] fixed point: largest fl32 mass, largest fl32 |vx|+|vy|+|vz| (bits)
-    unsigned long long *scratch;    // sorted: 2 n keyed items per resident CTA
+    unsigned long long *scratch;    // sorted: `words` per resident CTA (sort_scratch_size)
+    long long words;
     int slots;                      // resident CTAs of the mode's force kernel
 };
 #ifndef NB_FIX_NT
@@ -426,6 +427,29 @@ constexpr int kFixWaves = 4;
 constexpr int kSeqNT = 640;         // FP32 index order: threads per CTA
 constexpr int kSortNT = 256;        // FP32 sorted: one CTA per i
 constexpr int kSortCtas = 4;        // and at least this many per SM
+constexpr int kChunk = 2048, kChunks = 255;   // items aimed at in a chunk, and how many chunks at most
+
+// FP32 sorted: 8-byte words of scratch of a CTA (n keyed items; twice that where
+// every block takes the sort of all items, which moves them between two
+// arrays), and the CTAs.  All that fit the SMs (1820 active on 65536 bodies:
+// 5.3 ms with four an SM, 18.6 ms with a single larger one) unless their scratch is
+// more than a 32nd of the free memory, or 4 GiB: then as many as 16 n bytes an SM
+// hold, which is what one CTA an SM with two arrays takes.
+struct SortScratch {
+    long long words;
+    int slots;
+};
+inline SortScratch sort_scratch_size(long long n, int sms, int per_sm, unsigned long long free_bytes)
+{
+    SortScratch r;
+    r.words = n <= (long long)kChunks * kChunk ? n : 2 * n;
+    const long long part = (long long)(free_bytes / 32), least = 16 * n * sms, cap = 4LL << 30;
+    long long bytes = part > least ? part : least;
+    if (bytes > cap) bytes = cap;
+    const long long fit = bytes / (8 * r.words), all = (long long)sms * per_sm;
+    r.slots = (int)(fit < 1 ? 1 : (fit < all ? fit : all));
+    return r;
+}
 constexpr int kErrFixedScale = 64;  // device error word: fixed-point scales out of range
 constexpr int kErrInput = 65;       // device error word: a non-finite value or a negative mass
 

@@ -354,3 +354,34 @@ def test_sorted_equal_keys_in_a_chunk_bit_exact(nb, size):
         got = _gpu_force(nb, m[:k], x[:k], v[:k], EPS, few, nb.NB_SUM_FP32_SORTED, no_force=True)
         ref = oracle.force_summed(m[:k], x[:k], v[:k], EPS, few, mode=oracle.SUM_FP32_SORTED, nthreads=8)
         _assert_same(got, ref, "n=%d" % k)
+def test_sorted_scratch_size(nb):
+    # 8 n bytes for each of at most four CTAs an SM, beside what every context holds
+    import torch
+    n = 65536
+    m, x, v = plummer(n, 3, exact_virial_max=0)
+    held = []
+    for summation in (nb.NB_SUM_FP32, nb.NB_SUM_FP32_SORTED):
+        nb.Context(m, x, v, EPS, summation=summation, flags=nb.NB_INIT_NO_FORCE).nb_free()   # first use of the module
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        ctx = nb.Context(m, x, v, EPS, summation=summation, flags=nb.NB_INIT_NO_FORCE)
+        held.append(free - torch.cuda.mem_get_info()[0])
+        ctx.nb_free()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert held[1] - held[0] <= 4 * sms * 8 * n + (8 << 20)   # and the allocator's granules
+
+
+def test_sorted_in_the_scratch_bit_exact(nb):
+    # more keys in a bin than a chunk takes, several tiles of the scratch sort, and
+    # more active particles than CTAs
+    rng = np.random.RandomState(9)
+    n = 20000
+    m = np.full(n, 1.0 / n)
+    v = rng.normal(size=(n, 3))
+    x = rng.normal(size=(4, 3))[rng.randint(0, 4, n)]          # four points, keys equal in index order
+    x[:5] = rng.normal(size=(5, 3))
+    idx = sample_active(n, 700, 2)
+    got = _gpu_force(nb, m, x, v, EPS, idx, nb.NB_SUM_FP32_SORTED, no_force=True)
+    few = np.concatenate([idx[:6], idx[-6:]])
+    ref = oracle.force_summed(m, x, v, EPS, few, mode=oracle.SUM_FP32_SORTED, nthreads=8)
+    _assert_same([np.concatenate([g[:6], g[-6:]]) for g in got], ref, "scratch")

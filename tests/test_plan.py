@@ -25,6 +25,11 @@ int main() {
             std::printf("%d 0 0 0\n", combine_lanes(na, n));
             continue;
         }
+        if (kind == 's') {   // sorted sums: scratch words and CTAs (n, SMs = iblk, CTAs an SM = tile, free bytes = cap)
+            const SortScratch sc = sort_scratch_size(n, iblk, tile, (unsigned long long)cap);
+            std::printf("%lld %d 0 0\n", sc.words, sc.slots);
+            continue;
+        }
         if (kind == 'r') {   // regime for na active with jpar_max = n, small_max = iblk
             std::printf("%d 0 0 0\n", regime_of(na, n, iblk));
             continue;
@@ -349,3 +354,21 @@ def test_fine_plans(tmp_path):
         assert lanes in (1, 2, 4, 8, 16, 32) and (lanes == 1 or lanes <= S), c
         if na <= 20000:
             assert cand >= 0 and n_whole == 0 and regime == (1 if cand >= 16 else 2), c
+
+
+def test_sorted_scratch_fits_where_one_cta_an_sm_did(planner):
+    # with the memory short, no more than 16 n bytes an SM (or the 4 GiB that bound
+    # both); with plenty, every resident CTA has its scratch, at most twice that
+    # (the sort of all items needs two arrays above 522240 particles)
+    gib = 1 << 30
+    cases = [("s", 0, n, sms, 4, 0, 0, free) for n in (1, 300, 65536, 262144, 522240, 522241, 1 << 20, 1 << 28)
+             for sms in (1, 152) for free in (0, 1 << 20, gib, 16 * gib, 270 * gib)]
+    for c, (words, slots, _, _) in zip(cases, _run(planner, cases)):
+        n, sms, free = c[2], c[3], c[7]
+        used, least = 8 * words * slots, 16 * n * sms
+        assert words == (n if n <= 522240 else 2 * n)
+        assert 1 <= slots <= 4 * sms
+        assert slots == 1 or used <= min(4 * gib, max(least, free // 32)), c
+        assert slots == 4 * sms or used + 8 * words > min(4 * gib, max(least, free // 32)), c
+        if n <= 522240:
+            assert used <= 2 * least
