@@ -503,7 +503,7 @@ void enqueue_adj(nb_ctx *c, bool post, bool add, int slices, int pre, const Stat
 // per-stage graph instead.
 constexpr int kRunNotUsed = 1;
 
-int run_persistent(nb_ctx *c, long long te, long long max_steps)
+int run_persistent(nb_ctx *c, long long te, long long steps0, long long max_steps)
 {
     if (c->n > kRunMaxN || c->o.precision != NB_DS || (c->o.flags & NB_RUN_GRAPH) ||
         (c->o.summation != NB_SUM_COMPENSATED && c->o.summation != NB_SUM_FIXED))
@@ -545,21 +545,23 @@ int run_persistent(nb_ctx *c, long long te, long long max_steps)
     ra.flag = reinterpret_cast<unsigned long long *>(ra.maxrec + 2 * ra.ncta);
     ra.blk = reinterpret_cast<float4 *>(c->d_run_sync + 5LL * ra.ncta);
     for (;;) {
-        ra.max_steps = max_steps < kRunMaxSteps ? max_steps : kRunMaxSteps;
-        const long long steps0 = c->h_ctrl->steps;   // as of the caller's, or the last launch's, sync
+        // the mirror is as of the caller's, or the last launch's, sync
+        ra.max_steps = run_batch(max_steps, steps0, c->h_ctrl->steps, kRunMaxSteps);
+        const long long before = c->h_ctrl->steps;
         CK(cudaMemsetAsync(c->d_run_sync, 0, sizeof(ulonglong2) * (size_t)sync_count(), c->st));
         const cudaError_t e = launch_run(ra, c->o.summation, c->st);
         if (e == cudaErrorCooperativeLaunchTooLarge) {
-            // not every CTA can be resident now (a shared GPU): use the graph
+            // not every CTA can be resident now (a shared GPU): use the graph for
+            // the steps that are left
             cudaGetLastError();
             return kRunNotUsed;
         }
         if (e != cudaSuccess) return fail(c, NB_ECUDA, "persistent run launch: %s", cudaGetErrorString(e));
         c->launches += 1;
         const int rc = sync_ctrl(c);
-        const long long done = c->h_ctrl->steps - steps0;
-        max_steps -= done;
-        if (rc || done < ra.max_steps || max_steps <= 0 || c->h_ctrl->n_active == 0) return rc;
+        if (rc || c->h_ctrl->steps - before < ra.max_steps || c->h_ctrl->n_active == 0 ||
+            run_batch(max_steps, steps0, c->h_ctrl->steps, 1) <= 0)
+            return rc;
     }
 }
 
@@ -990,7 +992,7 @@ int nb_run(nb_ctx *c, double t_end, int64_t max_steps, int64_t *steps_out, int64
     if ((rc = sync_ctrl(c))) return rc;
     const long long steps0 = c->h_ctrl->steps, inter0 = c->h_ctrl->interactions;
     c->force_valid = false;
-    rc = run_persistent(c, te, max_steps);
+    rc = run_persistent(c, te, steps0, max_steps);
     if (rc != kRunNotUsed) {
         if (rc) {
             c->synchronous = false;
@@ -1002,10 +1004,10 @@ int nb_run(nb_ctx *c, double t_end, int64_t max_steps, int64_t *steps_out, int64
     }
     if (!c->step_exec && (rc = capture_steps(c, 1, &c->step_exec))) return rc;
     c->force_valid = false;
-    long long done = 0;
     const int batch = 32;
-    while (done < max_steps) {
-        const long long k = (max_steps - done) < batch ? (max_steps - done) : batch;
+    for (;;) {
+        const long long k = run_batch(max_steps, steps0, c->h_ctrl->steps, batch);
+        if (k <= 0) break;
         long long s = 0;
         if (k == batch) {   // a longer graph only where its capture pays
             if (!c->steps_exec && (rc = capture_steps(c, kGraphSteps, &c->steps_exec))) return rc;
@@ -1014,7 +1016,6 @@ int nb_run(nb_ctx *c, double t_end, int64_t max_steps, int64_t *steps_out, int64
         for (; s < k; ++s) CK(cudaGraphLaunch(c->step_exec, c->st));
         c->launches += k * c->step_nodes;
         if ((rc = sync_ctrl(c))) return rc;
-        done = c->h_ctrl->steps - steps0;
         if (c->h_ctrl->n_active == 0) break;
     }
     if (steps_out) *steps_out = c->h_ctrl->steps - steps0;

@@ -533,6 +533,13 @@ constexpr int kRunIndexBits = 14;   // particle index in a block record's tag, b
 constexpr int kRunPerLane = 8;      // CTAs at most: 32 times this
 // steps per launch at most: a tag's step number must not come round again
 constexpr long long kRunMaxSteps = 1LL << 17;
+// Steps of nb_run's next launch or batch: of the max_steps from counter value steps0
+// on, those that are left at counter value `steps`, whoever took the others.
+inline long long run_batch(long long max_steps, long long steps0, long long steps, long long limit)
+{
+    const long long left = max_steps - (steps - steps0);
+    return left < limit ? left : limit;
+}
 static_assert(kRunMaxN == 1 << kRunIndexBits && kRunMaxSteps < 1LL << (32 - kRunIndexBits), "tags");
 struct RunArgs {
     State s;

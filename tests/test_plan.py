@@ -30,6 +30,10 @@ int main() {
             std::printf("%lld %d 0 0\n", sc.words, sc.slots);
             continue;
         }
+        if (kind == 'b') {   // nb_run's batches: max_steps = cap, counter at start = na, now = n, limit = iblk
+            std::printf("%lld 0 0 0\n", run_batch(cap, na, n, iblk));
+            continue;
+        }
         if (kind == 'r') {   // regime for na active with jpar_max = n, small_max = iblk
             std::printf("%d 0 0 0\n", regime_of(na, n, iblk));
             continue;
@@ -372,3 +376,22 @@ def test_sorted_scratch_fits_where_one_cta_an_sm_did(planner):
         assert slots == 4 * sms or used + 8 * words > min(4 * gib, max(least, free // 32)), c
         if n <= 522240:
             assert used <= 2 * least
+
+
+def test_run_takes_no_more_than_its_steps(planner):
+    # a run of 131072 + 1 steps whose second persistent launch is refused: one step
+    # is left for the graphs; and batches of a run always end at max_steps
+    start = 77
+    assert _run(planner, [("b", start, start, 131072, 0, 0, 0, 131073)])[0][0] == 131072
+    assert _run(planner, [("b", start, start + 131072, 32, 0, 0, 0, 131073)])[0][0] == 1
+    assert _run(planner, [("b", start, start + 131073, 32, 0, 0, 0, 131073)])[0][0] == 0
+    for total in (0, 1, 31, 32, 33, 100):
+        taken = 0
+        while True:
+            k = _run(planner, [("b", start, start + taken, 32, 0, 0, 0, total)])[0][0]
+            if k <= 0:
+                break
+            assert k <= 32
+            taken += k
+        assert taken == total
+    assert _run(planner, [("b", 0, 5, 32, 0, 0, 0, 1 << 62)])[0][0] == 32
