@@ -314,9 +314,10 @@ __global__ void __launch_bounds__(kRunNT) k_run(RunArgs ra)
 {
     // this CTA's particles: state, end times, combined force of its block
     // members, j records
-    extern __shared__ double s_dyn[];
+    extern __shared__ float4 s_dyn[];
+    static_assert(alignof(decltype(s_dyn[0])) >= alignof(float4), "the records within need 16 bytes");
     const int per = ra.per;
-    double *const s_st = s_dyn;                                     // [12][per] x, v, a, k
+    double *const s_st = reinterpret_cast<double *>(s_dyn);         // [12][per] x, v, a, k
     double *const s_res = s_st + 12 * per;                          // [per][8]
     float4 *const s_p = reinterpret_cast<float4 *>(s_res + 8 * per);
     float4 *const s_l = s_p + per, *const s_v = s_l + per;

@@ -146,3 +146,12 @@ def test_device_wrappers_check_tensors_before_the_call():
     assert nb.nb._dev(raw, "float64", 3, "d_x").value == raw
     with pytest.raises(ValueError, match="required"):
         nb.nb._dev(None, "float64", 3, "d_x")
+
+
+def test_dynamic_shared_memory_is_declared_with_16_byte_alignment():
+    # the kernels lay float4 records into it
+    csrc = os.path.join(ROOT, "paper_cs_0702135_gb300", "csrc")
+    for name in sorted(os.listdir(csrc)):
+        text = open(os.path.join(csrc, name)).read()
+        for decl in re.findall(r"extern\s+__shared__\s+([^;]*);", text):
+            assert re.match(r"(__align__\(16\)\s+)?float4\b|__align__\((16|32)\)", decl), (name, decl)
