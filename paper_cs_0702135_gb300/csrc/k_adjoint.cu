@@ -494,6 +494,14 @@ __global__ void k_shared_done(State s, Ctrl *ctrl, int *act, long long steps, in
         act[i] = i;
     }
 }
+// Every particle at time t with the shared step.
+__global__ void k_shared_times(State s, long long t, int level)
+{
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < s.n; i += gridDim.x * blockDim.x) {
+        s.t[i] = t;
+        s.lev[i] = level;
+    }
+}
 __global__ void k_shared_ctrl(Ctrl *ctrl, int n, long long steps, int level)
 {
     ctrl->t_now += steps * (1LL << (kTickBits - level));
@@ -652,6 +660,11 @@ void launch_shared_done(const State &s, Ctrl *ctrl, int *act, long long steps, i
 {
     k_shared_done<<<grid_for(s.n, 256), 256, 0, st>>>(s, ctrl, act, steps, level);
     k_shared_ctrl<<<1, 1, 0, st>>>(ctrl, s.n, steps, level);
+}
+
+void launch_shared_times(const State &s, long long t, int level, cudaStream_t st)
+{
+    k_shared_times<<<grid_for(s.n, 256), 256, 0, st>>>(s, t, level);
 }
 
 void launch_adj_step(const AdjStep &q, cudaStream_t st)

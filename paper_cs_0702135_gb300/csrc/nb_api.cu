@@ -91,7 +91,7 @@ struct nb_ctx {
     bool traj_shared = false;       // made by the shared-step kernels
     // every particle at one time with level_fixed (else the scheduler picks blocks)
     bool synchronous = false;
-    long long traj_steps = 0, traj_ckpt = 0;
+    long long traj_steps = 0, traj_ckpt = 0, traj_t = 0;   // traj_t: its final time
 
     // measurement counters (nb_get_stats)
     long long launches = 0;
@@ -1227,13 +1227,13 @@ int nb_traj_forward(nb_ctx *c, int64_t steps, int64_t checkpoint_every)
         }
         launch_shared_done(c->S, c->d_ctrl, c->d_act, steps, c->o.level_fixed, c->st);
         c->launches += 3;
-        CK(cudaMemcpyAsync(c->d_tfin, c->d_t, sizeof(long long) * N, cudaMemcpyDeviceToDevice, c->st));
         CK(cudaGetLastError());
         c->force_valid = false;
         if ((rc = sync_ctrl(c))) return rc;
         c->traj_valid = true;
         c->traj_steps = steps;
         c->traj_ckpt = checkpoint_every;
+        c->traj_t = c->h_ctrl->t_now;
         return NB_OK;
     }
     enqueue_full_sweep(c);
@@ -1255,6 +1255,7 @@ int nb_traj_forward(nb_ctx *c, int64_t steps, int64_t checkpoint_every)
     c->traj_valid = true;
     c->traj_steps = steps;
     c->traj_ckpt = checkpoint_every;
+    c->traj_t = c->h_ctrl->t_now;
     return NB_OK;
 }
 
@@ -1339,17 +1340,23 @@ static int traj_backward_impl(nb_ctx *c, const double *xbar_T, const double *vba
     if (xbar0) CK(cudaMemcpyAsync(xbar0, cot(c, 0), sizeof(double) * 3 * N, kout, c->st));
     if (vbar0) CK(cudaMemcpyAsync(vbar0, cot(c, 1), sizeof(double) * 3 * N, kout, c->st));
     if (mbar) CK(cudaMemcpyAsync(mbar, cot(c, 4), sizeof(double) * N, kout, c->st));
-    // leave the context at the end of the trajectory, as after nb_traj_forward
+    // leave the context at the end of the trajectory, as after nb_traj_forward,
+    // wherever it went since
     launch_copy_state(c->S, state_view(c, c->d_fin), c->st);
-    CK(cudaMemcpyAsync(c->d_t, c->d_tfin, sizeof(long long) * N, cudaMemcpyDeviceToDevice, c->st));
+    if (c->traj_shared)
+        launch_shared_times(c->S, c->traj_t, c->o.level_fixed, c->st);
+    else
+        CK(cudaMemcpyAsync(c->d_t, c->d_tfin, sizeof(long long) * N, cudaMemcpyDeviceToDevice, c->st));
+    c->synchronous = c->traj_shared;
     CK(cudaStreamSynchronize(c->st));
-    if ((rc = sync_ctrl(c))) return rc;  // errors raised during the recomputation
-    c->h_ctrl->t_now = saved.t_now;
+    rc = sync_ctrl(c);  // errors raised during the recomputation
+    c->h_ctrl->t_now = c->traj_t;
     c->h_ctrl->steps = saved.steps;
     c->h_ctrl->interactions = saved.interactions;
     CK(cudaMemcpyAsync(c->d_ctrl, c->h_ctrl, sizeof(Ctrl), cudaMemcpyHostToDevice, c->st));
     c->force_valid = false;
-    return sync_ctrl(c);
+    const int rc_end = sync_ctrl(c);
+    return rc ? rc : rc_end;
 }
 
 int nb_traj_backward(nb_ctx *c, const double *xbar_T, const double *vbar_T, double *xbar0,

@@ -689,6 +689,7 @@ int launch_force_vjp(const VjpArgs &va, int precision, bool softened, bool combi
                      cudaStream_t st);
 void launch_shared_step(const SharedStep &q, cudaStream_t st);
 void launch_shared_done(const State &s, Ctrl *ctrl, int *act, long long steps, int level, cudaStream_t st);
+void launch_shared_times(const State &s, long long t, int level, cudaStream_t st);
 void launch_adj_step(const AdjStep &q, cudaStream_t st);
 void launch_adj_pre(const State &s, double dt, const double *xb, const double *vb, double *ab,
                     double *kb, int precision, const VjpRecDS &rec, const VjpRec64 &rec64,

@@ -263,3 +263,46 @@ def test_shared_steps_match_scheduled_steps(nb, n, precision):
     assert np.array_equal(sa["t"], sb["t"]) and np.array_equal(sa["level"], sb["level"])
     for a, b in [(sa[k], sb[k]) for k in ("x", "v", "a", "k")] + list(zip(ga, gb)):
         assert np.abs(a - b).max() <= 1e-11 * np.abs(b).max()
+
+
+@pytest.mark.parametrize("precision", ["ds", "f64"])
+@pytest.mark.parametrize("between", ["run", "state", "step"])
+def test_backward_returns_to_the_trajectory_from_elsewhere(nb, between, precision):
+    # The context went on after the trajectory: backward takes it back with its
+    # times, levels and system time, and a next trajectory starts from there.
+    n, eps, level = 96, 1 / 64, 8
+    m, x, v = plummer(n, 97)
+    r = np.random.default_rng(98)
+    xbT, vbT = r.normal(size=(n, 3)), r.normal(size=(n, 3))
+    p = {"ds": nb.NB_DS, "f64": nb.NB_FP64}[precision]
+    a, b = _ctx(nb, m, x, v, eps, p, level), _ctx(nb, m, x, v, eps, p, level)
+    try:
+        for c in (a, b):
+            c.nb_traj_forward(6, 4)
+        end = a.nb_get_state()
+        want = b.nb_traj_backward(xbT, vbT)
+        if between == "run":
+            assert a.nb_run(32 * 2.0 ** -level)[0] == 26
+        elif between == "step":
+            a.nb_step()
+        else:
+            t = np.full(n, 3 << 35, dtype=np.int64)
+            a.nb_set_state(x, v, x, v, t, np.full(n, level + 2, dtype=np.int32))
+        got = a.nb_traj_backward(xbT, vbT)
+        for g, w in zip(got, want):
+            assert np.array_equal(g, w)
+        st = a.nb_get_state()
+        for key in end:
+            assert np.array_equal(st[key], end[key]), key
+        assert a.nb_get_active()[1] == 6 << (40 - level)
+        for c in (a, b):
+            c.nb_traj_forward(5, 2)
+        sa, sb = a.nb_get_state(), b.nb_get_state()
+        for key in sa:
+            assert np.array_equal(sa[key], sb[key]), key
+        assert np.all(sa["t"] == 11 << (40 - level))
+        for g, w in zip(a.nb_traj_backward(xbT, vbT), b.nb_traj_backward(xbT, vbT)):
+            assert np.array_equal(g, w)
+    finally:
+        a.nb_free()
+        b.nb_free()
