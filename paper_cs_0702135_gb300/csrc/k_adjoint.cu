@@ -457,7 +457,7 @@ __global__ void __launch_bounds__(kShNT) k_shared_step(SharedStep q)
             if (q.mode == kShCorrect) {
                 bool bad = false;
                 AxisStep r = correct_axis(x, v, a, k, ap, kp, -q.level, bad);
-                if (bad) r = correct_axis_any(x, v, a, k, ap, kp, 1LL << (kTickBits - q.level));
+                if (bad) r = correct_axis_rest(x, v, a, k, ap, kp, 1LL << (kTickBits - q.level));
                 x = r.x, v = r.v;
             }
             a = ap, k = kp;

@@ -549,11 +549,7 @@ __global__ void __launch_bounds__(kRunNT) k_run(RunArgs ra)
                 bool bad = false;
                 split_ds_int(xp, h, l, bad);
                 u = to_float_int(vp, bad);
-                if (bad) {
-                    h = to_float_volatile(xp);
-                    l = to_float_volatile(__dsub_rn(xp, (double)h));
-                    u = to_float_volatile(vp);
-                }
+                if (bad) split_rest(xp, vp, h, l, u);
                 reinterpret_cast<float *>(&s_p[q])[c] = h;
                 reinterpret_cast<float *>(&s_l[q])[c] = l;
                 reinterpret_cast<float *>(&s_v[q])[c] = u;

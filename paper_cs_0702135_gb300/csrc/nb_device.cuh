@@ -240,11 +240,28 @@ __device__ __forceinline__ float to_float_volatile(double x)
     asm volatile("cvt.rn.f32.f64 %0, %1;" : "=f"(y) : "d"(x));
     return y;
 }
+// RN32(x) for an x that is bad: a zero (a system in a plane, a particle at rest) is
+// still a move of bits.
+__device__ __forceinline__ bool is_zero(double x) { return (__double_as_longlong(x) << 1) == 0; }
+__device__ __forceinline__ float to_float_rest(double x)
+{
+    return is_zero(x) ? __int_as_float(__double2hiint(x)) : to_float_volatile(x);
+}
 __device__ __forceinline__ float to_float_int(double x)
 {
     bool bad = false;
     const float y = to_float_int(x, bad);
-    return bad ? to_float_volatile(x) : y;
+    return bad ? to_float_rest(x) : y;
+}
+// A position's two words and a velocity where at least one of them was bad: what is
+// in range stays.
+__device__ __forceinline__ void split_rest(double x, double v, float &hi, float &lo, float &u)
+{
+    if (!exponent_in<-70, 190>(x)) {
+        hi = to_float_rest(x);
+        lo = is_zero(x) ? 0.0f : to_float_volatile(__dsub_rn(x, (double)hi));
+    }
+    if (!exponent_in<-70, 190>(v)) u = to_float_rest(v);
 }
 
 // A position split into double-single and a velocity in FP32, all axes.
@@ -259,11 +276,7 @@ __device__ __forceinline__ void split_record(const double x[3], const double v[3
     }
     if (bad)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            hi[c] = to_float_volatile(x[c]);
-            lo[c] = to_float_volatile(__dsub_rn(x[c], (double)hi[c]));
-            u[c] = to_float_volatile(v[c]);
-        }
+        for (int c = 0; c < 3; ++c) split_rest(x[c], v[c], hi[c], lo[c], u[c]);
 }
 
 __device__ __forceinline__ double norm3(double u0, double u1, double u2)
@@ -388,6 +401,18 @@ static __device__ __noinline__ AxisStep correct_axis_any(double x, double v, dou
     return r;
 }
 
+// Where correct_axis was bad: an axis at rest (a system in a plane) moves nothing, the
+// sums of its zeros being +0; else the general form.  128 bodies in a plane, graph
+// run: 27.7 us a step, 32.9 with the general form after the other, 31.7 with it alone.
+__device__ __forceinline__ AxisStep correct_axis_rest(double x, double v, double a, double k, double ap, double kp,
+                                                      long long ticks)
+{
+    const long long any = __double_as_longlong(v) | __double_as_longlong(a) | __double_as_longlong(k) |
+                          __double_as_longlong(ap) | __double_as_longlong(kp);
+    if (any == 0 && ticks > 0) return {is_zero(x) ? 0.0 : x, 0.0, 0.0, 0.0};
+    return correct_axis_any(x, v, a, k, ap, kp, ticks);
+}
+
 // e of a step of `ticks` = 2^(e + 40) ticks; false for any other step.
 __device__ __forceinline__ bool step_exponent(long long ticks, int &e)
 {
@@ -432,7 +457,7 @@ __device__ __forceinline__ bool correct_particle(const State &s, long long i, lo
                      k = ldst<CG>(&s.k[e]);
         bool bad = !block_step;
         AxisStep r = correct_axis(x, v, a, k, ap[c], kp[c], ex, bad);
-        if (bad) r = correct_axis_any(x, v, a, k, ap[c], kp[c], ticks);
+        if (bad) r = correct_axis_rest(x, v, a, k, ap[c], kp[c], ticks);
         s.x[e] = r.x;
         s.v[e] = r.v;
         s.a[e] = ap[c];
@@ -558,7 +583,7 @@ __device__ __forceinline__ bool correct_particle_quad(const State &s, long long 
     int ex;
     bool bad = !step_exponent(ticks, ex);
     AxisStep r = correct_axis(x, v, a, k, apc, kpc, ex, bad);
-    if (bad) r = correct_axis_any(x, v, a, k, apc, kpc, ticks);
+    if (bad) r = correct_axis_rest(x, v, a, k, apc, kpc, ticks);
     // every lane of the quad has read the old state before any lane stores
     __syncwarp();
     if (own) {

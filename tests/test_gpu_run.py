@@ -184,3 +184,32 @@ def test_bounded_wait_times_out_and_the_context_stays_usable(nb):
     finally:
         a.nb_free()
         b.nb_free()
+
+
+@pytest.mark.parametrize("n", [40, 300])
+@pytest.mark.parametrize("case", ["plane", "minus_plane", "line", "at_rest"])
+def test_zero_components_bit_exact(nb, case, n):
+    # coordinates that are and stay zero (of either sign) and particles that start
+    # at rest leave the integer forms of the corrector and of the records: force,
+    # persistent run and graph run with the oracle's bits
+    m, x, v = plummer(n, 53 + n)
+    if case == "at_rest":
+        v = np.zeros_like(v)
+    else:
+        z = -0.0 if case == "minus_plane" else 0.0
+        for c in (2,) if case != "line" else (1, 2):
+            x[:, c] = z
+            v[:, c] = z
+    eps = 1.0 / 16
+    for flags in (0, nb.NB_RUN_GRAPH):
+        orc = oracle.Integrator(m, x, v, eps, summation=oracle.SUM_FIXED, nthreads=8)
+        ctx = nb.Context(m, x, v, eps, summation=nb.NB_SUM_FIXED, flags=flags)
+        try:
+            assert ctx.nb_run(1.0, 40)[0] == 40
+            for _ in range(40):
+                orc.step()
+            st = ctx.nb_get_state()
+            for key, ref in (("x", orc.x), ("v", orc.v), ("a", orc.a), ("k", orc.k), ("t", orc.t), ("level", orc.lev)):
+                assert np.array_equal(st[key], ref), (key, flags)
+        finally:
+            ctx.nb_free()

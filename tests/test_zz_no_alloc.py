@@ -123,3 +123,20 @@ def test_noalloc_particles_over_lanes(nb, n, na, eps):
     ref = oracle.force(m, x, v, eps, idx, nthreads=os.cpu_count() or 1)
     mags = pair_magnitudes(m, x, v, eps, idx, chunk=8)
     assert_force_close(got, ref, mags, TOL_DS, "no-alloc n=%d n_active=%d eps=%g" % (n, na, eps))
+
+
+@pytest.mark.parametrize("na", [3, 32])
+def test_noalloc_zero_components_match_oracle(nb, na):
+    # a system in a plane, some particles at rest, zero and tiny values among the rest
+    torch = pytest.importorskip("torch")
+    n = 3001
+    m, x, v = plummer(n, 25)
+    x[:, 2] = 0.0
+    v[:, 2] = -0.0
+    v[::3] = 0.0
+    x[5, 0] = 1e-30
+    idx = sample_active(n, na, 8)
+    got = _noalloc(nb, torch, n, *[torch.from_numpy(q).cuda() for q in (m, x, v)], EPS, idx, calls=2)
+    ref = oracle.force(m, x, v, EPS, idx, nthreads=8)
+    assert_force_close(got, ref, pair_magnitudes(m, x, v, EPS, idx), TOL_DS, "plane na=%d" % na)
+    assert np.all(got[0][:, 2] == 0.0) and np.all(got[1][:, 2] == 0.0)
