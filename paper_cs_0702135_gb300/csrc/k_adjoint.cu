@@ -30,12 +30,7 @@ using namespace dev;
 
 constexpr int kVNT = 128;  // partners per tile; FP64: threads per CTA
 constexpr int kVDsNT = 64; // DS: threads per CTA
-#ifndef NB_VJP_U2
-#define NB_VJP_U2 4
-#endif
-#ifndef NB_VJP_U1
-#define NB_VJP_U1 4
-#endif
+constexpr int kVUnroll = 4;   // DS: partner unrolling
 
 // One particle's VJP record: (predicted) position and velocity, mass and the
 // cotangents of its acc and jerk, in the layout of the context's precision.
@@ -174,8 +169,7 @@ __global__ void __launch_bounds__(kVDsNT) k_force_vjp_ds(VjpArgs va)
                     for (int r = 0; r < R; ++r) vjp_pair_ds<SOFT, true>(Pq, K[r], eps2, t[r], jt + jj, k[r]);
                 }
             } else {
-                constexpr int U = R == 1 ? NB_VJP_U1 : NB_VJP_U2;
-#pragma unroll (U)
+#pragma unroll (kVUnroll)
                 for (int jj = 0; jj < kVNT; ++jj) {
                     VjpRec Pq;
                     Pq.ph = s_ph[jj]; Pq.pl = s_pl[jj]; Pq.v = s_v[jj]; Pq.ab = s_ab[jj]; Pq.kb = s_kb[jj];
@@ -212,7 +206,8 @@ __global__ void __launch_bounds__(kVDsNT) k_force_vjp_ds(VjpArgs va)
 // The DS sweep's particles per thread and slices.  Up to kVOneMax particles one
 // k per thread and slices of one tile: the sweep is then short of CTAs (4096:
 // 59 us, two k a thread 66, and 70 with 128-thread CTAs and slices of two tiles;
-// 1024: 15 against 23 us).  Above, two k per thread, each partner record
+// 1024: 15 against 23 us; at the line they meet, with the step's other kernel:
+// 8192 234 and 236 us, 10240 361 and 360, 16384 871 and 825).  Above, two k per thread, each partner record
 // read from shared memory serving two pairs, and slices that make about
 // kVWaves waves of the resident CTAs, dealt out as CTAs end (65536: 12.4 ms,
 // 12.9 ms with one k; one wave 14.8 ms, three 12.7 ms).
@@ -616,8 +611,6 @@ int vjp_slots(int precision, int sms)
                         : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_force_vjp_ds<2, true>, kVDsNT, 0);
     return e == cudaSuccess ? sms * (b > 0 ? b : 1) : sms;
 }
-
-int vjp_tile() { return kVNT; }
 
 int launch_force_vjp(const VjpArgs &va_in, int precision, bool softened, bool combine, int *slices,
                      cudaStream_t st)

@@ -34,7 +34,8 @@
 // Bound by latency: at N = 1024 a step was 36,000 clocks with the state in
 // global memory and three grid barriers (waits at barriers 15,000, force 6,500,
 // prediction 3,700, block list 3,600, partial sums 3,500, corrector 2,900),
-// 19.2 us a step with the copies around the run; now 14.1 us.
+// 19.2 us a step with the copies around the run; now 10.5 us (18.5 then, counted the
+// same way: 1/8 time unit with nb_set_state before it).
 //
 // Two summations: the compensated double-single sums (TwoSum-promoted FP32
 // partials, FP64 across CTAs) and the GRAPE-style fixed-point sums of k_sum.cu
@@ -682,7 +683,7 @@ int run_layout(int n, int sms, int blocks_per_sm, int *ncta, int *per)
 {
     // 32 particles per CTA up to 64 CTAs, then up to 64 particles per CTA
     // (64 CTAs at n = 4096), then one CTA per SM (measured on whole runs: more
-    // CTAs share the force and the predictor but add to every barrier and to
+    // CTAs share the force and the predictor but add to every exchange and to
     // the partials each block particle sums; above 4096 bodies the force
     // share wins)
     int p = (n + 63) / 64;

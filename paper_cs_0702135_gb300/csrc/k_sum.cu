@@ -397,7 +397,8 @@ __global__ void __launch_bounds__(kSeqNT, 1) k_force_seq(ForceArgs fa, JDS J, in
 // |mj dx/r^3| are sorted stably by j and the terms added in that order.
 //  1. a histogram of the keys over bins of 1/32 octave, and where a bin holds
 //     more than 2048 items (a particle far out sees all others at one distance)
-//     a second one of finer bins over the keys' own range;
+//     a second one of finer bins over the keys' own range: with bins of at most
+//     2048 a chunk stays within the 4096 items that shared memory takes;
 //  2. consecutive bins make chunks of up to 4096 items (about 2048 each); the
 //     items (key bits << 32 | j) go to their chunk in the CTA's scratch, keys
 //     evaluated again rather than stored and read: 8 bytes written and read

@@ -767,8 +767,7 @@ __device__ __forceinline__ void write_combined(const ForceOut &o, int c, int a, 
 // false when r2 = 0 (the terms are then not numbers and must be skipped).
 __device__ __forceinline__ bool pair_rn(const float4 &p, const float4 &l, const float4 &w,
                                         const float xh[3], const float xl[3], const float vi[3],
-                                        float eps2, float sa, float sk, float sp, float t[7],
-                                        float *key = nullptr)
+                                        float eps2, float sa, float sk, float sp, float t[7])
 {
     const float dx0 = __fadd_rn(__fsub_rn(p.x, xh[0]), __fsub_rn(l.x, xl[0]));
     const float dx1 = __fadd_rn(__fsub_rn(p.y, xh[1]), __fsub_rn(l.y, xl[1]));
@@ -792,7 +791,6 @@ __device__ __forceinline__ bool pair_rn(const float4 &p, const float4 &l, const 
     t[4] = __fmul_rn(fk, __fadd_rn(u1, __fmul_rn(b, dx1)));
     t[5] = __fmul_rn(fk, __fadd_rn(u2, __fmul_rn(b, dx2)));
     t[6] = -fp;
-    if (key) *key = fminf(__fmul_rn(mr3, __fsqrt_rn(d2)), FLT_MAX);
     return r2 != 0.0f;
 }
 
@@ -903,8 +901,8 @@ __device__ __forceinline__ float2 pair_rn2(const Side2 &J, const Side2 &N, float
     return r2;
 }
 
-// The sort keys of two pairs, min(mr3 sqrt(d2), FLT_MAX), as pair_rn's; r2 in
-// rr (a pair with r2 = 0 has no key).
+// The sort keys of two pairs, min(mr3 sqrt(d2), FLT_MAX) with pair_rn's operations;
+// r2 in rr (a pair with r2 = 0 has no key).
 __device__ __forceinline__ float2 pair_key2(const Side2 &J, const Side2 &N, float eps2, float2 &rr)
 {
     float2 dx[3];

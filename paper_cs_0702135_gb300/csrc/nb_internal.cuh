@@ -79,10 +79,7 @@ constexpr int kJparIC = 4;     // i per pass, j-parallel kernels
 constexpr int kJparIC1Max = 2;  // DS j-parallel kernel: one i per pass up to this block size
 constexpr int kJparMaxActive = 96;     // automatic mode, DS: j-parallel up to this block size
 constexpr int kJparMaxActive64 = 32;   // automatic mode, FP64
-#ifndef NB_U1
-#define NB_U1 2
-#endif
-constexpr int kIparSmallUnroll = NB_U1;  // its j unrolling (2, 4, 8: 169, 173, 171 us for 1820 active on 65536)
+constexpr int kIparSmallUnroll = 2;  // its j unrolling (2, 4, 8: 169, 173, 171 us for 1820 active on 65536)
 constexpr int kIparSmallR = 1;      // i per thread of the small-block DS i-parallel kernel
 constexpr int kSmallMaxActive = 1024;  // with a forced slice count: small-block kernel considered up to this size
 constexpr int kComp = 7;       // acc xyz, jerk xyz, pot
@@ -413,16 +410,15 @@ struct SumArgs {
     long long words;
     int slots;                      // resident CTAs of the mode's force kernel
 };
-#ifndef NB_FIX_NT
-#define NB_FIX_NT 64
-#endif
-constexpr int kFixNT = NB_FIX_NT;   // fixed point: threads per CTA, one i each (slices: multiples of it)
+constexpr int kFixNT = 64;   // fixed point: threads per CTA, one i each (slices: multiples of it)
 // fixed point: CTAs per SM the registers are held to (8, 9, 10, 12: 13.29, 13.23, 13.22, 13.36 ms
 // on 65536 bodies all active)
 constexpr int kFixCtas = 10;
 // fixed point: blocks of at least an eighth of the slots in i-blocks plan as if there were this
 // many times the slots, so that the items are short against the launch (1, 2, 4: 13.45, 13.45,
-// 13.29 ms); smaller blocks have too few j a slice for it
+// 13.29 ms); smaller blocks have too few j a slice for it (with and without, ms on 65536
+// bodies: 12288 active 2.55 and 2.59, 8192 1.75 and 1.79, 4096 0.90 and 0.93, 1820 0.48 and
+// 0.45: the two meet somewhat below the line)
 constexpr int kFixWaves = 4;
 constexpr int kSeqNT = 640;         // FP32 index order: threads per CTA
 constexpr int kSortNT = 256;        // FP32 sorted: one CTA per i
@@ -432,7 +428,7 @@ constexpr int kChunk = 2048, kChunks = 255;   // items aimed at in a chunk, and 
 // FP32 sorted: 8-byte words of scratch of a CTA (n keyed items; twice that where
 // every block takes the sort of all items, which moves them between two
 // arrays), and the CTAs.  All that fit the SMs (1820 active on 65536 bodies:
-// 5.3 ms with four an SM, 18.6 ms with a single larger one) unless their scratch is
+// 5.1 ms with four an SM, 18.6 ms with a single larger one) unless their scratch is
 // more than a 32nd of the free memory, or 4 GiB: then as many as 16 n bytes an SM
 // hold, which is what one CTA an SM with two arrays takes.
 struct SortScratch {
@@ -684,7 +680,6 @@ void launch_check_input(const double *p, long long cnt, bool nonneg, int *err, c
 
 // k_adjoint.cu
 int vjp_slots(int precision, int sms);
-int vjp_tile();
 int launch_force_vjp(const VjpArgs &va, int precision, bool softened, bool combine, int *slices,
                      cudaStream_t st);
 void launch_shared_step(const SharedStep &q, cudaStream_t st);
