@@ -379,7 +379,7 @@ __device__ __forceinline__ AxisStep correct_axis(double x, double v, double a, d
 }
 
 // The same for any step and any values.
-static __device__ __noinline__ AxisStep correct_axis_any(double x, double v, double a, double k, double ap, double kp,
+__device__ __forceinline__ AxisStep correct_axis_any(double x, double v, double a, double k, double ap, double kp,
                                                   long long ticks)
 {
     AxisStep r;
@@ -404,7 +404,7 @@ static __device__ __noinline__ AxisStep correct_axis_any(double x, double v, dou
 // Where correct_axis was bad: an axis at rest (a system in a plane) moves nothing, the
 // sums of its zeros being +0; else the general form.  128 bodies in a plane, graph
 // run: 27.7 us a step, 32.9 with the general form after the other, 31.7 with it alone.
-__device__ __forceinline__ AxisStep correct_axis_rest(double x, double v, double a, double k, double ap, double kp,
+static __device__ __noinline__ AxisStep correct_axis_rest(double x, double v, double a, double k, double ap, double kp,
                                                       long long ticks)
 {
     const long long any = __double_as_longlong(v) | __double_as_longlong(a) | __double_as_longlong(k) |
