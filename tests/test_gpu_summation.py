@@ -385,3 +385,26 @@ def test_sorted_in_the_scratch_bit_exact(nb):
     few = np.concatenate([idx[:6], idx[-6:]])
     ref = oracle.force_summed(m, x, v, EPS, few, mode=oracle.SUM_FP32_SORTED, nthreads=8)
     _assert_same([np.concatenate([g[:6], g[-6:]]) for g in got], ref, "scratch")
+
+
+@pytest.mark.parametrize("case", ["far_out", "far_out_close_pair", "wide_and_crowded"])
+def test_sorted_overfull_bins_bit_exact(nb, case):
+    # overfull bins of 1/32 octave: one distance for nearly all (finer bins over a
+    # range of one bin), the same beside a close neighbour (a range of many bins),
+    # and equal keys beside keys over more octaves than finer bins can take
+    rng = np.random.RandomState(12)
+    n = 9000
+    m = np.full(n, 1.0 / n)
+    x, v = rng.normal(size=(n, 3)) * 1e-3, rng.normal(size=(n, 3))
+    x[0] = [10.0, 0.0, 0.0]
+    if case == "far_out_close_pair":
+        x[1] = x[0] + [1e-3, 0.0, 0.0]
+        x[2] = [0.0, 1e3, 0.0]
+    elif case == "wide_and_crowded":
+        x[3:4000] = [1.0, 2.0, 3.0]
+        x[4000:] *= 10.0 ** rng.uniform(-3, 16, (n - 4000, 1))
+        m[4000:] *= 10.0 ** rng.uniform(-8, 0, n - 4000)
+    idx = np.array([0, 1, 2, 5000], dtype=np.int32)
+    got = _gpu_force(nb, m, x, v, EPS, idx, nb.NB_SUM_FP32_SORTED, no_force=True)
+    ref = oracle.force_summed(m, x, v, EPS, idx, mode=oracle.SUM_FP32_SORTED, nthreads=8)
+    _assert_same(got, ref, "sorted %s" % case)
